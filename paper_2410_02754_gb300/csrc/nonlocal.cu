@@ -5,8 +5,9 @@
 // done as three batched small contractions on the atom-support node lists:
 //   C   = P_a^H X        (per atom: npj x 2 x nvec, reduction over the support)
 //   C'  = Delta_a C      (2npj x 2npj times 2npj x nvec)
-//   Y  += P_a C'         (node-centric: every support node sums its atoms' terms,
-//                         a plain read-modify-write of Y, no atomics)
+//   Y  += P_a C'         (FP64: atom by atom with atomics; deterministic mode and the
+//                         FP32 SIMT engine: node-centric, every support node sums its
+//                         atoms' terms, a plain read-modify-write of Y)
 // P_a is the node-based projector table (one row per distinct free node of the
 // support, so nodes shared by several support cells are stored once).
 #include <algorithm>
@@ -32,77 +33,182 @@ __device__ __forceinline__ void catomic(double2* p, double2 v) {
 }
 
 constexpr int kStage = 64;      // support nodes staged in shared memory at a time
-constexpr int kCols = 128;      // threads (columns) per block
+constexpr int kCols = 128;      // threads per block
 
-// C[(c_off + 2chi + s) * nvec + v] += sum_j conj(P[j][chi]) X[node_j][s][v]
-template <typename T, int MAXPJ>
+// One block of the projection and of the atom-major expansion: kCols threads = CT
+// columns (a column is one spin of one vector) x NG node groups, over rows [j0, j0 + cnt)
+// of one atom's support.  Both kernels are bound by the FP64 pipe (about 2 FMAs per clock
+// and SM: 4 npj per column and node against one 16-byte load of X), so what matters is
+// that every lane has a column and every SM several blocks: with few columns the lanes go
+// to further nodes, and the grid splits a 1024-node chunk into nsub parts when chunks x
+// column tiles do not fill the SMs.  P rows are staged with an odd row stride, so the NG
+// rows a warp reads at once sit in distinct bank groups.  Measured on one GB300: the FP64
+// pipe is 85% busy in both; projection + expansion on 6 atoms x 18 projectors in 6^3 cells
+// at p = 6 with 64 vectors 20.0 -> 6.6 ms, on 24 atoms in 16^3 cells with one vector
+// 10.5 -> 0.6 ms (before: one chunk per block with all lanes as columns, and an expansion
+// that walked each shared node's incidence list).
+struct NlTile {
+  int atom, npj, j0, cnt, noff;
+  __device__ __forceinline__ NlTile(const int4* chunks, const int* atom_npj, int nsub) {
+    const int4 ch = chunks[blockIdx.x];    // (atom, first position, count, node offset of atom)
+    const int per = (ch.z + nsub - 1) / nsub;
+    const int o = min(ch.z, (int)blockIdx.z * per);
+    atom = ch.x;
+    npj = atom_npj[atom];
+    j0 = ch.y + o;
+    cnt = min(per, ch.z - o);
+    noff = ch.w;
+  }
+};
+
+// C[(c_off + 2chi + s) * nvec + v] += sum_j conj(P[j][chi]) X[node_j][s][v]: each thread
+// sums its nodes in registers, then the NG groups of a column are added by shuffles and
+// through shared memory in a fixed order, and one thread per (chi, column) adds the
+// block's sum to C (or stores it to Cpart, deterministic mode).
+template <typename T, int MAXPJ, int CT>
 __global__ void __launch_bounds__(kCols)
-nl_project(const cplx<T>* __restrict__ X, int ldx, int nvec, const int4* __restrict__ chunks,
-           const long long* __restrict__ nodes, const cplx<T>* __restrict__ P,
-           const int* __restrict__ atom_npj, const int* __restrict__ atom_pv_off,
-           const int* __restrict__ atom_c_off, cplx<T>* __restrict__ Cbuf, long long M,
-           cplx<T>* __restrict__ Cpart) {
+nl_project(const cplx<T>* __restrict__ X, int ldx, int nvec, int nsub,
+           const int4* __restrict__ chunks, const long long* __restrict__ nodes,
+           const cplx<T>* __restrict__ P, const int* __restrict__ atom_npj,
+           const int* __restrict__ atom_pv_off, const int* __restrict__ atom_c_off,
+           cplx<T>* __restrict__ Cbuf, long long M, cplx<T>* __restrict__ Cpart) {
   using C = cplx<T>;
-  __shared__ C Ps[kStage][MAXPJ];
+  constexpr int NG = kCols / CT, RS = MAXPJ | 1, NW = kCols / 32, RC = 8;
+  constexpr int NPS = kStage * RS, NRED = NW * CT * RC;
+  __shared__ C sh[NPS > NRED ? NPS : NRED];   // staged P rows, then the partial sums
   __shared__ long long Ns[kStage];
-  const int4 ch = chunks[blockIdx.x];      // (atom, first position, count, node offset of atom)
-  const int atom = ch.x, j0 = ch.y, cnt = ch.z, noff = ch.w;
-  const int npj = atom_npj[atom];
-  const C* Pa = P + atom_pv_off[atom];
-  const int col = blockIdx.y * kCols + threadIdx.x;
+  const NlTile t(chunks, atom_npj, nsub);
+  const C* Pa = P + atom_pv_off[t.atom];
+  const int lc = threadIdx.x % CT, grp = threadIdx.x / CT;
+  const int col = blockIdx.y * CT + lc;
   const bool ok = col < 2 * nvec;
   const int s = ok ? col / nvec : 0, v = ok ? col % nvec : 0;
   C acc[MAXPJ];
 #pragma unroll
   for (int c = 0; c < MAXPJ; ++c) acc[c] = cmake<C>(0, 0);
-  for (int jb = 0; jb < cnt; jb += kStage) {
-    const int nb = min(kStage, cnt - jb);
-    for (int t = threadIdx.x; t < nb * npj; t += kCols) {
-      const int jj = t / npj, c = t % npj;
-      Ps[jj][c] = Pa[(size_t)(j0 + jb + jj) * npj + c];
+  for (int jb = 0; jb < t.cnt; jb += kStage) {
+    const int nb = min(kStage, t.cnt - jb);
+    for (int i = threadIdx.x; i < nb * t.npj; i += kCols) {
+      const int jj = i / t.npj, c = i % t.npj;
+      sh[jj * RS + c] = Pa[(size_t)(t.j0 + jb + jj) * t.npj + c];
     }
-    for (int t = threadIdx.x; t < nb; t += kCols) Ns[t] = nodes[noff + j0 + jb + t];
+    for (int i = threadIdx.x; i < nb; i += kCols) Ns[i] = nodes[t.noff + t.j0 + jb + i];
     __syncthreads();
     if (ok) {
-      for (int t = 0; t < nb; t += 4) {
+      for (int i = grp; i < nb; i += 4 * NG) {
         C x[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u)
-          x[u] = (t + u < nb && GBC_IN_RANGE(GBC_SITE_NL_NODE, Ns[t + u], M))
-                     ? X[(Ns[t + u] * 2 + s) * ldx + v] : cmake<C>(0, 0);
+        for (int u = 0; u < 4; ++u) {
+          const int jj = i + u * NG;
+          x[u] = (jj < nb && GBC_IN_RANGE(GBC_SITE_NL_NODE, Ns[jj], M))
+                     ? X[(Ns[jj] * 2 + s) * ldx + v] : cmake<C>(0, 0);
+        }
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-          if (t + u >= nb) break;
+          const int jj = i + u * NG;
+          if (jj >= nb) break;
 #pragma unroll
           for (int c = 0; c < MAXPJ; ++c)
-            if (c < npj) cmac_conj(acc[c], Ps[t + u][c], x[u]);
+            if (c < t.npj) cmac_conj(acc[c], sh[jj * RS + c], x[u]);
         }
       }
     }
     __syncthreads();
   }
-  if (ok && Cpart) {   // this chunk's sums, rows 2chi + s (k_nl_chunk_sum adds them in order)
+  // add the node groups of each column: lanes of a warp, then the warps, RC projectors
+  // at a time
+  const int r0 = atom_c_off[t.atom];
 #pragma unroll
-    for (int c = 0; c < MAXPJ; ++c)
-      if (c < npj) Cpart[((size_t)blockIdx.x * 2 * MAXPJ + 2 * c + s) * nvec + v] = acc[c];
-  } else if (ok) {
-    const int r0 = atom_c_off[atom];
+  for (int c0 = 0; c0 < MAXPJ; c0 += RC) {
+    if (c0 >= t.npj) break;
 #pragma unroll
-    for (int c = 0; c < MAXPJ; ++c)
-      if (c < npj) catomic(&Cbuf[(size_t)(r0 + 2 * c + s) * nvec + v], acc[c]);
+    for (int c = c0; c < (c0 + RC < MAXPJ ? c0 + RC : MAXPJ); ++c) {
+      C a = acc[c];
+#pragma unroll
+      for (int o = 16; o >= CT; o >>= 1) {
+        a.x += __shfl_xor_sync(0xffffffffu, a.x, o);
+        a.y += __shfl_xor_sync(0xffffffffu, a.y, o);
+      }
+      if ((threadIdx.x & 31) < CT) sh[((threadIdx.x >> 5) * CT + lc) * RC + c - c0] = a;
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < CT * RC; i += kCols) {
+      const int c = c0 + i / CT, gc = blockIdx.y * CT + i % CT;
+      if (c >= t.npj || gc >= 2 * nvec) continue;
+      C a = cmake<C>(0, 0);
+#pragma unroll
+      for (int w = 0; w < NW; ++w) {
+        const C b = sh[(w * CT + i % CT) * RC + c - c0];
+        a.x += b.x;
+        a.y += b.y;
+      }
+      const int row = 2 * c + gc / nvec, gv = gc % nvec;
+      if (Cpart)   // this block's sums (k_nl_chunk_sum adds them in order)
+        Cpart[((size_t)(blockIdx.x * nsub + blockIdx.z) * 2 * MAXPJ + row) * nvec + gv] = a;
+      else
+        catomic(&Cbuf[(size_t)(r0 + row) * nvec + gv], a);
+    }
+    __syncthreads();
   }
 }
 
-// C[(c_off + r) * nvec + v] = sum over the atom's chunks k, in order, of Cpart[k][r][v]
+// Y[node][s][v] += sum_chi P[pos][chi] Cp[2chi+s][v], one atom's rows per block with FP64
+// atomics (the cell apply adds to the same rows the same way): the block's C' columns stay
+// in registers, and a node held by several atoms is updated once per atom instead of
+// walking its incidence list through dependent loads.
+template <int MAXPJ, int CT>
+__global__ void __launch_bounds__(kCols)
+nl_expand_add(double2* __restrict__ Y, int ldx, int nvec, int nsub,
+              const int4* __restrict__ chunks, const long long* __restrict__ nodes,
+              const double2* __restrict__ P, const int* __restrict__ atom_npj,
+              const int* __restrict__ atom_pv_off, const int* __restrict__ atom_c_off,
+              const double2* __restrict__ Cp, long long M) {
+  constexpr int NG = kCols / CT, RS = MAXPJ | 1;
+  __shared__ double2 sh[kStage * RS];
+  __shared__ long long Ns[kStage];
+  const NlTile t(chunks, atom_npj, nsub);
+  const double2* Pa = P + atom_pv_off[t.atom];
+  const int lc = threadIdx.x % CT, grp = threadIdx.x / CT;
+  const int col = blockIdx.y * CT + lc;
+  const bool ok = col < 2 * nvec;
+  const int s = ok ? col / nvec : 0, v = ok ? col % nvec : 0;
+  const double2* Ca = Cp + (size_t)(atom_c_off[t.atom] + s) * nvec + v;
+  double2 cp[MAXPJ];
+#pragma unroll
+  for (int c = 0; c < MAXPJ; ++c)
+    cp[c] = (ok && c < t.npj) ? Ca[(size_t)(2 * c) * nvec] : make_double2(0, 0);
+  for (int jb = 0; jb < t.cnt; jb += kStage) {
+    const int nb = min(kStage, t.cnt - jb);
+    for (int i = threadIdx.x; i < nb * t.npj; i += kCols) {
+      const int jj = i / t.npj, c = i % t.npj;
+      sh[jj * RS + c] = Pa[(size_t)(t.j0 + jb + jj) * t.npj + c];
+    }
+    for (int i = threadIdx.x; i < nb; i += kCols) Ns[i] = nodes[t.noff + t.j0 + jb + i];
+    __syncthreads();
+    if (ok) {
+#pragma unroll 2
+      for (int jj = grp; jj < nb; jj += NG) {
+        double2 a = make_double2(0, 0);
+#pragma unroll
+        for (int c = 0; c < MAXPJ; ++c)
+          if (c < t.npj) cmac(a, sh[jj * RS + c], cp[c]);
+        if (GBC_IN_RANGE(GBC_SITE_NL_NODE, Ns[jj], M)) catomic(&Y[(Ns[jj] * 2 + s) * ldx + v], a);
+      }
+    }
+    __syncthreads();
+  }
+}
+
+// C[(c_off + r) * nvec + v] = sum over the atom's chunk parts k, in order, of Cpart[k][r][v]
 template <typename T, int MAXPJ>
 __global__ void k_nl_chunk_sum(const cplx<T>* __restrict__ Cpart, cplx<T>* __restrict__ Cbuf,
                                const int* __restrict__ chunk_off, const int* __restrict__ atom_npj,
-                               const int* __restrict__ atom_c_off, int nvec) {
+                               const int* __restrict__ atom_c_off, int nvec, int nsub) {
   const int atom = blockIdx.x, r = blockIdx.y;
   const int v = blockIdx.z * blockDim.x + threadIdx.x;
   if (r >= 2 * atom_npj[atom] || v >= nvec) return;
   cplx<T> acc = cmake<cplx<T>>(0, 0);
-  for (int k = chunk_off[atom]; k < chunk_off[atom + 1]; ++k) {
+  for (int k = chunk_off[atom] * nsub; k < chunk_off[atom + 1] * nsub; ++k) {
     const cplx<T> p = Cpart[((size_t)k * 2 * MAXPJ + r) * nvec + v];
     acc.x += p.x;
     acc.y += p.y;
@@ -129,6 +235,7 @@ __global__ void nl_couple(const cplx<T>* __restrict__ Cbuf, cplx<T>* __restrict_
   Cp[base + (size_t)r * nvec] = acc;
 }
 
+// Node-major expansion (deterministic mode, and the overwrite mode of the FP32 SIMT engine):
 // Y[node][s][v] += sum over atoms whose support holds node of sum_chi P[pos][chi] Cp[2chi+s][v].
 // Every distinct support node is owned by the lowest-index atom whose support
 // holds it; the owner's block writes it once (plain read-modify-write, no
@@ -193,29 +300,71 @@ nl_expand(cplx<T>* __restrict__ Y, int ldx, int nvec, const int4* __restrict__ c
   }
 }
 
+// column tile (a power of two, at most a warp) and the parts a chunk is split into: about
+// eight blocks per SM, at least 64 nodes per part
+inline int nl_col_tile(int nvec) {
+  int ct = 2;
+  while (ct < 32 && ct < 2 * nvec) ct *= 2;
+  return ct;
+}
+inline int nl_parts(const ProjDev& pj, int nvec) {
+  const int ct = nl_col_tile(nvec);
+  const long long blocks = (long long)pj.nchunks * ((2 * nvec + ct - 1) / ct);
+  const long long want = (8LL * gbc_sm_count() + blocks - 1) / blocks;
+  return (int)std::max<long long>(1, std::min<long long>(16, want));
+}
+// f(std::integral_constant<int, CT>) for the column tile of nvec vectors
+template <typename F> inline void nl_with_tile(int nvec, F f) {
+  switch (nl_col_tile(nvec)) {
+    case 2: return f(std::integral_constant<int, 2>());
+    case 4: return f(std::integral_constant<int, 4>());
+    case 8: return f(std::integral_constant<int, 8>());
+    case 16: return f(std::integral_constant<int, 16>());
+    default: return f(std::integral_constant<int, 32>());
+  }
+}
+
 template <typename T, int MAXPJ>
 cudaError_t run_project(gbc_ctx* c, const cplx<T>* X, int nvec, int ldx, cplx<T>* Cbuf,
                         cudaStream_t s) {
   const ProjDev& pj = c->proj;
   const cplx<T>* P = std::is_same<T, double>::value ? (const cplx<T>*)pj.d_P64
                                                     : (const cplx<T>*)pj.d_P32;
-  // deterministic mode: per-chunk sums, then each atom's chunks added in order
+  const int nsub = nl_parts(pj, nvec);
+  // deterministic mode: per-part sums, then each atom's parts added in order
   cplx<T>* Cpart = nullptr;
   if (c->deterministic) {
-    if (gbc_ensure_work(c, 11, sizeof(cplx<T>) * pj.nchunks * 2 * MAXPJ * (size_t)nvec) != GBC_OK)
+    if (gbc_ensure_work(c, 11, sizeof(cplx<T>) * pj.nchunks * nsub * 2 * MAXPJ * (size_t)nvec) != GBC_OK)
       return cudaErrorMemoryAllocation;
     Cpart = (cplx<T>*)c->work[11];
   }
-  dim3 grid(pj.nchunks, (2 * nvec + kCols - 1) / kCols);
-  nl_project<T, MAXPJ><<<grid, kCols, 0, s>>>(X, ldx, nvec, pj.d_chunks, pj.d_nodes, P,
-                                              pj.d_atom_npj, pj.d_atom_pv_off, pj.d_atom_c_off,
-                                              Cbuf, c->mesh.M, Cpart);
-  if (!Cpart) return cudaGetLastError();
+  nl_with_tile(nvec, [&](auto ct) {
+    constexpr int CT = decltype(ct)::value;
+    dim3 grid(pj.nchunks, (2 * nvec + CT - 1) / CT, nsub);
+    nl_project<T, MAXPJ, CT><<<grid, kCols, 0, s>>>(X, ldx, nvec, nsub, pj.d_chunks, pj.d_nodes, P,
+                                                    pj.d_atom_npj, pj.d_atom_pv_off,
+                                                    pj.d_atom_c_off, Cbuf, c->mesh.M, Cpart);
+  });
   cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
+  if (!Cpart || e != cudaSuccess) return e;
   dim3 g2(pj.natoms, 2 * pj.max_npj, (nvec + kCols - 1) / kCols);
   k_nl_chunk_sum<T, MAXPJ><<<g2, kCols, 0, s>>>(Cpart, Cbuf, pj.d_chunk_off, pj.d_atom_npj,
-                                                pj.d_atom_c_off, nvec);
+                                                pj.d_atom_c_off, nvec, nsub);
+  return cudaGetLastError();
+}
+
+template <int MAXPJ>
+cudaError_t run_expand_add(const gbc_ctx* c, double2* Y, int nvec, int ldx, const double2* Cp,
+                           cudaStream_t s) {
+  const ProjDev& pj = c->proj;
+  const int nsub = nl_parts(pj, nvec);
+  nl_with_tile(nvec, [&](auto ct) {
+    constexpr int CT = decltype(ct)::value;
+    dim3 grid(pj.nchunks, (2 * nvec + CT - 1) / CT, nsub);
+    nl_expand_add<MAXPJ, CT><<<grid, kCols, 0, s>>>(Y, ldx, nvec, nsub, pj.d_chunks, pj.d_nodes,
+                                                    pj.d_P64, pj.d_atom_npj, pj.d_atom_pv_off,
+                                                    pj.d_atom_c_off, Cp, c->mesh.M);
+  });
   return cudaGetLastError();
 }
 
@@ -240,6 +389,11 @@ cudaError_t launch_nonlocal(gbc_ctx* c, const cplx<T>* X, cplx<T>* Y, int nvec, 
   if (e != cudaSuccess) return e;
   if constexpr (std::is_same<T, float>::value) {
     if (use_tc(c)) return launch_tc_expand(pj, Y, nvec, ldx, Cpbuf, s, overwrite, bpre, c->d_cell_ctr);
+  } else if (!overwrite && !c->deterministic) {
+    if (pj.max_npj <= 4) return run_expand_add<4>(c, Y, nvec, ldx, Cpbuf, s);
+    if (pj.max_npj <= 8) return run_expand_add<8>(c, Y, nvec, ldx, Cpbuf, s);
+    if (pj.max_npj <= 18) return run_expand_add<18>(c, Y, nvec, ldx, Cpbuf, s);
+    return run_expand_add<GBC_MAX_NPJ>(c, Y, nvec, ldx, Cpbuf, s);
   }
   const cplx<T>* P = std::is_same<T, double>::value ? (const cplx<T>*)pj.d_P64
                                                     : (const cplx<T>*)pj.d_P32;
