@@ -357,13 +357,13 @@ gbc_status gbc_tune(gbc_ctx* ctx, int nvec, void* stream);
 /* Vectors per CTA the cell apply of this context uses. */
 gbc_status gbc_get_tile(const gbc_ctx* ctx, int* vectors_per_cta);
 /* Set (overriding the tuner) / read the FP32 cell-apply variant, 0 ..
- * GBC_CELL_VARIANTS - 1: 0 = 2 vectors x 256 threads with registers for 4 CTAs
- * per SM, paired FP32 multiply-adds on (re, im); 1 = the same tile with
+ * GBC_CELL_VARIANTS - 1: 0 = 2 vectors per work item x 256 threads with registers
+ * for 2 CTAs per SM, paired FP32 multiply-adds on (re, im); 1 = the same with
  * registers for 3 CTAs per SM; 2 and 3 = variants 0 and 1 with scalar FP32
- * multiply-adds; 4 = 4 vectors x 512 threads with registers for 2 CTAs per SM,
- * scalar multiply-adds.  (One vector x 128 threads per CTA measured 1.5-2.5x
- * slower at p = 6 and is not compiled.)  gbc_get_cell_variant
- * also returns the variant's vectors and threads per CTA (either pointer may be
+ * multiply-adds; 4 = 4 vectors x 512 threads, one CTA per SM, paired
+ * multiply-adds.  A CTA's threads form independent groups that each work on one
+ * item (one cell, 2 or 4 vectors) at a time.  gbc_get_cell_variant also returns
+ * the variant's vectors per item and threads per CTA (either pointer may be
  * NULL).  GBC_EINVAL for a variant out of range. */
 #define GBC_CELL_VARIANTS 5
 gbc_status gbc_set_cell_variant(gbc_ctx* ctx, int variant);

@@ -4,29 +4,44 @@
 // Paper: Sec. IV.B.2 (extract X^(e) = R^(e) X, cell products, assemble
 // Y = sum_e R^(e)T Y^(e)) for the cell operator of Eq. FEHlocEl plus the k-terms
 // of Eq. FEHloc (per-cell Hermitian form), and Eq. chebfilt for the recurrence.
-// The arithmetic is the sum factorisation of the FP64 kernel (hx_local.cuh):
-// kinetic/k part K = G_x B_y B_z + B_x G_y B_z + B_x B_y G_z, potential part
-// N^T diag(w_q J [(V + |k|^2/2) I + B . sigma]) N, every 1-D operator in even-odd
-// form.  What differs is how it maps to the SM:
 //
-//  * complex values are float2 (re, im) and every real-matrix x complex-vector
-//    product is a paired FP32 multiply-add (one instruction for both parts);
-//  * per vector only three shared buffers: A (the gathered X^(e), n_p^3 nodes),
-//    T2 (n_p^3) and T1 (n_q^3 points), reused in place through the stages
-//      gather  X -> A
-//      Kz      A  -> T1 = B_z X, T2 = G_z X                     (z pencils)
-//      Ky      T1, T2 -> U1 = B_y T1, U2 = G_y T1 + B_y T2      (y pencils, in place)
-//      Kx+Ix   U1, U2, A -> T2 = G_x U1 + B_x U2 (kinetic result),
-//              T1 = N_x X                                       (x pencils, in place)
-//      Iy      T1 -> N_y T1                                     (y pencils, in place)
-//      Iz+W+Tz T1 -> N_z^T W N_z T1 with the 2x2 spin operator W at each point
-//              (z pencils; the two spins of a pencil on neighbouring lanes)
-//      Ty      T1 -> N_y^T T1                                   (y pencils, in place)
-//      Tx+out  T1 -> N_x^T T1 + T2, assembled                   (x pencils)
-//  * VB vectors per CTA, the vector index fastest across threads, so the gather
-//    and the scatter touch VB consecutive complex values of each node row; the
-//    gather of the next work item is issued (cp.async) as soon as A is free, so
-//    its latency hides behind the last four stages of the current item.
+// Algorithm: with N' = N diag(sqrt(w_q)) (nodes x Gauss points, so that the 1-D mass is
+// (h/2) N' N'^T) and the 1-D kinetic / k operators G_d,
+//   a  = N'_x^T X,  t1 = B_x X,  t2 = G_x X                      x pencils (n_p^2)
+//   u  = N'_y^T a;  c  = G_y t1 + B_y t2                          y pencils (n_q n_p; n_p^2)
+//   w  = N'_z F N'_z^T u + G'_z u;  k = B_z c                     z pencils (n_q^2; n_p^2)
+//   Y^(e) = N'_x N'_y w + k                                       y, then x pencils
+// where F = J [(V + |k|^2/2) I + B . sigma] at the Gauss points and G'_z = (h_x h_y / 4) G_z:
+// the z part of the kinetic term rides on the interpolated field (N'_x N'_y of G'_z u is
+// B_x B_y G_z X), so five stages and five kinetic 1-D products do what the separate kinetic
+// and potential passes of the dense form need seven for.  Every 1-D product is in even-odd
+// form, the products of one input sharing its even and odd parts and the products of one
+// output one accumulator.
+//
+// Mapping:
+//  * a thread owns a pencil of one vector, both spins: shared memory holds (up, down) of a
+//    point side by side, so every access is 16 bytes, the spin operator needs no exchange
+//    between lanes, and a table entry is used four times per load; complex values are
+//    float2 and a product is one paired multiply-add (or two scalar ones; both compiled);
+//  * per vector three buffers used in place: A (gathered X^(e), then t1), T2 (t2, c, k) and
+//    T1 (a, u, w);
+//  * the gather of the next work item (cp.async) starts when A is free, after the second
+//    stage, and hides behind the other three;
+//  * a CTA is several independent groups of threads, each with its own work items, buffers
+//    and named barrier, so one group's arithmetic fills the other's barrier waits at 128
+//    registers a thread; at p = 5 and 6 a warp owns whole z planes of the cell, which leaves
+//    two group barriers an item, both around the z stage; a helper warp takes the items from
+//    the work counter two ahead, so neither the atomic's latency nor the index divisions are
+//    waited for.
+//
+// Bounds at p = 6, k != 0 per cell and vector: 123,000 FP32 lane operations (960 cycles of
+// an SM's 128 lanes) and 103 KB of shared-memory traffic (806 cycles at 128 bytes).  Measured
+// on one GB300, 16^3 cells, p = 6, 256 vectors, k != 0, recurrence mode: 11.30 -> 7.62 ms a
+// launch (2290 cycles; the L1 data pipe is 73% busy, issue 54%), from 12.3 -> 6.6 thousand
+// warp instructions per cell and vector pair.  The steps: five stages and 16-byte two-spin
+// pencils 9.29, index work once per pencil 9.07, items decoded once and fields staged 8.34,
+// planes owned by warps 7.62.  Other sizes: 12^3 cells, p = 5, 96 vectors 1144 -> 815 us;
+// p = 4 812 -> 460; 10^3 cells, p = 3, 128 vectors 460 -> 212; p = 7, 64 vectors 1167 -> 1048.
 //
 // Assembly modes (per system):
 //  * accumulate: Y += H^loc X with FP32 atomics on every node;
@@ -59,17 +74,17 @@ template <int NP, int NQ, bool PACKED> struct CellTables {
   template <int NO, int NI>
   using M = typename std::conditional<PACKED, EO2<NO, NI>, EO<float, NO, NI>>::type;
   M<NP, NP> B[3];    // 1-D Gauss mass
-  M<NP, NP> Gr[3];   // 1/2 A_d
-  M<NP, NP> Gi[3];   // -1/2 k_d (C^ - C^T)
-  M<NQ, NP> Ni;      // interpolation to the Gauss points
-  M<NP, NQ> Nt;      // testing back to the nodes
+  M<NP, NP> Gr[3];   // 1/2 A_d (z: times h_x h_y / 4)
+  M<NP, NP> Gi[3];   // -1/2 k_d (C^ - C^T) (z: times h_x h_y / 4)
+  M<NQ, NP> Ni;      // N'^T: interpolation to the Gauss points times sqrt(w_q)
+  M<NP, NQ> Nt;      // N'
 };
 
 // One system of a launch.
 struct CellSys {
   const float2* X;      // block applied to
   float2* Y;            // accumulator
-  const float* fields;  // [E][NQ^3][4] w_q J (V + |k|^2/2), w_q J B_x, B_y, B_z
+  const float* fields;  // [E][NQ^3][4] J (V + |k|^2/2), J B_x, J B_y, J B_z
   float2* Xout;         // recurrence mode: X_{k+1} (may alias Xprev)
   const float2* Xprev;  // recurrence mode: X_{k-1}, or null on the first step
   const float* invmd;   // recurrence mode: 1 / M_D per node
@@ -103,405 +118,559 @@ __device__ __forceinline__ void cp_async8(void* dst, const void* src, int src_by
                "l"(src), "r"(src_bytes)
                : "memory");
 }
+// 16-byte asynchronous global -> shared copy (both addresses 16-byte aligned)
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)),
+               "l"(src)
+               : "memory");
+}
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-// y = M x for a centro-symmetric (S = 1) or centro-antisymmetric (S = -1) M
-template <int S, int NO, int NI>
-__device__ __forceinline__ void eo2_apply(const EO2<NO, NI>& M, const float2 (&x)[NI],
-                                          float2 (&y)[NO]) {
-  constexpr int HI = NI / 2, HO = (NO + 1) / 2;
-  static_assert(HI >= 1, "NI >= 2");
-  float2 e[HI], o[HI];
+// products and sums of complex values held as float2: paired instructions for a duplicated
+// table entry (float2), scalar ones for a plain entry
+__device__ __forceinline__ float2 m_mul(float2 m, float2 x) { return p_mul(m, x); }
+__device__ __forceinline__ float2 m_fma(float2 m, float2 x, float2 a) { return p_fma(m, x, a); }
+__device__ __forceinline__ float2 m_mul(float m, float2 x) { return make_float2(m * x.x, m * x.y); }
+__device__ __forceinline__ float2 m_fma(float m, float2 x, float2 a) {
+  return make_float2(fmaf(m, x.x, a.x), fmaf(m, x.y, a.y));
+}
+template <bool PACKED> __device__ __forceinline__ float2 c_add(float2 a, float2 b) {
+  return PACKED ? p_add(a, b) : make_float2(a.x + b.x, a.y + b.y);
+}
+template <bool PACKED> __device__ __forceinline__ float2 c_sub(float2 a, float2 b) {
+  return PACKED ? p_sub(a, b) : make_float2(a.x - b.x, a.y - b.y);
+}
+__device__ __forceinline__ float2 lo2(float4 v) { return make_float2(v.x, v.y); }
+__device__ __forceinline__ float2 hi2(float4 v) { return make_float2(v.z, v.w); }
+__device__ __forceinline__ float4 cat2(float2 a, float2 b) { return make_float4(a.x, a.y, b.x, b.y); }
+
+// even and odd parts (and the middle point of an odd count) of a pencil of NI points, both
+// spins: e_j = x_j + x_{NI-1-j}, o_j = x_j - x_{NI-1-j}
+template <int NI> struct Parts {
+  static constexpr int HI = NI / 2;
+  float2 e[2][HI], o[2][HI], m[2];
+};
+template <bool PACKED, int NI>
+__device__ __forceinline__ void set_part(Parts<NI>& s, int j, float4 a, float4 b) {
+  s.e[0][j] = c_add<PACKED>(lo2(a), lo2(b));
+  s.o[0][j] = c_sub<PACKED>(lo2(a), lo2(b));
+  s.e[1][j] = c_add<PACKED>(hi2(a), hi2(b));
+  s.o[1][j] = c_sub<PACKED>(hi2(a), hi2(b));
+}
+template <bool PACKED, int NI, typename F>
+__device__ __forceinline__ void load_parts(Parts<NI>& s, F ld) {
 #pragma unroll
-  for (int j = 0; j < HI; ++j) {
-    e[j] = p_add(x[j], x[NI - 1 - j]);
-    o[j] = p_sub(x[j], x[NI - 1 - j]);
+  for (int j = 0; j < NI / 2; ++j) set_part<PACKED>(s, j, ld(j), ld(NI - 1 - j));
+  if (NI & 1) {
+    const float4 c = ld(NI / 2);
+    s.m[0] = lo2(c);
+    s.m[1] = hi2(c);
   }
+}
+
+// rows i and NO-1-i of a product, as even and odd accumulators of both spins:
+// y_i = ae + ao, y_{NO-1-i} = ae - ao (the middle row of an odd NO is ae alone)
+struct Acc { float2 e[2], o[2]; };
+// FIRST: a = M x, else a += M x, for a centro-symmetric M
+template <bool FIRST, int NO, int NI, typename MT>
+__device__ __forceinline__ void row_sym(const MT& M, int i, const Parts<NI>& s, Acc& a) {
+  constexpr int HI = NI / 2;
 #pragma unroll
-  for (int i = 0; i < HO; ++i) {
-    float2 ae = p_mul(M.E[i][0], e[0]);
-    float2 ao = p_mul(M.O[i][0], o[0]);
+  for (int j = 0; j < HI; ++j)
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      a.e[q] = (FIRST && j == 0) ? m_mul(M.E[i][j], s.e[q][j]) : m_fma(M.E[i][j], s.e[q][j], a.e[q]);
+      if (NO - 1 - i != i)
+        a.o[q] = (FIRST && j == 0) ? m_mul(M.O[i][j], s.o[q][j]) : m_fma(M.O[i][j], s.o[q][j], a.o[q]);
+    }
+  if (NI & 1) {
+#pragma unroll
+    for (int q = 0; q < 2; ++q) a.e[q] = m_fma(M.Mid[i], s.m[q], a.e[q]);
+  }
+}
+// a += i M x for a centro-antisymmetric M (its odd chain feeds the even accumulator and the
+// even chain the odd one)
+template <int NO, int NI, typename MT>
+__device__ __forceinline__ void row_anti(const MT& M, int i, const Parts<NI>& s, Acc& a) {
+  constexpr int HI = NI / 2;
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    float2 te = m_mul(M.E[i][0], s.e[q][0]), to = m_mul(M.O[i][0], s.o[q][0]);
 #pragma unroll
     for (int j = 1; j < HI; ++j) {
-      ae = p_fma(M.E[i][j], e[j], ae);
-      ao = p_fma(M.O[i][j], o[j], ao);
+      te = m_fma(M.E[i][j], s.e[q][j], te);
+      to = m_fma(M.O[i][j], s.o[q][j], to);
     }
-    if (NI & 1) ae = p_fma(M.Mid[i], x[HI], ae);
-    y[i] = p_add(ae, ao);
-    if (NO - 1 - i != i) y[NO - 1 - i] = S > 0 ? p_sub(ae, ao) : p_sub(ao, ae);
+    if (NI & 1) te = m_fma(M.Mid[i], s.m[q], te);
+    a.e[q].x -= to.y;
+    a.e[q].y += to.x;
+    if (NO - 1 - i != i) {
+      a.o[q].x -= te.y;
+      a.o[q].y += te.x;
+    }
+  }
+}
+// st(row, both spins) for the two rows of a
+template <bool PACKED, int NO, typename F>
+__device__ __forceinline__ void put_rows(int i, const Acc& a, F st) {
+  if (NO - 1 - i == i) {
+    st(i, cat2(a.e[0], a.e[1]));
+  } else {
+    st(i, cat2(c_add<PACKED>(a.e[0], a.o[0]), c_add<PACKED>(a.e[1], a.o[1])));
+    st(NO - 1 - i, cat2(c_sub<PACKED>(a.e[0], a.o[0]), c_sub<PACKED>(a.e[1], a.o[1])));
   }
 }
 
-// the same with plain FP32 entries: two scalar multiply-adds per complex product
-template <int S, int NO, int NI>
-__device__ __forceinline__ void eo2_apply(const EO<float, NO, NI>& M, const float2 (&x)[NI],
-                                          float2 (&y)[NO]) {
-  constexpr int HI = NI / 2, HO = (NO + 1) / 2;
-  static_assert(HI >= 1, "NI >= 2");
-  float2 e[HI], o[HI];
-#pragma unroll
-  for (int j = 0; j < HI; ++j) {
-    e[j] = make_float2(x[j].x + x[NI - 1 - j].x, x[j].y + x[NI - 1 - j].y);
-    o[j] = make_float2(x[j].x - x[NI - 1 - j].x, x[j].y - x[NI - 1 - j].y);
-  }
-#pragma unroll
-  for (int i = 0; i < HO; ++i) {
-    float er = M.E[i][0] * e[0].x, ei = M.E[i][0] * e[0].y;
-    float orr = M.O[i][0] * o[0].x, oi = M.O[i][0] * o[0].y;
-#pragma unroll
-    for (int j = 1; j < HI; ++j) {
-      er = fmaf(M.E[i][j], e[j].x, er);
-      ei = fmaf(M.E[i][j], e[j].y, ei);
-      orr = fmaf(M.O[i][j], o[j].x, orr);
-      oi = fmaf(M.O[i][j], o[j].y, oi);
-    }
-    if (NI & 1) {
-      er = fmaf(M.Mid[i], x[HI].x, er);
-      ei = fmaf(M.Mid[i], x[HI].y, ei);
-    }
-    y[i] = make_float2(er + orr, ei + oi);
-    if (NO - 1 - i != i)
-      y[NO - 1 - i] = S > 0 ? make_float2(er - orr, ei - oi) : make_float2(orr - er, oi - ei);
-  }
-}
-
-// y = (Gr + i Gi) x, Gr symmetric, Gi antisymmetric (Gi only at k != 0)
-template <bool KPT, int N, typename MT>
-__device__ __forceinline__ void g2_apply(const MT& Gr, const MT& Gi, const float2 (&x)[N],
-                                         float2 (&y)[N]) {
-  eo2_apply<1>(Gr, x, y);
-  if (KPT) {
-    float2 t[N];
-    eo2_apply<-1>(Gi, x, t);
-#pragma unroll
-    for (int i = 0; i < N; ++i) y[i] = make_float2(y[i].x - t[i].y, y[i].y + t[i].x);
-  }
-}
-
-// Point strides (y, z) of the n_p^3 buffers (A, T2) and of the n_q^3 buffer (T1).
-// With the unit order of the stages (vector fastest, then spin, then pencil) a
-// half-warp touches 4 pencils x 2 spins x 2 vectors; these strides put those 16
-// 8-byte accesses in 16 distinct bank pairs for every stage's pencil direction
-// (found by enumerating strides against a model of the 64-bit shared-memory
-// wavefronts); the n_p^3 buffers are dense for odd n_p.
+// Point strides (y, z) of the n_p^3 buffers (A, T2) and of T1 (up to n_q x n_q x n_p
+// points).  A quarter-warp's 16-byte accesses (VB vectors, then neighbouring pencils) fall
+// in the 8 distinct bank groups when neighbouring pencils are an odd number of points
+// apart, which these strides give in every stage's pencil direction, and the vectors
+// start 8 / VB groups apart (cell_vpoints).
 template <int NP> struct CellLayout;
 template <> struct CellLayout<3> { static constexpr int AY = 3, AZ = 9, QY = 5, QZ = 23; };
 template <> struct CellLayout<4> { static constexpr int AY = 5, AZ = 21, QY = 5, QZ = 25; };
-template <> struct CellLayout<5> { static constexpr int AY = 5, AZ = 25, QY = 9, QZ = 57; };
+template <> struct CellLayout<5> { static constexpr int AY = 5, AZ = 25, QY = 7, QZ = 43; };
 template <> struct CellLayout<6> { static constexpr int AY = 7, AZ = 43, QY = 7, QZ = 51; };
-template <> struct CellLayout<7> { static constexpr int AY = 7, AZ = 49, QY = 9, QZ = 75; };
-template <> struct CellLayout<8> { static constexpr int AY = 9, AZ = 73, QY = 9, QZ = 81; };
+template <> struct CellLayout<7> { static constexpr int AY = 7, AZ = 49, QY = 9, QZ = 73; };
+template <> struct CellLayout<8> { static constexpr int AY = 9, AZ = 72, QY = 9, QZ = 81; };
 template <int NP> __host__ __device__ constexpr int cell_bufa() {   // points of A / T2
   return (NP - 1) * (1 + CellLayout<NP>::AY + CellLayout<NP>::AZ) + 1;
 }
 template <int NP> __host__ __device__ constexpr int cell_bufq() {   // points of T1
-  return NP * (1 + CellLayout<NP>::QY + CellLayout<NP>::QZ) + 1;
+  return NP * (1 + CellLayout<NP>::QY) + (NP - 1) * CellLayout<NP>::QZ + 1;
 }
-
-template <int NP, int NQ, int VB> __host__ __device__ constexpr int cell_vstride() {
-  // float2 elements per vector: [A | T2 | T1], two spins per point, padded so that the
-  // VB vectors of a lane group start in distinct quarters (VB = 4: 4 mod 16) or halves
-  // (VB = 2: 8 mod 16) of a 128-byte bank row (the same wavefront model as the strides)
+template <int NP, int VB> __host__ __device__ constexpr int cell_vpoints() {
+  // points per vector: [A | T2 | T1], padded to 8 / VB mod 8
   static_assert(VB == 2 || VB == 4, "VB");
-  constexpr int n = 2 * (2 * cell_bufa<NP>() + cell_bufq<NP>());
-  constexpr int r = VB == 4 ? 4 : 8;
-  return n + ((16 + r - n % 16) % 16);
+  constexpr int n = 2 * cell_bufa<NP>() + cell_bufq<NP>(), r = 8 / VB;
+  return n + ((8 + r - n % 8) % 8);
 }
-// vector buffers, then the node-offset tables of the current and the next work item
-template <int NP, int NQ, int VB> constexpr size_t hx_cell_smem() {
-  return sizeof(float2) * (size_t)VB * cell_vstride<NP, NQ, VB>() + sizeof(int) * 2 * 3 * NP + 16;
+// Threads of a group: about one per pencil of a vector's x stage.  At p = 3 and 4 small
+// groups are worth more than full rounds (12^3 cells, p = 4, 96 vectors: 446 us a launch at
+// 128 threads, 642 at 256).
+template <int NP, int VB> __host__ __device__ constexpr int cell_group_threads() {
+  constexpr int g4[9] = {0, 0, 0, 64, 128, 128, 256, 256, 256};
+  constexpr int g2[9] = {0, 0, 0, 32, 64, 64, 128, 128, 128};
+  return VB == 4 ? g4[NP] : g2[NP];
+}
+// Whether each warp owns whole z planes of a cell (see cell_body): where a plane's pencils
+// fill a warp and a warp is left over (p = 6, 4 vectors: 28 to 32 lanes, 8.34 -> 7.62 ms a
+// launch on 16^3 cells, 256 vectors; p = 5: 872 -> 815 us on 12^3 cells, 96 vectors).  At
+// p = 7 a plane has 36 pencils a vector quad and every warp a plane (1048 -> 1090 us), at
+// p <= 4 it leaves lanes idle (460 -> 575 us).
+template <int NP> __host__ __device__ constexpr bool cell_planes() { return NP == 6 || NP == 7; }
+// a work item: system, cell, first vector; e < 0: none
+struct alignas(16) CellItem { int q, e, v0, pad; };
+constexpr int kCellSlots = 4;    // item records and offset tables in flight
+// one group: vector buffers, the cell's fields (FS), the item records and node offsets
+template <int NP, int VB, bool FS> __host__ __device__ constexpr size_t cell_group_smem() {
+  return sizeof(float4) * ((size_t)VB * cell_vpoints<NP, VB>() +
+                           (FS ? (NP + 1) * (NP + 1) * (NP + 1) : 0)) +
+         kCellSlots * (sizeof(CellItem) + sizeof(int) * 3 * 8);
+}
+// 1 / M_D of a cell's interior nodes: one table per CTA
+template <int NP> __host__ __device__ constexpr size_t cell_mass_smem() {
+  return (sizeof(float) * (NP - 2) * (NP - 2) * (NP - 2) + 15) / 16 * 16;
+}
+// the fields are staged in shared memory where MINB CTAs per SM still fit with them
+template <int NP, int VB, int NT, int MINB> __host__ __device__ constexpr bool cell_stage_fields() {
+  return MINB * (NT / cell_group_threads<NP, VB>() * cell_group_smem<NP, VB, true>() +
+                 cell_mass_smem<NP>() + 1024) <= 228 * 1024;
+}
+template <int NP, int VB, int NT, int MINB> __host__ __device__ constexpr size_t cell_smem() {
+  return NT / cell_group_threads<NP, VB>() * cell_group_smem<NP, VB, cell_stage_fields<NP, VB, NT, MINB>()>() +
+         cell_mass_smem<NP>();
 }
 constexpr int kNoNode = -(1 << 29);   // offset of a direction with no free node (Dirichlet face)
 
 // The work items [0, nitems) of the systems sys[0 .. nsys) (item0 ascending), taken
-// from the counter *ctr (zero at launch) one atomic increment at a time, so CTAs
+// from the counter *ctr (zero at launch) one atomic increment at a time, so groups
 // that finish early take more and the items in flight stay close to each other in
-// the order (cell-major, vector chunks of a cell adjacent).
-template <int NP, int NQ, bool KPT, int VB, int NT, bool PACKED>
+// the order (cell-major, vector chunks of a cell adjacent).  GT: threads of a group.
+template <int NP, int NQ, bool KPT, int VB, int GT, bool PACKED, bool FS>
 __device__ __forceinline__ void cell_body(const CellSys* __restrict__ sys, int nsys,
                                           long long nitems, const CellTables<NP, NQ, PACKED>& tb,
                                           unsigned long long* __restrict__ ctr) {
   constexpr int BA = cell_bufa<NP>();
   constexpr int NQ3 = NQ * NQ * NQ;
-  constexpr int VS = cell_vstride<NP, NQ, VB>();
+  constexpr int VS = cell_vpoints<NP, VB>();
+  constexpr int HP = (NP + 1) / 2, HQ = (NQ + 1) / 2;   // row pairs
   using L = CellLayout<NP>;
-  extern __shared__ __align__(16) float2 sm[];
-  // spin s of point pidx of vector v: Buf(v)[2 * pidx + s]
+  extern __shared__ __align__(16) unsigned char sm_raw[];
+  const int group = threadIdx.x / GT;
+  float4* sm = reinterpret_cast<float4*>(sm_raw + group * cell_group_smem<NP, VB, FS>());
+  // both spins of point pidx of vector v: Buf(v)[pidx]
   auto Ab = [&](int v) { return sm + v * VS; };
-  auto T2b = [&](int v) { return sm + v * VS + 2 * BA; };
-  auto T1b = [&](int v) { return sm + v * VS + 4 * BA; };
+  auto T2b = [&](int v) { return sm + v * VS + BA; };
+  auto T1b = [&](int v) { return sm + v * VS + 2 * BA; };
   auto pa = [](int x, int y, int z) { return x + y * L::AY + z * L::AZ; };
   auto pq = [](int x, int y, int z) { return x + y * L::QY + z * L::QZ; };
-  const int tid = threadIdx.x;
-  auto locate = [&](long long it) {
-    int q = 0;
-    if (nsys == 1) return q;   // one system: skip the scan over the descriptor slots
+  // odd groups number their warps backwards: a stage's last, partly filled round then falls
+  // on other schedulers than the even groups'
+  const int tid0 = threadIdx.x % GT;
+  const int tid = (group & 1) == 0 ? tid0 : ((GT / 32 - 1 - tid0 / 32) * 32 + (tid0 & 31));
+  auto sync = [&]() {   // the group's own barrier
+    if (GT == 32) __syncwarp();
+    else asm volatile("bar.sync %0, %1;" ::"r"(1 + group), "n"(GT) : "memory");
+  };
+  // the work item with index ``it``
+  auto decode = [&](long long it) {
+    CellItem r{0, -1, 0, 0};
+    if (it >= nitems) return r;
+    if (nsys > 1) {   // one system: skip the scan over the descriptor slots
 #pragma unroll
-    for (int r = 1; r < GBC_MAX_SYS; ++r)
-      if (r < nsys && it >= sys[r].item0) q = r;
-    return q;
+      for (int k = 1; k < GBC_MAX_SYS; ++k)
+        if (k < nsys && it >= sys[k].item0) r.q = k;
+    }
+    const long long li = it - sys[r.q].item0;
+    r.e = (int)(li / sys[r.q].vchunks);
+    r.v0 = (int)(li - (long long)r.e * sys[r.q].vchunks) * VB;
+    return r;
   };
 
-  // node index of local node (ix, iy, iz) of a work item's cell:
-  // noff[b][0][ix] + noff[b][1][iy] + noff[b][2][iz], negative where the node is
-  // on a Dirichlet face; b alternates between the current and the next item
-  int* noff = reinterpret_cast<int*>(sm + VB * VS);
-  auto offsets = [&](long long it, int b) {
-    if (tid < 3 * NP) {
-      const CellSys& g = sys[locate(it)];
-      const int e = (int)((it - g.item0) / g.vchunks);
-      const int dd = tid / NP, i = tid % NP;
-      const int c = dd == 0 ? e % g.mesh.ncell[0]
-                  : dd == 1 ? (e / g.mesh.ncell[0]) % g.mesh.ncell[1]
-                            : e / (g.mesh.ncell[0] * g.mesh.ncell[1]);
-      const int gc = c * g.mesh.p + i;
+  // records of the items in flight, item n in slot n % kCellSlots, with the node offsets of
+  // its cell: local node (ix, iy, iz) is noff[0][ix] + noff[1][iy] + noff[2][iz], negative
+  // where the node is on a Dirichlet face
+  float4* fsm = sm + VB * VS;
+  CellItem* rec = reinterpret_cast<CellItem*>(fsm + (FS ? NQ3 : 0));
+  int* noff0 = reinterpret_cast<int*>(rec + kCellSlots);
+  auto noff = [&](int n) { return noff0 + (n % kCellSlots) * 24; };
+  // 1 / M_D of a cell's interior nodes, after the last group's buffers: a node inside one cell
+  // has the same mass in every cell of a launch (all of its systems share p and the edges)
+  constexpr int NIN = NP - 2;
+  float* wint = reinterpret_cast<float*>(sm_raw + blockDim.x / GT * cell_group_smem<NP, VB, FS>());
+  {
+    const MeshDev& m = sys[0].mesh;
+    for (int i = threadIdx.x; i < NIN * NIN * NIN; i += blockDim.x) {
+      const int x = i % NIN + m.periodic[0], y = (i / NIN) % NIN + m.periodic[1],
+                z = i / (NIN * NIN) + m.periodic[2];
+      wint[i] = __ldg(sys[0].invmd + ((long long)z * m.nfree[1] + y) * m.nfree[0] + x);
+    }
+    __syncthreads();
+  }
+  const int lane = tid & 31, warp = tid / 32;
+  constexpr int NW = GT / 32;
+  // PL: the x and y stages, the gather and the assembly of the planes z0 .. z0 + nz - 1 are
+  // one warp's, ordered by warp barriers alone; otherwise all planes belong to the group
+  constexpr bool PL = cell_planes<NP>();
+  // the helper warp stages the fields and posts items before the x stage; at p = 7 it has a
+  // full share of pencils, and all threads stage and it posts after the z stage
+  constexpr bool EARLY = NP < 8;
+  constexpr int PZW = PL ? (NP + NW - 1) / NW : NP;
+  const int z0 = PL ? min(NP, warp * PZW) : 0, nz = PL ? min(NP - z0, PZW) : NP;
+  constexpr int US = PL ? 32 : GT;           // threads that share a plane's units
+  const int ut = PL ? lane : tid;
+  auto psync = [&]() {
+    if (PL) __syncwarp();
+    else sync();
+  };
+  const bool helper = warp == NW - 1;
+
+  // warp ``helper``: write the record and the offsets of item n, the counter's value ``it``
+  auto post = [&](int n, long long it) {
+    CellItem r{0, -1, 0, 0};
+    if (lane == 0) {
+      r = decode(it);
+      rec[n % kCellSlots] = r;
+    }
+    r.q = __shfl_sync(0xffffffffu, r.q, 0);
+    r.e = __shfl_sync(0xffffffffu, r.e, 0);
+    if (r.e >= 0 && lane < 3 * NP) {
+      const MeshDev& m = sys[r.q].mesh;
+      const int dd = lane / NP, i = lane % NP;
+      const int c = dd == 0 ? r.e % m.ncell[0]
+                  : dd == 1 ? (r.e / m.ncell[0]) % m.ncell[1] : r.e / (m.ncell[0] * m.ncell[1]);
+      const int gc = c * m.p + i;
       int f;
-      if (g.mesh.periodic[dd]) {
-        f = gc >= g.mesh.period[dd] ? gc - g.mesh.period[dd] : gc;
-      } else {
-        f = (gc == 0 || gc == g.mesh.period[dd]) ? -1 : gc - 1;
-      }
-      const int scale = dd == 0 ? 1 : dd == 1 ? g.mesh.nfree[0] : g.mesh.nfree[0] * g.mesh.nfree[1];
-      noff[b * 3 * NP + tid] = f < 0 ? kNoNode : f * scale;
+      if (m.periodic[dd]) f = gc >= m.period[dd] ? gc - m.period[dd] : gc;
+      else f = (gc == 0 || gc == m.period[dd]) ? -1 : gc - 1;
+      const int scale = dd == 0 ? 1 : dd == 1 ? m.nfree[0] : m.nfree[0] * m.nfree[1];
+      noff(n)[dd * 8 + i] = f < 0 ? kNoNode : f * scale;
     }
   };
-  // asynchronous gather of X^(e) of work item ``it`` into A: thread -> (vector,
-  // spin, node), vector fastest; absent nodes (Dirichlet faces) and vectors
-  // beyond nvec are zero-filled
-  auto gather = [&](long long it, int b) {
-    const CellSys& g = sys[locate(it)];
-    const int vb0 = (int)((it - g.item0) % g.vchunks) * VB;
-    const int* no = noff + b * 3 * NP;
-    for (int i = tid; i < VB * 2 * NP * NP * NP; i += NT) {
-      const int v = i % VB, r = i / VB, s = r & 1, n = r >> 1;
-      const int ix = n % NP, iy = (n / NP) % NP, iz = n / (NP * NP);
-      const int I = no[ix] + no[NP + iy] + no[2 * NP + iz];
-      const bool ok = I >= 0 && vb0 + v < g.nvec && GBC_IN_RANGE(GBC_SITE_CELL_GATHER, I, g.mesh.M);
-      cp_async8(&Ab(v)[2 * pa(ix, iy, iz) + s],
-                ok ? &g.X[((long long)I * 2 + s) * g.ldx + vb0 + v] : g.X, ok ? 8 : 0);
+  // asynchronous gather of the thread's planes of item n into A: thread -> (vector, spin, x
+  // pencil), vector fastest; absent nodes (Dirichlet faces) and vectors beyond nvec are
+  // zero-filled
+  auto gather = [&](int n) {
+    const CellItem it = rec[n % kCellSlots];
+    const CellSys& g = sys[it.q];
+    const int* no = noff(n);
+    const long long step = 2 * (long long)g.ldx;
+    for (int i = ut; i < VB * 2 * NP * nz; i += US) {
+      const int v = i % VB, s = (i / VB) & 1, pen = i / (2 * VB);
+      const int y = pen % NP, z = z0 + pen / NP;
+      const int Iyz = no[8 + y] + no[16 + z];
+      const bool ok0 = Iyz >= 0 && it.v0 + v < g.nvec;
+      float2* dst = reinterpret_cast<float2*>(&Ab(v)[pa(0, y, z)]) + s;
+      const float2* src = g.X + (long long)s * g.ldx + it.v0 + v;
+      // nodes x = 1 .. NP-2 are consecutive; the two on x faces may wrap or be absent
+      const int I1 = Iyz + no[1];
+      const float2* p = src + I1 * step;
+#pragma unroll
+      for (int x = 1; x < NP - 1; ++x, p += step) {
+        const bool ok = ok0 && GBC_IN_RANGE(GBC_SITE_CELL_GATHER, I1 + x - 1, g.mesh.M);
+        cp_async8(dst + 2 * x, ok ? p : g.X, ok ? 8 : 0);
+      }
+#pragma unroll
+      for (int x = 0; x < NP; x += NP - 1) {
+        const int I = Iyz + no[x];
+        const bool ok = ok0 && I >= 0 && GBC_IN_RANGE(GBC_SITE_CELL_GATHER, I, g.mesh.M);
+        cp_async8(dst + 2 * x, ok ? src + I * step : g.X, ok ? 8 : 0);
+      }
     }
     cp_async_commit();
   };
 
-  // the next item's index; tid 0 writes it before a barrier that every thread
-  // passes after its last read of the previous value (the stage barriers below)
-  long long* s_next = reinterpret_cast<long long*>(noff + 2 * 3 * NP);
-  if (tid == 0) *s_next = (long long)atomicAdd(ctr, 1ULL);
-  __syncthreads();
-  const long long first = *s_next;
-  __syncthreads();
-  if (first < nitems) {
-    offsets(first, 0);
-    __syncthreads();
-    gather(first, 0);
+  // fields of an item's cell into shared memory
+  auto stage_fields = [&](const CellItem& it, int t, int nt) {
+    if (!FS) return;
+    const float4* src = reinterpret_cast<const float4*>(sys[it.q].fields) + (size_t)it.e * NQ3;
+    for (int i = t; i < NQ3; i += nt) cp_async16(fsm + i, src + i);
+    cp_async_commit();
+  };
+
+  // Items are taken two ahead by the helper warp.
+  auto take = [&]() {
+    long long it = 0;
+    if (lane == 0) it = (long long)atomicAdd(ctr, 1ULL);
+    return it;
+  };
+  if (helper) {
+    post(0, take());
+    post(1, take());
   }
-  int buf = 0;
-  long long next = first;
-  for (long long item = first; item < nitems; item = next, buf ^= 1) {
-    const CellSys& d = sys[locate(item)];
-    const long long li = item - d.item0;
-    const int e = (int)(li / d.vchunks);
-    const int vbase = (int)(li % d.vchunks) * VB;
-    const int* no = noff + buf * 3 * NP;
-    if (tid == 0) *s_next = (long long)atomicAdd(ctr, 1ULL);
-    cp_async_wait_all();
-    __syncthreads();
-    next = *s_next;
-    if (next < nitems) offsets(next, buf ^ 1);   // read after the next two barriers
-
-    // ---- Kz: T1 = B_z X, T2 = G_z X
-    for (int u = tid; u < VB * 2 * NP * NP; u += NT) {
-      const int v = u % VB, s = (u / VB) & 1, pen = u / (2 * VB);
-      const int x = pen % NP, y = pen / NP;
-      float2 in[NP], t1[NP], t2[NP];
-#pragma unroll
-      for (int j = 0; j < NP; ++j) in[j] = Ab(v)[2 * pa(x, y, j) + s];
-      eo2_apply<1>(tb.B[2], in, t1);
-      g2_apply<KPT>(tb.Gr[2], tb.Gi[2], in, t2);
-#pragma unroll
-      for (int i = 0; i < NP; ++i) {
-        T1b(v)[2 * pq(x, y, i) + s] = t1[i];
-        T2b(v)[2 * pa(x, y, i) + s] = t2[i];
-      }
-    }
-    __syncthreads();
-
-    // ---- Ky (in place): U1 = B_y T1, U2 = G_y T1 + B_y T2
-    for (int u = tid; u < VB * 2 * NP * NP; u += NT) {
-      const int v = u % VB, s = (u / VB) & 1, pen = u / (2 * VB);
-      const int x = pen % NP, z = pen / NP;
-      float2 t1[NP], t2[NP], u1[NP], u2[NP], w2[NP];
-#pragma unroll
-      for (int j = 0; j < NP; ++j) {
-        t1[j] = T1b(v)[2 * pq(x, j, z) + s];
-        t2[j] = T2b(v)[2 * pa(x, j, z) + s];
-      }
-      eo2_apply<1>(tb.B[1], t1, u1);
-      g2_apply<KPT>(tb.Gr[1], tb.Gi[1], t1, u2);
-      eo2_apply<1>(tb.B[1], t2, w2);
-#pragma unroll
-      for (int i = 0; i < NP; ++i) {
-        T1b(v)[2 * pq(x, i, z) + s] = u1[i];
-        T2b(v)[2 * pa(x, i, z) + s] = p_add(u2[i], w2[i]);
-      }
-    }
-    __syncthreads();
-
-    // ---- Kx + Ix (in place, x pencils): T2 = G_x U1 + B_x U2, T1 = N_x X
-    for (int u = tid; u < VB * 2 * NP * NP; u += NT) {
-      const int v = u % VB, s = (u / VB) & 1, pen = u / (2 * VB);
-      const int y = pen % NP, z = pen / NP;
-      {
-        float2 u1[NP], u2[NP], yk[NP], w2[NP];
-#pragma unroll
-        for (int j = 0; j < NP; ++j) {
-          u1[j] = T1b(v)[2 * pq(j, y, z) + s];
-          u2[j] = T2b(v)[2 * pa(j, y, z) + s];
-        }
-        g2_apply<KPT>(tb.Gr[0], tb.Gi[0], u1, yk);
-        eo2_apply<1>(tb.B[0], u2, w2);
-#pragma unroll
-        for (int i = 0; i < NP; ++i) T2b(v)[2 * pa(i, y, z) + s] = p_add(yk[i], w2[i]);
-      }
-      {
-        float2 in[NP], out[NQ];
-#pragma unroll
-        for (int j = 0; j < NP; ++j) in[j] = Ab(v)[2 * pa(j, y, z) + s];
-        eo2_apply<1>(tb.Ni, in, out);
-#pragma unroll
-        for (int q = 0; q < NQ; ++q) T1b(v)[2 * pq(q, y, z) + s] = out[q];
-      }
-    }
-    __syncthreads();
-    // A is free from here on: start the next item's gather behind the remaining stages
-    if (next < nitems) gather(next, buf ^ 1);
-
-    // ---- Iy (in place): T1 (nq, np, np) -> (nq, nq, np)
-    for (int u = tid; u < VB * 2 * NQ * NP; u += NT) {
-      const int v = u % VB, s = (u / VB) & 1, pen = u / (2 * VB);
-      const int x = pen % NQ, z = pen / NQ;
-      float2 in[NP], out[NQ];
-#pragma unroll
-      for (int j = 0; j < NP; ++j) in[j] = T1b(v)[2 * pq(x, j, z) + s];
-      eo2_apply<1>(tb.Ni, in, out);
-#pragma unroll
-      for (int q = 0; q < NQ; ++q) T1b(v)[2 * pq(x, q, z) + s] = out[q];
-    }
-    __syncthreads();
-
-    // ---- Iz + spin operator + Tz (z pencils, in place); spin fastest, so the
-    // two spins of a pencil sit on neighbouring lanes and swap values by shuffle
-    {
-      const float* __restrict__ fld = d.fields + (size_t)e * 4 * NQ3;
-      constexpr int UNITS = VB * 2 * NQ * NQ;
-      constexpr int ROUNDS = (UNITS + NT - 1) / NT;
+  sync();
+  if (rec[0].e >= 0) {
+    gather(0);
+    if (!EARLY) stage_fields(rec[0], tid, GT);
+  }
 #pragma unroll 1
-      for (int r = 0; r < ROUNDS; ++r) {
-        const int uu = tid + r * NT;
-        const bool act = uu < UNITS;
-        const int u = act ? uu : (uu & 1);
-        const int s = u & 1, v = (u >> 1) % VB, pen = (u >> 1) / VB;
-        const int x = pen % NQ, y = pen / NQ;
-        float2 in[NP], own[NQ];
+  for (int n = 0;; ++n) {
+    const CellItem item = rec[n % kCellSlots];
+    if (item.e < 0) break;
+    const CellSys& d = sys[item.q];
+    const int e = item.e;
+    const int vbase = item.v0;
+    const int* no = noff(n);
+    long long taken = 0;
+    if (helper) taken = take();
+    if (EARLY && helper) {
+      stage_fields(item, lane, 32);
+      post(n + 2, taken);
+    }
+    cp_async_wait_all();
+    psync();
+
+    // ---- x pencils: T1 = N'^T X, A = B_x X (in place), T2 = G_x X
+    for (int u = ut; u < VB * NP * nz; u += US) {
+      const int v = u % VB, pen = u / VB;
+      const int y = pen % NP, z = z0 + pen / NP;
+      float4 *A = Ab(v) + pa(0, y, z), *K = T2b(v) + pa(0, y, z), *Q = T1b(v) + pq(0, y, z);
+      Parts<NP> s;
+      load_parts<PACKED>(s, [&](int j) { return A[j]; });
 #pragma unroll
-        for (int j = 0; j < NP; ++j) in[j] = T1b(v)[2 * pq(x, y, j) + s];
-        eo2_apply<1>(tb.Ni, in, own);
-        const float sg = s ? -1.f : 1.f;
-        float2 w[NQ];
+      for (int i = 0; i < HQ; ++i) {
+        Acc a;
+        row_sym<true, NQ>(tb.Ni, i, s, a);
+        put_rows<PACKED, NQ>(i, a, [&](int r, float4 val) { Q[r] = val; });
+      }
 #pragma unroll
-        for (int q = 0; q < NQ; ++q) {
-          float2 oth;
-          oth.x = __shfl_xor_sync(0xffffffffu, own[q].x, 1);
-          oth.y = __shfl_xor_sync(0xffffffffu, own[q].y, 1);
-          const int qq = (q * NQ + y) * NQ + x;
-          const float4 F = __ldg(reinterpret_cast<const float4*>(fld) + qq);
-          const float V = F.x, bx = F.y, by = F.z, bz = F.w;
-          // up:   (V + bz) u + bx d + by (d.y, -d.x)
-          // down: (V - bz) d + bx u - by (u.y, -u.x)
-          float2 o = p_mul(dup(V + sg * bz), own[q]);
-          o = p_fma(dup(bx), oth, o);
-          w[q] = p_fma(make_float2(sg * by, -sg * by), make_float2(oth.y, oth.x), o);
-        }
-        float2 out[NP];
-        eo2_apply<1>(tb.Nt, w, out);
-        if (act) {
-#pragma unroll
-          for (int i = 0; i < NP; ++i) T1b(v)[2 * pq(x, y, i) + s] = out[i];
-        }
+      for (int i = 0; i < HP; ++i) {
+        Acc a;
+        row_sym<true, NP>(tb.B[0], i, s, a);
+        put_rows<PACKED, NP>(i, a, [&](int r, float4 val) { A[r] = val; });
+        row_sym<true, NP>(tb.Gr[0], i, s, a);
+        if (KPT) row_anti<NP>(tb.Gi[0], i, s, a);
+        put_rows<PACKED, NP>(i, a, [&](int r, float4 val) { K[r] = val; });
       }
     }
-    __syncthreads();
+    psync();
 
-    // ---- Ty (in place): T1 (nq, nq, np) -> (nq, np, np)
-    for (int u = tid; u < VB * 2 * NQ * NP; u += NT) {
-      const int v = u % VB, s = (u / VB) & 1, pen = u / (2 * VB);
-      const int x = pen % NQ, z = pen / NQ;
-      float2 in[NQ], out[NP];
+    // ---- y pencils (in place): T1 = N'^T T1; T2 = G_y A + B_y T2
+    for (int u = ut; u < VB * NQ * nz; u += US) {
+      const int v = u % VB, pen = u / VB;
+      float4* Q = T1b(v) + pq(pen % NQ, 0, z0 + pen / NQ);
+      Parts<NP> s;
+      load_parts<PACKED>(s, [&](int j) { return Q[j * L::QY]; });
 #pragma unroll
-      for (int q = 0; q < NQ; ++q) in[q] = T1b(v)[2 * pq(x, q, z) + s];
-      eo2_apply<1>(tb.Nt, in, out);
-#pragma unroll
-      for (int i = 0; i < NP; ++i) T1b(v)[2 * pq(x, i, z) + s] = out[i];
+      for (int i = 0; i < HQ; ++i) {
+        Acc a;
+        row_sym<true, NQ>(tb.Ni, i, s, a);
+        put_rows<PACKED, NQ>(i, a, [&](int r, float4 val) { Q[r * L::QY] = val; });
+      }
     }
-    __syncthreads();
+    // (the threads left idle by the last round above take the first units here)
+    for (int u = (ut + US - VB * NQ * nz % US) % US; u < VB * NP * nz; u += US) {
+      const int v = u % VB, pen = u / VB;
+      const int o = pa(pen % NP, 0, z0 + pen / NP);
+      const float4* A = Ab(v) + o;
+      float4* K = T2b(v) + o;
+      Parts<NP> s1, s2;
+      load_parts<PACKED>(s1, [&](int j) { return A[j * L::AY]; });
+      load_parts<PACKED>(s2, [&](int j) { return K[j * L::AY]; });
+#pragma unroll
+      for (int i = 0; i < HP; ++i) {
+        Acc a;
+        row_sym<true, NP>(tb.Gr[1], i, s1, a);
+        if (KPT) row_anti<NP>(tb.Gi[1], i, s1, a);
+        row_sym<false, NP>(tb.B[1], i, s2, a);
+        put_rows<PACKED, NP>(i, a, [&](int r, float4 val) { K[r * L::AY] = val; });
+      }
+    }
+    psync();
+    // the planes of A are free: start the next item's gather
+    if (rec[(n + 1) % kCellSlots].e >= 0) gather(n + 1);
+    if (PL) sync();
 
-    // ---- Tx, add the kinetic part, assemble (vector fastest across threads)
-    for (int u = tid; u < VB * 2 * NP * NP; u += NT) {
-      const int v = u % VB, s = (u / VB) & 1, pen = u / (2 * VB);
-      const int y = pen % NP, z = pen / NP;
-      const int vec = vbase + v;
-      float2 in[NQ], out[NP];
+    // ---- z pencils (in place): T1 = N' F N'^T T1 + G'_z T1; T2 = B_z T2
+    constexpr int UZ = VB * NQ * NQ;
+    {
+      const float4* __restrict__ fld = reinterpret_cast<const float4*>(d.fields) + (size_t)e * NQ3;
+      for (int u = tid; u < UZ; u += GT) {
+        const int v = u % VB, pen = u / VB;
+        const int x = pen % NQ, y = pen / NQ;
+        float4* Q = T1b(v) + pq(x, y, 0);
+        Parts<NP> s;
+        load_parts<PACKED>(s, [&](int j) { return Q[j * L::QZ]; });
+        // up:   (V + bz) u + (bx - i by) d
+        // down: (V - bz) d + (bx + i by) u
+        auto spin_op = [&](int q, float4 o) {
+          const float4 F = FS ? fsm[(q * NQ + y) * NQ + x] : __ldg(fld + (q * NQ + y) * NQ + x);
+          const float vp = F.x + F.w, vm = F.x - F.w;
+          return make_float4(fmaf(F.z, o.w, fmaf(F.y, o.z, vp * o.x)),
+                             fmaf(-F.z, o.z, fmaf(F.y, o.w, vp * o.y)),
+                             fmaf(-F.z, o.y, fmaf(F.y, o.x, vm * o.z)),
+                             fmaf(F.z, o.x, fmaf(F.y, o.y, vm * o.w)));
+        };
+        Parts<NQ> w;
 #pragma unroll
-      for (int q = 0; q < NQ; ++q) in[q] = T1b(v)[2 * pq(q, y, z) + s];
-      eo2_apply<1>(tb.Nt, in, out);
-      if (vec >= d.nvec) continue;
-      const bool yz_in = y > 0 && y < NP - 1 && z > 0 && z < NP - 1;
-      const int Iyz = no[NP + y] + no[2 * NP + z];
-#pragma unroll
-      for (int i = 0; i < NP; ++i) out[i] = p_add(out[i], T2b(v)[2 * pa(i, y, z) + s]);
-      if (d.cheb && yz_in) {
-        // nodes x = 1 .. NP-2 of this pencil are interior to the cell: every load is
-        // issued before the first update (X_out may alias X_prev), so their latencies
-        // overlap
-        constexpr int NIN = NP - 2;
-        float2 yv[NIN], xv[NIN], pv[NIN];
-        float wv[NIN];
-#pragma unroll
-        for (int j = 0; j < NIN; ++j) {
-          const int I = Iyz + no[1 + j];
-          const long long o = ((long long)I * 2 + s) * d.ldx + vec;
-          if (GBC_IN_RANGE(GBC_SITE_CELL_STORE, I, d.mesh.M)) {
-            yv[j] = d.Y[o];
-            xv[j] = __ldg(&d.X[o]);
-            wv[j] = __ldg(d.invmd + I);
-            pv[j] = d.Xprev ? d.Xprev[o] : make_float2(0.f, 0.f);
+        for (int i = 0; i < HQ; ++i) {
+          Acc a;
+          float4 r0, r1;
+          row_sym<true, NQ>(tb.Ni, i, s, a);
+          put_rows<PACKED, NQ>(i, a, [&](int r, float4 val) {
+            if (r == i) r0 = spin_op(r, val);
+            else r1 = spin_op(r, val);
+          });
+          if (NQ - 1 - i == i) {
+            w.m[0] = lo2(r0);
+            w.m[1] = hi2(r0);
           } else {
-            yv[j] = xv[j] = pv[j] = make_float2(0.f, 0.f);
-            wv[j] = 0.f;
+            set_part<PACKED>(w, i, r0, r1);
           }
         }
 #pragma unroll
-        for (int j = 0; j < NIN; ++j) {
-          const int I = Iyz + no[1 + j];
-          const long long o = ((long long)I * 2 + s) * d.ldx + vec;
-          const float2 yt = p_add(yv[j], out[1 + j]);
-          const float2 xn = p_fma(dup(-d.cb), pv[j],
-                                  p_mul(dup(d.ca), p_fma(dup(-d.cc), xv[j], p_mul(dup(wv[j]), yt))));
-          if (GBC_IN_RANGE(GBC_SITE_CELL_STORE, I, d.mesh.M)) d.Xout[o] = xn;
+        for (int i = 0; i < HP; ++i) {
+          Acc a;
+          row_sym<true, NP>(tb.Nt, i, w, a);
+          row_sym<false, NP>(tb.Gr[2], i, s, a);
+          if (KPT) row_anti<NP>(tb.Gi[2], i, s, a);
+          put_rows<PACKED, NP>(i, a, [&](int r, float4 val) { Q[r * L::QZ] = val; });
         }
+      }
+    }
+    for (int u = (tid + GT - UZ % GT) % GT; u < VB * NP * NP; u += GT) {
+      const int v = u % VB, pen = u / VB;
+      float4* K = T2b(v) + pa(pen % NP, pen / NP, 0);
+      Parts<NP> s;
+      load_parts<PACKED>(s, [&](int j) { return K[j * L::AZ]; });
 #pragma unroll
-        for (int i = 0; i < NP; i += NP - 1) {   // the pencil's two face nodes
-          const int I = Iyz + no[i];
-          if (I >= 0 && GBC_IN_RANGE(GBC_SITE_CELL_STORE, I, d.mesh.M))
-            atomicAdd(&d.Y[((long long)I * 2 + s) * d.ldx + vec], out[i]);
+      for (int i = 0; i < HP; ++i) {
+        Acc a;
+        row_sym<true, NP>(tb.B[2], i, s, a);
+        put_rows<PACKED, NP>(i, a, [&](int r, float4 val) { K[r * L::AZ] = val; });
+      }
+    }
+    sync();
+
+    if (!EARLY) {
+      if (helper) post(n + 2, taken);
+      const CellItem next = rec[(n + 1) % kCellSlots];
+      if (next.e >= 0) stage_fields(next, tid, GT);
+    }
+    // ---- y pencils of the planes (in place): T1 = N' T1
+    for (int u = ut; u < VB * NQ * nz; u += US) {
+      const int v = u % VB, pen = u / VB;
+      float4* Q = T1b(v) + pq(pen % NQ, 0, z0 + pen / NQ);
+      Parts<NQ> s;
+      load_parts<PACKED>(s, [&](int j) { return Q[j * L::QY]; });
+#pragma unroll
+      for (int i = 0; i < HP; ++i) {
+        Acc a;
+        row_sym<true, NP>(tb.Nt, i, s, a);
+        put_rows<PACKED, NP>(i, a, [&](int r, float4 val) { Q[r * L::QY] = val; });
+      }
+    }
+    psync();
+
+    // ---- x pencils: N' T1 + T2, assembled (vector fastest across threads)
+    for (int u = ut; u < VB * NP * nz; u += US) {
+      const int v = u % VB, pen = u / VB;
+      const int y = pen % NP, z = z0 + pen / NP;
+      const int vec = vbase + v;
+      if (vec >= d.nvec) continue;
+      float4 out[NP];
+      {
+        const float4* Q = T1b(v) + pq(0, y, z);
+        const float4* K = T2b(v) + pa(0, y, z);
+        Parts<NQ> s;
+        load_parts<PACKED>(s, [&](int j) { return Q[j]; });
+#pragma unroll
+        for (int i = 0; i < HP; ++i) {
+          Acc a;
+          row_sym<true, NP>(tb.Nt, i, s, a);
+          put_rows<PACKED, NP>(i, a, [&](int r, float4 val) {
+            const float4 k = K[r];
+            out[r] = cat2(c_add<PACKED>(lo2(val), lo2(k)), c_add<PACKED>(hi2(val), hi2(k)));
+          });
         }
-      } else {
+      }
+      const bool yz_in = y > 0 && y < NP - 1 && z > 0 && z < NP - 1;
+      const int Iyz = no[8 + y] + no[16 + z];
 #pragma unroll
-        for (int i = 0; i < NP; ++i) {
-          const int I = Iyz + no[i];
-          if (I >= 0 && GBC_IN_RANGE(GBC_SITE_CELL_STORE, I, d.mesh.M))
-            atomicAdd(&d.Y[((long long)I * 2 + s) * d.ldx + vec], out[i]);
+      for (int s = 0; s < 2; ++s) {
+        if (d.cheb && yz_in) {
+          // nodes x = 1 .. NP-2 of this pencil are interior to the cell: every load is
+          // issued before the first update (X_out may alias X_prev), so their latencies
+          // overlap
+          float2 yv[NIN], xv[NIN], pv[NIN];
+          const long long step = 2 * (long long)d.ldx;
+          const int I1 = Iyz + no[1];   // consecutive from here
+          const long long o1 = I1 * step + (long long)s * d.ldx + vec;
+          const float* w = wint + ((z - 1) * NIN + y - 1) * NIN;
+#pragma unroll
+          for (int j = 0; j < NIN; ++j) {
+            const long long o = o1 + j * step;
+            if (GBC_IN_RANGE(GBC_SITE_CELL_STORE, I1 + j, d.mesh.M)) {
+              yv[j] = d.Y[o];
+              xv[j] = __ldg(&d.X[o]);
+              pv[j] = d.Xprev ? d.Xprev[o] : make_float2(0.f, 0.f);
+            } else {
+              yv[j] = xv[j] = pv[j] = make_float2(0.f, 0.f);
+            }
+          }
+#pragma unroll
+          for (int j = 0; j < NIN; ++j) {
+            const long long o = o1 + j * step;
+            const float2 yt = p_add(yv[j], s ? hi2(out[1 + j]) : lo2(out[1 + j]));
+            const float2 xn = p_fma(dup(-d.cb), pv[j],
+                                    p_mul(dup(d.ca), p_fma(dup(-d.cc), xv[j], p_mul(dup(w[j]), yt))));
+            if (GBC_IN_RANGE(GBC_SITE_CELL_STORE, I1 + j, d.mesh.M)) d.Xout[o] = xn;
+          }
+#pragma unroll
+          for (int i = 0; i < NP; i += NP - 1) {   // the pencil's two face nodes
+            const int I = Iyz + no[i];
+            if (I >= 0 && GBC_IN_RANGE(GBC_SITE_CELL_STORE, I, d.mesh.M))
+              atomicAdd(&d.Y[((long long)I * 2 + s) * d.ldx + vec], s ? hi2(out[i]) : lo2(out[i]));
+          }
+        } else {
+#pragma unroll
+          for (int i = 0; i < NP; ++i) {
+            const int I = Iyz + no[i];
+            if (I >= 0 && GBC_IN_RANGE(GBC_SITE_CELL_STORE, I, d.mesh.M))
+              atomicAdd(&d.Y[((long long)I * 2 + s) * d.ldx + vec], s ? hi2(out[i]) : lo2(out[i]));
+          }
         }
       }
     }
@@ -509,13 +678,15 @@ __device__ __forceinline__ void cell_body(const CellSys* __restrict__ sys, int n
 }
 
 // One persistent launch over systems that share p, the cell edges and the k-point;
-// the CTAs take their work items from the zeroed counter *ctr in ascending order.
+// the groups of the CTAs take their work items from the zeroed counter *ctr in ascending
+// order.
 template <int NP, int NQ, bool KPT, int VB, int NT, int MINB, bool PACKED>
 __global__ void __launch_bounds__(NT, MINB)
 hx_cell_kernel(const __grid_constant__ CellArgs a,
                const __grid_constant__ CellTables<NP, NQ, PACKED> tb,
                unsigned long long* __restrict__ ctr) {
-  cell_body<NP, NQ, KPT, VB, NT, PACKED>(a.sys, a.nsys, a.nitems, tb, ctr);
+  cell_body<NP, NQ, KPT, VB, cell_group_threads<NP, VB>(), PACKED, cell_stage_fields<NP, VB, NT, MINB>()>(
+      a.sys, a.nsys, a.nitems, tb, ctr);
 }
 
 template <int NO, int NI>
@@ -535,6 +706,23 @@ template <int NP, int NQ, bool PACKED>
 inline bool make_cell_tables(const gbc_ctx* c, CellTables<NP, NQ, PACKED>* t) {
   TablesEO<float, NP, NQ> f;
   if (!make_tables_eo<float, NP, NQ>(c, &f)) return false;
+  // N' = N diag(sqrt(w_q)) and its transpose; the z kinetic operators carry the x and y
+  // edges that the mass products of N' leave out
+  const HostTables& h = c->tab;
+  std::vector<double> Ni(NQ * NP), Nt(NP * NQ);
+  for (int i = 0; i < NP; ++i)
+    for (int q = 0; q < NQ; ++q)
+      Ni[q * NP + i] = Nt[i * NQ + q] = h.N1[i * NQ + q] * std::sqrt(h.gq_w[q]);
+  if (!make_eo<float, NQ, NP>(Ni, 1, &f.Ni) || !make_eo<float, NP, NQ>(Nt, 1, &f.Nt)) return false;
+  const double hxy = 0.25 * c->h[0] * c->h[1], hz = c->h[2];
+  std::vector<double> Gr(NP * NP), Gi(NP * NP);
+  for (int i = 0; i < NP; ++i)
+    for (int j = 0; j < NP; ++j) {
+      Gr[i * NP + j] = hxy * 0.5 * (2.0 / hz) * h.Ah[i * NP + j];
+      Gi[i * NP + j] = -hxy * 0.5 * c->k[2] * (h.Ch[i * NP + j] - h.Ch[j * NP + i]);
+    }
+  if (!make_eo<float, NP, NP>(Gr, 1, &f.Gr[2]) || !make_eo<float, NP, NP>(Gi, -1, &f.Gi[2]))
+    return false;
   for (int d = 0; d < 3; ++d) {
     cvt_table(f.B[d], t->B[d]);
     cvt_table(f.Gr[d], t->Gr[d]);
@@ -590,7 +778,8 @@ cudaError_t launch_cell_group_p(const CellJob* jobs, int n, cudaStream_t s) {
   CellTables<NP, NQ, PACKED> tb;
   if (!make_cell_tables<NP, NQ, PACKED>(c0, &tb)) return cudaErrorInvalidValue;
   const bool kpt = (c0->k[0] != 0.0 || c0->k[1] != 0.0 || c0->k[2] != 0.0);
-  constexpr size_t smem = hx_cell_smem<NP, NQ, VB>();
+  constexpr size_t smem = cell_smem<NP, VB, NT, MINB>();
+  constexpr int groups = NT / cell_group_threads<NP, VB>();
   int dev = 0, nsm = 0, per_sm = 0;
   cudaError_t err = cudaGetDevice(&dev);
   if (err != cudaSuccess) return err;
@@ -604,7 +793,8 @@ cudaError_t launch_cell_group_p(const CellJob* jobs, int n, cudaStream_t s) {
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NT, smem);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
-    const long long nblk = std::min<long long>(item, (long long)nsm * per_sm);
+    const long long nblk =
+        std::min<long long>((item + groups - 1) / groups, (long long)nsm * per_sm);
     e = cudaMemsetAsync(ctr, 0, sizeof(unsigned long long), s);
     if (e != cudaSuccess) return e;
     kern<<<(unsigned)nblk, NT, smem, s>>>(a, tb, ctr);

@@ -10,9 +10,9 @@ cudaError_t launch_cell_f32_v4(const CellJob* jobs, int n, cudaStream_t s);
 
 
 CellVariant cell_variant(int v) {
-  static const CellVariant tab[GBC_CELL_VARIANTS] = {{2, 256, 4, 1}, {2, 256, 3, 1},
-                                                     {2, 256, 4, 0}, {2, 256, 3, 0},
-                                                     {4, 512, 2, 0}};
+  static const CellVariant tab[GBC_CELL_VARIANTS] = {{2, 256, 2, 1}, {2, 256, 3, 1},
+                                                     {2, 256, 2, 0}, {2, 256, 3, 0},
+                                                     {4, 512, 1, 1}};
   return tab[(v >= 0 && v < GBC_CELL_VARIANTS) ? v : 0];
 }
 

@@ -154,7 +154,8 @@ __global__ void k_mass(const MeshDev m, const double* mx, const double* my, cons
 }
 
 // fields[e][c][q] = w_q J * {V + |k|^2/2, bx, by, bz}[e][q] (FP64); the FP32 copy is
-// [e][q][c], one float4 per quadrature point
+// [e][q][c], one float4 per quadrature point, without w_q (the FP32 interpolation tables
+// carry its square root on both sides)
 __global__ void k_fields(const double* raw, long long E, int nq, double jac, double k2half,
                          const double* __restrict__ wq, double* f64, float* f32) {
   const long long nq3 = (long long)nq * nq * nq;
@@ -169,7 +170,7 @@ __global__ void k_fields(const double* raw, long long E, int nq, double jac, dou
     if (c == 0) val += k2half;
     const double o = w * val;
     f64[(e * 4 + c) * nq3 + q] = o;
-    f32[(e * nq3 + q) * 4 + c] = (float)o;   // FP32: one float4 per point
+    f32[(e * nq3 + q) * 4 + c] = (float)(jac * val);
   }
 }
 

@@ -455,7 +455,8 @@ gbc_status tcl_tables(gbc_ctx* c, TclState* t, int mode) {
     const int qx = q % nq, qy = (q / nq) % nq, qz = q / (nq * nq);
     for (int n = 0; n < np3; ++n) {
       const int ix = n % np, iy = (n / np) % np, iz = n / (np * np);
-      const double v = h.N1[ix * nq + qx] * h.N1[iy * nq + qy] * h.N1[iz * nq + qz];
+      const double v = h.N1[ix * nq + qx] * h.N1[iy * nq + qy] * h.N1[iz * nq + qz] *
+                       std::sqrt(h.gq_w[qx] * h.gq_w[qy] * h.gq_w[qz]);
       n3[(size_t)q * t->NPP + n] = v;
       b2[(size_t)n * t->KT + q] = v;   // N3^T
     }

@@ -1,0 +1,55 @@
+"""FP32 cell apply at the orders and shapes where its thread groups, plane ownership and
+tables change: p = 3, 4, 5 (group sizes) and p = 6 (planes owned by warps), unequal cell
+edges (the z kinetic operator carries the x and y edges), Dirichlet faces in every
+direction, ragged vector chunks and several systems in one launch.
+
+Tolerances as test_gpu_batch.py: H.X relative Frobenius 1e-5, degree-3 filter 2e-5."""
+import numpy as np
+import pytest
+
+import synthetic as syn
+from oracle import chfsi as oc
+from oracle import fe
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def g():
+    import __graft_entry__ as ge
+    ge.build()
+    import paper_2410_02754_gb300 as pkg
+    return pkg
+
+
+def rel(a, b):
+    return float(np.linalg.norm(a - b) / np.linalg.norm(b))
+
+
+CASES = [((3, 2, 1), 3, (1, 0, 1), (0.1, 0.0, -0.2), 3), ((1, 2, 3), 4, (0, 1, 0), (0.0, 0.0, 0.0), 9),
+         ((2, 1, 2), 5, (1, 1, 0), (0.0, 0.2, 0.1), 5), ((2, 3, 1), 6, (0, 0, 0), (0.05, 0.1, 0.2), 6)]
+
+
+@pytest.mark.parametrize("var", [0, 1, 2, 4])
+@pytest.mark.parametrize("case", CASES, ids=lambda c: f"p{c[1]}")
+def test_cell_groups(g, var, case):
+    ncell, p, per, k, nvec = case
+    prob = syn.make_problem(ncell=ncell, h=(0.9, 1.3, 1.1), p=p, periodic=per, k=k, natoms=1, rc=0.8,
+                            seed=31)
+    d = fe.Discretisation(prob)
+    X = syn.random_block(d.mesh.nnodes, nvec, 8)
+    c = g.Context(0)
+    c.set_problem(prob)
+    c.set_precision(1)
+    c.set_cell_variant(var)
+    Xd = torch.from_numpy(X).to(torch.complex64).cuda()
+    Yd = torch.empty_like(Xd)
+    c.apply_h(Xd, Yd)
+    c.sync_status()
+    assert rel(Yd.cpu().numpy(), d.apply_h(X)) < 1e-5
+    bounds = (1.0, 90.0, -2.0)
+    c.filter(Xd, 3, *bounds)
+    c.sync_status()
+    assert rel(Xd.cpu().numpy().astype(np.complex128), oc.cheb_filter(d.apply_htilde, X, 3, *bounds)) < 2e-5
+    c.close()
