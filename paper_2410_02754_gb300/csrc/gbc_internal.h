@@ -202,7 +202,7 @@ struct gbc_ctx {
   double* d_invmd = nullptr;         // [M]
   float* d_invmd32 = nullptr;
   double* d_rawfields = nullptr;     // [4][E][nq^3] user fields (V, bx, by, bz)
-  double* d_fields64 = nullptr;      // [E][4][nq^3] w_q J (V + |k|^2/2), w_q J B_d
+  double* d_fields64 = nullptr;      // [E][nq^3][4] J (V + |k|^2/2), J B_x, J B_y, J B_z
   float* d_fields32 = nullptr;
   ProjDev proj;
   // workspaces

@@ -222,44 +222,6 @@ __device__ __forceinline__ void put_rows(int i, const Acc& a, F st) {
   }
 }
 
-// Point strides (y, z) of the n_p^3 buffers (A, T2) and of T1 (up to n_q x n_q x n_p
-// points).  A quarter-warp's 16-byte accesses (VB vectors, then neighbouring pencils) fall
-// in the 8 distinct bank groups when neighbouring pencils are an odd number of points
-// apart, which these strides give in every stage's pencil direction, and the vectors
-// start 8 / VB groups apart (cell_vpoints).
-template <int NP> struct CellLayout;
-template <> struct CellLayout<3> { static constexpr int AY = 3, AZ = 9, QY = 5, QZ = 23; };
-template <> struct CellLayout<4> { static constexpr int AY = 5, AZ = 21, QY = 5, QZ = 25; };
-template <> struct CellLayout<5> { static constexpr int AY = 5, AZ = 25, QY = 7, QZ = 43; };
-template <> struct CellLayout<6> { static constexpr int AY = 7, AZ = 43, QY = 7, QZ = 51; };
-template <> struct CellLayout<7> { static constexpr int AY = 7, AZ = 49, QY = 9, QZ = 73; };
-template <> struct CellLayout<8> { static constexpr int AY = 9, AZ = 72, QY = 9, QZ = 81; };
-template <int NP> __host__ __device__ constexpr int cell_bufa() {   // points of A / T2
-  return (NP - 1) * (1 + CellLayout<NP>::AY + CellLayout<NP>::AZ) + 1;
-}
-template <int NP> __host__ __device__ constexpr int cell_bufq() {   // points of T1
-  return NP * (1 + CellLayout<NP>::QY) + (NP - 1) * CellLayout<NP>::QZ + 1;
-}
-template <int NP, int VB> __host__ __device__ constexpr int cell_vpoints() {
-  // points per vector: [A | T2 | T1], padded to 8 / VB mod 8
-  static_assert(VB == 2 || VB == 4, "VB");
-  constexpr int n = 2 * cell_bufa<NP>() + cell_bufq<NP>(), r = 8 / VB;
-  return n + ((8 + r - n % 8) % 8);
-}
-// Threads of a group: about one per pencil of a vector's x stage.  At p = 3 and 4 small
-// groups are worth more than full rounds (12^3 cells, p = 4, 96 vectors: 446 us a launch at
-// 128 threads, 642 at 256).
-template <int NP, int VB> __host__ __device__ constexpr int cell_group_threads() {
-  constexpr int g4[9] = {0, 0, 0, 64, 128, 128, 256, 256, 256};
-  constexpr int g2[9] = {0, 0, 0, 32, 64, 64, 128, 128, 128};
-  return VB == 4 ? g4[NP] : g2[NP];
-}
-// Whether each warp owns whole z planes of a cell (see cell_body): where a plane's pencils
-// fill a warp and a warp is left over (p = 6, 4 vectors: 28 to 32 lanes, 8.34 -> 7.62 ms a
-// launch on 16^3 cells, 256 vectors; p = 5: 872 -> 815 us on 12^3 cells, 96 vectors).  At
-// p = 7 a plane has 36 pencils a vector quad and every warp a plane (1048 -> 1090 us), at
-// p <= 4 it leaves lanes idle (460 -> 575 us).
-template <int NP> __host__ __device__ constexpr bool cell_planes() { return NP == 6 || NP == 7; }
 // a work item: system, cell, first vector; e < 0: none
 struct alignas(16) CellItem { int q, e, v0, pad; };
 constexpr int kCellSlots = 4;    // item records and offset tables in flight
@@ -282,11 +244,10 @@ template <int NP, int VB, int NT, int MINB> __host__ __device__ constexpr size_t
   return NT / cell_group_threads<NP, VB>() * cell_group_smem<NP, VB, cell_stage_fields<NP, VB, NT, MINB>()>() +
          cell_mass_smem<NP>();
 }
-constexpr int kNoNode = -(1 << 29);   // offset of a direction with no free node (Dirichlet face)
 
-// The work items [0, nitems) of the systems sys[0 .. nsys) (item0 ascending), taken
-// from the counter *ctr (zero at launch) one atomic increment at a time, so groups
-// that finish early take more and the items in flight stay close to each other in
+// The work items [0, nitems) of the systems sys[0 .. nsys) (item0 ascending), after each
+// group's first taken from the counter *ctr (zero at launch) one at a time, so groups that
+// finish early take more and the items in flight stay close to each other in
 // the order (cell-major, vector chunks of a cell adjacent).  GT: threads of a group.
 template <int NP, int NQ, bool KPT, int VB, int GT, bool PACKED, bool FS>
 __device__ __forceinline__ void cell_body(const CellSys* __restrict__ sys, int nsys,
@@ -430,14 +391,16 @@ __device__ __forceinline__ void cell_body(const CellSys* __restrict__ sys, int n
     cp_async_commit();
   };
 
-  // Items are taken two ahead by the helper warp.
+  // Items are taken two ahead by the helper warp.  A group's first item is its own: those of a
+  // CTA are gridDim.x apart, so few items spread over the SMs.
+  const long long ngroups = (long long)gridDim.x * (blockDim.x / GT);
   auto take = [&]() {
     long long it = 0;
-    if (lane == 0) it = (long long)atomicAdd(ctr, 1ULL);
+    if (lane == 0) it = ngroups + (long long)atomicAdd(ctr, 1ULL);
     return it;
   };
   if (helper) {
-    post(0, take());
+    post(0, (long long)group * gridDim.x + blockIdx.x);
     post(1, take());
   }
   sync();
@@ -706,23 +669,6 @@ template <int NP, int NQ, bool PACKED>
 inline bool make_cell_tables(const gbc_ctx* c, CellTables<NP, NQ, PACKED>* t) {
   TablesEO<float, NP, NQ> f;
   if (!make_tables_eo<float, NP, NQ>(c, &f)) return false;
-  // N' = N diag(sqrt(w_q)) and its transpose; the z kinetic operators carry the x and y
-  // edges that the mass products of N' leave out
-  const HostTables& h = c->tab;
-  std::vector<double> Ni(NQ * NP), Nt(NP * NQ);
-  for (int i = 0; i < NP; ++i)
-    for (int q = 0; q < NQ; ++q)
-      Ni[q * NP + i] = Nt[i * NQ + q] = h.N1[i * NQ + q] * std::sqrt(h.gq_w[q]);
-  if (!make_eo<float, NQ, NP>(Ni, 1, &f.Ni) || !make_eo<float, NP, NQ>(Nt, 1, &f.Nt)) return false;
-  const double hxy = 0.25 * c->h[0] * c->h[1], hz = c->h[2];
-  std::vector<double> Gr(NP * NP), Gi(NP * NP);
-  for (int i = 0; i < NP; ++i)
-    for (int j = 0; j < NP; ++j) {
-      Gr[i * NP + j] = hxy * 0.5 * (2.0 / hz) * h.Ah[i * NP + j];
-      Gi[i * NP + j] = -hxy * 0.5 * c->k[2] * (h.Ch[i * NP + j] - h.Ch[j * NP + i]);
-    }
-  if (!make_eo<float, NP, NP>(Gr, 1, &f.Gr[2]) || !make_eo<float, NP, NP>(Gi, -1, &f.Gi[2]))
-    return false;
   for (int d = 0; d < 3; ++d) {
     cvt_table(f.B[d], t->B[d]);
     cvt_table(f.Gr[d], t->Gr[d]);
@@ -779,7 +725,6 @@ cudaError_t launch_cell_group_p(const CellJob* jobs, int n, cudaStream_t s) {
   if (!make_cell_tables<NP, NQ, PACKED>(c0, &tb)) return cudaErrorInvalidValue;
   const bool kpt = (c0->k[0] != 0.0 || c0->k[1] != 0.0 || c0->k[2] != 0.0);
   constexpr size_t smem = cell_smem<NP, VB, NT, MINB>();
-  constexpr int groups = NT / cell_group_threads<NP, VB>();
   int dev = 0, nsm = 0, per_sm = 0;
   cudaError_t err = cudaGetDevice(&dev);
   if (err != cudaSuccess) return err;
@@ -793,8 +738,7 @@ cudaError_t launch_cell_group_p(const CellJob* jobs, int n, cudaStream_t s) {
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NT, smem);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
-    const long long nblk =
-        std::min<long long>((item + groups - 1) / groups, (long long)nsm * per_sm);
+    const long long nblk = std::min<long long>(item, (long long)nsm * per_sm);
     e = cudaMemsetAsync(ctr, 0, sizeof(unsigned long long), s);
     if (e != cudaSuccess) return e;
     kern<<<(unsigned)nblk, NT, smem, s>>>(a, tb, ctr);

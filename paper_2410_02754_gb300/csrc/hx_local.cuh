@@ -1,20 +1,28 @@
-// Cell-level apply of the local spinor Hamiltonian, matrix-free (sum
-// factorisation), with atomic assembly into the global block.
+// Cell-level apply of the local spinor Hamiltonian for FP64 blocks (matrix-free, sum
+// factorisation), with atomic assembly into the global block or a per-cell result, and the
+// even-odd 1-D tables that the FP32 form (hx_cell.cuh) shares.
 //
 // Paper: Sec. IV.B.2 (extract X^(e) = R^(e) X, cell products, assemble
 // Y = sum_e R^(e)T Y^(e)) with the cell operator of Eq. FEHlocEl plus the
 // k-terms of Eq. FEHloc in per-cell Hermitian form.  The dense cell matrix
-// (N o V^eff) N^T of Sec. IV.B.1 is applied in factored form: interpolate to
-// the Gauss points with N (n_p -> n_q per direction), multiply by
-// w_q J [ (V + |k|^2/2) I + B . sigma ], test back with N^T.  The kinetic and
-// -i k.grad parts use the tensor structure of the shared reference matrices:
-//   K^k = sum_d G_d (x) B (x) B  (G_d in direction d, B in the other two),
-//   G_d = 1/2 A_d - (i/2) k_d (C^ - C^T),
-// applied as 7 one-dimensional contractions.
+// (N o V^eff) N^T of Sec. IV.B.1 is applied in factored form, as in hx_cell.cuh:
+//   a  = N'_x^T X,  t1 = B_x X,  t2 = G_x X                      x pencils
+//   u  = N'_y^T a;  c  = G_y t1 + B_y t2                          y pencils
+//   w  = N'_z F N'_z^T u + G'_z u;  k = B_z c                     z pencils
+//   Y^(e) = N'_x N'_y w + k                                       y, then x pencils
+// N' = N diag(sqrt(w_q)), G_d = 1/2 A_d - (i/2) k_d (C^ - C^T), G'_z = (h_x h_y / 4) G_z,
+// F = J [(V + |k|^2/2) I + B . sigma].
 //
-// Thread mapping: a CTA owns one cell and VB vectors; 64 "lanes" per vector
-// walk the pencils of each 1-D contraction.  Each vector has three padded
-// n_q^3 shared-memory buffers; per-point data are the two spin components.
+// Bound by the FP64 pipe (2 FMAs per clock and SM), so what counts is the number of FP64
+// instructions and that no lane of one is idle: a warp's instruction takes its 16 cycles
+// whether 2 or 32 lanes have a pencil.  A group of threads works on two (cell, vector) pairs
+// at a time, one thread per pencil and spin; with the two pairs and two spins side by side
+// the n_p^2 pencils of a stage fill 6.1 of 7 warps (p = 6; one pair a CTA filled 3.1 of 4), and
+// the pairs may be of different cells, so a block of one vector fills the lanes as well.  Two
+// independent groups per CTA (more at small p) keep the pipe busy across each other's
+// barriers; at p = 5 and 6 a warp owns whole z planes and only the z stage is between group
+// barriers.  Measured on one GB300 against one pair a CTA in seven stages: 6^3 cells, p = 6,
+// 64 vectors, k != 0: 4.84 -> 3.46 ms a launch; 16^3 cells, one vector, k = 0: 1.21 -> 0.92 ms.
 #pragma once
 
 #include <algorithm>
@@ -27,42 +35,27 @@
 namespace gbc {
 
 // One system of a launch: its blocks, fields, mesh and the first global work item.
-template <typename T> struct SysDesc {
-  const cplx<T>* X;
-  cplx<T>* Y;
-  cplx<T>* Ycell;    // non-null: per-cell results [E][n_p^3][2][nvec] instead of assembly
-  const T* fields;   // [E][4][NQ^3]
-  int ldx, nvec, vchunks, pad;
-  long long item0;   // work items of this system: [item0, item0 + E * vchunks)
+struct SysDesc {
+  const double2* X;
+  double2* Y;
+  double2* Ycell;        // non-null: per-cell results [E][n_p^3][2][nvec] instead of assembly
+  const double* fields;  // [E][NQ^3][4] J (V + |k|^2/2), J B_x, J B_y, J B_z
+  int ldx, nvec;
+  long long item0;       // work items (pairs of (cell, vector)s): [item0, item0 + ceil(E nvec / 2))
   MeshDev mesh;
 };
 
 // A launch covers up to GBC_MAX_BATCH systems that share p, the cell edges and
 // the k-point (hence the 1-D tables); items run over all systems.
-template <typename T> struct LocalArgs {
-  SysDesc<T> sys[GBC_MAX_BATCH];
+struct LocalArgs {
+  SysDesc sys[GBC_MAX_BATCH];
   int nsys;
   long long nitems;
 };
 
-template <typename C> __device__ __forceinline__ C cadd(C a, C b) { a.x += b.x; a.y += b.y; return a; }
-
-template <typename T> __device__ __forceinline__ void atomic_add_c(cplx<T>* p, cplx<T> v);
-template <> __device__ __forceinline__ void atomic_add_c<float>(float2* p, float2 v) {
-  atomicAdd(p, v);
-}
-template <> __device__ __forceinline__ void atomic_add_c<double>(double2* p, double2 v) {
+__device__ __forceinline__ void atomic_add_c(double2* p, double2 v) {
   atomicAdd(&p->x, v.x);
   atomicAdd(&p->y, v.y);
-}
-
-// point (x, y, z) -> index in a padded per-vector buffer
-// padded strides: y by NQ + 1, z by (NQ + 1) NQ + 1 points
-template <int NQ> __device__ __forceinline__ int pidx(int x, int y, int z) {
-  return x + y * (NQ + 1) + z * ((NQ + 1) * NQ + 1);
-}
-template <int NQ> __host__ __device__ constexpr int pbuf_points() {   // max pidx + 1
-  return (NQ - 1) * (1 + (NQ + 1) + ((NQ + 1) * NQ + 1)) + 1;
 }
 
 // ---------------------------------------------------------------------------
@@ -88,61 +81,11 @@ template <typename T, int NO, int NI> struct EO {
 
 template <typename T, int NP, int NQ> struct TablesEO {
   EO<T, NP, NP> B[3];    // 1-D Gauss mass h_d/2 B^               (symmetric)
-  EO<T, NP, NP> Gr[3];   // 1/2 A_d                                (symmetric)
-  EO<T, NP, NP> Gi[3];   // -1/2 k_d (C^ - C^T)                    (antisymmetric)
-  EO<T, NQ, NP> Ni;      // interpolation: y_q = sum_i l_i(xi_q) x_i (symmetric)
-  EO<T, NP, NQ> Nt;      // testing:       y_i = sum_q l_i(xi_q) x_q (symmetric)
+  EO<T, NP, NP> Gr[3];   // 1/2 A_d (z: times h_x h_y / 4)          (symmetric)
+  EO<T, NP, NP> Gi[3];   // -1/2 k_d (C^ - C^T) (z: the same)       (antisymmetric)
+  EO<T, NQ, NP> Ni;      // N'^T: interpolation times sqrt(w_q)      (symmetric)
+  EO<T, NP, NQ> Nt;      // N'                                       (symmetric)
 };
-
-template <int S, typename T, int NO, int NI, typename C>
-__device__ __forceinline__ void eo_apply(const EO<T, NO, NI>& M, const C (&x)[NI], C (&y)[NO]) {
-  constexpr int HI = NI / 2, HO = (NO + 1) / 2;
-  C e[HI > 0 ? HI : 1], o[HI > 0 ? HI : 1];
-#pragma unroll
-  for (int j = 0; j < HI; ++j) {
-    e[j].x = x[j].x + x[NI - 1 - j].x;
-    e[j].y = x[j].y + x[NI - 1 - j].y;
-    o[j].x = x[j].x - x[NI - 1 - j].x;
-    o[j].y = x[j].y - x[NI - 1 - j].y;
-  }
-#pragma unroll
-  for (int i = 0; i < HO; ++i) {
-    T er = 0, ei = 0, orr = 0, oi = 0;
-#pragma unroll
-    for (int j = 0; j < HI; ++j) {
-      er += M.E[i][j] * e[j].x;
-      ei += M.E[i][j] * e[j].y;
-      orr += M.O[i][j] * o[j].x;
-      oi += M.O[i][j] * o[j].y;
-    }
-    if (NI & 1) {
-      er += M.Mid[i] * x[HI].x;
-      ei += M.Mid[i] * x[HI].y;
-    }
-    y[i].x = er + orr;
-    y[i].y = ei + oi;
-    if (NO - 1 - i != i) {
-      y[NO - 1 - i].x = S * (er - orr);
-      y[NO - 1 - i].y = S * (ei - oi);
-    }
-  }
-}
-
-// complex operator Gr + i Gi (Gr symmetric, Gi antisymmetric) on complex data
-template <bool KPT, typename T, int N, typename C>
-__device__ __forceinline__ void g_apply(const EO<T, N, N>& Gr, const EO<T, N, N>& Gi,
-                                        const C (&x)[N], C (&y)[N]) {
-  eo_apply<1>(Gr, x, y);
-  if (KPT) {
-    C t[N];
-    eo_apply<-1>(Gi, x, t);
-#pragma unroll
-    for (int i = 0; i < N; ++i) {
-      y[i].x -= t[i].y;
-      y[i].y += t[i].x;
-    }
-  }
-}
 
 // host: even-odd split of a dense row-major NO x NI matrix (checks the symmetry)
 template <typename T, int NO, int NI>
@@ -172,13 +115,14 @@ inline bool make_tables_eo(const gbc_ctx* c, TablesEO<T, NP, NQ>* t) {
   const HostTables& h = c->tab;
   bool ok = true;
   for (int d = 0; d < 3; ++d) {
-    const double hd = c->h[d];
+    // the mass products of N' leave out the edges, which the z operators carry for x and y
+    const double hd = c->h[d], f = d == 2 ? 0.25 * c->h[0] * c->h[1] : 1.0;
     std::vector<double> B(NP * NP), Gr(NP * NP), Gi(NP * NP);
     for (int i = 0; i < NP; ++i)
       for (int j = 0; j < NP; ++j) {
         B[i * NP + j] = 0.5 * hd * h.Bh[i * NP + j];
-        Gr[i * NP + j] = 0.5 * (2.0 / hd) * h.Ah[i * NP + j];
-        Gi[i * NP + j] = -0.5 * c->k[d] * (h.Ch[i * NP + j] - h.Ch[j * NP + i]);
+        Gr[i * NP + j] = f * 0.5 * (2.0 / hd) * h.Ah[i * NP + j];
+        Gi[i * NP + j] = -f * 0.5 * c->k[d] * (h.Ch[i * NP + j] - h.Ch[j * NP + i]);
       }
     ok = ok && make_eo<T, NP, NP>(B, 1, &t->B[d]) && make_eo<T, NP, NP>(Gr, 1, &t->Gr[d]) &&
          make_eo<T, NP, NP>(Gi, -1, &t->Gi[d]);
@@ -186,293 +130,452 @@ inline bool make_tables_eo(const gbc_ctx* c, TablesEO<T, NP, NQ>* t) {
   std::vector<double> Ni(NQ * NP), Nt(NP * NQ);
   for (int i = 0; i < NP; ++i)
     for (int q = 0; q < NQ; ++q) {
-      Ni[q * NP + i] = h.N1[i * NQ + q];
-      Nt[i * NQ + q] = h.N1[i * NQ + q];
+      Ni[q * NP + i] = Nt[i * NQ + q] = h.N1[i * NQ + q] * std::sqrt(h.gq_w[q]);
     }
   ok = ok && make_eo<T, NQ, NP>(Ni, 1, &t->Ni) && make_eo<T, NP, NQ>(Nt, 1, &t->Nt);
   return ok;
 }
 
-template <typename T, int NP, int NQ, bool KPT, int VB>
-__global__ void __launch_bounds__(VB * 64, sizeof(T) == 4 ? 4 : 2)
-hx_local_kernel(const __grid_constant__ LocalArgs<T> a, const TablesEO<T, NP, NQ> tb) {
-  using C = cplx<T>;
-  constexpr int TPV = 64;
-  constexpr int NT = VB * TPV;
-  constexpr int BUF = pbuf_points<NQ>();             // points per padded buffer
-  constexpr int NQ3 = NQ * NQ * NQ;
-  // per-vector stride = 8 (mod 16) complex: threads of neighbouring work units
-  // (vector fastest, then spin, then pencil) fall into distinct banks
-  constexpr int VBASE = 3 * BUF * 2;
-  constexpr int VSTRIDE = VBASE + ((24 - VBASE % 16) % 16);
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  C* buf = reinterpret_cast<C*>(smem_raw);
-  auto Ab = [&](int v) { return buf + v * VSTRIDE; };
-  auto Bb = [&](int v) { return buf + v * VSTRIDE + BUF * 2; };
-  auto Cb = [&](int v) { return buf + v * VSTRIDE + 2 * BUF * 2; };
 
-  const int v0 = threadIdx.x % VB;      // vector of this thread for gathering
-  const int lane = threadIdx.x / VB;
-  const long long nitems = a.nitems;
-  auto locate = [&](long long it) {
-    int q = 0;
+// ---------------------------------------------------------------------------
+// layout and grouping shared with the FP32 form (16-byte elements: here one spin of one
+// (cell, vector), there both spins of one vector)
+// ---------------------------------------------------------------------------
+// Point strides (y, z) of the n_p^3 buffers (A, T2) and of T1 (up to n_q x n_q x n_p
+// points).  A quarter-warp's 16-byte accesses (VB vectors, then neighbouring pencils) fall
+// in the 8 distinct bank groups when neighbouring pencils are an odd number of points
+// apart, which these strides give in every stage's pencil direction, and the vectors
+// start 8 / VB groups apart (cell_vpoints).
+template <int NP> struct CellLayout;
+template <> struct CellLayout<3> { static constexpr int AY = 3, AZ = 9, QY = 5, QZ = 23; };
+template <> struct CellLayout<4> { static constexpr int AY = 5, AZ = 21, QY = 5, QZ = 25; };
+template <> struct CellLayout<5> { static constexpr int AY = 5, AZ = 25, QY = 7, QZ = 43; };
+template <> struct CellLayout<6> { static constexpr int AY = 7, AZ = 43, QY = 7, QZ = 51; };
+template <> struct CellLayout<7> { static constexpr int AY = 7, AZ = 49, QY = 9, QZ = 73; };
+template <> struct CellLayout<8> { static constexpr int AY = 9, AZ = 72, QY = 9, QZ = 81; };
+template <int NP> __host__ __device__ constexpr int cell_bufa() {   // points of A / T2
+  return (NP - 1) * (1 + CellLayout<NP>::AY + CellLayout<NP>::AZ) + 1;
+}
+template <int NP> __host__ __device__ constexpr int cell_bufq() {   // points of T1
+  return NP * (1 + CellLayout<NP>::QY) + (NP - 1) * CellLayout<NP>::QZ + 1;
+}
+template <int NP, int VB> __host__ __device__ constexpr int cell_vpoints() {
+  // points per vector: [A | T2 | T1], padded to 8 / VB mod 8
+  static_assert(VB == 2 || VB == 4, "VB");
+  constexpr int n = 2 * cell_bufa<NP>() + cell_bufq<NP>(), r = 8 / VB;
+  return n + ((8 + r - n % 8) % 8);
+}
+// Threads of a group: about one per pencil of a vector's x stage.  At p = 3 and 4 small
+// groups are worth more than full rounds (12^3 cells, p = 4, 96 vectors: 446 us a launch at
+// 128 threads, 642 at 256).
+template <int NP, int VB> __host__ __device__ constexpr int cell_group_threads() {
+  constexpr int g4[9] = {0, 0, 0, 64, 128, 128, 256, 256, 256};
+  constexpr int g2[9] = {0, 0, 0, 32, 64, 64, 128, 128, 128};
+  return VB == 4 ? g4[NP] : g2[NP];
+}
+// Whether each warp owns whole z planes of a cell (see cell_body): where a plane's pencils
+// fill a warp and a warp is left over (p = 6, 4 vectors: 28 to 32 lanes, 8.34 -> 7.62 ms a
+// launch on 16^3 cells, 256 vectors; p = 5: 872 -> 815 us on 12^3 cells, 96 vectors).  At
+// p = 7 a plane has 36 pencils a vector quad and every warp a plane (1048 -> 1090 us), at
+// p <= 4 it leaves lanes idle (460 -> 575 us).
+template <int NP> __host__ __device__ constexpr bool cell_planes() { return NP == 6 || NP == 7; }
+constexpr int kNoNode = -(1 << 29);   // offset of a direction with no free node (Dirichlet face)
+
+// ---------------------------------------------------------------------------
+// the FP64 kernel
+// ---------------------------------------------------------------------------
+// even and odd parts (and the middle point of an odd count) of a pencil of NI points
+template <int NI> struct PartsD {
+  static constexpr int HI = NI / 2;
+  double2 e[HI], o[HI], m;
+};
+template <int NI> __device__ __forceinline__ void set_part(PartsD<NI>& s, int j, double2 a, double2 b) {
+  s.e[j] = make_double2(a.x + b.x, a.y + b.y);
+  s.o[j] = make_double2(a.x - b.x, a.y - b.y);
+}
+template <int NI, typename F> __device__ __forceinline__ void load_parts(PartsD<NI>& s, F ld) {
 #pragma unroll
-    for (int r = 1; r < GBC_MAX_BATCH; ++r)
-      if (r < a.nsys && it >= a.sys[r].item0) q = r;
-    return q;
+  for (int j = 0; j < NI / 2; ++j) set_part(s, j, ld(j), ld(NI - 1 - j));
+  if (NI & 1) s.m = ld(NI / 2);
+}
+// rows i and NO-1-i of a product: y_i = e + o, y_{NO-1-i} = e - o (the middle row is e)
+struct AccD { double2 e, o; };
+template <bool FIRST, int NO, int NI>
+__device__ __forceinline__ void row_sym(const EO<double, NO, NI>& M, int i, const PartsD<NI>& s, AccD& a) {
+#pragma unroll
+  for (int j = 0; j < NI / 2; ++j) {
+    if (FIRST && j == 0) {
+      a.e = make_double2(M.E[i][j] * s.e[j].x, M.E[i][j] * s.e[j].y);
+      if (NO - 1 - i != i) a.o = make_double2(M.O[i][j] * s.o[j].x, M.O[i][j] * s.o[j].y);
+    } else {
+      a.e.x += M.E[i][j] * s.e[j].x;
+      a.e.y += M.E[i][j] * s.e[j].y;
+      if (NO - 1 - i != i) {
+        a.o.x += M.O[i][j] * s.o[j].x;
+        a.o.y += M.O[i][j] * s.o[j].y;
+      }
+    }
+  }
+  if (NI & 1) {
+    a.e.x += M.Mid[i] * s.m.x;
+    a.e.y += M.Mid[i] * s.m.y;
+  }
+}
+// a += i M x for a centro-antisymmetric M (the odd chain feeds the even accumulator and the
+// even chain the odd one)
+template <int NO, int NI>
+__device__ __forceinline__ void row_anti(const EO<double, NO, NI>& M, int i, const PartsD<NI>& s, AccD& a) {
+#pragma unroll
+  for (int j = 0; j < NI / 2; ++j) {
+    a.e.x -= M.O[i][j] * s.o[j].y;
+    a.e.y += M.O[i][j] * s.o[j].x;
+    if (NO - 1 - i != i) {
+      a.o.x -= M.E[i][j] * s.e[j].y;
+      a.o.y += M.E[i][j] * s.e[j].x;
+    }
+  }
+  if ((NI & 1) && NO - 1 - i != i) {
+    a.o.x -= M.Mid[i] * s.m.y;
+    a.o.y += M.Mid[i] * s.m.x;
+  }
+}
+template <int NO, typename F> __device__ __forceinline__ void put_rows(int i, const AccD& a, F st) {
+  if (NO - 1 - i == i) {
+    st(i, a.e);
+  } else {
+    st(i, make_double2(a.e.x + a.o.x, a.e.y + a.o.y));
+    st(NO - 1 - i, make_double2(a.e.x - a.o.x, a.e.y - a.o.y));
+  }
+}
+__device__ __forceinline__ void cp_async16z(void* dst, const void* src, int src_bytes) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)),
+               "l"(src), "r"(src_bytes)
+               : "memory");
+}
+
+constexpr int kHxThreads = 512;
+// one group: 4 lane vectors (two (cell, vector)s x two spins) of [A | T2 | T1], the node
+// offsets and records of three items
+struct HxItem { int q, e[2], v[2], pad[3]; };   // system, cells (negative: none), vectors
+constexpr int kHxSlots = 3;
+template <int NP> __host__ __device__ constexpr size_t hx_group_smem() {
+  return sizeof(double2) * 4 * (size_t)cell_vpoints<NP, 4>() + kHxSlots * (sizeof(HxItem) + 2 * 24 * sizeof(int));
+}
+template <int NP> __host__ __device__ constexpr int hx_groups() { return kHxThreads / cell_group_threads<NP, 4>(); }
+
+template <int NP, int NQ, bool KPT>
+__global__ void __launch_bounds__(kHxThreads, 1)
+hx_local_kernel(const __grid_constant__ LocalArgs a, const __grid_constant__ TablesEO<double, NP, NQ> tb) {
+  constexpr int GT = cell_group_threads<NP, 4>(), NW = GT / 32;
+  constexpr int BA = cell_bufa<NP>(), VS = cell_vpoints<NP, 4>();
+  constexpr int NQ3 = NQ * NQ * NQ, HP = (NP + 1) / 2, HQ = (NQ + 1) / 2;
+  using L = CellLayout<NP>;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int group = threadIdx.x / GT;
+  double2* sm = reinterpret_cast<double2*>(smem_raw + group * hx_group_smem<NP>());
+  // lane vector w = 2 * slot + spin: point pidx at Buf(w)[pidx]
+  auto Ab = [&](int w) { return sm + w * VS; };
+  auto T2b = [&](int w) { return sm + w * VS + BA; };
+  auto T1b = [&](int w) { return sm + w * VS + 2 * BA; };
+  HxItem* rec0 = reinterpret_cast<HxItem*>(sm + 4 * VS);
+  int* noff0 = reinterpret_cast<int*>(rec0 + kHxSlots);
+  auto pa = [](int x, int y, int z) { return x + y * L::AY + z * L::AZ; };
+  auto pq = [](int x, int y, int z) { return x + y * L::QY + z * L::QZ; };
+  // odd groups number their warps backwards, so partly filled rounds fall on other schedulers
+  const int tid0 = threadIdx.x % GT;
+  const int tid = (group & 1) == 0 ? tid0 : ((NW - 1 - tid0 / 32) * 32 + (tid0 & 31));
+  const int lane = tid & 31, warp = tid / 32;
+  auto sync = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(1 + group), "n"(GT) : "memory"); };
+  constexpr bool PL = cell_planes<NP>();
+  constexpr int PZW = PL ? (NP + NW - 1) / NW : NP;
+  const int z0 = PL ? min(NP, warp * PZW) : 0, nz = PL ? min(NP - z0, PZW) : NP;
+  constexpr int US = PL ? 32 : GT;
+  const int ut = PL ? lane : tid;
+  auto psync = [&]() {
+    if (PL) __syncwarp();
+    else sync();
+  };
+  const long long ngroups = (long long)gridDim.x * hx_groups<NP>();
+  // a CTA's groups take items gridDim.x apart, so few items spread over the SMs
+  const long long first = (long long)group * gridDim.x + blockIdx.x;
+
+  auto rec = [&](int n) -> HxItem& { return rec0[n % kHxSlots]; };
+  auto noff = [&](int n, int slot) { return noff0 + (n % kHxSlots) * 48 + slot * 24; };
+  // the group's last warp: record and node offsets of the group's n-th item
+  // (noff[0][ix] + noff[8 + iy] + noff[16 + iz], negative on a Dirichlet face)
+  auto post = [&](int n) {
+    const long long it = first + n * ngroups;
+    HxItem r{0, {-1, -1}, {0, 0}, {0, 0, 0}};
+    if (it < a.nitems) {
+      for (int k = 1; k < a.nsys; ++k)
+        if (it >= a.sys[k].item0) r.q = k;
+      const SysDesc& g = a.sys[r.q];
+      const long long li = 2 * (it - g.item0), n2 = (long long)g.mesh.E * g.nvec;
+      for (int i = 0; i < 2; ++i)
+        if (li + i < n2) {
+          r.e[i] = (int)((li + i) / g.nvec);
+          r.v[i] = (int)((li + i) - (long long)r.e[i] * g.nvec);
+        }
+    }
+    if (lane == 0) rec(n) = r;
+    if (lane < 3 * NP) {
+      const MeshDev& m = a.sys[r.q].mesh;
+      const int dd = lane / NP, i = lane % NP;
+      for (int sl = 0; sl < 2; ++sl) {
+        const int e = r.e[sl];
+        if (e < 0) continue;
+        const int c = dd == 0 ? e % m.ncell[0] : dd == 1 ? (e / m.ncell[0]) % m.ncell[1] : e / (m.ncell[0] * m.ncell[1]);
+        const int gc = c * m.p + i;
+        int f;
+        if (m.periodic[dd]) f = gc >= m.period[dd] ? gc - m.period[dd] : gc;
+        else f = (gc == 0 || gc == m.period[dd]) ? -1 : gc - 1;
+        const int scale = dd == 0 ? 1 : dd == 1 ? m.nfree[0] : m.nfree[0] * m.nfree[1];
+        noff(n, sl)[dd * 8 + i] = f < 0 ? kNoNode : f * scale;
+      }
+    }
+  };
+  // asynchronous gather of the thread's planes of item n into A, one (lane vector, x pencil)
+  // at a time; zeros on Dirichlet faces and for an absent second (cell, vector)
+  auto gather = [&](int n) {
+    const HxItem it = rec(n);
+    const SysDesc& g = a.sys[it.q];
+    for (int i = ut; i < 4 * NP * nz; i += US) {
+      const int w = i & 3, pen = i >> 2, sl = w >> 1;
+      const int y = pen % NP, z = z0 + pen / NP;
+      const int* no = noff(n, sl);
+      const bool have = (sl ? it.e[1] : it.e[0]) >= 0;
+      const int Iyz = have ? no[8 + y] + no[16 + z] : kNoNode;
+      double2* dst = &Ab(w)[pa(0, y, z)];
+      const double2* src = g.X + (long long)(w & 1) * g.ldx + (sl ? it.v[1] : it.v[0]);
+#pragma unroll
+      for (int x = 0; x < NP; ++x) {
+        const int I = have ? Iyz + no[x] : -1;
+        const bool ok = I >= 0 && GBC_IN_RANGE(GBC_SITE_HX64, I, g.mesh.M);
+        cp_async16z(dst + x, ok ? src + 2 * (long long)I * g.ldx : g.X, ok ? 16 : 0);
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
   };
 
-  // work units of the single-spin stages: u -> (vector, spin, pencil), vector fastest
-  constexpr int XU = VB * NP * NP * 2;          // units of the x-pencil stages
-  constexpr int XR = (XU + NT - 1) / NT;        // rounds per thread
+  const bool helper = warp == NW - 1;
+  if (helper) {
+    post(0);
+    post(1);
+  }
+  sync();
+  if (rec(0).e[0] >= 0) gather(0);
+#pragma unroll 1
+  for (int n = 0;; ++n) {
+    const HxItem item = rec(n);
+    if (item.e[0] < 0) break;
+    const SysDesc& d = a.sys[item.q];
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    psync();
 
-  for (long long item = blockIdx.x; item < nitems; item += gridDim.x) {
-    const SysDesc<T>& d = a.sys[locate(item)];
-    const long long li = item - d.item0;
-    const int e = (int)(li / d.vchunks);
-    const int vbase = (int)(li % d.vchunks) * VB;
-    const int nx = d.mesh.ncell[0], ny = d.mesh.ncell[1];
-    const int cx = e % nx, cy = (e / nx) % ny, cz = e / (nx * ny);
+    // ---- x pencils: T1 = N'^T X, A = B_x X (in place), T2 = G_x X
+    for (int u = ut; u < 4 * NP * nz; u += US) {
+      const int w = u & 3, pen = u >> 2;
+      const int y = pen % NP, z = z0 + pen / NP;
+      double2 *A = Ab(w) + pa(0, y, z), *K = T2b(w) + pa(0, y, z), *Q = T1b(w) + pq(0, y, z);
+      PartsD<NP> s;
+      load_parts(s, [&](int j) { return A[j]; });
+#pragma unroll
+      for (int i = 0; i < HQ; ++i) {
+        AccD r;
+        row_sym<true, NQ>(tb.Ni, i, s, r);
+        put_rows<NQ>(i, r, [&](int k, double2 v) { Q[k] = v; });
+      }
+#pragma unroll
+      for (int i = 0; i < HP; ++i) {
+        AccD r;
+        row_sym<true, NP>(tb.B[0], i, s, r);
+        put_rows<NP>(i, r, [&](int k, double2 v) { A[k] = v; });
+        row_sym<true, NP>(tb.Gr[0], i, s, r);
+        if (KPT) row_anti<NP>(tb.Gi[0], i, s, r);
+        put_rows<NP>(i, r, [&](int k, double2 v) { K[k] = v; });
+      }
+    }
+    psync();
 
-    // ---- extract X^(e) (both spins) into A
-    {
-      const int vec = vbase + v0;
-      const bool vok = vec < d.nvec;
-      for (int i = lane; i < NP * NP * NP; i += TPV) {
-        const int ix = i % NP, iy = (i / NP) % NP, iz = i / (NP * NP);
-        const long long I = gbc_node(d.mesh, cx, cy, cz, ix, iy, iz);
-        C u = cmake<C>(0, 0), dn = cmake<C>(0, 0);
-        if (I >= 0 && vok && GBC_IN_RANGE(GBC_SITE_HX64, I, d.mesh.M)) {
-          u = d.X[(I * 2 + 0) * d.ldx + vec];
-          dn = d.X[(I * 2 + 1) * d.ldx + vec];
-        }
-        const int q = pidx<NQ>(ix, iy, iz);
-        Ab(v0)[2 * q] = u;
-        Ab(v0)[2 * q + 1] = dn;
+    // ---- y pencils (in place): T1 = N'^T T1; T2 = G_y A + B_y T2
+    for (int u = ut; u < 4 * NQ * nz; u += US) {
+      double2* Q = T1b(u & 3) + pq((u >> 2) % NQ, 0, z0 + (u >> 2) / NQ);
+      PartsD<NP> s;
+      load_parts(s, [&](int j) { return Q[j * L::QY]; });
+#pragma unroll
+      for (int i = 0; i < HQ; ++i) {
+        AccD r;
+        row_sym<true, NQ>(tb.Ni, i, s, r);
+        put_rows<NQ>(i, r, [&](int k, double2 v) { Q[k * L::QY] = v; });
       }
     }
-    const T* __restrict__ fld = d.fields + (size_t)e * 4 * NQ3;   // read through L1
-    __syncthreads();
+    for (int u = (ut + US - 4 * NQ * nz % US) % US; u < 4 * NP * nz; u += US) {
+      const int w = u & 3, o = pa((u >> 2) % NP, 0, z0 + (u >> 2) / NP);
+      const double2* A = Ab(w) + o;
+      double2* K = T2b(w) + o;
+      PartsD<NP> s1, s2;
+      load_parts(s1, [&](int j) { return A[j * L::AY]; });
+      load_parts(s2, [&](int j) { return K[j * L::AY]; });
+#pragma unroll
+      for (int i = 0; i < HP; ++i) {
+        AccD r;
+        row_sym<true, NP>(tb.Gr[1], i, s1, r);
+        if (KPT) row_anti<NP>(tb.Gi[1], i, s1, r);
+        row_sym<false, NP>(tb.B[1], i, s2, r);
+        put_rows<NP>(i, r, [&](int k, double2 v) { K[k * L::AY] = v; });
+      }
+    }
+    psync();
+    // the planes of A are free: start the next item's gather behind the remaining stages
+    if (rec(n + 1).e[0] >= 0) gather(n + 1);
+    if (PL) sync();
 
-    // ===== kinetic / k part: Y = G_x(B_y B_z X) + B_x(G_y B_z X + B_y G_z X)
-    // z-stage: T1 = B_z X -> Bb, T2 = G_z X -> Cb
-    for (int u = threadIdx.x; u < VB * NP * NP * 2; u += NT) {
-      const int v = u % VB, s = (u / VB) & 1, pen = u / (2 * VB);
-      const int x = pen % NP, y = pen / NP;
-      C in[NP], t1[NP], t2[NP];
+    // ---- z pencils (in place): T1 = N' F N'^T T1 + G'_z T1; the two spins of a pencil are on
+    // neighbouring lanes and swap their values by shuffle
+    constexpr int UZ = 4 * NQ * NQ, ROUNDS = (UZ + GT - 1) / GT;
+#pragma unroll 1
+    for (int rd = 0; rd < ROUNDS; ++rd) {
+      const int uu = tid + rd * GT;
+      const bool act = uu < UZ;
+      const int u = act ? uu : (uu & 1);
+      const int w = u & 3, x = (u >> 2) % NQ, y = (u >> 2) / NQ;
+      double2* Q = T1b(w) + pq(x, y, 0);
+      const int e = max(0, (w >> 1) ? item.e[1] : item.e[0]);
+      const double2* __restrict__ fld = reinterpret_cast<const double2*>(d.fields) + 2 * (size_t)e * NQ3;
+      PartsD<NP> s;
+      load_parts(s, [&](int j) { return Q[j * L::QZ]; });
+      // up:   (V + bz) u + (bx - i by) d
+      // down: (V - bz) d + (bx + i by) u
+      auto spin_op = [&](int q, double2 own) {
+        const double2 oth = make_double2(__shfl_xor_sync(0xffffffffu, own.x, 1),
+                                         __shfl_xor_sync(0xffffffffu, own.y, 1));
+        const double2 f0 = __ldg(fld + 2 * ((q * NQ + y) * NQ + x)), f1 = __ldg(fld + 2 * ((q * NQ + y) * NQ + x) + 1);
+        const double dg = (w & 1) ? f0.x - f1.y : f0.x + f1.y, by = (w & 1) ? -f1.x : f1.x;
+        return make_double2(dg * own.x + f0.y * oth.x + by * oth.y, dg * own.y + f0.y * oth.y - by * oth.x);
+      };
+      PartsD<NQ> t;
 #pragma unroll
-      for (int j = 0; j < NP; ++j) in[j] = Ab(v)[2 * pidx<NQ>(x, y, j) + s];
-      eo_apply<1>(tb.B[2], in, t1);
-      g_apply<KPT>(tb.Gr[2], tb.Gi[2], in, t2);
+      for (int i = 0; i < HQ; ++i) {
+        AccD r;
+        double2 r0, r1;
+        row_sym<true, NQ>(tb.Ni, i, s, r);
+        put_rows<NQ>(i, r, [&](int k, double2 v) {
+          if (k == i) r0 = spin_op(k, v);
+          else r1 = spin_op(k, v);
+        });
+        if (NQ - 1 - i == i) t.m = r0;
+        else set_part(t, i, r0, r1);
+      }
 #pragma unroll
-      for (int i = 0; i < NP; ++i) {
-        Bb(v)[2 * pidx<NQ>(x, y, i) + s] = t1[i];
-        Cb(v)[2 * pidx<NQ>(x, y, i) + s] = t2[i];
+      for (int i = 0; i < HP; ++i) {
+        AccD r;
+        row_sym<true, NP>(tb.Nt, i, t, r);
+        row_sym<false, NP>(tb.Gr[2], i, s, r);
+        if (KPT) row_anti<NP>(tb.Gi[2], i, s, r);
+        if (act) put_rows<NP>(i, r, [&](int k, double2 v) { Q[k * L::QZ] = v; });
       }
     }
-    __syncthreads();
-    // y-stage (in place): U1 = B_y T1 -> Bb, U2 = G_y T1 + B_y T2 -> Cb
-    for (int u = threadIdx.x; u < VB * NP * NP * 2; u += NT) {
-      const int v = u % VB, s = (u / VB) & 1, pen = u / (2 * VB);
-      const int x = pen % NP, z = pen / NP;
-      C t1[NP], t2[NP], u1[NP], u2[NP], w2[NP];
+    // T2 = B_z T2 (the threads left idle by the last round above take the first units)
+    for (int u = (tid + GT - UZ % GT) % GT; u < 4 * NP * NP; u += GT) {
+      double2* K = T2b(u & 3) + pa((u >> 2) % NP, (u >> 2) / NP, 0);
+      PartsD<NP> s;
+      load_parts(s, [&](int j) { return K[j * L::AZ]; });
 #pragma unroll
-      for (int j = 0; j < NP; ++j) {
-        t1[j] = Bb(v)[2 * pidx<NQ>(x, j, z) + s];
-        t2[j] = Cb(v)[2 * pidx<NQ>(x, j, z) + s];
-      }
-      eo_apply<1>(tb.B[1], t1, u1);
-      g_apply<KPT>(tb.Gr[1], tb.Gi[1], t1, u2);
-      eo_apply<1>(tb.B[1], t2, w2);
-#pragma unroll
-      for (int i = 0; i < NP; ++i) {
-        Bb(v)[2 * pidx<NQ>(x, i, z) + s] = u1[i];
-        Cb(v)[2 * pidx<NQ>(x, i, z) + s] = cadd(u2[i], w2[i]);
+      for (int i = 0; i < HP; ++i) {
+        AccD r;
+        row_sym<true, NP>(tb.B[2], i, s, r);
+        put_rows<NP>(i, r, [&](int k, double2 v) { K[k * L::AZ] = v; });
       }
     }
-    __syncthreads();
-    // x-stage: Y = G_x U1 + B_x U2, kept in registers per work unit
-    C yacc[XR][NP];
-#pragma unroll
-    for (int r = 0; r < XR; ++r) {
-      const int u = threadIdx.x + r * NT;
-      if (u >= XU) break;
-      const int v = u % VB, s = (u / VB) & 1, pen = u / (2 * VB);
-      const int y = pen % NP, z = pen / NP;
-      C u1[NP], u2[NP], w2[NP];
-#pragma unroll
-      for (int j = 0; j < NP; ++j) {
-        u1[j] = Bb(v)[2 * pidx<NQ>(j, y, z) + s];
-        u2[j] = Cb(v)[2 * pidx<NQ>(j, y, z) + s];
-      }
-      g_apply<KPT>(tb.Gr[0], tb.Gi[0], u1, yacc[r]);
-      eo_apply<1>(tb.B[0], u2, w2);
-#pragma unroll
-      for (int i = 0; i < NP; ++i) yacc[r][i] = cadd(yacc[r][i], w2[i]);
-    }
-    __syncthreads();
+    if (helper) post(n + 2);   // read after the group barrier that follows
+    sync();
 
-    // ===== V_eff / B_xc part through the Gauss points
-    // interp x: A (np,np,np) -> Bb (nq,np,np)
-    for (int u = threadIdx.x; u < VB * NP * NP * 2; u += NT) {
-      const int v = u % VB, s = (u / VB) & 1, pen = u / (2 * VB);
-      const int y = pen % NP, z = pen / NP;
-      C in[NP], out[NQ];
+    // ---- y pencils (in place): T1 = N' T1
+    for (int u = ut; u < 4 * NQ * nz; u += US) {
+      double2* Q = T1b(u & 3) + pq((u >> 2) % NQ, 0, z0 + (u >> 2) / NQ);
+      PartsD<NQ> s;
+      load_parts(s, [&](int j) { return Q[j * L::QY]; });
 #pragma unroll
-      for (int j = 0; j < NP; ++j) in[j] = Ab(v)[2 * pidx<NQ>(j, y, z) + s];
-      eo_apply<1>(tb.Ni, in, out);
-#pragma unroll
-      for (int q = 0; q < NQ; ++q) Bb(v)[2 * pidx<NQ>(q, y, z) + s] = out[q];
-    }
-    __syncthreads();
-    // interp y: Bb (nq,np,np) -> Cb (nq,nq,np)
-    for (int u = threadIdx.x; u < VB * NQ * NP * 2; u += NT) {
-      const int v = u % VB, s = (u / VB) & 1, pen = u / (2 * VB);
-      const int x = pen % NQ, z = pen / NQ;
-      C in[NP], out[NQ];
-#pragma unroll
-      for (int j = 0; j < NP; ++j) in[j] = Bb(v)[2 * pidx<NQ>(x, j, z) + s];
-      eo_apply<1>(tb.Ni, in, out);
-#pragma unroll
-      for (int q = 0; q < NQ; ++q) Cb(v)[2 * pidx<NQ>(x, q, z) + s] = out[q];
-    }
-    __syncthreads();
-    // interp z + pointwise spin operator: Cb (nq,nq,np) -> Bb (nq,nq,nq), both spins
-    for (int u = threadIdx.x; u < VB * NQ * NQ; u += NT) {
-      const int v = u % VB, pen = u / VB;
-      const int x = pen % NQ, y = pen / NQ;
-      C iu[NP], id[NP], ou[NQ], od[NQ];
-#pragma unroll
-      for (int j = 0; j < NP; ++j) {
-        iu[j] = Cb(v)[2 * pidx<NQ>(x, y, j)];
-        id[j] = Cb(v)[2 * pidx<NQ>(x, y, j) + 1];
-      }
-      eo_apply<1>(tb.Ni, iu, ou);
-      eo_apply<1>(tb.Ni, id, od);
-#pragma unroll
-      for (int q = 0; q < NQ; ++q) {
-        const int qq = (q * NQ + y) * NQ + x;
-        const T V = __ldg(fld + qq), bx = __ldg(fld + NQ3 + qq), by = __ldg(fld + 2 * NQ3 + qq),
-                bz = __ldg(fld + 3 * NQ3 + qq);
-        const T ur = ou[q].x, ui = ou[q].y, dr = od[q].x, di = od[q].y;
-        // [(V + bz) u + (bx - i by) d ; (bx + i by) u + (V - bz) d]
-        Bb(v)[2 * pidx<NQ>(x, y, q)] =
-            cmake<C>((V + bz) * ur + bx * dr + by * di, (V + bz) * ui + bx * di - by * dr);
-        Bb(v)[2 * pidx<NQ>(x, y, q) + 1] =
-            cmake<C>(bx * ur - by * ui + (V - bz) * dr, bx * ui + by * ur + (V - bz) * di);
+      for (int i = 0; i < HP; ++i) {
+        AccD r;
+        row_sym<true, NP>(tb.Nt, i, s, r);
+        put_rows<NP>(i, r, [&](int k, double2 v) { Q[k * L::QY] = v; });
       }
     }
-    __syncthreads();
-    // test z: Bb (nq,nq,nq) -> Cb (nq,nq,np)
-    for (int u = threadIdx.x; u < VB * NQ * NQ * 2; u += NT) {
-      const int v = u % VB, s = (u / VB) & 1, pen = u / (2 * VB);
-      const int x = pen % NQ, y = pen / NQ;
-      C in[NQ], out[NP];
+    psync();
+
+    // ---- x pencils: N' T1 + T2, assembled
+    for (int u = ut; u < 4 * NP * nz; u += US) {
+      const int w = u & 3, pen = u >> 2, sl = w >> 1, sp = w & 1;
+      const int y = pen % NP, z = z0 + pen / NP;
+      const int e = sl ? item.e[1] : item.e[0], vec = sl ? item.v[1] : item.v[0];
+      if (e < 0) continue;
+      const double2 *Q = T1b(w) + pq(0, y, z), *K = T2b(w) + pa(0, y, z);
+      const int* no = noff(n, sl);
+      const int Iyz = no[8 + y] + no[16 + z];
+      PartsD<NQ> s;
+      load_parts(s, [&](int j) { return Q[j]; });
 #pragma unroll
-      for (int q = 0; q < NQ; ++q) in[q] = Bb(v)[2 * pidx<NQ>(x, y, q) + s];
-      eo_apply<1>(tb.Nt, in, out);
-#pragma unroll
-      for (int i = 0; i < NP; ++i) Cb(v)[2 * pidx<NQ>(x, y, i) + s] = out[i];
-    }
-    __syncthreads();
-    // test y: Cb (nq,nq,np) -> Bb (nq,np,np)
-    for (int u = threadIdx.x; u < VB * NQ * NP * 2; u += NT) {
-      const int v = u % VB, s = (u / VB) & 1, pen = u / (2 * VB);
-      const int x = pen % NQ, z = pen / NQ;
-      C in[NQ], out[NP];
-#pragma unroll
-      for (int q = 0; q < NQ; ++q) in[q] = Cb(v)[2 * pidx<NQ>(x, q, z) + s];
-      eo_apply<1>(tb.Nt, in, out);
-#pragma unroll
-      for (int i = 0; i < NP; ++i) Bb(v)[2 * pidx<NQ>(x, i, z) + s] = out[i];
-    }
-    __syncthreads();
-    // test x: Bb (nq,np,np) -> add into the x-stage registers, then assemble
-#pragma unroll
-    for (int r = 0; r < XR; ++r) {
-      const int u = threadIdx.x + r * NT;
-      if (u >= XU) break;
-      const int v = u % VB, s = (u / VB) & 1, pen = u / (2 * VB);
-      const int y = pen % NP, z = pen / NP;
-      C in[NQ], out[NP];
-#pragma unroll
-      for (int q = 0; q < NQ; ++q) in[q] = Bb(v)[2 * pidx<NQ>(q, y, z) + s];
-      eo_apply<1>(tb.Nt, in, out);
-      const int vec = vbase + v;
-      if (vec < d.nvec) {
-#pragma unroll
-        for (int i = 0; i < NP; ++i) {
-          const long long I = gbc_node(d.mesh, cx, cy, cz, i, y, z);
-          if (I < 0 || !GBC_IN_RANGE(GBC_SITE_HX64, I, d.mesh.M)) continue;
+      for (int i = 0; i < HP; ++i) {
+        AccD r;
+        row_sym<true, NP>(tb.Nt, i, s, r);
+        put_rows<NP>(i, r, [&](int x, double2 v) {
+          const double2 k = K[x];
+          const double2 o = make_double2(v.x + k.x, v.y + k.y);
+          const int I = Iyz + no[x];
+          if (I < 0 || !GBC_IN_RANGE(GBC_SITE_HX64, I, d.mesh.M)) return;
           if (d.Ycell)
-            d.Ycell[(((long long)e * (NP * NP * NP) + i + NP * (y + NP * z)) * 2 + s) * d.nvec + vec] =
-                cadd(yacc[r][i], out[i]);
+            d.Ycell[(((long long)e * (NP * NP * NP) + x + NP * (y + NP * z)) * 2 + sp) * d.nvec + vec] = o;
           else
-            atomic_add_c<T>(&d.Y[(I * 2 + s) * d.ldx + vec], cadd(yacc[r][i], out[i]));
-        }
+            atomic_add_c(&d.Y[((long long)I * 2 + sp) * d.ldx + vec], o);
+        });
       }
     }
-  }  // item loop
+  }
 }
 
-template <typename T, int NP, int NQ, int VB> constexpr size_t hx_local_smem() {
-  constexpr int BUF = pbuf_points<NQ>();
-  constexpr int VBASE = 3 * BUF * 2;
-  constexpr int VSTRIDE = VBASE + ((24 - VBASE % 16) % 16);
-  return sizeof(cplx<T>) * (size_t)VB * VSTRIDE;
-}
-
-template <typename T, int NP, int VB>
+template <int NP>
 cudaError_t launch_hx_group_p(const HxJob* jobs, int n, cudaStream_t s) {
-  static_assert(std::is_same<T, double>::value, "FP64 only (the FP32 cell apply is hx_cell.cuh)");
   constexpr int NQ = NP + 1;   // nq = p + 2
   if (n < 1 || n > GBC_MAX_BATCH) return cudaErrorInvalidValue;
-  LocalArgs<T> a;
+  LocalArgs a;
   long long item = 0;
   for (int i = 0; i < GBC_MAX_BATCH; ++i) {
-    SysDesc<T>& d = a.sys[i];
+    SysDesc& d = a.sys[i];
     if (i >= n) {
       d = a.sys[0];
       d.item0 = 0x7fffffffffffffffLL;
       continue;
     }
     const gbc_ctx* c = jobs[i].c;
-    d.X = (const cplx<T>*)jobs[i].X;
-    d.Y = (cplx<T>*)jobs[i].Y;
-    d.Ycell = (cplx<T>*)jobs[i].Ycell;
-    d.fields = (const T*)c->d_fields64;
+    d.X = (const double2*)jobs[i].X;
+    d.Y = (double2*)jobs[i].Y;
+    d.Ycell = (double2*)jobs[i].Ycell;
+    d.fields = c->d_fields64;
     d.ldx = jobs[i].ldx;
     d.nvec = jobs[i].nvec;
-    d.vchunks = (jobs[i].nvec + VB - 1) / VB;
-    d.pad = 0;
     d.item0 = item;
     d.mesh = c->mesh;
-    item += (long long)c->mesh.E * d.vchunks;
+    item += ((long long)c->mesh.E * d.nvec + 1) / 2;
   }
   a.nsys = n;
   a.nitems = item;
   if (item <= 0) return cudaSuccess;
   const gbc_ctx* c0 = jobs[0].c;
-  TablesEO<T, NP, NQ> tb;
-  if (!make_tables_eo<T, NP, NQ>(c0, &tb)) return cudaErrorInvalidValue;
+  TablesEO<double, NP, NQ> tb;
+  if (!make_tables_eo<double, NP, NQ>(c0, &tb)) return cudaErrorInvalidValue;
   const bool kpt = (c0->k[0] != 0.0 || c0->k[1] != 0.0 || c0->k[2] != 0.0);
-  constexpr size_t smem = hx_local_smem<T, NP, NQ, VB>();
-  int dev = 0, nsm = 0, per_sm = 0;
-  cudaError_t err = cudaGetDevice(&dev);
-  if (err != cudaSuccess) return err;
-  err = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  if (err != cudaSuccess) return err;
+  constexpr size_t smem = hx_groups<NP>() * hx_group_smem<NP>();
+  static_assert(smem <= 227 * 1024, "shared memory of the FP64 cell apply");
   auto run = [&](auto kern) -> cudaError_t {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, VB * 64, smem);
-    if (e != cudaSuccess) return e;
-    const long long nblk = std::min<long long>(item, (long long)nsm * std::max(per_sm, 1));
-    kern<<<(unsigned)nblk, VB * 64, smem, s>>>(a, tb);
+    const long long nblk = std::min<long long>(item, gbc_sm_count());
+    kern<<<(unsigned)nblk, kHxThreads, smem, s>>>(a, tb);
     return cudaGetLastError();
   };
-  if (kpt) return run(hx_local_kernel<T, NP, NQ, true, VB>);
-  return run(hx_local_kernel<T, NP, NQ, false, VB>);
+  if (kpt) return run(hx_local_kernel<NP, NQ, true>);
+  return run(hx_local_kernel<NP, NQ, false>);
 }
 
 // Deterministic assembly: Y[I][s][v] += the results of every cell holding node I, added
@@ -531,16 +634,17 @@ __global__ void k_cell_gather(cplx<T>* __restrict__ Y, const cplx<T>* __restrict
   }
 }
 
-// dispatch on p (nq = p + 2) for a fixed VB
-template <typename T, int VB>
-cudaError_t launch_hx_group(const HxJob* jobs, int n, cudaStream_t s) {
+// dispatch on p (nq = p + 2)
+inline cudaError_t launch_hx_group(const HxJob* jobs, int n, cudaStream_t s) {
+  for (int i = 0; i < n; ++i)   // node offsets are 32-bit
+    if (jobs[i].c->mesh.M >= (1LL << 29)) return cudaErrorInvalidValue;
   switch (jobs[0].c->mesh.p) {
-    case 2: return launch_hx_group_p<T, 3, VB>(jobs, n, s);
-    case 3: return launch_hx_group_p<T, 4, VB>(jobs, n, s);
-    case 4: return launch_hx_group_p<T, 5, VB>(jobs, n, s);
-    case 5: return launch_hx_group_p<T, 6, VB>(jobs, n, s);
-    case 6: return launch_hx_group_p<T, 7, VB>(jobs, n, s);
-    case 7: return launch_hx_group_p<T, 8, VB>(jobs, n, s);
+    case 2: return launch_hx_group_p<3>(jobs, n, s);
+    case 3: return launch_hx_group_p<4>(jobs, n, s);
+    case 4: return launch_hx_group_p<5>(jobs, n, s);
+    case 5: return launch_hx_group_p<6>(jobs, n, s);
+    case 6: return launch_hx_group_p<7>(jobs, n, s);
+    case 7: return launch_hx_group_p<8>(jobs, n, s);
     default: return cudaErrorInvalidValue;
   }
 }

@@ -1,8 +1,8 @@
-// FP64 instantiations of the matrix-free cell apply (p = 2..7, nq = p + 2, one vector per CTA).
+// FP64 instantiations of the matrix-free cell apply (p = 2..7, nq = p + 2).
 #include "hx_local.cuh"
 
 cudaError_t launch_hx_local_group_f64(const HxJob* jobs, int n, int /*vb*/, cudaStream_t s) {
-  return gbc::launch_hx_group<double, 1>(jobs, n, s);
+  return gbc::launch_hx_group(jobs, n, s);
 }
 
 cudaError_t launch_cell_gather_f64(const gbc_ctx* c, const double2* Ycell, double2* Y, int nvec,

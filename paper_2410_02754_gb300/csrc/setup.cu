@@ -153,24 +153,18 @@ __global__ void k_mass(const MeshDev m, const double* mx, const double* my, cons
   invmd32[I] = (float)(1.0 / v);
 }
 
-// fields[e][c][q] = w_q J * {V + |k|^2/2, bx, by, bz}[e][q] (FP64); the FP32 copy is
-// [e][q][c], one float4 per quadrature point, without w_q (the FP32 interpolation tables
-// carry its square root on both sides)
+// fields[e][q][c] = J * {V + |k|^2/2, bx, by, bz}[e][q] in FP64 and FP32 (the interpolation
+// tables carry sqrt(w_q) on both sides of them)
 __global__ void k_fields(const double* raw, long long E, int nq, double jac, double k2half,
-                         const double* __restrict__ wq, double* f64, float* f32) {
+                         double* f64, float* f32) {
   const long long nq3 = (long long)nq * nq * nq;
   const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (i >= E * nq3) return;
-  const long long e = i / nq3;
-  const int q = (int)(i % nq3);
-  const int qx = q % nq, qy = (q / nq) % nq, qz = q / (nq * nq);
-  const double w = wq[qx] * wq[qy] * wq[qz] * jac;
   for (int c = 0; c < 4; ++c) {
     double val = raw[(size_t)c * E * nq3 + i];
     if (c == 0) val += k2half;
-    const double o = w * val;
-    f64[(e * 4 + c) * nq3 + q] = o;
-    f32[(e * nq3 + q) * 4 + c] = (float)(jac * val);
+    f64[i * 4 + c] = jac * val;
+    f32[i * 4 + c] = (float)(jac * val);
   }
 }
 
@@ -264,15 +258,12 @@ gbc_status setup_fields(gbc_ctx* c) {
   const long long n = (long long)m.E * nq3;
   if (!c->d_fields64) GBC_CU(c, cudaMalloc(&c->d_fields64, sizeof(double) * 4 * n));
   if (!c->d_fields32) GBC_CU(c, cudaMalloc(&c->d_fields32, sizeof(float) * 4 * n));
-  double* dwq = nullptr;
-  GBC_TRY(upload(c, (void**)&dwq, c->tab.gq_w.data(), sizeof(double) * nq));
   const double jac = c->h[0] * c->h[1] * c->h[2] / 8.0;
   const double k2 = 0.5 * (c->k[0] * c->k[0] + c->k[1] * c->k[1] + c->k[2] * c->k[2]);
-  k_fields<<<(unsigned)((n + 255) / 256), 256>>>(c->d_rawfields, m.E, nq, jac, k2, dwq,
+  k_fields<<<(unsigned)((n + 255) / 256), 256>>>(c->d_rawfields, m.E, nq, jac, k2,
                                                   c->d_fields64, c->d_fields32);
   GBC_CU(c, cudaGetLastError());
   GBC_CU(c, cudaDeviceSynchronize());
-  cudaFree(dwq);
   return GBC_OK;
 }
 
