@@ -210,63 +210,128 @@ gbc_status filter_t(gbc_ctx* c, cplx<T>* X, int nvec, int ldx, int m, double lT,
   return GBC_OK;
 }
 
-template <typename T>
-gbc_status cholgs_t(gbc_ctx* c, cplx<T>* X, int nvec, int ldx, cudaStream_t s) {
-  const size_t nn = (size_t)nvec * nvec;
-  GBC_TRY(gbc_ensure_work(c, 3, sizeof(double2) * 2 * nn + sizeof(double) * nvec + 256));
-  double2* S = (double2*)c->work[3];
-  double2* Q = S + nn;
+// Gram matrices and rotations: split products on the tensor cores (split_gemm.cu) from these
+// column counts on, below them FP64 (FP64 block) or float-float arithmetic (FP32 block).
+// Measured, split against direct: FP64 Gram at 16 columns 0.06 / 0.07 ms (1728 nodes) and
+// 1.36 / 5.22 ms (216,000 nodes), rotation 0.04 / 0.11 and 0.74 / 4.8 ms; FP32 Gram 1.34 /
+// 0.83 ms at 32 columns and 0.147 / 0.171 ms at 64 (216,000 and 13,824 nodes), FP32 rotation
+// 0.56 / 0.64 ms at 16 and 0.56 / 1.29 at 32 (216,000 nodes), 0.033 / 0.023 at 16 (1728).
+template <typename T> constexpr int split_gram_cols() { return sizeof(T) == 8 ? 16 : 64; }
+template <typename T> constexpr int split_rotate_cols() { return sizeof(T) == 8 ? 16 : 32; }
+
+// S = X^H diag(md) Y, both triangles
+template <typename T, typename TY>
+gbc_status gram(gbc_ctx* c, const cplx<T>* X, int ldx, const cplx<TY>* Y, int ldy, const double* md,
+                int nvec, double2* S, cudaStream_t s) {
   {
     TimerScope ts(c, FAM_GRAM, s);
-    GBC_CU(c, launch_gram<T>(X, X, c->d_md, c->mesh.M, nvec, ldx, S, s));
+    if (nvec >= split_gram_cols<T>()) {
+      GBC_TRY((launch_gram_split<T, TY>(c, X, ldx, Y, ldy, md, c->mesh.M, nvec, S, s)));
+    } else if constexpr (std::is_same<T, double>::value) {
+      GBC_CU(c, launch_gram<double>(X, Y, md, c->mesh.M, nvec, ldx, S, s));
+    } else {
+      GBC_CU(c, launch_gram_ff<TY>(X, ldx, Y, ldy, md, c->mesh.M, nvec, S, s));
+    }
   }
   GBC_CU(c, launch_hermitize(S, nvec, s));
-  {
-    TimerScope ts(c, FAM_DENSE, s);
-    GBC_TRY(dense_cholesky_inv_h(c, S, nvec, Q, s));
-  }
-  const size_t bytes = sizeof(cplx<T>) * 2 * (size_t)c->mesh.M * ldx;
-  GBC_TRY(gbc_ensure_work(c, 1, bytes));
-  cplx<T>* W = (cplx<T>*)c->work[1];
-  {
-    TimerScope ts(c, FAM_ROTATE, s);
-    GBC_CU(c, launch_rotate<T>(X, Q, W, c->mesh.M, nvec, ldx, s));
-  }
-  GBC_CU(c, launch_copy_block<T>(W, X, c->mesh.M, nvec, ldx, s));
-  GBC_CU(c, cudaStreamSynchronize(s));
   return GBC_OK;
 }
 
+// X <- X Q.  diag: the diagonal of X's Gram matrix (null: the columns have one size);
+// qsplit: 2 nvec^2 float2 of scratch
 template <typename T>
-gbc_status rr_t(gbc_ctx* c, cplx<T>* X, int nvec, int ldx, double* ritz, cudaStream_t s) {
-  const size_t nn = (size_t)nvec * nvec;
-  const size_t bytes = sizeof(cplx<T>) * 2 * (size_t)c->mesh.M * ldx;
-  GBC_TRY(gbc_ensure_work(c, 0, bytes));
-  GBC_TRY(gbc_ensure_work(c, 1, bytes));
-  GBC_TRY(gbc_ensure_work(c, 3, sizeof(double2) * 2 * nn + sizeof(double) * nvec + 256));
-  double2* Hp = (double2*)c->work[3];
-  double2* Q = Hp + nn;
-  double* ev = (double*)(Q + nn);
-  cplx<T>* HX = (cplx<T>*)c->work[0];
-  GBC_TRY(apply_h_t<T>(c, X, HX, nvec, ldx, s));
-  {
-    TimerScope ts(c, FAM_GRAM, s);
-    GBC_CU(c, launch_gram<T>(X, HX, nullptr, c->mesh.M, nvec, ldx, Hp, s));
+gbc_status rotate(gbc_ctx* c, cplx<T>* X, int nvec, int ldx, const double2* Q, const double2* diag,
+                  float2* qsplit, cudaStream_t s) {
+  if (nvec >= split_rotate_cols<T>()) {
+    TimerScope ts(c, FAM_ROTATE, s);
+    return launch_rotate_split<T>(c, X, Q, c->mesh.M, nvec, ldx, diag, s);
   }
-  GBC_CU(c, launch_hermitize(Hp, nvec, s));
-  {
-    TimerScope ts(c, FAM_DENSE, s);
-    GBC_TRY(dense_eigh(c, Hp, nvec, ev, Q, s));
-  }
+  GBC_TRY(gbc_ensure_work(c, 1, sizeof(cplx<T>) * 2 * (size_t)c->mesh.M * ldx));
   cplx<T>* W = (cplx<T>*)c->work[1];
   {
     TimerScope ts(c, FAM_ROTATE, s);
-    GBC_CU(c, launch_rotate<T>(X, Q, W, c->mesh.M, nvec, ldx, s));
+    if constexpr (std::is_same<T, double>::value)
+      GBC_CU(c, launch_rotate<double>(X, Q, W, c->mesh.M, nvec, ldx, s));
+    else
+      GBC_CU(c, launch_rotate_ff(X, Q, qsplit, W, c->mesh.M, nvec, ldx, s));
   }
   GBC_CU(c, launch_copy_block<T>(W, X, c->mesh.M, nvec, ldx, s));
-  GBC_CU(c, cudaMemcpyAsync(ritz, ev, sizeof(double) * nvec, cudaMemcpyDeviceToHost, s));
-  GBC_CU(c, cudaStreamSynchronize(s));
   return GBC_OK;
+}
+
+// waits for the stream; a bounded wait of the split products that expired
+gbc_status finish_dense(gbc_ctx* c, cudaStream_t s) {
+  int err = 0;
+  GBC_CU(c, split_error(&err, s));
+  if (err) return gbc_fail(c, GBC_ETIMEOUT, "a tensor-core wait expired; the block is invalid");
+  return GBC_OK;
+}
+
+// small dense scratch of CholGS / Rayleigh-Ritz (work slot 3): two n x n matrices, the FP32
+// pairs of Q, a diagonal and n doubles
+struct DenseScratch {
+  double2 *S, *Q, *diag;
+  float2* qsplit;
+  double* ev;
+};
+gbc_status dense_scratch(gbc_ctx* c, int nvec, DenseScratch* d) {
+  const size_t nn = (size_t)nvec * nvec;
+  GBC_TRY(gbc_ensure_work(c, 3, sizeof(double2) * (3 * nn + nvec) + sizeof(double) * nvec + 256));
+  d->S = (double2*)c->work[3];
+  d->Q = d->S + nn;
+  d->qsplit = (float2*)(d->Q + nn);
+  d->diag = d->Q + 2 * nn;
+  d->ev = (double*)(d->diag + nvec);
+  return GBC_OK;
+}
+
+// Cholesky-Gram-Schmidt.  FP64 blocks: FP64 throughout.  The mixed path keeps complex64
+// blocks for the filter, but S = X^H M_D X and the rotation are FP64-accurate (the rotated
+// block is rounded to FP32 once).
+template <typename T>
+gbc_status cholgs_t(gbc_ctx* c, cplx<T>* X, int nvec, int ldx, cudaStream_t s) {
+  DenseScratch d;
+  GBC_TRY(dense_scratch(c, nvec, &d));
+  GBC_TRY((gram<T, T>(c, X, ldx, X, ldx, c->d_md, nvec, d.S, s)));
+  GBC_CU(c, cudaMemcpy2DAsync(d.diag, sizeof(double2), d.S, sizeof(double2) * (nvec + 1), sizeof(double2),
+                              nvec, cudaMemcpyDeviceToDevice, s));
+  {
+    TimerScope ts(c, FAM_DENSE, s);
+    GBC_TRY(dense_cholesky_inv_h(c, d.S, nvec, d.Q, s));
+  }
+  GBC_TRY(rotate<T>(c, X, nvec, ldx, d.Q, d.diag, d.qsplit, s));
+  return finish_dense(c, s);
+}
+
+// Rayleigh-Ritz: Hp = X^H (H X), Hp Q = Q Lambda, X <- X Q.  HX is the FP64 H.X of X; an FP32
+// block is applied as its FP64 copy (an FP32 H.X would put a first-order error
+// eps32 * ||H~|| into X^H H X and hence into the Ritz values).
+template <typename T>
+gbc_status rr_t(gbc_ctx* c, cplx<T>* X, int nvec, int ldx, double* ritz, cudaStream_t s) {
+  const bool f64 = std::is_same<T, double>::value;
+  const int ldh = f64 ? ldx : nvec;
+  const size_t bytes = sizeof(double2) * 2 * (size_t)c->mesh.M * ldh;
+  DenseScratch d;
+  GBC_TRY(dense_scratch(c, nvec, &d));
+  GBC_TRY(gbc_ensure_work(c, 0, bytes));
+  double2* HX = (double2*)c->work[0];
+  const double2* X64;
+  if constexpr (std::is_same<T, double>::value) {
+    X64 = X;
+  } else {
+    GBC_TRY(gbc_ensure_work(c, 4, bytes));
+    GBC_CU(c, launch_convert_block(X, ldx, (double2*)c->work[4], nvec, c->mesh.M, nvec, s));
+    X64 = (const double2*)c->work[4];
+  }
+  GBC_TRY(apply_h_t<double>(c, X64, HX, nvec, ldh, s));
+  GBC_TRY((gram<T, double>(c, X, ldx, HX, ldh, nullptr, nvec, d.S, s)));
+  {
+    TimerScope ts(c, FAM_DENSE, s);
+    GBC_TRY(dense_eigh(c, d.S, nvec, d.ev, d.Q, s));
+  }
+  GBC_TRY(rotate<T>(c, X, nvec, ldx, d.Q, nullptr, d.qsplit, s));
+  GBC_CU(c, cudaMemcpyAsync(ritz, d.ev, sizeof(double) * nvec, cudaMemcpyDeviceToHost, s));
+  return finish_dense(c, s);
 }
 
 // Residual-split filter (Hamiltonian-times-residual form of the recurrence):
@@ -340,76 +405,6 @@ gbc_status filter_split_t(gbc_ctx* c, cplx<T>* X, int nvec, int ldx, int m, doub
   }
   cplx<T>* Zm = (m & 1) ? Za : Zb;
   GBC_CU(c, launch_split_final<T>(X, Zm, d_Dm, c->mesh.M, nvec, ldx, s));
-  return GBC_OK;
-}
-
-// The mixed path keeps complex64 blocks for the filter but runs CholGS and
-// CholGS and Rayleigh-Ritz of an FP32 block.  The projected matrices are FP64-
-// accurate: S = X^H M_D X and Hp = X^H (H X) are accumulated in float-float
-// arithmetic on the FP32 pipes; Rayleigh-Ritz needs an FP64 H.X (an FP32 one
-// would put a first-order error eps32 * ||H~|| into X^H H X and hence into the
-// Ritz values), computed on an FP64 copy of X (work slot 4).  The rotations
-// X <- X Q act on the FP32 block in float-float arithmetic as well: the FP64
-// product rounded to FP32.
-gbc_status rotate_mixed(gbc_ctx* c, float2* X, int nvec, int ldx, const double2* Q, float2* Qsplit,
-                        cudaStream_t s) {
-  const size_t bytes = sizeof(float2) * 2 * (size_t)c->mesh.M * ldx;
-  GBC_TRY(gbc_ensure_work(c, 1, bytes));
-  float2* W = (float2*)c->work[1];
-  {
-    TimerScope ts(c, FAM_ROTATE, s);
-    GBC_CU(c, launch_rotate_ff(X, Q, Qsplit, W, c->mesh.M, nvec, ldx, s));
-  }
-  GBC_CU(c, launch_copy_block<float>(W, X, c->mesh.M, nvec, ldx, s));
-  return GBC_OK;
-}
-
-gbc_status cholgs_mixed(gbc_ctx* c, float2* X, int nvec, int ldx, cudaStream_t s) {
-  const size_t nn = (size_t)nvec * nvec;
-  GBC_TRY(gbc_ensure_work(c, 3, sizeof(double2) * 3 * nn + sizeof(double) * nvec + 256));
-  double2* S = (double2*)c->work[3];
-  double2* Q = S + nn;
-  float2* Qsplit = (float2*)(Q + nn);   // 2 nn float2
-  {
-    TimerScope ts(c, FAM_GRAM, s);
-    GBC_CU(c, launch_gram_ff<float>(X, ldx, X, ldx, c->d_md, c->mesh.M, nvec, S, s));
-  }
-  GBC_CU(c, launch_hermitize(S, nvec, s));
-  {
-    TimerScope ts(c, FAM_DENSE, s);
-    GBC_TRY(dense_cholesky_inv_h(c, S, nvec, Q, s));
-  }
-  GBC_TRY(rotate_mixed(c, X, nvec, ldx, Q, Qsplit, s));
-  GBC_CU(c, cudaStreamSynchronize(s));
-  return GBC_OK;
-}
-
-gbc_status rr_mixed(gbc_ctx* c, float2* X, int nvec, int ldx, double* ritz, cudaStream_t s) {
-  const size_t nn = (size_t)nvec * nvec;
-  const size_t bytes64 = sizeof(double2) * 2 * (size_t)c->mesh.M * nvec;
-  GBC_TRY(gbc_ensure_work(c, 4, bytes64));
-  GBC_TRY(gbc_ensure_work(c, 0, bytes64));
-  GBC_TRY(gbc_ensure_work(c, 3, sizeof(double2) * 3 * nn + sizeof(double) * nvec + 256));
-  double2* X64 = (double2*)c->work[4];
-  double2* HX = (double2*)c->work[0];
-  double2* Hp = (double2*)c->work[3];
-  double2* Q = Hp + nn;
-  float2* Qsplit = (float2*)(Q + nn);
-  double* ev = (double*)(Q + 2 * nn);
-  GBC_CU(c, launch_convert_block(X, ldx, X64, nvec, c->mesh.M, nvec, s));
-  GBC_TRY(apply_h_t<double>(c, X64, HX, nvec, nvec, s));
-  {
-    TimerScope ts(c, FAM_GRAM, s);
-    GBC_CU(c, launch_gram_ff<double>(X, ldx, HX, nvec, nullptr, c->mesh.M, nvec, Hp, s));
-  }
-  GBC_CU(c, launch_hermitize(Hp, nvec, s));
-  {
-    TimerScope ts(c, FAM_DENSE, s);
-    GBC_TRY(dense_eigh(c, Hp, nvec, ev, Q, s));
-  }
-  GBC_TRY(rotate_mixed(c, X, nvec, ldx, Q, Qsplit, s));
-  GBC_CU(c, cudaMemcpyAsync(ritz, ev, sizeof(double) * nvec, cudaMemcpyDeviceToHost, s));
-  GBC_CU(c, cudaStreamSynchronize(s));
   return GBC_OK;
 }
 
@@ -729,7 +724,7 @@ gbc_status gbc_cholgs(gbc_ctx* c, void* X, int nvec, int ldx, void* stream) {
   GBC_TRY(gbc_prepare(c));
   cudaStream_t s = (cudaStream_t)stream;
   if (c->prec == GBC_FP64) return cholgs_t<double>(c, (double2*)X, nvec, ldx, s);
-  return cholgs_mixed(c, (float2*)X, nvec, ldx, s);
+  return cholgs_t<float>(c, (float2*)X, nvec, ldx, s);
 }
 
 gbc_status gbc_rayleigh_ritz(gbc_ctx* c, void* X, int nvec, int ldx, double* ritz, void* stream) {
@@ -740,7 +735,7 @@ gbc_status gbc_rayleigh_ritz(gbc_ctx* c, void* X, int nvec, int ldx, double* rit
   GBC_TRY(gbc_prepare(c));
   cudaStream_t s = (cudaStream_t)stream;
   if (c->prec == GBC_FP64) return rr_t<double>(c, (double2*)X, nvec, ldx, ritz, s);
-  return rr_mixed(c, (float2*)X, nvec, ldx, ritz, s);
+  return rr_t<float>(c, (float2*)X, nvec, ldx, ritz, s);
 }
 
 gbc_status gbc_lanczos_bounds(gbc_ctx* c, const void* v0, int steps, double* lmin, double* lmax,

@@ -846,13 +846,13 @@ cudaError_t launch_divmass(double2* y, const double* invmd, long long M, cudaStr
   template cudaError_t launch_cheb_step<T>(const cplx<T>*, const cplx<T>*, const cplx<T>*,      \
                                            cplx<T>*, const T*, long long, int, int, double,     \
                                            double, double, cudaStream_t);                        \
-  template cudaError_t launch_gram<T>(const cplx<T>*, const cplx<T>*, const double*, long long, \
-                                      int, int, double2*, cudaStream_t);                        \
-  template cudaError_t launch_rotate<T>(const cplx<T>*, const double2*, cplx<T>*, long long,    \
-                                        int, int, cudaStream_t);                                 \
   template cudaError_t launch_copy_block<T>(const cplx<T>*, cplx<T>*, long long, int, int,      \
                                             cudaStream_t);
 INST(float)
 INST(double)
+template cudaError_t launch_gram<double>(const double2*, const double2*, const double*, long long,
+                                         int, int, double2*, cudaStream_t);
+template cudaError_t launch_rotate<double>(const double2*, const double2*, double2*, long long, int,
+                                           int, cudaStream_t);
 
 GBC_CHECK_WORD_ACCESSOR(gbc_check_word_blas)

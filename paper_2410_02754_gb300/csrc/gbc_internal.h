@@ -209,8 +209,8 @@ struct gbc_ctx {
   // 0 H.X accumulator, 1 second block, 2 nonlocal coefficients, 3 small dense,
   // 4-7 FP64 copies / residual-split blocks, 8 backward block pool, 9 backward
   // accumulators; deterministic mode: 10 per-cell results, 11 projection partials,
-  // 12 reduction partials
-  static constexpr int kWorkSlots = 13;
+  // 12 reduction partials; 13 digit slices of the split products
+  static constexpr int kWorkSlots = 14;
   void* work[kWorkSlots] = {};
   size_t work_bytes[kWorkSlots] = {};
   bool deterministic = false;        // FP64 kernels: fixed-order sums instead of atomics
@@ -413,6 +413,17 @@ cudaError_t launch_gram(const cplx<T>* X, const cplx<T>* Y, const double* md, lo
 template <typename T>
 cudaError_t launch_rotate(const cplx<T>* X, const double2* Q, cplx<T>* Out, long long M, int nvec,
                           int ldx, cudaStream_t s);
+// split_gemm.cu : Gram matrices and in-place rotations as exact split products on the tensor
+// cores (FP64-accurate; work slot 13)
+struct CUtensorMap_st;
+bool tc_make_map_bf16(CUtensorMap_st* m, const void* p, long long rows, int cols, int box_rows);
+template <typename T>
+gbc_status launch_rotate_split(gbc_ctx* c, cplx<T>* X, const double2* Q, long long M, int n, int ldx,
+                               const double2* diag, cudaStream_t s);
+template <typename TX, typename TY>
+gbc_status launch_gram_split(gbc_ctx* c, const cplx<TX>* X, int ldx, const cplx<TY>* Y, int ldy,
+                             const double* md, long long M, int n, double2* Sm, cudaStream_t s);
+cudaError_t split_error(int* err, cudaStream_t s);
 // residual-split filter kernels
 template <typename T>
 cudaError_t launch_split_init(const double2* HX, const double2* X64, const double* invmd,

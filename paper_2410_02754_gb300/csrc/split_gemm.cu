@@ -1,0 +1,656 @@
+// Gram matrices and block rotations of CholGS / Rayleigh-Ritz as exact split products on the
+// tcgen05 tensor cores (BF16 digits, FP32 accumulation without rounding, integer recombination).
+//
+// Paper: Sec. III.B.2 (X^H M X, X^H H X, U = X Q).  Method: the error-free transformation of a
+// matrix product by splitting both factors (Ozaki, Ogita, Oishi, Rump, Numer. Algorithms 59,
+// 2012), with balanced base-256 digits: a value x with |x| < 2^E is
+//   x = 2^(E-6) sum_k d_k 256^-k,  |d_0| <= 65, d_k in [-128, 127],
+// so every digit is a BF16 number and a product of two digits an integer below 2^14; S digits
+// carry 8 S - 2 bits below 2^E.  The partial products of order t = i + j <= S - 1,
+// G_t = sum_{i+j=t} A_i B_j, are integers that FP32 holds exactly while (t + 1) K 2^14 <= 2^24;
+// the accumulators are read out (to 64-bit integers) every kFlush K chunks to keep that, and
+// sum_t G_t 256^-t is rounded once at the end.  Exponents are per row of A and B: per block
+// row and per column of Q for a rotation, per column of the block (over all rows) for a Gram
+// matrix.  A row with an infinity or a NaN is marked and gives NaN, as in FP arithmetic.
+//
+//  * rotation of an orthonormal FP32 block by a unitary matrix (Rayleigh-Ritz): S = 4 (30 bits
+//    below the row's largest entry, an error of at most sqrt(n) 2^-33 of a column's norm), 10
+//    digit products, rounded to FP32 once;
+//  * everything else (Gram matrices, FP64 blocks, the triangular rotation of CholGS, whose
+//    terms can cancel; its columns are first brought to a common size by powers of two):
+//    S = 7 (54 bits), 28 digit products.
+//
+// GB300's FP64 pipe gives 1.05 TFLOP/s and float-float arithmetic on the FP32 pipes about 6;
+// 28 BF16 products at 1.9 PFLOP/s are an FP64-accurate 68 TFLOP/s.  Per tile (128 x 128 for
+// S = 4, 128 x 64 for S = 7) every order has its own accumulator in tensor memory and all S
+// digit slices of a 64-wide K chunk are in shared memory at once (one TMA box each), so a
+// slice is loaded once per tile and used in up to S products.  The products run from the
+// outermost digit pairs (0, j), (i, 0) inwards: after step m the slices m and S-1-m are free,
+// and their next chunk loads behind the remaining steps.
+#include <algorithm>
+#include <cmath>
+#include <cuda.h>
+
+#include "gbc_internal.h"
+#include "tc.cuh"
+
+namespace {
+
+__device__ int g_split_err;   // set when a bounded wait expired
+
+constexpr int kTM = 128;              // tile rows
+constexpr int kKC = 64;               // K chunk: one 128-byte swizzled row
+constexpr int kBad = 0x7fffffff;      // exponent of a row with an infinity or a NaN
+template <int S> struct SplitCfg {
+  static constexpr int N = S <= 4 ? 128 : 64;             // tile columns
+  static constexpr int FLUSH = S <= 4 ? 4 : 2;            // K chunks between read-outs
+  static constexpr int ABYTES = kTM * 128, SLICE = ABYTES + N * 128;
+  static constexpr size_t SMEM = 1024 + (size_t)S * SLICE + 256;
+  static_assert(S * N <= 512, "tensor memory columns");
+  static_assert((long long)S * FLUSH * kKC << 14 <= 1LL << 24, "exact accumulation");
+};
+
+enum { ROT32 = 0, ROT64 = 1, GRAM = 2 };
+struct SplitArgs {
+  int rows_a, rows_b;      // rows of a slice of A and B
+  int nchunk, kper;        // K chunks; chunks per CTA (GRAM: split over blockIdx.y)
+  int ntn;                 // column tiles
+  const int *ea, *eb;      // unit exponents (E - 6) of the rows of A and B
+  long long rows;          // rotation: valid rows of the chunk
+  int n;                   // complex columns
+  int ldo;                 // rotation: complex leading dimension of out
+  void* out;
+};
+
+// 2^e as a double (|e| < 1000)
+__device__ __forceinline__ double pow2d(int e) {
+  return __hiloint2double((1023 + max(-1000, min(1000, e))) << 20, 0);
+}
+
+template <int S, int MODE>
+__global__ void __launch_bounds__(320, 1)
+k_split_gemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb,
+             const SplitArgs a) {
+  using G = SplitCfg<S>;
+  constexpr int N = G::N;
+  int m0, n0, k0 = 0, nk = a.nchunk;
+  if (MODE == GRAM) {   // tiles that reach the diagonal or above it, row by row
+    int I = 0, t = blockIdx.x, first = 0;
+    while (t >= a.ntn - first) {
+      t -= a.ntn - first;
+      ++I;
+      first = I * (kTM / N);
+    }
+    m0 = I * kTM;
+    n0 = (first + t) * N;
+    k0 = blockIdx.y * a.kper;
+    nk = min(a.kper, a.nchunk - k0);
+    if (nk <= 0) return;
+  } else {
+    m0 = (int)(blockIdx.x / a.ntn) * kTM;
+    n0 = (int)(blockIdx.x % a.ntn) * N;
+  }
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  unsigned char* st = reinterpret_cast<unsigned char*>(
+      (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  uint64_t* full = reinterpret_cast<uint64_t*>(st + S * G::SLICE);   // [S] slice landed
+  uint64_t* empty = full + S;                                        // [S] slice free
+  uint64_t* accf = empty + S;                                        // accumulators complete
+  uint64_t* acce = accf + 1;                                         // accumulators read out
+  uint64_t* drain = acce + 1;                                        // every MMA complete
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(drain + 1);
+  int* fail = reinterpret_cast<int*>(tslot + 1);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  auto A = [&](int s) { return tc::smem_u32(st + s * G::SLICE); };
+  auto B = [&](int s) { return tc::smem_u32(st + s * G::SLICE + G::ABYTES); };
+  auto failed = [&]() { return *reinterpret_cast<volatile int*>(fail) != 0; };
+
+  if (warp == 0) {
+    tc::tmem_alloc(tc::smem_u32(tslot), 512);
+    tc::tmem_relinquish();
+  }
+  if (threadIdx.x == 32) {
+    for (int s = 0; s < S; ++s) {
+      tc::mbar_init(tc::smem_u32(&full[s]), 1);
+      tc::mbar_init(tc::smem_u32(&empty[s]), 1);
+    }
+    tc::mbar_init(tc::smem_u32(accf), 1);
+    tc::mbar_init(tc::smem_u32(acce), 8);
+    tc::mbar_init(tc::smem_u32(drain), 1);
+    *fail = 0;
+    tc::fence_mbar_init();
+  }
+  tc::fence_before_sync();
+  __syncthreads();
+  tc::fence_after_sync();
+  const uint32_t tmem = *tslot;
+  const int nwin = (nk + G::FLUSH - 1) / G::FLUSH;
+
+  if (warp == 0 && lane == 0) {
+    // producer: slices in the order in which the MMA steps free them
+    int issued[S];
+#pragma unroll
+    for (int s = 0; s < S; ++s) issued[s] = 0;
+    for (int c = 0; c < nk && !failed(); ++c) {
+#pragma unroll
+      for (int o = 0; o < S; ++o) {
+        const int s = (o & 1) ? S - 1 - o / 2 : o / 2;
+        if (c > 0 && !tc::mbar_wait_bounded(tc::smem_u32(&empty[s]), (c - 1) & 1)) atomicExch(fail, 1);
+        if (failed()) break;
+        const uint32_t fb = tc::smem_u32(&full[s]);
+        tc::mbar_arrive_expect_tx(fb, G::SLICE);
+        tc::tma_load_2d(A(s), &ta, (k0 + c) * kKC, s * a.rows_a + m0, fb);
+        tc::tma_load_2d(B(s), &tb, (k0 + c) * kKC, s * a.rows_b + n0, fb);
+        issued[s] = c + 1;
+      }
+    }
+    if (failed())   // let the copies in flight land first
+#pragma unroll
+      for (int s = 0; s < S; ++s)
+        if (issued[s]) tc::mbar_wait_bounded(tc::smem_u32(&full[s]), (issued[s] - 1) & 1);
+  } else if (warp == 1 && lane == 0) {
+    constexpr uint32_t idesc = tc::idesc_bf16(kTM, N);
+    for (int c = 0; c < nk && !failed(); ++c) {
+      const bool first = c % G::FLUSH == 0;
+      if (first && c > 0) {
+        if (!tc::mbar_wait_bounded(tc::smem_u32(acce), (c / G::FLUSH - 1) & 1)) atomicExch(fail, 1);
+        tc::fence_after_sync();
+      }
+      auto pair = [&](int i, int j, bool fresh) {
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk)
+          tc::mma_bf16(tmem + (i + j) * N, tc::sdesc_sw128(A(i) + kk * 32),
+                       tc::sdesc_sw128(B(j) + kk * 32), idesc, (fresh && kk == 0) ? 0u : 1u);
+      };
+      auto need = [&](int s) {
+        if (!tc::mbar_wait_bounded(tc::smem_u32(&full[s]), c & 1)) atomicExch(fail, 1);
+        tc::fence_after_sync();
+      };
+#pragma unroll
+      for (int m = 0; 2 * m <= S - 1; ++m) {
+        // pairs whose smaller index is m; the others in the order of their arrival
+#pragma unroll
+        for (int o = 2 * m; o < S; ++o) {
+          const int s = (o & 1) ? S - 1 - o / 2 : o / 2;
+          if (m == 0) need(s);
+          if (s < m || s + m > S - 1) continue;
+          pair(m, s, first && m == 0);
+          if (s != m) pair(s, m, false);
+        }
+        tc::mma_commit(tc::smem_u32(&empty[m]));
+        if (S - 1 - m != m) tc::mma_commit(tc::smem_u32(&empty[S - 1 - m]));
+      }
+      if ((c + 1) % G::FLUSH == 0 || c + 1 == nk) tc::mma_commit(tc::smem_u32(accf));
+    }
+    // tensor memory is given back only after the issued MMAs (also after a failure)
+    tc::mma_commit(tc::smem_u32(drain));
+    if (!tc::mbar_wait_bounded(tc::smem_u32(drain), 0)) atomicExch(fail, 1);
+  } else if (warp >= 2) {
+    const int g = warp & 3, half = (warp - 2) >> 2;
+    constexpr int NC = N / 2;                        // columns of a thread
+    const uint32_t tl = tmem + ((uint32_t)(g * 32) << 16) + (uint32_t)(half * NC);
+    // orders 0..3 and 4..S-1 as 64-bit integers, in units of 256^-3 and 256^-(S-1)
+    long long hi[NC], lo[S > 4 ? NC : 1];
+#pragma unroll
+    for (int i = 0; i < NC; ++i) {
+      hi[i] = 0;
+      if (S > 4) lo[i] = 0;
+    }
+    bool ok = true;
+    for (int w = 0; w < nwin && ok; ++w) {
+      ok = tc::mbar_wait_bounded(tc::smem_u32(accf), w & 1);
+      if (!ok) atomicExch(fail, 1);
+      ok = ok && !failed();
+      tc::fence_after_sync();
+      if (ok) {
+#pragma unroll
+        for (int c0 = 0; c0 < NC; c0 += 8) {
+          uint32_t r[S][8];
+#pragma unroll
+          for (int t = 0; t < S; ++t) tc::tmem_ld8_nowait(tl + t * N + c0, r[t]);
+          tc::tmem_wait_ld();
+#pragma unroll
+          for (int i = 0; i < 8; ++i)
+#pragma unroll
+            for (int t = 0; t < S; ++t) {
+              const int v = __float2int_rn(__uint_as_float(r[t][i]));
+              if (t < 4) hi[c0 + i] += (long long)v * (1 << (8 * (3 - t)));
+              else lo[c0 + i] += (long long)v * (1 << (8 * (S - 1 - t)));
+            }
+        }
+      }
+      tc::fence_before_sync();
+      if (lane == 0) tc::mbar_arrive(tc::smem_u32(acce));
+    }
+    if (ok) {
+      const int mr = m0 + g * 32 + lane;
+      const int ea = a.ea[mr];
+      const int cb = n0 + half * NC;
+      const int* eb = a.eb + cb;
+      // the sum as one integer W in units of 2^(ea + eb - 24 - sh): exact where |hi| < 2^38 (or
+      // S = 4), else cut 2^-53 below its leading bit; converted (and rounded) once
+      auto value = [&](int i, int& sh) {
+        if (S == 4) {
+          sh = 0;
+          return hi[i];
+        }
+        const bool small = llabs(hi[i]) < (1LL << 38);
+        sh = small ? 24 : 15;
+        return small ? (hi[i] << 24) + lo[S > 4 ? i : 0] : (hi[i] << 15) + (lo[S > 4 ? i : 0] >> 9);
+      };
+      if (MODE == ROT32) {
+        if (mr < a.rows) {
+          float2* o = reinterpret_cast<float2*>(a.out) + (size_t)mr * a.ldo + cb / 2;
+#pragma unroll
+          for (int i = 0; i < NC; i += 2) {
+            if (cb + i >= 2 * a.n) break;
+            float v[2];
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+              int sh;
+              const float f = __ll2float_rn(value(i + q, sh));
+              const int e = eb[i + q];
+              v[q] = (ea == kBad || e == kBad) ? NAN : scalbnf(f, ea + e - 24 - sh);
+            }
+            o[i / 2] = make_float2(v[0], v[1]);
+          }
+        }
+      } else {
+#pragma unroll
+        for (int i = 0; i < NC; i += 2) {
+          if (cb + i >= 2 * a.n) break;
+          double v[2];
+#pragma unroll
+          for (int q = 0; q < 2; ++q) {
+            int sh;
+            v[q] = __ll2double_rn(value(i + q, sh));
+            const int e = eb[i + q], x = ea + e - 24 - sh;
+            if (ea == kBad || e == kBad) v[q] = NAN;
+            else if (abs(x) > 900) v[q] = scalbn(v[q], x);
+            else if (v[q] != 0.0)   // a multiplication by 2^x on the integer pipe (1 <= |v| < 2^63)
+              v[q] = __hiloint2double(__double2hiint(v[q]) + (x << 20), __double2loint(v[q]));
+          }
+          if (MODE == ROT64) {
+            if (mr < a.rows)
+              reinterpret_cast<double2*>(a.out)[(size_t)mr * a.ldo + (cb + i) / 2] = make_double2(v[0], v[1]);
+          } else {
+            // conj(x) y of complex columns (mr / 2, (cb + i) / 2): re = rr + ii, im = ri - ir
+            const int ci = mr >> 1, cj = (cb + i) >> 1;
+            if (ci < a.n && ci <= cj) {
+              double2* s = reinterpret_cast<double2*>(a.out) + (size_t)ci * a.n + cj;
+              atomicAdd(&s->x, (mr & 1) ? v[1] : v[0]);
+              atomicAdd(&s->y, (mr & 1) ? -v[0] : v[1]);
+            }
+          }
+        }
+      }
+    }
+  }
+  tc::fence_before_sync();
+  __syncthreads();
+  if (failed() && threadIdx.x == 0) atomicExch(&g_split_err, 1);
+  if (warp == 0) tc::tmem_dealloc(tmem, 512);
+}
+
+// ---------------------------------------------------------------------------
+// splitting
+// ---------------------------------------------------------------------------
+// largest-magnitude key of a value (ordered as an unsigned integer) and its exponent E
+// (|x| < 2^E), kBad for an infinity or a NaN
+__device__ __forceinline__ unsigned mag_key(float x) { return __float_as_uint(x) & 0x7fffffffu; }
+__device__ __forceinline__ unsigned mag_key(double x) {
+  return (unsigned)__double2hiint(x) & 0x7fffffffu;
+}
+template <typename T> __device__ __forceinline__ int key_exponent(unsigned k) {
+  if (sizeof(T) == 4) {
+    if (k >= 0x7f800000u) return kBad;
+    return k == 0 ? 0 : max((int)(k >> 23), 1) - 126;
+  }
+  if (k >= 0x7ff00000u) return kBad;
+  return k == 0 ? 0 : max((int)(k >> 20), 1) - 1022;
+}
+// x as a fixed-point integer with unit 2^(E - 6 - 8 (S - 1)), rounded to nearest
+template <int S, typename T> __device__ __forceinline__ long long to_fixed(T x, int E) {
+  long long m;
+  int sh;
+  bool neg;
+  if (sizeof(T) == 4) {
+    const unsigned b = __float_as_uint((float)x);
+    const int ex = (b >> 23) & 0xff;
+    m = (b & 0x7fffffu) | (ex ? 0x800000u : 0u);
+    neg = b >> 31;
+    sh = max(ex, 1) - 150;
+  } else {
+    const long long b = __double_as_longlong((double)x);
+    const int ex = (int)((b >> 52) & 0x7ff);
+    m = (b & 0xfffffffffffffLL) | (ex ? 0x10000000000000LL : 0LL);
+    neg = b < 0;
+    sh = max(ex, 1) - 1075;
+  }
+  sh += 6 + 8 * (S - 1) - E;
+  if (sh >= 0) m <<= min(sh, 40);
+  else m = sh < -60 ? 0 : (m + (1LL << (-sh - 1))) >> -sh;
+  return neg ? -m : m;
+}
+// the biased digits of q (byte k of the result is digit S-1-k plus 128)
+template <int S> __device__ __forceinline__ unsigned long long digits(long long q) {
+  return (unsigned long long)q + (0x8080808080808080ULL >> (64 - 8 * S));
+}
+// digit s (0 = leading) of two values, as two BF16 (a low, b high)
+template <int S>
+__device__ __forceinline__ unsigned pack2(unsigned long long a, unsigned long long b, int s) {
+  const int sh = 8 * (S - 1 - s);
+  const float fa = __uint_as_float(0x4B000000u | ((unsigned)(a >> sh) & 255u)) - 8388736.f;
+  const float fb = __uint_as_float(0x4B000000u | ((unsigned)(b >> sh) & 255u)) - 8388736.f;
+  return __byte_perm(__float_as_uint(fa), __float_as_uint(fb), 0x7632);
+}
+
+// rows of a block (2n reals each) -> digits [S][rows_pad][kp] and unit exponents, one warp per
+// row; rows >= rows are written as zeros.  cs: exponents that multiply the columns (or null).
+template <int S, typename T>
+__global__ void __launch_bounds__(256)
+k_split_rows(const cplx<T>* __restrict__ X, int ldx, int n, long long rows, int rows_pad, int kp,
+             const int* __restrict__ cs, uint16_t* __restrict__ D, int* __restrict__ eu) {
+  const int lane = threadIdx.x & 31;
+  const long long r = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
+  if (r >= rows_pad) return;
+  constexpr int IT = 512 / 64;                 // n <= 512: 64 complex columns per iteration
+  T v[IT][4];
+  unsigned key = 0;
+#pragma unroll
+  for (int i = 0; i < IT; ++i) {
+    if (i * 128 >= kp) break;
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const int c = i * 64 + 2 * lane + q;
+      cplx<T> x = cmake<cplx<T>>(0, 0);
+      if (r < rows && c < n) {
+        x = X[r * ldx + c];
+        if (cs) {
+          const T f = (T)pow2d(cs[c]);
+          x.x *= f;
+          x.y *= f;
+        }
+      }
+      v[i][2 * q] = x.x;
+      v[i][2 * q + 1] = x.y;
+      key = max(key, max(mag_key(x.x), mag_key(x.y)));
+    }
+  }
+  key = __reduce_max_sync(0xffffffffu, key);
+  const int E = key_exponent<T>(key);
+  if (lane == 0) eu[r] = E == kBad ? kBad : E - 6;
+#pragma unroll
+  for (int i = 0; i < IT; ++i) {
+    if (i * 128 >= kp) break;
+    const int k = i * 128 + 4 * lane;
+    if (k >= kp) continue;
+    unsigned long long d[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) d[q] = digits<S>(E == kBad ? 0 : to_fixed<S>(v[i][q], E));
+#pragma unroll
+    for (int s = 0; s < S; ++s)
+      *reinterpret_cast<uint2*>(&D[((size_t)s * rows_pad + r) * kp + k]) =
+          make_uint2(pack2<S>(d[0], d[1], s), pack2<S>(d[2], d[3], s));
+  }
+}
+
+// Q (n x n, rows scaled by 2^-cs) -> the real right factor of the rotation: row 2j + part of
+// output column j's part, over the reals k of a block row; one warp per output row
+template <int S>
+__global__ void __launch_bounds__(256)
+k_split_q(const double2* __restrict__ Q, int n, int rows_pad, int kp, const int* __restrict__ cs,
+          uint16_t* __restrict__ D, int* __restrict__ eu) {
+  const int lane = threadIdx.x & 31;
+  const int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (r >= rows_pad) return;
+  const int j = r >> 1, part = r & 1;
+  auto at = [&](int i) {   // (factor of x_i.re, factor of x_i.im) in output part ``part``
+    if (j >= n || i >= n) return make_double2(0, 0);
+    double2 q = Q[(size_t)i * n + j];
+    if (cs) {
+      const double f = pow2d(-cs[i]);
+      q.x *= f;
+      q.y *= f;
+    }
+    return part ? make_double2(q.y, q.x) : make_double2(q.x, -q.y);
+  };
+  unsigned key = 0;
+  for (int i = lane; i < n; i += 32) {
+    const double2 q = at(i);
+    key = max(key, max(mag_key(q.x), mag_key(q.y)));
+  }
+  key = __reduce_max_sync(0xffffffffu, key);
+  const int E = key_exponent<double>(key);
+  if (lane == 0) eu[r] = E == kBad ? kBad : E - 6;
+  for (int i = lane; 2 * i < kp; i += 32) {
+    const double2 q = at(i);
+    const unsigned long long a = digits<S>(E == kBad ? 0 : to_fixed<S>(q.x, E)),
+                             b = digits<S>(E == kBad ? 0 : to_fixed<S>(q.y, E));
+#pragma unroll
+    for (int s = 0; s < S; ++s)
+      *reinterpret_cast<unsigned*>(&D[((size_t)s * rows_pad + r) * kp + 2 * i]) = pack2<S>(a, b, s);
+  }
+}
+
+// exponents that bring the columns to a common size: 2^cs[i] ~ max_j sqrt(S_jj) / sqrt(S_ii)
+__global__ void k_col_scale(const double2* __restrict__ diag, int n, int* __restrict__ cs) {
+  __shared__ int big;
+  if (threadIdx.x == 0) big = -100000;
+  __syncthreads();
+  auto half_exp = [&](int i) {   // exponent of the norm; a column that is zero or not finite: none
+    const unsigned k = mag_key(diag[i].x);
+    const int e = (int)(k >> 20);
+    return (e == 0 || e == 0x7ff) ? -100000 : (e - 1023) / 2;
+  };
+  for (int i = threadIdx.x; i < n; i += blockDim.x) atomicMax(&big, half_exp(i));
+  __syncthreads();
+  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    const int e = half_exp(i);
+    cs[i] = e == -100000 ? 0 : min(60, big - e);
+  }
+}
+
+// largest magnitude key of every real column over all rows (WEIGHT: of |x| w rounded up by a
+// factor of two)
+template <typename T, bool WEIGHT>
+__global__ void __launch_bounds__(256)
+k_col_max(const cplx<T>* __restrict__ X, int ldx, int n, long long rows,
+          const double* __restrict__ md, unsigned* __restrict__ key) {
+  const int c = blockIdx.y * 32 + (threadIdx.x & 31);
+  const long long step = (long long)gridDim.x * 8;
+  unsigned kx = 0, ky = 0;
+  if (c < n)
+    for (long long r = blockIdx.x * 8LL + (threadIdx.x >> 5); r < rows; r += step) {
+      cplx<T> x = X[r * ldx + c];
+      if (WEIGHT) {
+        const T w = 2 * (T)md[r >> 1];
+        x.x *= w;
+        x.y *= w;
+      }
+      kx = max(kx, mag_key(x.x));
+      ky = max(ky, mag_key(x.y));
+    }
+  __shared__ unsigned sk[2][8][32];
+  sk[0][threadIdx.x >> 5][threadIdx.x & 31] = kx;
+  sk[1][threadIdx.x >> 5][threadIdx.x & 31] = ky;
+  __syncthreads();
+  if (threadIdx.x < 64) {
+    const int p = threadIdx.x >> 5, l = threadIdx.x & 31;
+    unsigned k = 0;
+    for (int w = 0; w < 8; ++w) k = max(k, sk[p][w][l]);
+    const int cc = blockIdx.y * 32 + l;
+    if (cc < n && k) atomicMax(&key[2 * cc + p], k);
+  }
+}
+
+// columns of a block over the rows [r0, r0 + rows_pad) -> digits [S][cols_pad][rows_pad] (rows
+// contiguous), rows >= rows as zeros; blocks of 64 rows x 32 complex columns are transposed
+// through shared memory.  WEIGHT: x w (FP64 product).
+template <int S, typename T, bool WEIGHT>
+__global__ void __launch_bounds__(256)
+k_split_cols(const cplx<T>* __restrict__ X, int ldx, int n, long long r0, long long rows,
+             int rows_pad, int cols_pad, const double* __restrict__ md,
+             const unsigned* __restrict__ key, uint16_t* __restrict__ D, int* __restrict__ eu) {
+  using V = typename std::conditional<WEIGHT, double, T>::type;
+  __shared__ V xs[64][65];                      // [real column][row]
+  const int rb = blockIdx.x * 64, cb = blockIdx.y * 32;
+  for (int i = threadIdx.x; i < 64 * 32; i += 256) {
+    const int c = i & 31, rr = i >> 5;
+    const long long r = rb + rr;
+    V a = 0, b = 0;
+    if (r < rows && cb + c < n) {
+      const cplx<T> x = X[(r0 + r) * ldx + cb + c];
+      const double w = WEIGHT ? md[(r0 + r) >> 1] : 1.0;
+      a = WEIGHT ? (V)((double)x.x * w) : (V)x.x;
+      b = WEIGHT ? (V)((double)x.y * w) : (V)x.y;
+    }
+    xs[2 * c][rr] = a;
+    xs[2 * c + 1][rr] = b;
+  }
+  __syncthreads();
+  const int c = threadIdx.x >> 2, q = threadIdx.x & 3;   // real column, group of 16 rows
+  const int col = 2 * cb + c;
+  const int E = col < 2 * n ? key_exponent<T>(key[col]) : 0;
+  if (q == 0 && blockIdx.x == 0) eu[col] = E == kBad ? kBad : E - 6;
+  unsigned long long d[16];
+#pragma unroll
+  for (int i = 0; i < 16; ++i)
+    d[i] = digits<S>(E == kBad ? 0 : to_fixed<S>(xs[c][q * 16 + i], E));
+#pragma unroll
+  for (int s = 0; s < S; ++s) {
+    uint4* o = reinterpret_cast<uint4*>(&D[((size_t)s * cols_pad + col) * rows_pad + rb + q * 16]);
+    o[0] = make_uint4(pack2<S>(d[0], d[1], s), pack2<S>(d[2], d[3], s), pack2<S>(d[4], d[5], s),
+                      pack2<S>(d[6], d[7], s));
+    o[1] = make_uint4(pack2<S>(d[8], d[9], s), pack2<S>(d[10], d[11], s), pack2<S>(d[12], d[13], s),
+                      pack2<S>(d[14], d[15], s));
+  }
+}
+
+inline int up(int x, int m) { return (x + m - 1) / m * m; }
+
+template <int S, int MODE>
+cudaError_t run_split_gemm(const uint16_t* A, const uint16_t* B, int kpad, const SplitArgs& a, dim3 grid,
+                           cudaStream_t s) {
+  using G = SplitCfg<S>;
+  CUtensorMap ta, tb;
+  if (!tc_make_map_bf16(&ta, A, (long long)S * a.rows_a, kpad, kTM) ||
+      !tc_make_map_bf16(&tb, B, (long long)S * a.rows_b, kpad, G::N))
+    return cudaErrorInvalidValue;
+  auto k = k_split_gemm<S, MODE>;
+  const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM);
+  if (e != cudaSuccess) return e;
+  k<<<grid, 320, G::SMEM, s>>>(ta, tb, a);
+  return cudaGetLastError();
+}
+
+constexpr size_t kChunkBytes = size_t(256) << 20;   // digit buffer of a chunk of rows
+
+}  // namespace
+
+cudaError_t split_error(int* err, cudaStream_t s) {
+  cudaError_t e = cudaMemcpyFromSymbolAsync(err, g_split_err, sizeof(int), 0, cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  if (e != cudaSuccess || *err == 0) return e;
+  const int zero = 0;
+  return cudaMemcpyToSymbol(g_split_err, &zero, sizeof(int));
+}
+
+// X <- X Q in place, chunk of rows by chunk
+template <int S, typename T>
+static gbc_status rotate_split(gbc_ctx* c, cplx<T>* X, const double2* Q, long long M, int n, int ldx,
+                               const double2* diag, cudaStream_t s) {
+  constexpr int MODE = sizeof(T) == 4 ? ROT32 : ROT64;
+  using G = SplitCfg<S>;
+  const long long rows = 2 * M;
+  const int kp = up(2 * n, kKC), nb = up(2 * n, G::N);
+  const long long per = std::max<long long>(kTM, (long long)(kChunkBytes / (2 * S * (size_t)kp)) / kTM * kTM);
+  const int rc = (int)std::min<long long>(per, (rows + kTM - 1) / kTM * kTM);
+  const size_t ab = (size_t)2 * S * rc * kp, bb = (size_t)2 * S * nb * kp;
+  GBC_TRY(gbc_ensure_work(c, 13, ab + bb + sizeof(int) * ((size_t)rc + nb + n) + 1024));
+  uint16_t* A = (uint16_t*)c->work[13];
+  uint16_t* B = (uint16_t*)((char*)A + ab);
+  int* ea = (int*)((char*)B + bb);
+  int* eb = ea + rc;
+  int* cs = diag ? eb + nb : nullptr;
+  if (cs) k_col_scale<<<1, 256, 0, s>>>(diag, n, cs);
+  k_split_q<S><<<(nb + 7) / 8, 256, 0, s>>>(Q, n, nb, kp, cs, B, eb);
+  GBC_CU(c, cudaGetLastError());
+  for (long long r0 = 0; r0 < rows; r0 += rc) {
+    const long long nr = std::min<long long>(rc, rows - r0);
+    const int rp = up((int)nr, kTM);
+    k_split_rows<S, T><<<(rp + 7) / 8, 256, 0, s>>>(X + r0 * ldx, ldx, n, nr, rp, kp, cs, A, ea);
+    GBC_CU(c, cudaGetLastError());
+    SplitArgs a{rp, nb, kp / kKC, kp / kKC, nb / G::N, ea, eb, nr, n, ldx, X + r0 * ldx};
+    GBC_CU(c, (run_split_gemm<S, MODE>(A, B, kp, a, dim3((unsigned)(rp / kTM * a.ntn)), s)));
+  }
+  return GBC_OK;
+}
+// diag: the diagonal of X's Gram matrix (the columns' sizes squared), or null for orthonormal
+// columns and a unitary Q
+template <typename T>
+gbc_status launch_rotate_split(gbc_ctx* c, cplx<T>* X, const double2* Q, long long M, int n, int ldx,
+                               const double2* diag, cudaStream_t s) {
+  if (sizeof(T) == 4 && !diag) return rotate_split<4, T>(c, X, Q, M, n, ldx, diag, s);
+  return rotate_split<7, T>(c, X, Q, M, n, ldx, diag, s);
+}
+template gbc_status launch_rotate_split<float>(gbc_ctx*, float2*, const double2*, long long, int, int,
+                                               const double2*, cudaStream_t);
+template gbc_status launch_rotate_split<double>(gbc_ctx*, double2*, const double2*, long long, int, int,
+                                                const double2*, cudaStream_t);
+
+// Sm (upper triangle) = X^H diag(md) Y (md may be null: weight 1)
+template <typename TX, typename TY>
+gbc_status launch_gram_split(gbc_ctx* c, const cplx<TX>* X, int ldx, const cplx<TY>* Y, int ldy,
+                             const double* md, long long M, int n, double2* Sm, cudaStream_t s) {
+  constexpr int S = 7;
+  using G = SplitCfg<S>;
+  const long long rows = 2 * M;
+  const int ma = up(2 * n, kTM), nb = ma;    // both padded to a row tile
+  const size_t rowb = (size_t)2 * S * (ma + nb);
+  const int win = G::FLUSH * kKC;
+  const long long per = std::max<long long>(win, (long long)(kChunkBytes / rowb) / win * win);
+  const int rc = (int)std::min<long long>(per, (rows + win - 1) / win * win);
+  const size_t ab = (size_t)2 * S * ma * rc, bb = (size_t)2 * S * nb * rc;
+  GBC_TRY(gbc_ensure_work(c, 13, ab + bb + sizeof(int) * 4 * (size_t)ma + 1024));
+  uint16_t* A = (uint16_t*)c->work[13];
+  uint16_t* B = (uint16_t*)((char*)A + ab);
+  int* ea = (int*)((char*)B + bb);
+  int* eb = ea + ma;
+  unsigned* ka = (unsigned*)(eb + nb);
+  unsigned* kb = ka + ma;
+  GBC_CU(c, cudaMemsetAsync(Sm, 0, sizeof(double2) * (size_t)n * n, s));
+  GBC_CU(c, cudaMemsetAsync(ka, 0, sizeof(unsigned) * 2 * (size_t)ma, s));
+  const unsigned ncb = (unsigned)((n + 31) / 32);
+  const dim3 gm((unsigned)std::max<long long>(1, std::min<long long>((rows + 63) / 64, 16LL * gbc_sm_count() / ncb + 1)), ncb);
+  if (md) k_col_max<TX, true><<<gm, 256, 0, s>>>(X, ldx, n, rows, md, ka);
+  else k_col_max<TX, false><<<gm, 256, 0, s>>>(X, ldx, n, rows, md, ka);
+  k_col_max<TY, false><<<gm, 256, 0, s>>>(Y, ldy, n, rows, nullptr, kb);
+  GBC_CU(c, cudaGetLastError());
+  int tiles = 0;
+  const int ntn = nb / G::N;
+  for (int I = 0; I < ma / kTM; ++I) tiles += ntn - I * (kTM / G::N);
+  for (long long r0 = 0; r0 < rows; r0 += rc) {
+    const long long nr = std::min<long long>(rc, rows - r0);
+    const int rp = up((int)nr, win);
+    const dim3 gs((unsigned)(rp / 64), (unsigned)(ma / 64));
+    if (md) k_split_cols<S, TX, true><<<gs, 256, 0, s>>>(X, ldx, n, r0, nr, rp, ma, md, ka, A, ea);
+    else k_split_cols<S, TX, false><<<gs, 256, 0, s>>>(X, ldx, n, r0, nr, rp, ma, md, ka, A, ea);
+    k_split_cols<S, TY, false><<<gs, 256, 0, s>>>(Y, ldy, n, r0, nr, rp, nb, nullptr, kb, B, eb);
+    GBC_CU(c, cudaGetLastError());
+    // K split so that the CTAs fill the SMs about once, in whole read-out windows
+    const int nwin = rp / win;
+    const int split = std::max(1, std::min(nwin, gbc_sm_count() / std::max(1, tiles)));
+    const int kper = (nwin + split - 1) / split * G::FLUSH;
+    SplitArgs a{ma, nb, rp / kKC, kper, ntn, ea, eb, nr, n, 0, Sm};
+    GBC_CU(c, (run_split_gemm<S, GRAM>(A, B, rp, a,
+                                       dim3((unsigned)tiles, (unsigned)((rp / kKC + kper - 1) / kper)), s)));
+  }
+  return GBC_OK;
+}
+template gbc_status launch_gram_split<float, float>(gbc_ctx*, const float2*, int, const float2*, int,
+                                                    const double*, long long, int, double2*, cudaStream_t);
+template gbc_status launch_gram_split<float, double>(gbc_ctx*, const float2*, int, const double2*, int,
+                                                     const double*, long long, int, double2*, cudaStream_t);
+template gbc_status launch_gram_split<double, double>(gbc_ctx*, const double2*, int, const double2*, int,
+                                                      const double*, long long, int, double2*, cudaStream_t);

@@ -44,29 +44,6 @@ __device__ int g_tcl_err;   // set when a bounded wait of the GEMM expired
 
 constexpr int kBM = 128;    // rows of D per CTA
 
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const void* tmap, int x, int y,
-                                            uint32_t mbar) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes "
-      "[%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
-      "l"(tmap), "r"(x), "r"(y), "r"(mbar)
-      : "memory");
-}
-
-__host__ __device__ constexpr uint32_t idesc_bf16(int M, int N) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) |
-         ((uint32_t)(M >> 4) << 24);
-}
-
-__device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc,
-                                         uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-
 template <int MODE, int BN> struct GemmCfg {
   static constexpr int PL = MODE ? 2 : 1;               // planes (hi, lo) per operand
   static constexpr int ABYTES = kBM * 128;              // one 128-byte K slice of A
@@ -134,18 +111,18 @@ k_tcl_gemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUten
       if (*reinterpret_cast<volatile int*>(fail)) break;
       const uint32_t fb = tc::smem_u32(&full[s]);
       tc::mbar_arrive_expect_tx(fb, G::STAGE);
-      tma_load_2d(A(s, 0), &ta, ax0 + kt * KE, (int)m0, fb);
-      tma_load_2d(B(s, 0), &tb, kt * KE, n0, fb);
+      tc::tma_load_2d(A(s, 0), &ta, ax0 + kt * KE, (int)m0, fb);
+      tc::tma_load_2d(B(s, 0), &tb, kt * KE, n0, fb);
       if (MODE) {
-        tma_load_2d(A(s, 1), &ta_lo, ax0 + kt * KE, (int)m0, fb);
-        tma_load_2d(B(s, 1), &tb_lo, kt * KE, n0, fb);
+        tc::tma_load_2d(A(s, 1), &ta_lo, ax0 + kt * KE, (int)m0, fb);
+        tc::tma_load_2d(B(s, 1), &tb_lo, kt * KE, n0, fb);
       }
     }
     if (*reinterpret_cast<volatile int*>(fail))   // let the copies in flight land first
       for (int j = kt > G::STAGES ? kt - G::STAGES : 0; j < kt; ++j)
         tc::mbar_wait_bounded(tc::smem_u32(&full[j % G::STAGES]), (j / G::STAGES) & 1);
   } else if (warp == 1 && lane == 0) {
-    constexpr uint32_t idesc = MODE ? idesc_bf16(kBM, BN) : tc::idesc_tf32(kBM, BN);
+    constexpr uint32_t idesc = MODE ? tc::idesc_bf16(kBM, BN) : tc::idesc_tf32(kBM, BN);
     int kt = 0;
     for (; kt < nkt; ++kt) {
       const int s = kt % G::STAGES;
@@ -159,9 +136,9 @@ k_tcl_gemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUten
         const uint32_t o = kk * 32;
         const uint32_t acc = (kt > 0 || kk > 0) ? 1u : 0u;
         if (MODE) {
-          mma_bf16(tmem, tc::sdesc_sw128(A(s, 0) + o), tc::sdesc_sw128(B(s, 0) + o), idesc, acc);
-          mma_bf16(tmem, tc::sdesc_sw128(A(s, 0) + o), tc::sdesc_sw128(B(s, 1) + o), idesc, 1u);
-          mma_bf16(tmem, tc::sdesc_sw128(A(s, 1) + o), tc::sdesc_sw128(B(s, 0) + o), idesc, 1u);
+          tc::mma_bf16(tmem, tc::sdesc_sw128(A(s, 0) + o), tc::sdesc_sw128(B(s, 0) + o), idesc, acc);
+          tc::mma_bf16(tmem, tc::sdesc_sw128(A(s, 0) + o), tc::sdesc_sw128(B(s, 1) + o), idesc, 1u);
+          tc::mma_bf16(tmem, tc::sdesc_sw128(A(s, 1) + o), tc::sdesc_sw128(B(s, 0) + o), idesc, 1u);
         } else {
           tc::mma_tf32(tmem, tc::sdesc_sw128(A(s, 0) + o), tc::sdesc_sw128(B(s, 0) + o), idesc, acc);
         }
@@ -577,6 +554,10 @@ gbc_status tcl_apply(gbc_ctx* c, const float2* X, float2* Y, int nvec, int ldx, 
 }
 
 // bounded-wait flag of the tensor-core cell apply (cleared on read)
+bool tc_make_map_bf16(CUtensorMap* m, const void* p, long long rows, int cols, int box_rows) {
+  return make_map(m, p, rows, cols, box_rows, 1);
+}
+
 cudaError_t tcl_error(int* err, cudaStream_t s) {
   cudaError_t e = cudaMemcpyFromSymbolAsync(err, g_tcl_err, sizeof(int), 0, cudaMemcpyDeviceToHost, s);
   if (e != cudaSuccess) return e;

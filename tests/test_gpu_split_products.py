@@ -1,0 +1,104 @@
+"""CholGS and Rayleigh-Ritz through the split tensor-core products (16 columns and more), at
+the edges of their tiles (64- and 128-wide, padded columns, the largest block), with a padded
+leading dimension, columns and rows of very different size, and blocks that are not finite or
+not of full rank.
+
+FP64 blocks: X^H M X = I and the span to 1e-12 (the FP64 rounding of test_gpu_parity.py).  FP32
+blocks: one rounding to FP32 per entry, so the rotated columns agree with the FP64 result to
+2^-23 of a column (a rounding error is at most 2^-24 of an entry, and the input is exact)."""
+import numpy as np
+import pytest
+
+import synthetic as syn
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def g():
+    import __graft_entry__ as ge
+    ge.build()
+    import paper_2410_02754_gb300 as pkg
+    return pkg
+
+
+def block(M, n, seed):
+    """Columns from 1 to 1e-3, rows falling off by 1e-1.5, neighbouring columns overlapping."""
+    X = syn.random_block(M, n, seed)
+    X[:, :, 1:] += 0.4 * X[:, :, :-1]
+    return X * np.logspace(0, -1.5, M)[:, None, None] * np.logspace(0, -3, n)
+
+
+def context(g, prec, ncell=(3, 3, 3), p=5):
+    prob = syn.make_problem(ncell=ncell, h=(1.0, 1.1, 0.9), p=p, k=(0.1, 0.0, 0.0), natoms=1, rc=1.0, seed=4)
+    ctx = g.Context(0)
+    ctx.set_problem(prob)
+    ctx.set_precision(prec)
+    return ctx, prob
+
+
+def device(X, prec, ldx):
+    out = torch.zeros(X.shape[:2] + (ldx,), dtype=torch.complex64 if prec else torch.complex128, device="cuda")
+    out[:, :, :X.shape[2]] = torch.from_numpy(X).to(out.dtype).cuda()
+    return out
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("n,ldx", [(15, 15), (16, 17), (33, 33), (64, 64), (65, 70), (129, 129), (512, 512)])
+def test_cholgs_tiles(g, prec, n, ldx):
+    ctx, prob = context(g, prec)
+    M = prob.nnodes
+    Xd = device(block(M, n, 3), prec, ldx)
+    X = Xd[:, :, :n].cpu().numpy().astype(np.complex128).reshape(2 * M, n)   # the exact input
+    md = np.repeat(ctx.mass(), 2)[:, None]
+    L = np.linalg.cholesky(X.conj().T @ (md * X))
+    ref = np.linalg.solve(L.conj(), X.T).T          # X L^-H
+    ctx.cholgs(Xd, nvec=n)
+    Y = Xd[:, :, :n].cpu().numpy().astype(np.complex128).reshape(2 * M, n)
+    if prec == 0:
+        G = Y.conj().T @ (md * Y)
+        assert np.abs(G - np.eye(n)).max() < 1e-12
+    err = np.linalg.norm(Y - ref, axis=0) / np.linalg.norm(ref, axis=0)
+    assert err.max() < (1e-12 if prec == 0 else 2.0 ** -23)
+    if ldx > n:
+        assert not Xd[:, :, n:].any()
+    ctx.close()
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("n", [16, 63, 130])
+def test_rayleigh_ritz_tiles(g, prec, n):
+    from oracle import fe
+    ctx, prob = context(g, prec, (2, 2, 3), 4)
+    d = fe.Discretisation(prob)
+    Xd = device(block(prob.nnodes, n, 5), prec, n)
+    ctx.cholgs(Xd)
+    X = Xd.cpu().numpy().astype(np.complex128)
+    flat = X.reshape(-1, n)
+    ref = np.linalg.eigvalsh(flat.conj().T @ d.apply_h(X).reshape(-1, n))
+    ritz = ctx.rayleigh_ritz(Xd)
+    assert np.abs(ritz - ref).max() < 1e-11 * np.abs(ref).max()
+    Y = Xd.cpu().numpy().astype(np.complex128)
+    Hp = Y.reshape(-1, n).conj().T @ d.apply_h(Y).reshape(-1, n)
+    off = Hp - np.diag(np.diag(Hp))
+    assert np.abs(off).max() < (1e-11 if prec == 0 else 1e-5) * np.abs(ref).max()
+    ctx.close()
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+def test_cholgs_refuses_what_it_refused(g, prec):
+    ctx, prob = context(g, prec, (2, 2, 2), 3)
+    for bad in (np.inf, np.nan, 0.0):
+        X = syn.random_block(prob.nnodes, 20, 6)
+        if bad == 0.0:
+            X[:, :, 7] = 0.0
+        else:
+            X[11, 1, 7] = bad
+        Xd = device(X, prec, 20)
+        keep = Xd.clone()
+        with pytest.raises(g.GbcError) as e:
+            ctx.cholgs(Xd)
+        assert e.value.status == 5                       # GBC_ENOTPD, the block unchanged
+        assert torch.equal(torch.view_as_real(Xd).nan_to_num(), torch.view_as_real(keep).nan_to_num())
+    ctx.close()
