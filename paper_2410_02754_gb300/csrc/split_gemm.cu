@@ -24,9 +24,10 @@
 // 28 BF16 products at 1.9 PFLOP/s are an FP64-accurate 68 TFLOP/s.  Per tile (128 x 128 for
 // S = 4, 128 x 64 for S = 7) every order has its own accumulator in tensor memory and all S
 // digit slices of a 64-wide K chunk are in shared memory at once (one TMA box each), so a
-// slice is loaded once per tile and used in up to S products.  The products run from the
-// outermost digit pairs (0, j), (i, 0) inwards: after step m the slices m and S-1-m are free,
-// and their next chunk loads behind the remaining steps.
+// slice is loaded once per tile and used in up to S products.  Step i multiplies A_i with all
+// of B_0 .. B_{S-1-i} in instructions of up to 256 columns (one product per instruction, 64
+// columns, ran at a quarter of this rate); A_i's next chunk then loads behind the other steps,
+// B is double-buffered.
 #include <algorithm>
 #include <cmath>
 #include <cuda.h>
@@ -44,17 +45,19 @@ constexpr int kBad = 0x7fffffff;      // exponent of a row with an infinity or a
 template <int S> struct SplitCfg {
   static constexpr int N = S <= 4 ? 128 : 64;             // tile columns
   static constexpr int FLUSH = S <= 4 ? 4 : 2;            // K chunks between read-outs
-  static constexpr int ABYTES = kTM * 128, SLICE = ABYTES + N * 128;
-  static constexpr size_t SMEM = 1024 + (size_t)S * SLICE + 256;
+  static constexpr int ABYTES = kTM * 128, BBYTES = N * 128;
+  static constexpr size_t SMEM = 1024 + (size_t)S * (ABYTES + 2 * BBYTES) + 256;
   static_assert(S * N <= 512, "tensor memory columns");
   static_assert((long long)S * FLUSH * kKC << 14 <= 1LL << 24, "exact accumulation");
+  static_assert(SMEM <= 227 * 1024, "shared memory");
 };
 
 enum { ROT32 = 0, ROT64 = 1, GRAM = 2 };
 struct SplitArgs {
   int rows_a, rows_b;      // rows of a slice of A and B
-  int nchunk, kper;        // K chunks; chunks per CTA (GRAM: split over blockIdx.y)
+  int nchunk, kper;        // K chunks; chunks per work item (GRAM: a part of them)
   int ntn;                 // column tiles
+  int ntiles, nwork;       // tiles; work items (tiles, GRAM: x K parts)
   const int *ea, *eb;      // unit exponents (E - 6) of the rows of A and B
   long long rows;          // rotation: valid rows of the chunk
   int n;                   // complex columns
@@ -67,42 +70,51 @@ __device__ __forceinline__ double pow2d(int e) {
   return __hiloint2double((1023 + max(-1000, min(1000, e))) << 20, 0);
 }
 
+// Persistent: CTAs take work items blockIdx.x, + gridDim.x, ...; the roles run on across items.
 template <int S, int MODE>
 __global__ void __launch_bounds__(320, 1)
 k_split_gemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb,
              const SplitArgs a) {
   using G = SplitCfg<S>;
   constexpr int N = G::N;
-  int m0, n0, k0 = 0, nk = a.nchunk;
-  if (MODE == GRAM) {   // tiles that reach the diagonal or above it, row by row
-    int I = 0, t = blockIdx.x, first = 0;
-    while (t >= a.ntn - first) {
-      t -= a.ntn - first;
-      ++I;
-      first = I * (kTM / N);
+  struct Item { int m0, n0, k0, nk; };
+  auto decode = [&](int w) {
+    Item it{0, 0, 0, a.nchunk};
+    if (MODE == GRAM) {   // tiles that reach the diagonal or above it, row by row
+      int I = 0, t = w % a.ntiles, first = 0;
+      while (t >= a.ntn - first) {
+        t -= a.ntn - first;
+        ++I;
+        first = I * (kTM / N);
+      }
+      it.m0 = I * kTM;
+      it.n0 = (first + t) * N;
+      it.k0 = (w / a.ntiles) * a.kper;
+      it.nk = min(a.kper, a.nchunk - it.k0);
+    } else {   // column tiles of a row tile next to each other (its digits stay in L2)
+      it.m0 = w / a.ntn * kTM;
+      it.n0 = w % a.ntn * N;
     }
-    m0 = I * kTM;
-    n0 = (first + t) * N;
-    k0 = blockIdx.y * a.kper;
-    nk = min(a.kper, a.nchunk - k0);
-    if (nk <= 0) return;
-  } else {
-    m0 = (int)(blockIdx.x / a.ntn) * kTM;
-    n0 = (int)(blockIdx.x % a.ntn) * N;
-  }
+    return it;
+  };
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* st = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-  uint64_t* full = reinterpret_cast<uint64_t*>(st + S * G::SLICE);   // [S] slice landed
-  uint64_t* empty = full + S;                                        // [S] slice free
-  uint64_t* accf = empty + S;                                        // accumulators complete
+  uint64_t* fulla = reinterpret_cast<uint64_t*>(st + S * (G::ABYTES + 2 * G::BBYTES));   // [S]
+  uint64_t* emptya = fulla + S;                                                          // [S]
+  uint64_t* fullb = emptya + S;                                                          // [2]
+  uint64_t* emptyb = fullb + 2;                                                          // [2]
+  uint64_t* accf = emptyb + 2;                                       // accumulators complete
   uint64_t* acce = accf + 1;                                         // accumulators read out
   uint64_t* drain = acce + 1;                                        // every MMA complete
   uint32_t* tslot = reinterpret_cast<uint32_t*>(drain + 1);
   int* fail = reinterpret_cast<int*>(tslot + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  auto A = [&](int s) { return tc::smem_u32(st + s * G::SLICE); };
-  auto B = [&](int s) { return tc::smem_u32(st + s * G::SLICE + G::ABYTES); };
+  // A: one buffer per digit slice; B: two buffers of all slices back to back
+  auto A = [&](int s) { return tc::smem_u32(st + s * G::ABYTES); };
+  auto B = [&](int buf, int s) {
+    return tc::smem_u32(st + S * G::ABYTES + (buf * S + s) * G::BBYTES);
+  };
   auto failed = [&]() { return *reinterpret_cast<volatile int*>(fail) != 0; };
 
   if (warp == 0) {
@@ -111,8 +123,12 @@ k_split_gemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUt
   }
   if (threadIdx.x == 32) {
     for (int s = 0; s < S; ++s) {
-      tc::mbar_init(tc::smem_u32(&full[s]), 1);
-      tc::mbar_init(tc::smem_u32(&empty[s]), 1);
+      tc::mbar_init(tc::smem_u32(&fulla[s]), 1);
+      tc::mbar_init(tc::smem_u32(&emptya[s]), 1);
+    }
+    for (int s = 0; s < 2; ++s) {
+      tc::mbar_init(tc::smem_u32(&fullb[s]), 1);
+      tc::mbar_init(tc::smem_u32(&emptyb[s]), 1);
     }
     tc::mbar_init(tc::smem_u32(accf), 1);
     tc::mbar_init(tc::smem_u32(acce), 8);
@@ -124,63 +140,76 @@ k_split_gemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUt
   __syncthreads();
   tc::fence_after_sync();
   const uint32_t tmem = *tslot;
-  const int nwin = (nk + G::FLUSH - 1) / G::FLUSH;
 
   if (warp == 0 && lane == 0) {
-    // producer: slices in the order in which the MMA steps free them
-    int issued[S];
+    // producer: chunk q of the CTA; A slice s once step s of chunk q - 1 is done, B buffer
+    // q & 1 once chunk q - 2 is done
+    int q = 0, ib = 0, ia[S];
 #pragma unroll
-    for (int s = 0; s < S; ++s) issued[s] = 0;
-    for (int c = 0; c < nk && !failed(); ++c) {
-#pragma unroll
-      for (int o = 0; o < S; ++o) {
-        const int s = (o & 1) ? S - 1 - o / 2 : o / 2;
-        if (c > 0 && !tc::mbar_wait_bounded(tc::smem_u32(&empty[s]), (c - 1) & 1)) atomicExch(fail, 1);
+    for (int s = 0; s < S; ++s) ia[s] = 0;
+    for (int w = blockIdx.x; w < a.nwork && !failed(); w += gridDim.x) {
+      const Item it = decode(w);
+      for (int c = 0; c < it.nk && !failed(); ++c, ++q) {
+        const int x = (it.k0 + c) * kKC, buf = q & 1;
+        if (q > 1 && !tc::mbar_wait_bounded(tc::smem_u32(&emptyb[buf]), (q / 2 - 1) & 1)) atomicExch(fail, 1);
         if (failed()) break;
-        const uint32_t fb = tc::smem_u32(&full[s]);
-        tc::mbar_arrive_expect_tx(fb, G::SLICE);
-        tc::tma_load_2d(A(s), &ta, (k0 + c) * kKC, s * a.rows_a + m0, fb);
-        tc::tma_load_2d(B(s), &tb, (k0 + c) * kKC, s * a.rows_b + n0, fb);
-        issued[s] = c + 1;
+        const uint32_t fb = tc::smem_u32(&fullb[buf]);
+        tc::mbar_arrive_expect_tx(fb, S * G::BBYTES);
+#pragma unroll
+        for (int s = 0; s < S; ++s) tc::tma_load_2d(B(buf, s), &tb, x, s * a.rows_b + it.n0, fb);
+        ib = q + 1;
+#pragma unroll
+        for (int s = 0; s < S; ++s) {
+          if (q > 0 && !tc::mbar_wait_bounded(tc::smem_u32(&emptya[s]), (q - 1) & 1)) atomicExch(fail, 1);
+          if (failed()) break;
+          const uint32_t fa = tc::smem_u32(&fulla[s]);
+          tc::mbar_arrive_expect_tx(fa, G::ABYTES);
+          tc::tma_load_2d(A(s), &ta, x, s * a.rows_a + it.m0, fa);
+          ia[s] = q + 1;
+        }
       }
     }
-    if (failed())   // let the copies in flight land first
+    if (failed()) {   // let the copies in flight land first
 #pragma unroll
       for (int s = 0; s < S; ++s)
-        if (issued[s]) tc::mbar_wait_bounded(tc::smem_u32(&full[s]), (issued[s] - 1) & 1);
+        if (ia[s]) tc::mbar_wait_bounded(tc::smem_u32(&fulla[s]), (ia[s] - 1) & 1);
+      for (int j = max(0, ib - 2); j < ib; ++j)
+        tc::mbar_wait_bounded(tc::smem_u32(&fullb[j & 1]), (j / 2) & 1);
+    }
   } else if (warp == 1 && lane == 0) {
-    constexpr uint32_t idesc = tc::idesc_bf16(kTM, N);
-    for (int c = 0; c < nk && !failed(); ++c) {
-      const bool first = c % G::FLUSH == 0;
-      if (first && c > 0) {
-        if (!tc::mbar_wait_bounded(tc::smem_u32(acce), (c / G::FLUSH - 1) & 1)) atomicExch(fail, 1);
-        tc::fence_after_sync();
-      }
-      auto pair = [&](int i, int j, bool fresh) {
+    int q = 0, win = 0;
+    for (int w = blockIdx.x; w < a.nwork && !failed(); w += gridDim.x) {
+      const Item it = decode(w);
+      for (int c = 0; c < it.nk && !failed(); ++c, ++q) {
+        const bool first = c % G::FLUSH == 0;
+        if (first && win > 0 && !tc::mbar_wait_bounded(tc::smem_u32(acce), (win - 1) & 1)) atomicExch(fail, 1);
+        const int buf = q & 1;
+        if (!tc::mbar_wait_bounded(tc::smem_u32(&fullb[buf]), (q / 2) & 1)) atomicExch(fail, 1);
 #pragma unroll
-        for (int kk = 0; kk < 4; ++kk)
-          tc::mma_bf16(tmem + (i + j) * N, tc::sdesc_sw128(A(i) + kk * 32),
-                       tc::sdesc_sw128(B(j) + kk * 32), idesc, (fresh && kk == 0) ? 0u : 1u);
-      };
-      auto need = [&](int s) {
-        if (!tc::mbar_wait_bounded(tc::smem_u32(&full[s]), c & 1)) atomicExch(fail, 1);
-        tc::fence_after_sync();
-      };
+        for (int i = 0; i < S; ++i) {
+          if (!tc::mbar_wait_bounded(tc::smem_u32(&fulla[i]), q & 1)) atomicExch(fail, 1);
+          tc::fence_after_sync();
+          // A_i against B_0 .. B_{S-1-i} at once: the slices are consecutive rows of one operand
+          // and their orders i .. S-1 consecutive accumulators, so an instruction is up to 256
+          // columns wide (64 columns take as long as 256)
 #pragma unroll
-      for (int m = 0; 2 * m <= S - 1; ++m) {
-        // pairs whose smaller index is m; the others in the order of their arrival
+          for (int kk = 0; kk < 4; ++kk)
 #pragma unroll
-        for (int o = 2 * m; o < S; ++o) {
-          const int s = (o & 1) ? S - 1 - o / 2 : o / 2;
-          if (m == 0) need(s);
-          if (s < m || s + m > S - 1) continue;
-          pair(m, s, first && m == 0);
-          if (s != m) pair(s, m, false);
+            for (int j = 0; j < S - i; j += 256 / N) {
+              constexpr int W = 256 / N;
+              const int cnt = S - i - j < W ? S - i - j : W;
+              tc::mma_bf16(tmem + (i + j) * N, tc::sdesc_sw128(A(i) + kk * 32),
+                           tc::sdesc_sw128(B(buf, j) + kk * 32), tc::idesc_bf16(kTM, cnt * N),
+                           (first && i == 0 && kk == 0) ? 0u : 1u);
+            }
+          tc::mma_commit(tc::smem_u32(&emptya[i]));
         }
-        tc::mma_commit(tc::smem_u32(&empty[m]));
-        if (S - 1 - m != m) tc::mma_commit(tc::smem_u32(&empty[S - 1 - m]));
+        tc::mma_commit(tc::smem_u32(&emptyb[buf]));
+        if ((c + 1) % G::FLUSH == 0 || c + 1 == it.nk) {
+          tc::mma_commit(tc::smem_u32(accf));
+          ++win;
+        }
       }
-      if ((c + 1) % G::FLUSH == 0 || c + 1 == nk) tc::mma_commit(tc::smem_u32(accf));
     }
     // tensor memory is given back only after the issued MMAs (also after a failure)
     tc::mma_commit(tc::smem_u32(drain));
@@ -189,97 +218,105 @@ k_split_gemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUt
     const int g = warp & 3, half = (warp - 2) >> 2;
     constexpr int NC = N / 2;                        // columns of a thread
     const uint32_t tl = tmem + ((uint32_t)(g * 32) << 16) + (uint32_t)(half * NC);
-    // orders 0..3 and 4..S-1 as 64-bit integers, in units of 256^-3 and 256^-(S-1)
-    long long hi[NC], lo[S > 4 ? NC : 1];
-#pragma unroll
-    for (int i = 0; i < NC; ++i) {
-      hi[i] = 0;
-      if (S > 4) lo[i] = 0;
-    }
+    int win = 0;
     bool ok = true;
-    for (int w = 0; w < nwin && ok; ++w) {
-      ok = tc::mbar_wait_bounded(tc::smem_u32(accf), w & 1);
-      if (!ok) atomicExch(fail, 1);
-      ok = ok && !failed();
-      tc::fence_after_sync();
-      if (ok) {
+    for (int w = blockIdx.x; w < a.nwork && ok; w += gridDim.x) {
+      const Item it = decode(w);
+      // orders 0..3 and 4..S-1 as 64-bit integers, in units of 256^-3 and 256^-(S-1)
+      long long hi[NC], lo[S > 4 ? NC : 1];
 #pragma unroll
-        for (int c0 = 0; c0 < NC; c0 += 8) {
-          uint32_t r[S][8];
-#pragma unroll
-          for (int t = 0; t < S; ++t) tc::tmem_ld8_nowait(tl + t * N + c0, r[t]);
-          tc::tmem_wait_ld();
-#pragma unroll
-          for (int i = 0; i < 8; ++i)
-#pragma unroll
-            for (int t = 0; t < S; ++t) {
-              const int v = __float2int_rn(__uint_as_float(r[t][i]));
-              if (t < 4) hi[c0 + i] += (long long)v * (1 << (8 * (3 - t)));
-              else lo[c0 + i] += (long long)v * (1 << (8 * (S - 1 - t)));
-            }
-        }
+      for (int i = 0; i < NC; ++i) {
+        hi[i] = 0;
+        if (S > 4) lo[i] = 0;
       }
-      tc::fence_before_sync();
-      if (lane == 0) tc::mbar_arrive(tc::smem_u32(acce));
-    }
-    if (ok) {
-      const int mr = m0 + g * 32 + lane;
-      const int ea = a.ea[mr];
-      const int cb = n0 + half * NC;
-      const int* eb = a.eb + cb;
-      // the sum as one integer W in units of 2^(ea + eb - 24 - sh): exact where |hi| < 2^38 (or
-      // S = 4), else cut 2^-53 below its leading bit; converted (and rounded) once
-      auto value = [&](int i, int& sh) {
-        if (S == 4) {
-          sh = 0;
-          return hi[i];
+      const int nwin = (it.nk + G::FLUSH - 1) / G::FLUSH;
+      for (int v = 0; v < nwin && ok; ++v, ++win) {
+        ok = tc::mbar_wait_bounded(tc::smem_u32(accf), win & 1);
+        if (!ok) atomicExch(fail, 1);
+        ok = ok && !failed();
+        tc::fence_after_sync();
+        if (ok) {
+#pragma unroll
+          for (int c0 = 0; c0 < NC; c0 += 8) {
+            uint32_t r[S][8];
+#pragma unroll
+            for (int t = 0; t < S; ++t) tc::tmem_ld8_nowait(tl + t * N + c0, r[t]);
+            tc::tmem_wait_ld();
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+#pragma unroll
+              for (int t = 0; t < S; ++t) {
+                const int x = __float2int_rn(__uint_as_float(r[t][i]));
+                if (t < 4) hi[c0 + i] += (long long)x * (1 << (8 * (3 - t)));
+                else lo[c0 + i] += (long long)x * (1 << (8 * (S - 1 - t)));
+              }
+          }
         }
-        const bool small = llabs(hi[i]) < (1LL << 38);
-        sh = small ? 24 : 15;
-        return small ? (hi[i] << 24) + lo[S > 4 ? i : 0] : (hi[i] << 15) + (lo[S > 4 ? i : 0] >> 9);
-      };
-      if (MODE == ROT32) {
-        if (mr < a.rows) {
-          float2* o = reinterpret_cast<float2*>(a.out) + (size_t)mr * a.ldo + cb / 2;
+        tc::fence_before_sync();
+        if (lane == 0) tc::mbar_arrive(tc::smem_u32(acce));
+      }
+      if (ok) {
+        const int mr = it.m0 + g * 32 + lane;
+        const int ea = a.ea[mr];
+        const int cb = it.n0 + half * NC;
+        const int* eb = a.eb + cb;
+        // a rotation's sum (|hi| < 2^47) as one integer in units of 2^(ea + eb - 24 - sh): exact
+        // where |hi| < 2^38 (or S = 4), else cut 2^-53 below its leading bit; rounded once
+        auto value = [&](int i, int& sh) {
+          if (S == 4) {
+            sh = 0;
+            return hi[i];
+          }
+          const bool small = llabs(hi[i]) < (1LL << 38);
+          sh = small ? 24 : 15;
+          return small ? (hi[i] << 24) + lo[S > 4 ? i : 0] : (hi[i] << 15) + (lo[S > 4 ? i : 0] >> 9);
+        };
+        if (MODE == ROT32) {
+          if (mr < a.rows) {
+            float2* o = reinterpret_cast<float2*>(a.out) + (size_t)mr * a.ldo + cb / 2;
+#pragma unroll
+            for (int i = 0; i < NC; i += 2) {
+              if (cb + i >= 2 * a.n) break;
+              float v[2];
+#pragma unroll
+              for (int q = 0; q < 2; ++q) {
+                int sh;
+                const float f = __ll2float_rn(value(i + q, sh));
+                const int e = eb[i + q];
+                v[q] = (ea == kBad || e == kBad) ? NAN : scalbnf(f, ea + e - 24 - sh);
+              }
+              o[i / 2] = make_float2(v[0], v[1]);
+            }
+          }
+        } else {
 #pragma unroll
           for (int i = 0; i < NC; i += 2) {
             if (cb + i >= 2 * a.n) break;
-            float v[2];
+            double v[2];
 #pragma unroll
             for (int q = 0; q < 2; ++q) {
-              int sh;
-              const float f = __ll2float_rn(value(i + q, sh));
-              const int e = eb[i + q];
-              v[q] = (ea == kBad || e == kBad) ? NAN : scalbnf(f, ea + e - 24 - sh);
+              int sh = 0;
+              if (MODE == GRAM)   // hi may use all of its 53 bits here: hi + 2^-24 lo, rounded once
+                v[q] = fma(__ll2double_rn(lo[S > 4 ? i + q : 0]), pow2d(-24), __ll2double_rn(hi[i + q]));
+              else
+                v[q] = __ll2double_rn(value(i + q, sh));
+              const int e = eb[i + q], x = ea + e - 24 - sh;
+              if (ea == kBad || e == kBad) v[q] = NAN;
+              else if (abs(x) > 900) v[q] = scalbn(v[q], x);
+              else if (v[q] != 0.0)   // a multiplication by 2^x on the integer pipe (2^-24 <= |v| < 2^63)
+                v[q] = __hiloint2double(__double2hiint(v[q]) + (x << 20), __double2loint(v[q]));
             }
-            o[i / 2] = make_float2(v[0], v[1]);
-          }
-        }
-      } else {
-#pragma unroll
-        for (int i = 0; i < NC; i += 2) {
-          if (cb + i >= 2 * a.n) break;
-          double v[2];
-#pragma unroll
-          for (int q = 0; q < 2; ++q) {
-            int sh;
-            v[q] = __ll2double_rn(value(i + q, sh));
-            const int e = eb[i + q], x = ea + e - 24 - sh;
-            if (ea == kBad || e == kBad) v[q] = NAN;
-            else if (abs(x) > 900) v[q] = scalbn(v[q], x);
-            else if (v[q] != 0.0)   // a multiplication by 2^x on the integer pipe (1 <= |v| < 2^63)
-              v[q] = __hiloint2double(__double2hiint(v[q]) + (x << 20), __double2loint(v[q]));
-          }
-          if (MODE == ROT64) {
-            if (mr < a.rows)
-              reinterpret_cast<double2*>(a.out)[(size_t)mr * a.ldo + (cb + i) / 2] = make_double2(v[0], v[1]);
-          } else {
-            // conj(x) y of complex columns (mr / 2, (cb + i) / 2): re = rr + ii, im = ri - ir
-            const int ci = mr >> 1, cj = (cb + i) >> 1;
-            if (ci < a.n && ci <= cj) {
-              double2* s = reinterpret_cast<double2*>(a.out) + (size_t)ci * a.n + cj;
-              atomicAdd(&s->x, (mr & 1) ? v[1] : v[0]);
-              atomicAdd(&s->y, (mr & 1) ? -v[0] : v[1]);
+            if (MODE == ROT64) {
+              if (mr < a.rows)
+                reinterpret_cast<double2*>(a.out)[(size_t)mr * a.ldo + (cb + i) / 2] = make_double2(v[0], v[1]);
+            } else {
+              // conj(x) y of complex columns (mr / 2, (cb + i) / 2): re = rr + ii, im = ri - ir
+              const int ci = mr >> 1, cj = (cb + i) >> 1;
+              if (ci < a.n && ci <= cj) {
+                double2* s = reinterpret_cast<double2*>(a.out) + (size_t)ci * a.n + cj;
+                atomicAdd(&s->x, (mr & 1) ? v[1] : v[0]);
+                atomicAdd(&s->y, (mr & 1) ? -v[0] : v[1]);
+              }
             }
           }
         }
@@ -530,7 +567,7 @@ k_split_cols(const cplx<T>* __restrict__ X, int ldx, int n, long long r0, long l
 inline int up(int x, int m) { return (x + m - 1) / m * m; }
 
 template <int S, int MODE>
-cudaError_t run_split_gemm(const uint16_t* A, const uint16_t* B, int kpad, const SplitArgs& a, dim3 grid,
+cudaError_t run_split_gemm(const uint16_t* A, const uint16_t* B, int kpad, const SplitArgs& a,
                            cudaStream_t s) {
   using G = SplitCfg<S>;
   CUtensorMap ta, tb;
@@ -540,11 +577,13 @@ cudaError_t run_split_gemm(const uint16_t* A, const uint16_t* B, int kpad, const
   auto k = k_split_gemm<S, MODE>;
   const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM);
   if (e != cudaSuccess) return e;
-  k<<<grid, 320, G::SMEM, s>>>(ta, tb, a);
+  k<<<(unsigned)std::min(a.nwork, gbc_sm_count()), 320, G::SMEM, s>>>(ta, tb, a);
   return cudaGetLastError();
 }
 
-constexpr size_t kChunkBytes = size_t(256) << 20;   // digit buffer of a chunk of rows
+// digit buffer of a chunk of rows: 884,736 x 256 CholGS 72 / 66 ms at 80 / 256 MB (fewer, longer
+// launches; that the digits stay in L2 at 80 MB does not make up for it)
+constexpr size_t kChunkBytes = size_t(512) << 20;
 
 }  // namespace
 
@@ -581,8 +620,9 @@ static gbc_status rotate_split(gbc_ctx* c, cplx<T>* X, const double2* Q, long lo
     const int rp = up((int)nr, kTM);
     k_split_rows<S, T><<<(rp + 7) / 8, 256, 0, s>>>(X + r0 * ldx, ldx, n, nr, rp, kp, cs, A, ea);
     GBC_CU(c, cudaGetLastError());
-    SplitArgs a{rp, nb, kp / kKC, kp / kKC, nb / G::N, ea, eb, nr, n, ldx, X + r0 * ldx};
-    GBC_CU(c, (run_split_gemm<S, MODE>(A, B, kp, a, dim3((unsigned)(rp / kTM * a.ntn)), s)));
+    const int ntn = nb / G::N, tiles = rp / kTM * ntn;
+    SplitArgs a{rp, nb, kp / kKC, kp / kKC, ntn, tiles, tiles, ea, eb, nr, n, ldx, X + r0 * ldx};
+    GBC_CU(c, (run_split_gemm<S, MODE>(A, B, kp, a, s)));
   }
   return GBC_OK;
 }
@@ -642,9 +682,9 @@ gbc_status launch_gram_split(gbc_ctx* c, const cplx<TX>* X, int ldx, const cplx<
     const int nwin = rp / win;
     const int split = std::max(1, std::min(nwin, gbc_sm_count() / std::max(1, tiles)));
     const int kper = (nwin + split - 1) / split * G::FLUSH;
-    SplitArgs a{ma, nb, rp / kKC, kper, ntn, ea, eb, nr, n, 0, Sm};
-    GBC_CU(c, (run_split_gemm<S, GRAM>(A, B, rp, a,
-                                       dim3((unsigned)tiles, (unsigned)((rp / kKC + kper - 1) / kper)), s)));
+    const int parts = (rp / kKC + kper - 1) / kper;
+    SplitArgs a{ma, nb, rp / kKC, kper, ntn, tiles, tiles * parts, ea, eb, nr, n, 0, Sm};
+    GBC_CU(c, (run_split_gemm<S, GRAM>(A, B, rp, a, s)));
   }
   return GBC_OK;
 }
