@@ -17,14 +17,26 @@
 
 namespace {
 
+// acc += conj(p) x and acc += p x, two multiply-adds per part (written out: the sum of two
+// products added to acc compiles to three operations, which the FP64 pipe feels)
 template <typename C> __device__ __forceinline__ void cmac_conj(C& acc, C p, C x) {
-  // acc += conj(p) * x
-  acc.x += p.x * x.x + p.y * x.y;
-  acc.y += p.x * x.y - p.y * x.x;
+  acc.x = fma(p.x, x.x, fma(p.y, x.y, acc.x));
+  acc.y = fma(p.x, x.y, fma(-p.y, x.x, acc.y));
 }
 template <typename C> __device__ __forceinline__ void cmac(C& acc, C p, C x) {
-  acc.x += p.x * x.x - p.y * x.y;
-  acc.y += p.x * x.y + p.y * x.x;
+  acc.x = fma(p.x, x.x, fma(-p.y, x.y, acc.x));
+  acc.y = fma(p.x, x.y, fma(p.y, x.x, acc.y));
+}
+// the same with a real p
+__device__ __forceinline__ void cmac_conj(double2& acc, double p, double2 x) {
+  acc.x += p * x.x;
+  acc.y += p * x.y;
+}
+__device__ __forceinline__ void cmac(double2& acc, double p, double2 x) { cmac_conj(acc, p, x); }
+// the part of a table entry that a kernel multiplies with
+template <typename PT, typename C> __device__ __forceinline__ PT p_entry(C p) {
+  if constexpr (std::is_same<PT, double>::value) return p.x;
+  else return p;
 }
 __device__ __forceinline__ void catomic(float2* p, float2 v) { atomicAdd(p, v); }
 __device__ __forceinline__ void catomic(double2* p, double2 v) {
@@ -44,9 +56,10 @@ constexpr int kCols = 128;      // threads per block
 // column tiles do not fill the SMs.  P rows are staged with an odd row stride, so the NG
 // rows a warp reads at once sit in distinct bank groups.  Measured on one GB300: the FP64
 // pipe is 85% busy in both; projection + expansion on 6 atoms x 18 projectors in 6^3 cells
-// at p = 6 with 64 vectors 20.0 -> 6.6 ms, on 24 atoms in 16^3 cells with one vector
-// 10.5 -> 0.6 ms (before: one chunk per block with all lanes as columns, and an expansion
-// that walked each shared node's incidence list).
+// at p = 6 with 64 vectors, k != 0: 20.0 -> 6.6 ms, with the multiply-adds written as FMAs
+// 4.0 ms; on 24 atoms in 16^3 cells with one vector, k = 0: 10.5 -> 0.59 ms, with real tables
+// 0.29 ms (before: one chunk per block with all lanes as columns, and an expansion that walked
+// each shared node's incidence list).
 struct NlTile {
   int atom, npj, j0, cnt, noff;
   __device__ __forceinline__ NlTile(const int4* chunks, const int* atom_npj, int nsub) {
@@ -65,7 +78,8 @@ struct NlTile {
 // sums its nodes in registers, then the NG groups of a column are added by shuffles and
 // through shared memory in a fixed order, and one thread per (chi, column) adds the
 // block's sum to C (or stores it to Cpart, deterministic mode).
-template <typename T, int MAXPJ, int CT>
+// REALP: the table's imaginary parts are zero (k = 0: no Bloch phases), half the FP64 work.
+template <typename T, int MAXPJ, int CT, bool REALP>
 __global__ void __launch_bounds__(kCols)
 nl_project(const cplx<T>* __restrict__ X, int ldx, int nvec, int nsub,
            const int4* __restrict__ chunks, const long long* __restrict__ nodes,
@@ -75,7 +89,12 @@ nl_project(const cplx<T>* __restrict__ X, int ldx, int nvec, int nsub,
   using C = cplx<T>;
   constexpr int NG = kCols / CT, RS = MAXPJ | 1, NW = kCols / 32, RC = 8;
   constexpr int NPS = kStage * RS, NRED = NW * CT * RC;
-  __shared__ C sh[NPS > NRED ? NPS : NRED];   // staged P rows, then the partial sums
+  using PT = typename std::conditional<REALP, double, C>::type;
+  // staged P rows, then the partial sums
+  __shared__ __align__(16) unsigned char sh_raw[NPS * sizeof(PT) > NRED * sizeof(C) ? NPS * sizeof(PT)
+                                                                                     : NRED * sizeof(C)];
+  PT* ps = reinterpret_cast<PT*>(sh_raw);
+  C* sh = reinterpret_cast<C*>(sh_raw);
   __shared__ long long Ns[kStage];
   const NlTile t(chunks, atom_npj, nsub);
   const C* Pa = P + atom_pv_off[t.atom];
@@ -90,7 +109,7 @@ nl_project(const cplx<T>* __restrict__ X, int ldx, int nvec, int nsub,
     const int nb = min(kStage, t.cnt - jb);
     for (int i = threadIdx.x; i < nb * t.npj; i += kCols) {
       const int jj = i / t.npj, c = i % t.npj;
-      sh[jj * RS + c] = Pa[(size_t)(t.j0 + jb + jj) * t.npj + c];
+      ps[jj * RS + c] = p_entry<PT>(Pa[(size_t)(t.j0 + jb + jj) * t.npj + c]);
     }
     for (int i = threadIdx.x; i < nb; i += kCols) Ns[i] = nodes[t.noff + t.j0 + jb + i];
     __syncthreads();
@@ -109,7 +128,7 @@ nl_project(const cplx<T>* __restrict__ X, int ldx, int nvec, int nsub,
           if (jj >= nb) break;
 #pragma unroll
           for (int c = 0; c < MAXPJ; ++c)
-            if (c < t.npj) cmac_conj(acc[c], sh[jj * RS + c], x[u]);
+            if (c < t.npj) cmac_conj(acc[c], ps[jj * RS + c], x[u]);
         }
       }
     }
@@ -156,7 +175,7 @@ nl_project(const cplx<T>* __restrict__ X, int ldx, int nvec, int nsub,
 // atomics (the cell apply adds to the same rows the same way): the block's C' columns stay
 // in registers, and a node held by several atoms is updated once per atom instead of
 // walking its incidence list through dependent loads.
-template <int MAXPJ, int CT>
+template <int MAXPJ, int CT, bool REALP>
 __global__ void __launch_bounds__(kCols)
 nl_expand_add(double2* __restrict__ Y, int ldx, int nvec, int nsub,
               const int4* __restrict__ chunks, const long long* __restrict__ nodes,
@@ -164,7 +183,8 @@ nl_expand_add(double2* __restrict__ Y, int ldx, int nvec, int nsub,
               const int* __restrict__ atom_pv_off, const int* __restrict__ atom_c_off,
               const double2* __restrict__ Cp, long long M) {
   constexpr int NG = kCols / CT, RS = MAXPJ | 1;
-  __shared__ double2 sh[kStage * RS];
+  using PT = typename std::conditional<REALP, double, double2>::type;
+  __shared__ PT sh[kStage * RS];
   __shared__ long long Ns[kStage];
   const NlTile t(chunks, atom_npj, nsub);
   const double2* Pa = P + atom_pv_off[t.atom];
@@ -181,7 +201,7 @@ nl_expand_add(double2* __restrict__ Y, int ldx, int nvec, int nsub,
     const int nb = min(kStage, t.cnt - jb);
     for (int i = threadIdx.x; i < nb * t.npj; i += kCols) {
       const int jj = i / t.npj, c = i % t.npj;
-      sh[jj * RS + c] = Pa[(size_t)(t.j0 + jb + jj) * t.npj + c];
+      sh[jj * RS + c] = p_entry<PT>(Pa[(size_t)(t.j0 + jb + jj) * t.npj + c]);
     }
     for (int i = threadIdx.x; i < nb; i += kCols) Ns[i] = nodes[t.noff + t.j0 + jb + i];
     __syncthreads();
@@ -231,6 +251,7 @@ __global__ void nl_couple(const cplx<T>* __restrict__ Cbuf, cplx<T>* __restrict_
   const C* D = delta + atom_delta_off[atom] + (size_t)r * n2;
   const size_t base = (size_t)atom_c_off[atom] * nvec + v;
   C acc = cmake<C>(0, 0);
+#pragma unroll 12   // the loads of 12 terms in flight (36 at 18 projectors: latency is all it takes)
   for (int c = 0; c < n2; ++c) cmac(acc, D[c], Cbuf[base + (size_t)c * nvec]);
   Cp[base + (size_t)r * nvec] = acc;
 }
@@ -313,6 +334,8 @@ inline int nl_parts(const ProjDev& pj, int nvec) {
   const long long want = (8LL * gbc_sm_count() + blocks - 1) / blocks;
   return (int)std::max<long long>(1, std::min<long long>(16, want));
 }
+// the FP64 tables are real (e^{-ik.r} = 1)
+inline bool real_tables(const gbc_ctx* c) { return c->k[0] == 0.0 && c->k[1] == 0.0 && c->k[2] == 0.0; }
 // f(std::integral_constant<int, CT>) for the column tile of nvec vectors
 template <typename F> inline void nl_with_tile(int nvec, F f) {
   switch (nl_col_tile(nvec)) {
@@ -341,9 +364,14 @@ cudaError_t run_project(gbc_ctx* c, const cplx<T>* X, int nvec, int ldx, cplx<T>
   nl_with_tile(nvec, [&](auto ct) {
     constexpr int CT = decltype(ct)::value;
     dim3 grid(pj.nchunks, (2 * nvec + CT - 1) / CT, nsub);
-    nl_project<T, MAXPJ, CT><<<grid, kCols, 0, s>>>(X, ldx, nvec, nsub, pj.d_chunks, pj.d_nodes, P,
-                                                    pj.d_atom_npj, pj.d_atom_pv_off,
-                                                    pj.d_atom_c_off, Cbuf, c->mesh.M, Cpart);
+    auto run = [&](auto kern) {
+      kern<<<grid, kCols, 0, s>>>(X, ldx, nvec, nsub, pj.d_chunks, pj.d_nodes, P, pj.d_atom_npj,
+                                  pj.d_atom_pv_off, pj.d_atom_c_off, Cbuf, c->mesh.M, Cpart);
+    };
+    if constexpr (std::is_same<T, double>::value) {
+      if (real_tables(c)) return run(nl_project<T, MAXPJ, CT, true>);
+    }
+    run(nl_project<T, MAXPJ, CT, false>);
   });
   cudaError_t e = cudaGetLastError();
   if (!Cpart || e != cudaSuccess) return e;
@@ -361,9 +389,12 @@ cudaError_t run_expand_add(const gbc_ctx* c, double2* Y, int nvec, int ldx, cons
   nl_with_tile(nvec, [&](auto ct) {
     constexpr int CT = decltype(ct)::value;
     dim3 grid(pj.nchunks, (2 * nvec + CT - 1) / CT, nsub);
-    nl_expand_add<MAXPJ, CT><<<grid, kCols, 0, s>>>(Y, ldx, nvec, nsub, pj.d_chunks, pj.d_nodes,
-                                                    pj.d_P64, pj.d_atom_npj, pj.d_atom_pv_off,
-                                                    pj.d_atom_c_off, Cp, c->mesh.M);
+    auto run = [&](auto kern) {
+      kern<<<grid, kCols, 0, s>>>(Y, ldx, nvec, nsub, pj.d_chunks, pj.d_nodes, pj.d_P64, pj.d_atom_npj,
+                                  pj.d_atom_pv_off, pj.d_atom_c_off, Cp, c->mesh.M);
+    };
+    if (real_tables(c)) run(nl_expand_add<MAXPJ, CT, true>);
+    else run(nl_expand_add<MAXPJ, CT, false>);
   });
   return cudaGetLastError();
 }
