@@ -751,55 +751,52 @@ gbc_status gbc_lanczos_bounds(gbc_ctx* c, const void* v0, int steps, double* lmi
   GBC_TRY(gbc_ensure_work(c, 0, vb));
   GBC_TRY(gbc_ensure_work(c, 1, vb * (steps + 1)));
   const int kmax = steps;
-  GBC_TRY(gbc_ensure_work(c, 3, sizeof(double2) * (2 * (size_t)kmax * kmax + 8 * kmax + 64) +
+  GBC_TRY(gbc_ensure_work(c, 3, sizeof(double2) * (2 * (size_t)kmax * kmax + 4 * kmax + 64) +
                                     sizeof(double) * kmax));
   double2* w = (double2*)c->work[0];
   double2* V = (double2*)c->work[1];
   double2* T = (double2*)c->work[3];                 // kmax x kmax tridiagonal (complex storage)
   double2* Qt = T + (size_t)kmax * kmax;
-  double2* coef = Qt + (size_t)kmax * kmax;         // scratch inner products
-  double* ev = (double*)(coef + 8 * kmax + 64);
+  double2* coef = Qt + (size_t)kmax * kmax;          // inner products of a pass
+  double2* d_alpha = coef + kmax + 1;                // alpha_j, beta_j^2
+  double2* d_beta2 = d_alpha + kmax;
+  double* ev = (double*)(coef + 4 * kmax + 64);
   const long long n2 = 2 * M;
   // v_1 = v0 / ||v0||_M
   double2 h;
   double2* part = nullptr;   // deterministic mode: block sums added in order
   if (c->deterministic) {
-    GBC_TRY(gbc_ensure_work(c, 12, mdot_part_bytes(M)));
+    GBC_TRY(gbc_ensure_work(c, 12, mdots_part_bytes(M)));
     part = (double2*)c->work[12];
   }
-  GBC_CU(c, launch_mdot((const double2*)v0, (const double2*)v0, c->d_md, M, coef, s, part));
+  GBC_CU(c, launch_mdots((const double2*)v0, n2, 1, (const double2*)v0, c->d_md, M, coef, s, part));
   GBC_CU(c, cudaMemcpyAsync(&h, coef, sizeof(double2), cudaMemcpyDeviceToHost, s));
   GBC_CU(c, cudaStreamSynchronize(s));
   if (!(h.x > 0)) return gbc_fail(c, GBC_EINVAL, "zero start vector");
-  GBC_CU(c, launch_scale_c(V, (const double2*)v0, 1.0 / std::sqrt(h.x), n2, s));
-  std::vector<double> alpha(kmax), beta(kmax);
+  GBC_CU(c, launch_normalise(V, (const double2*)v0, coef, n2, s));
   for (int j = 0; j < kmax; ++j) {
     double2* vj = V + (size_t)j * n2;
     // w = M_D^-1 H v_j
     GBC_TRY(apply_h_t<double>(c, vj, w, 1, 1, s));
     GBC_CU(c, launch_divmass(w, c->d_invmd, M, s));
-    // alpha_j = <v_j, w>_M ; w -= alpha v_j + beta_{j-1} v_{j-1}; two passes of full
-    // reorthogonalisation against v_0..v_j
-    GBC_CU(c, launch_mdot(vj, w, c->d_md, M, coef, s, part));
-    GBC_CU(c, cudaMemcpyAsync(&h, coef, sizeof(double2), cudaMemcpyDeviceToHost, s));
-    GBC_CU(c, cudaStreamSynchronize(s));
-    alpha[j] = h.x;
-    GBC_CU(c, launch_axpy_c(w, vj, coef, 1.0, n2, s));
+    // two passes of full (classical Gram-Schmidt) orthogonalisation against v_0..v_j; alpha_j
+    // = <v_j, w>_M is the last inner product of the first
     for (int pass = 0; pass < 2; ++pass) {
-      for (int i = 0; i <= j; ++i) {
-        double2* vi = V + (size_t)i * n2;
-        GBC_CU(c, launch_mdot(vi, w, c->d_md, M, coef + 1 + i, s, part));
-        GBC_CU(c, launch_axpy_c(w, vi, coef + 1 + i, 1.0, n2, s));
-      }
+      GBC_CU(c, launch_mdots(V, n2, j + 1, w, c->d_md, M, coef, s, part));
+      if (pass == 0)
+        GBC_CU(c, cudaMemcpyAsync(d_alpha + j, coef + j, sizeof(double2), cudaMemcpyDeviceToDevice, s));
+      GBC_CU(c, launch_maxpys(w, V, n2, j + 1, coef, n2, s));
     }
-    GBC_CU(c, launch_mdot(w, w, c->d_md, M, coef, s, part));
-    GBC_CU(c, cudaMemcpyAsync(&h, coef, sizeof(double2), cudaMemcpyDeviceToHost, s));
-    GBC_CU(c, cudaStreamSynchronize(s));
-    beta[j] = std::sqrt(std::max(h.x, 0.0));
-    if (j + 1 <= kmax) {
-      const double inv = beta[j] > 0 ? 1.0 / beta[j] : 0.0;
-      GBC_CU(c, launch_scale_c(V + (size_t)(j + 1) * n2, w, inv, n2, s));
-    }
+    GBC_CU(c, launch_mdots(w, n2, 1, w, c->d_md, M, d_beta2 + j, s, part));
+    GBC_CU(c, launch_normalise(V + (size_t)(j + 1) * n2, w, d_beta2 + j, n2, s));
+  }
+  std::vector<double2> ab(2 * (size_t)kmax);
+  GBC_CU(c, cudaMemcpyAsync(ab.data(), d_alpha, sizeof(double2) * ab.size(), cudaMemcpyDeviceToHost, s));
+  GBC_CU(c, cudaStreamSynchronize(s));
+  std::vector<double> alpha(kmax), beta(kmax);
+  for (int j = 0; j < kmax; ++j) {
+    alpha[j] = ab[j].x;
+    beta[j] = std::sqrt(std::max(ab[kmax + j].x, 0.0));
   }
   // eigenvalues of the tridiagonal T_k on the device
   std::vector<double2> Th((size_t)kmax * kmax, make_double2(0, 0));

@@ -467,12 +467,15 @@ cudaError_t launch_rotate_ff(const float2* X, const double2* Q, float2* Qsplit, 
                              long long M, int nvec, int ldx, cudaStream_t s);
 // Hermitian matrix from its upper triangle (the lower one mirrored, real diagonal)
 cudaError_t launch_hermitize(double2* A, int n, cudaStream_t s);
-// lanczos helpers
-// deterministic mode (part: scratch of mdot_part_bytes(n)): block sums added in order
-cudaError_t launch_mdot(const double2* a, const double2* b, const double* md, long long n,
-                        double2* out, cudaStream_t s, double2* part = nullptr);
-size_t mdot_part_bytes(long long n);
-cudaError_t launch_axpy_c(double2* y, const double2* x, const double2* alpha_dev, double alpha_scale,
-                          long long n, cudaStream_t s);
-cudaError_t launch_scale_c(double2* y, const double2* x, double scale, long long n, cudaStream_t s);
+// lanczos helpers: out[i] = <v_i, w> in the M_D inner product, v_i = V + i * stride, i < nv
+// (part: scratch of mdots_part_bytes(n), deterministic mode: block sums added in order);
+// w -= sum_i c[i] v_i; y = x / sqrt(nrm2->x) (0 where that is not positive)
+cudaError_t launch_mdots(const double2* V, long long stride, int nv, const double2* w,
+                         const double* md, long long n, double2* out, cudaStream_t s,
+                         double2* part = nullptr);
+size_t mdots_part_bytes(long long n);
+cudaError_t launch_maxpys(double2* w, const double2* V, long long stride, int nv, const double2* c,
+                          long long n2, cudaStream_t s);
+cudaError_t launch_normalise(double2* y, const double2* x, const double2* nrm2, long long n,
+                             cudaStream_t s);
 cudaError_t launch_divmass(double2* y, const double* invmd, long long M, cudaStream_t s);
