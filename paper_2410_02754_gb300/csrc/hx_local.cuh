@@ -301,8 +301,9 @@ hx_local_kernel(const __grid_constant__ LocalArgs a, const __grid_constant__ Tab
 
   auto rec = [&](int n) -> HxItem& { return rec0[n % kHxSlots]; };
   auto noff = [&](int n, int slot) { return noff0 + (n % kHxSlots) * 48 + slot * 24; };
-  // the group's last warp: record and node offsets of the group's n-th item
-  // (noff[0][ix] + noff[8 + iy] + noff[16 + iz], negative on a Dirichlet face)
+  // the group's last warp: record and node coordinates of the group's n-th item: node
+  // (ix, iy, iz) is (no[8 + iy] + no[16 + iz]) * nfree[0] + no[ix], negative terms on a
+  // Dirichlet face (a mesh may have more nodes than an int counts)
   auto post = [&](int n) {
     const long long it = first + n * ngroups;
     HxItem r{0, {-1, -1}, {0, 0}, {0, 0, 0}};
@@ -329,7 +330,7 @@ hx_local_kernel(const __grid_constant__ LocalArgs a, const __grid_constant__ Tab
         int f;
         if (m.periodic[dd]) f = gc >= m.period[dd] ? gc - m.period[dd] : gc;
         else f = (gc == 0 || gc == m.period[dd]) ? -1 : gc - 1;
-        const int scale = dd == 0 ? 1 : dd == 1 ? m.nfree[0] : m.nfree[0] * m.nfree[1];
+        const int scale = dd < 2 ? 1 : m.nfree[1];
         noff(n, sl)[dd * 8 + i] = f < 0 ? kNoNode : f * scale;
       }
     }
@@ -347,11 +348,11 @@ hx_local_kernel(const __grid_constant__ LocalArgs a, const __grid_constant__ Tab
       const int Iyz = have ? no[8 + y] + no[16 + z] : kNoNode;
       double2* dst = &Ab(w)[pa(0, y, z)];
       const double2* src = g.X + (long long)(w & 1) * g.ldx + (sl ? it.v[1] : it.v[0]);
+      const long long I0 = (long long)Iyz * g.mesh.nfree[0];
 #pragma unroll
       for (int x = 0; x < NP; ++x) {
-        const int I = have ? Iyz + no[x] : -1;
-        const bool ok = I >= 0 && GBC_IN_RANGE(GBC_SITE_HX64, I, g.mesh.M);
-        cp_async16z(dst + x, ok ? src + 2 * (long long)I * g.ldx : g.X, ok ? 16 : 0);
+        const bool ok = Iyz >= 0 && no[x] >= 0 && GBC_IN_RANGE(GBC_SITE_HX64, I0 + no[x], g.mesh.M);
+        cp_async16z(dst + x, ok ? src + 2 * (I0 + no[x]) * g.ldx : g.X, ok ? 16 : 0);
       }
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
@@ -522,12 +523,12 @@ hx_local_kernel(const __grid_constant__ LocalArgs a, const __grid_constant__ Tab
         put_rows<NP>(i, r, [&](int x, double2 v) {
           const double2 k = K[x];
           const double2 o = make_double2(v.x + k.x, v.y + k.y);
-          const int I = Iyz + no[x];
-          if (I < 0 || !GBC_IN_RANGE(GBC_SITE_HX64, I, d.mesh.M)) return;
+          const long long I = (long long)Iyz * d.mesh.nfree[0] + no[x];
+          if (Iyz < 0 || no[x] < 0 || !GBC_IN_RANGE(GBC_SITE_HX64, I, d.mesh.M)) return;
           if (d.Ycell)
             d.Ycell[(((long long)e * (NP * NP * NP) + x + NP * (y + NP * z)) * 2 + sp) * d.nvec + vec] = o;
           else
-            atomic_add_c(&d.Y[((long long)I * 2 + sp) * d.ldx + vec], o);
+            atomic_add_c(&d.Y[(I * 2 + sp) * d.ldx + vec], o);
         });
       }
     }
@@ -631,21 +632,6 @@ __global__ void k_cell_gather(cplx<T>* __restrict__ Y, const cplx<T>* __restrict
     cplx<T>& o = Y[(I * 2 + s) * ldx + v];
     o.x += acc.x;
     o.y += acc.y;
-  }
-}
-
-// dispatch on p (nq = p + 2)
-inline cudaError_t launch_hx_group(const HxJob* jobs, int n, cudaStream_t s) {
-  for (int i = 0; i < n; ++i)   // node offsets are 32-bit
-    if (jobs[i].c->mesh.M >= (1LL << 29)) return cudaErrorInvalidValue;
-  switch (jobs[0].c->mesh.p) {
-    case 2: return launch_hx_group_p<3>(jobs, n, s);
-    case 3: return launch_hx_group_p<4>(jobs, n, s);
-    case 4: return launch_hx_group_p<5>(jobs, n, s);
-    case 5: return launch_hx_group_p<6>(jobs, n, s);
-    case 6: return launch_hx_group_p<7>(jobs, n, s);
-    case 7: return launch_hx_group_p<8>(jobs, n, s);
-    default: return cudaErrorInvalidValue;
   }
 }
 
