@@ -7,31 +7,37 @@
 //   X_f[J] = sum_I N^{p_c}_I(r_J) X_c[I],
 //
 // per cell a tensor product of the 1-D matrix T[j][i] = l^{p_c}_i(x^{p_f}_j),
-// applied in three sum-factorised stages.
+// applied in three sum-factorised stages, each 1-D product in even-odd form (the GLL nodes are
+// symmetric).  p_f = p_c is the identity: a copy.
 //
-// One CTA per (cell, tile of VT vectors), 128 threads = VT vector lanes x G
-// pencil groups, so every global access of a node row is one contiguous
-// VT-vector segment (64 bytes: two full 32-byte sectors; the tile is kept this
-// small so that six CTAs fit an SM's shared memory and their gathers overlap).
-// Per spin: stage the coarse cell in shared memory with asynchronous copies
-// (every load of the cell in flight at once, zero-fill for absent nodes),
-// x stage -> B, y stage -> A, z stage -> global.  A cell writes only
-// the fine nodes it owns (local index < p_f in every direction); with the
-// periodic wrap and the Dirichlet faces this writes every free fine node
-// exactly once, with no atomics.  HBM-bound: the coarse block is read and the
-// fine block written once (shared coarse nodes are re-read from L2).
-#include "gbc_internal.h"
+// One CTA per (cell, tile of kLanes 16-byte elements a node row: 8 FP32 or 4 FP64 vectors), the
+// tiles of a cell next to each other so that they share its node rows' sectors in L2.  A thread
+// owns a pencil of one element (two FP32 vectors or one FP64 vector), so shared-memory accesses
+// are 16 bytes and FP32 products paired multiply-adds on (re, im).  Per spin: stage the coarse
+// cell in shared memory with asynchronous copies (every load of the cell in flight at once,
+// zero-fill for absent nodes), x stage -> B, y stage -> A, z stage -> global.  Neighbouring
+// pencils are an odd number of points apart in every stage, so a quarter-warp's accesses (4
+// elements x 2 pencils) cover all banks.  A cell writes only the fine nodes it owns (local
+// index < p_f in every direction); with the periodic wrap and the Dirichlet faces this writes
+// every free fine node exactly once, with no atomics.  HBM-bound in the limit (the coarse block
+// read and the fine block written once).  Measured on one GB300, 16^3 cells, p = 5 -> 6, 256 FP32
+// vectors: 2.91 ms with dense scalar products on 8-byte elements (issue-bound), 1.53 ms now.
+#include "hx_cell.cuh"
 
 namespace {
 
-template <typename T, int NC, int NF> struct TwoGridTab {
-  T t[NF][NC];   // l^{p_c}_i(x^{p_f}_j)
-};
+using namespace gbc;
 
-// asynchronous global -> shared copy of one complex value (8 or 16 bytes);
-// src_bytes = 0 writes zeros
-template <int N>
-__device__ __forceinline__ void cp_async_n(void* dst, const void* src, int src_bytes) {
+constexpr int kLanes = 4;       // 16-byte elements of a node row per CTA
+constexpr int kThreads = 192;
+
+template <typename T> __host__ __device__ constexpr int vecs_per_elem() { return sizeof(T) == 4 ? 2 : 1; }
+template <typename T, int NC, int NF> struct TwoGridTab;
+template <int NC, int NF> struct TwoGridTab<float, NC, NF> { EO2<NF, NC> t; };
+template <int NC, int NF> struct TwoGridTab<double, NC, NF> { EO<double, NF, NC> t; };
+
+// asynchronous global -> shared copy of N bytes, of which src_bytes are read and the rest zero
+template <int N> __device__ __forceinline__ void cp_async_n(void* dst, const void* src, int src_bytes) {
   static_assert(N == 8 || N == 16, "8- or 16-byte copies");
   if (N == 16)
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(
@@ -45,104 +51,144 @@ __device__ __forceinline__ void cp_async_n(void* dst, const void* src, int src_b
                  : "memory");
 }
 
-template <typename T, int NC, int NF, int VT>
-__global__ void __launch_bounds__(128)
-k_prolongate(const MeshDev mc, const MeshDev mf, const cplx<T>* __restrict__ Xc, int ldxc,
-             cplx<T>* __restrict__ Xf, int ldxf, int nvec, const TwoGridTab<T, NC, NF> tb) {
-  using C = cplx<T>;
-  constexpr int G = 128 / VT;                          // pencil groups
-  constexpr int ASZ = (NC * NC * NC > NF * NF * NC ? NC * NC * NC : NF * NF * NC);
-  constexpr int BSZ = NF * NC * NC;
+// one 1-D product: ld(j) -> the NC inputs, st(row, value) for the NF outputs
+template <int NC, int NF, typename L, typename S>
+__device__ __forceinline__ void line(const TwoGridTab<float, NC, NF>& tb, L ld, S st) {
+  Parts<NC> s;
+  load_parts<true>(s, ld);
+#pragma unroll
+  for (int i = 0; i < (NF + 1) / 2; ++i) {
+    Acc a;
+    row_sym<true, NF>(tb.t, i, s, a);
+    put_rows<true, NF>(i, a, st);
+  }
+}
+template <int NC, int NF, typename L, typename S>
+__device__ __forceinline__ void line(const TwoGridTab<double, NC, NF>& tb, L ld, S st) {
+  PartsD<NC> s;
+  load_parts(s, ld);
+#pragma unroll
+  for (int i = 0; i < (NF + 1) / 2; ++i) {
+    AccD a;
+    row_sym<true, NF>(tb.t, i, s, a);
+    put_rows<NF>(i, a, st);
+  }
+}
+
+template <int NC> __host__ __device__ constexpr int odd_stride() { return NC | 1; }   // of A's x pencils
+template <int NC, int NF> __host__ __device__ constexpr int points_a() {
+  return NC * NC * odd_stride<NC>() > NF * NF * NC ? NC * NC * odd_stride<NC>() : NF * NF * NC;
+}
+
+// al_in / al_out: the node rows of Xc / Xf are 16-byte aligned
+template <typename T, int NC, int NF>
+__global__ void __launch_bounds__(kThreads)
+k_prolongate(const __grid_constant__ MeshDev mc, const __grid_constant__ MeshDev mf, const cplx<T>* __restrict__ Xc, int ldxc,
+             cplx<T>* __restrict__ Xf, int ldxf, int nvec, int ntiles, int al_in, int al_out,
+             const __grid_constant__ TwoGridTab<T, NC, NF> tb) {
+  using E = typename std::conditional<sizeof(T) == 4, float4, double2>::type;
+  constexpr int VE = vecs_per_elem<T>();
+  constexpr int RS = odd_stride<NC>();
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  C* A = reinterpret_cast<C*>(smem_raw);               // [ASZ][VT]
-  C* B = A + ASZ * VT;                                 // [BSZ][VT]
-  const int v = threadIdx.x % VT, grp = threadIdx.x / VT;
-  const int e = blockIdx.x;
-  const int vec = blockIdx.y * VT + v;
-  const bool vok = vec < nvec;
-  const int cx = e % mc.ncell[0], cy = (e / mc.ncell[0]) % mc.ncell[1];
-  const int cz = e / (mc.ncell[0] * mc.ncell[1]);
+  E* A = reinterpret_cast<E*>(smem_raw);               // [points_a][kLanes]
+  E* B = A + points_a<NC, NF>() * kLanes;              // [NF NC NC][kLanes]
+  __shared__ long long off[3][8];                      // coarse node offsets, < 0: no free node
+  const int e = blockIdx.x / ntiles;
+  const int vec0 = (blockIdx.x % ntiles) * kLanes * VE;
+  const int cx = e % mc.ncell[0], cy = (e / mc.ncell[0]) % mc.ncell[1], cz = e / (mc.ncell[0] * mc.ncell[1]);
+  if (threadIdx.x < 3 * NC) {
+    const int d = threadIdx.x / NC, i = threadIdx.x % NC;
+    const int g = (d == 0 ? cx : d == 1 ? cy : cz) * mc.p + i;
+    int f;
+    if (mc.periodic[d]) f = g >= mc.period[d] ? g - mc.period[d] : g;
+    else f = (g == 0 || g == mc.period[d]) ? -1 : g - 1;
+    const long long scale = d == 0 ? 1 : d == 1 ? mc.nfree[0] : (long long)mc.nfree[0] * mc.nfree[1];
+    off[d][i] = f < 0 ? -(1LL << 60) : f * scale;
+  }
+  __syncthreads();
   for (int s = 0; s < 2; ++s) {
-    // coarse cell nodes (ix fastest) -> A
-    for (int i = grp; i < NC * NC * NC; i += G) {
-      const int ix = i % NC, iy = (i / NC) % NC, iz = i / (NC * NC);
-      const long long I = gbc_node(mc, cx, cy, cz, ix, iy, iz);
-      const bool ok = I >= 0 && vok;
-      cp_async_n<sizeof(C)>(&A[i * VT + v], ok ? &Xc[(I * 2 + s) * ldxc + vec] : Xc,
-                            ok ? (int)sizeof(C) : 0);
+    // coarse cell nodes (x pencils) -> A
+    for (int u = threadIdx.x; u < NC * NC * kLanes; u += kThreads) {
+      const int l = u % kLanes, pid = u / kLanes;
+      const long long Iyz = off[1][pid % NC] + off[2][pid / NC];
+      const int v = vec0 + l * VE;
+      const int have = max(0, min(VE, nvec - v));      // vectors of the element
+#pragma unroll
+      for (int x = 0; x < NC; ++x) {
+        const long long I = Iyz + off[0][x];
+        const bool ok = I >= 0 && have > 0;
+        const cplx<T>* src = ok ? Xc + (I * 2 + s) * ldxc + v : Xc;
+        E* dst = &A[(pid * RS + x) * kLanes + l];
+        if (sizeof(T) == 8 || al_in) {
+          cp_async_n<16>(dst, src, ok ? have * (int)sizeof(cplx<T>) : 0);
+        } else {
+          cp_async_n<8>(dst, src, ok ? 8 : 0);
+          cp_async_n<8>(reinterpret_cast<char*>(dst) + 8, ok && have > 1 ? src + 1 : Xc, ok && have > 1 ? 8 : 0);
+        }
+      }
     }
     asm volatile("cp.async.commit_group;\ncp.async.wait_all;" ::: "memory");
     __syncthreads();
     // x: A [z][y][x] (NC^3) -> B [z][y][xq] (NC^2 NF)
-    for (int pid = grp; pid < NC * NC; pid += G) {
-      C in[NC];
-#pragma unroll
-      for (int j = 0; j < NC; ++j) in[j] = A[(pid * NC + j) * VT + v];
-#pragma unroll
-      for (int q = 0; q < NF; ++q) {
-        T r = 0, im = 0;
-#pragma unroll
-        for (int j = 0; j < NC; ++j) {
-          r += tb.t[q][j] * in[j].x;
-          im += tb.t[q][j] * in[j].y;
-        }
-        B[(pid * NF + q) * VT + v] = cmake<C>(r, im);
-      }
+    for (int u = threadIdx.x; u < NC * NC * kLanes; u += kThreads) {
+      const int l = u % kLanes, pid = u / kLanes;
+      line(tb, [&](int j) { return A[(pid * RS + j) * kLanes + l]; },
+           [&](int q, E r) { B[(pid * NF + q) * kLanes + l] = r; });
     }
     __syncthreads();
     // y: B [z][y][xq] -> A [z][yq][xq] (NC NF^2)
-    for (int pid = grp; pid < NF * NC; pid += G) {
-      const int xq = pid % NF, z = pid / NF;
-      C in[NC];
-#pragma unroll
-      for (int j = 0; j < NC; ++j) in[j] = B[((z * NC + j) * NF + xq) * VT + v];
-#pragma unroll
-      for (int q = 0; q < NF; ++q) {
-        T r = 0, im = 0;
-#pragma unroll
-        for (int j = 0; j < NC; ++j) {
-          r += tb.t[q][j] * in[j].x;
-          im += tb.t[q][j] * in[j].y;
-        }
-        A[((z * NF + q) * NF + xq) * VT + v] = cmake<C>(r, im);
-      }
+    for (int u = threadIdx.x; u < NF * NC * kLanes; u += kThreads) {
+      const int l = u % kLanes, xq = (u / kLanes) % NF, z = u / (kLanes * NF);
+      line(tb, [&](int j) { return B[((z * NC + j) * NF + xq) * kLanes + l]; },
+           [&](int q, E r) { A[((z * NF + q) * NF + xq) * kLanes + l] = r; });
     }
     __syncthreads();
-    // z: A [z][yq][xq] -> owned fine nodes (xq, yq, zq < p_f)
-    for (int pid = grp; pid < (NF - 1) * (NF - 1); pid += G) {
-      const int xq = pid % (NF - 1), yq = pid / (NF - 1);
-      C in[NC];
-#pragma unroll
-      for (int j = 0; j < NC; ++j) in[j] = A[((j * NF + yq) * NF + xq) * VT + v];
-#pragma unroll
-      for (int q = 0; q < NF - 1; ++q) {
-        T r = 0, im = 0;
-#pragma unroll
-        for (int j = 0; j < NC; ++j) {
-          r += tb.t[q][j] * in[j].x;
-          im += tb.t[q][j] * in[j].y;
-        }
-        const long long J = gbc_node(mf, cx, cy, cz, xq, yq, q);
-        if (J >= 0 && vok) Xf[(J * 2 + s) * ldxf + vec] = cmake<C>(r, im);
-      }
+    // z: A [z][yq][xq] -> owned fine nodes (xq, yq, zq < p_f); no wrap there, so the nodes of a
+    // z pencil are a constant distance apart
+    for (int u = threadIdx.x; u < (NF - 1) * (NF - 1) * kLanes; u += kThreads) {
+      const int l = u % kLanes, xq = (u / kLanes) % (NF - 1), yq = u / (kLanes * (NF - 1));
+      const int fx = cx * mf.p + xq - (mf.periodic[0] ? 0 : 1);
+      const int fy = cy * mf.p + yq - (mf.periodic[1] ? 0 : 1);
+      const int fz = cz * mf.p - (mf.periodic[2] ? 0 : 1);
+      const int v = vec0 + l * VE;
+      const bool in = fx >= 0 && fy >= 0 && v < nvec;
+      const long long row = ((long long)fz * mf.nfree[1] + fy) * mf.nfree[0] + fx;
+      cplx<T>* dst = Xf + (row * 2 + s) * ldxf + v;
+      const long long step = (long long)mf.nfree[0] * mf.nfree[1] * 2 * ldxf;
+      line(tb, [&](int j) { return A[((j * NF + yq) * NF + xq) * kLanes + l]; },
+           [&](int q, E r) {
+             if (q == NF - 1 || !in || fz + q < 0) return;
+             cplx<T>* o = dst + q * step;
+             if constexpr (sizeof(T) == 8) {
+               *o = r;
+             } else if (al_out && v + 1 < nvec) {
+               *reinterpret_cast<float4*>(o) = r;
+             } else {
+               o[0] = make_float2(r.x, r.y);
+               if (v + 1 < nvec) o[1] = make_float2(r.z, r.w);
+             }
+           });
     }
     __syncthreads();   // A is restaged by the next spin
   }
 }
 
-template <typename T, int NC, int NF> constexpr int vt_of() { return sizeof(T) == 4 ? 8 : 4; }
-
-template <typename T, int NC, int NF> constexpr size_t prolongate_smem() {
-  constexpr int VT = vt_of<T, NC, NF>();
-  constexpr int ASZ = (NC * NC * NC > NF * NF * NC ? NC * NC * NC : NF * NF * NC);
-  return sizeof(cplx<T>) * (size_t)VT * (ASZ + NF * NC * NC);
+// p -> p: columns 0 .. nvec-1 of every row
+template <typename T>
+__global__ void k_copy_cols(const cplx<T>* __restrict__ X, int ldx, cplx<T>* __restrict__ Out, int ldo,
+                            long long rows, int nvec) {
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < rows * nvec;
+       i += (long long)gridDim.x * blockDim.x) {
+    const long long r = i / nvec;
+    const int v = (int)(i - r * nvec);
+    Out[r * ldo + v] = X[r * ldx + v];
+  }
 }
 
 template <typename T, int NC, int NF>
 cudaError_t launch_prolongate_t(const gbc_ctx* cc, const gbc_ctx* cf, const cplx<T>* Xc, int ldxc,
                                 cplx<T>* Xf, int ldxf, int nvec, cudaStream_t s) {
-  constexpr int VT = vt_of<T, NC, NF>();
-  TwoGridTab<T, NC, NF> tb;   // coarse Lagrange basis at the fine GLL nodes
+  std::vector<double> m((size_t)NF * NC);   // coarse Lagrange basis at the fine GLL nodes
   const std::vector<double>& xc = cc->tab.gll_x;
   const std::vector<double>& xf = cf->tab.gll_x;
   for (int j = 0; j < NF; ++j)
@@ -150,14 +196,23 @@ cudaError_t launch_prolongate_t(const gbc_ctx* cc, const gbc_ctx* cf, const cplx
       double l = 1.0;
       for (int k = 0; k < NC; ++k)
         if (k != i) l *= (xf[j] - xc[k]) / (xc[i] - xc[k]);
-      tb.t[j][i] = (T)l;
+      m[j * NC + i] = l;
     }
-  constexpr size_t smem = prolongate_smem<T, NC, NF>();
-  auto k = k_prolongate<T, NC, NF, VT>;
+  EO<T, NF, NC> eo;
+  if (!make_eo<T, NF, NC>(m, 1, &eo)) return cudaErrorInvalidValue;
+  TwoGridTab<T, NC, NF> tb;
+  if constexpr (sizeof(T) == 4) cvt_table(eo, tb.t);
+  else tb.t = eo;
+  constexpr size_t smem = 16 * (size_t)kLanes * (points_a<NC, NF>() + NF * NC * NC);
+  auto k = k_prolongate<T, NC, NF>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  dim3 grid(cf->mesh.E, (nvec + VT - 1) / VT);
-  k<<<grid, 128, smem, s>>>(cc->mesh, cf->mesh, Xc, ldxc, Xf, ldxf, nvec, tb);
+  constexpr int VT = kLanes * vecs_per_elem<T>();
+  const long long ntiles = (nvec + VT - 1) / VT, blocks = (long long)cf->mesh.E * ntiles;
+  if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
+  auto aligned = [](const void* p, int ld) { return ((uintptr_t)p & 15) == 0 && (ld & 1) == 0; };
+  k<<<(unsigned)blocks, kThreads, smem, s>>>(cc->mesh, cf->mesh, Xc, ldxc, Xf, ldxf, nvec, (int)ntiles,
+                                             aligned(Xc, ldxc), aligned(Xf, ldxf), tb);
   return cudaGetLastError();
 }
 
@@ -167,10 +222,16 @@ cudaError_t launch_prolongate(const gbc_ctx* cc, const gbc_ctx* cf, const void* 
   const int pc = cc->mesh.p, pf = cf->mesh.p;
   const cplx<T>* xc = (const cplx<T>*)Xc;
   cplx<T>* xf = (cplx<T>*)Xf;
-#define GBC_TG(PC, PF) \
-  if (pc == PC && pf == PF) return launch_prolongate_t<T, PC + 1, PF + 1>(cc, cf, xc, ldxc, xf, ldxf, nvec, s);
-  GBC_TG(2, 2) GBC_TG(2, 3) GBC_TG(3, 3) GBC_TG(3, 4) GBC_TG(4, 4) GBC_TG(4, 5)
-  GBC_TG(5, 5) GBC_TG(5, 6) GBC_TG(6, 6) GBC_TG(6, 7) GBC_TG(7, 7)
+  if (pc == pf) {
+    const long long n = 2 * cf->mesh.M * nvec;
+    const unsigned grid = (unsigned)std::min<long long>((n + 255) / 256, 64LL * gbc_sm_count());
+    k_copy_cols<T><<<grid, 256, 0, s>>>(xc, ldxc, xf, ldxf, 2 * cf->mesh.M, nvec);
+    return cudaGetLastError();
+  }
+#define GBC_TG(PC) \
+  if (pc == PC && pf == PC + 1) \
+    return launch_prolongate_t<T, PC + 1, PC + 2>(cc, cf, xc, ldxc, xf, ldxf, nvec, s);
+  GBC_TG(2) GBC_TG(3) GBC_TG(4) GBC_TG(5) GBC_TG(6)
 #undef GBC_TG
   return cudaErrorInvalidValue;
 }
