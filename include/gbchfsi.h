@@ -208,7 +208,8 @@ gbc_status gbc_rayleigh_ritz(gbc_ctx* ctx, void* X, int nvec, int ldx, double* r
  * gB = 3 consecutive arrays x, y, z, written; layout as gbc_set_fields),
  * gDelta (host, the concatenated Delta matrices, complex128, Hermitian part,
  * written; may be NULL).  p <= 6.  Synchronous.  Uses library workspace of
- * (2 ceil(degree/ckpt_every) + max(ckpt_every, 3) + 4) blocks. */
+ * (2 ceil(degree/ckpt_every) + max(ckpt_every, 3) + 4) blocks and the projector
+ * coefficients (2 npj per atom and vector) of every degree. */
 gbc_status gbc_filter_vjp(gbc_ctx* ctx, const void* X0, const void* GY, void* GX, double* gV,
                           double* gB, double* gDelta, int nvec, int ldx, int degree, double lT,
                           double lmax, double lmin, int ckpt_every, void* stream);

@@ -113,10 +113,11 @@ gbc_status check_block(gbc_ctx* c, const void* X, int nvec, int ldx) {
   return GBC_OK;
 }
 
-// Y = H X in the context precision (Y zeroed first)
+// Y = H X in the context precision (Y zeroed first).  C: P^H X is left there (null: in work
+// slot 2)
 template <typename T>
 gbc_status apply_h_t(gbc_ctx* c, const cplx<T>* X, cplx<T>* Y, int nvec, int ldx, cudaStream_t s,
-                     bool zero = true) {
+                     bool zero = true, cplx<T>* C = nullptr) {
   if (zero) GBC_CU(c, cudaMemsetAsync(Y, 0, sizeof(cplx<T>) * 2 * (size_t)c->mesh.M * ldx, s));
   if (nvec == 0) return GBC_OK;
   cudaError_t e;
@@ -146,19 +147,54 @@ gbc_status apply_h_t(gbc_ctx* c, const cplx<T>* X, cplx<T>* Y, int nvec, int ldx
     cplx<T>* C2 = C1 + (size_t)c->proj.rows_total * nvec;
     {
       TimerScope ts(c, FAM_NONLOCAL, s);
-      e = launch_nonlocal<T>(c, X, Y, nvec, ldx, C1, C2, s);
+      e = launch_nonlocal<T>(c, X, Y, nvec, ldx, C ? C : C1, C2, s);
     }
     if (e != cudaSuccess) return gbc_cuda_fail(c, e, "nonlocal");
   }
   return GBC_OK;
 }
 
-// X <- p_m(H~) X in place, the sigma-scaled three-term recurrence of Eq. chebfilt.
+// One step of the recurrence of Eq. chebfilt, out = a (M_D^-1 H cur - cc cur) - b prev (out may
+// be prev; prev null: b = 0), with the accumulator Y, which is zero before the first step of a
+// sequence and left ready for the next.
 // FP64: the H.X accumulation (cell apply, nonlocal step) then one recurrence
 // pass over every row.  FP32: the recurrence is fused into the applies -- the
 // nonlocal step writes P C' into the accumulator's support rows, the cell apply
 // finishes the rows interior to a cell in its epilogue, and a row pass finishes
-// the rows on cell faces (see hx_cell.cuh).
+// the rows on cell faces (see hx_cell.cuh).  C: P^H cur is left there (null: in work slot 2).
+template <typename T>
+gbc_status recur_t(gbc_ctx* c, const cplx<T>* cur, const cplx<T>* prev, cplx<T>* out, cplx<T>* Y,
+                   int nvec, int ldx, double a, double cc, double b, cudaStream_t s,
+                   cplx<T>* C = nullptr) {
+  const T* invmd = std::is_same<T, double>::value ? (const T*)c->d_invmd : (const T*)c->d_invmd32;
+  if (std::is_same<T, double>::value || nvec == 0 || c->prec != GBC_FP32) {
+    GBC_TRY(apply_h_t<T>(c, cur, Y, nvec, ldx, s, false, C));
+    TimerScope ts(c, FAM_CHEB, s);
+    GBC_CU(c, launch_cheb_step<T>(Y, cur, prev, out, invmd, c->mesh.M, nvec, ldx, a, cc, b, s));
+    return GBC_OK;
+  }
+  if (c->proj.natoms > 0) {
+    size_t xoff = 0;
+    GBC_TRY(gbc_ensure_work(c, 2, nl_work_bytes(c, nvec, ldx, sizeof(cplx<T>), &xoff)));
+    cplx<T>* C1 = (cplx<T>*)c->work[2];
+    cplx<T>* C2 = C1 + (size_t)c->proj.rows_total * nvec;
+    void* bpre = xoff ? (char*)c->work[2] + xoff : nullptr;
+    TimerScope ts(c, FAM_NONLOCAL, s);
+    GBC_CU(c, launch_nonlocal<T>(c, cur, Y, nvec, ldx, C ? C : C1, C2, s, true, bpre));
+  }
+  {
+    TimerScope ts(c, FAM_HX_LOCAL, s);
+    CellJob j{c, cur, Y, nvec, ldx, out, prev, a, cc, b};
+    GBC_CU(c, launch_cell_f32(&j, 1, c->cell_var, s));
+  }
+  TimerScope ts(c, FAM_CHEB, s);
+  GBC_CU(c, launch_cheb_rows<T>(Y, cur, prev, out, invmd, c->d_face_rows, c->nface,
+                                c->proj.natoms > 0 ? c->nface_supp : 0, c->mesh.M, nvec, ldx,
+                                a, cc, b, s));
+  return GBC_OK;
+}
+
+// X <- p_m(H~) X in place, the sigma-scaled three-term recurrence of Eq. chebfilt.
 template <typename T>
 gbc_status filter_t(gbc_ctx* c, cplx<T>* X, int nvec, int ldx, int m, double lT, double lmax,
                     double lmin, cudaStream_t s) {
@@ -171,7 +207,6 @@ gbc_status filter_t(gbc_ctx* c, cplx<T>* X, int nvec, int ldx, int m, double lT,
   GBC_TRY(gbc_ensure_work(c, 1, bytes));
   cplx<T>* Y = (cplx<T>*)c->work[0];
   cplx<T>* W = (cplx<T>*)c->work[1];
-  const T* invmd = std::is_same<T, double>::value ? (const T*)c->d_invmd : (const T*)c->d_invmd32;
   GBC_CU(c, cudaMemsetAsync(Y, 0, bytes, s));
   // step k: X_{k+1} = a_k (M_D^-1 H X_k - c X_k) - b_k X_{k-1}; X_1 -> W, then
   // X_{k+1} written over X_{k-1}
@@ -181,30 +216,7 @@ gbc_status filter_t(gbc_ctx* c, cplx<T>* X, int nvec, int ldx, int m, double lT,
     cplx<T>* out = k == 0 ? W : prev;
     const double a = k == 0 ? sig[0] / e : 2.0 * sig[k] / e;
     const double b = k == 0 ? 0.0 : sig[k - 1] * sig[k];
-    if (std::is_same<T, double>::value || nvec == 0 || c->prec != GBC_FP32) {
-      GBC_TRY(apply_h_t<T>(c, cur, Y, nvec, ldx, s, false));
-      TimerScope ts(c, FAM_CHEB, s);
-      GBC_CU(c, launch_cheb_step<T>(Y, cur, prev, out, invmd, c->mesh.M, nvec, ldx, a, cc, b, s));
-      continue;
-    }
-    if (c->proj.natoms > 0) {
-      size_t xoff = 0;
-      GBC_TRY(gbc_ensure_work(c, 2, nl_work_bytes(c, nvec, ldx, sizeof(cplx<T>), &xoff)));
-      cplx<T>* C1 = (cplx<T>*)c->work[2];
-      cplx<T>* C2 = C1 + (size_t)c->proj.rows_total * nvec;
-      void* bpre = xoff ? (char*)c->work[2] + xoff : nullptr;
-      TimerScope ts(c, FAM_NONLOCAL, s);
-      GBC_CU(c, launch_nonlocal<T>(c, cur, Y, nvec, ldx, C1, C2, s, true, bpre));
-    }
-    {
-      TimerScope ts(c, FAM_HX_LOCAL, s);
-      CellJob j{c, cur, Y, nvec, ldx, out, prev, a, cc, b};
-      GBC_CU(c, launch_cell_f32(&j, 1, c->cell_var, s));
-    }
-    TimerScope ts(c, FAM_CHEB, s);
-    GBC_CU(c, launch_cheb_rows<T>(Y, cur, prev, out, invmd, c->d_face_rows, c->nface,
-                                  c->proj.natoms > 0 ? c->nface_supp : 0, c->mesh.M, nvec, ldx,
-                                  a, cc, b, s));
+    GBC_TRY(recur_t<T>(c, cur, prev, out, Y, nvec, ldx, a, cc, b, s));
   }
   if (m & 1) GBC_CU(c, launch_copy_block<T>(W, X, c->mesh.M, nvec, ldx, s));
   return GBC_OK;
@@ -417,6 +429,15 @@ gbc_status gbc_apply_h_dev(gbc_ctx* c, const void* X, void* Y, int nvec, int ldx
   if (c->prec == GBC_FP64)
     return apply_h_t<double>(c, (const double2*)X, (double2*)Y, nvec, ldx, s, zero);
   return apply_h_t<float>(c, (const float2*)X, (float2*)Y, nvec, ldx, s, zero);
+}
+
+gbc_status gbc_recur_dev(gbc_ctx* c, const void* cur, const void* prev, void* out, void* Y, int nvec,
+                         int ldx, double a, double cc, double b, void* C, cudaStream_t s) {
+  if (c->prec == GBC_FP64)
+    return recur_t<double>(c, (const double2*)cur, (const double2*)prev, (double2*)out, (double2*)Y,
+                           nvec, ldx, a, cc, b, s, (double2*)C);
+  return recur_t<float>(c, (const float2*)cur, (const float2*)prev, (float2*)out, (float2*)Y, nvec,
+                        ldx, a, cc, b, s, (float2*)C);
 }
 
 // ---------------------------------------------------------------------------

@@ -269,6 +269,11 @@ bool gbc_is_device_ptr(const void* p);
 gbc_status gbc_apply_h_dev(gbc_ctx* c, const void* X, void* Y, int nvec, int ldx, bool zero,
                            cudaStream_t s);
 
+// one recurrence step out = a (M_D^-1 H cur - cc cur) - b prev in the context precision, with the
+// accumulator Y (zero before the first step of a sequence); C (or null) receives P^H cur
+gbc_status gbc_recur_dev(gbc_ctx* c, const void* cur, const void* prev, void* out, void* Y, int nvec,
+                         int ldx, double a, double cc, double b, void* C, cudaStream_t s);
+
 // ---------------------------------------------------------------------------
 // launchers implemented in the .cu files
 // ---------------------------------------------------------------------------

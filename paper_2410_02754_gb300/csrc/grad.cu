@@ -139,20 +139,14 @@ cudaError_t quad_grad(const gbc_ctx* c, const cplx<T>* A, const cplx<T>* B, cons
                               pointwise, s);
 }
 
-// projector-coefficient outer products for the Delta gradient
+// projector-coefficient outer products for the Delta gradient, from Ca = P^H A and Cb = P^H B
 template <typename T>
-gbc_status delta_grad(gbc_ctx* c, const cplx<T>* A, const cplx<T>* B, const double* wv, double f,
-                      int nvec, int ldx, cplx<T>* Ca, cplx<T>* Cb, double2* gD, cudaStream_t s) {
+gbc_status delta_grad(gbc_ctx* c, const cplx<T>* Ca, const cplx<T>* Cb, const double* wv, double f,
+                      int nvec, double2* gD, cudaStream_t s) {
   const ProjDev& pj = c->proj;
   if (pj.natoms == 0) return GBC_OK;
-  GBC_CU(c, launch_nl_project<T>(c, A, nvec, ldx, Ca, s));
-  const cplx<T>* Cbp = Ca;
-  if (B != A) {
-    GBC_CU(c, launch_nl_project<T>(c, B, nvec, ldx, Cb, s));
-    Cbp = Cb;
-  }
   dim3 grid(pj.natoms, 2 * pj.max_npj);
-  k_delta_grad<T><<<grid, 2 * pj.max_npj, 0, s>>>(Ca, Cbp, wv, f, nvec, pj.d_atom_npj,
+  k_delta_grad<T><<<grid, 2 * pj.max_npj, 0, s>>>(Ca, Cb, wv, f, nvec, pj.d_atom_npj,
                                                   pj.d_atom_c_off, pj.d_atom_delta_off, gD);
   GBC_CU(c, cudaGetLastError());
   return GBC_OK;
@@ -163,20 +157,21 @@ gbc_status delta_grad(gbc_ctx* c, const cplx<T>* A, const cplx<T>* B, const doub
 struct GradScratch {
   double* g;
   double2* gD;
-  void* Ca;
-  void* Cb;
+  char* coef;      // projector coefficients P^H X, ncoef sets of coef_bytes
+  size_t coef_bytes;
   double* wv;
   double* dots;
 };
 
-gbc_status grad_scratch(gbc_ctx* c, int nvec, GradScratch* gs) {
+gbc_status grad_scratch(gbc_ctx* c, int nvec, int ncoef, GradScratch* gs) {
   const size_t nq3 = (size_t)c->nq * c->nq * c->nq;
   const size_t ng = (size_t)c->mesh.E * 4 * nq3;
   const size_t nd = c->proj.natoms ? (size_t)c->proj.delta_off[c->proj.natoms] : 0;
   const size_t el = c->prec == GBC_FP64 ? sizeof(double2) : sizeof(float2);
   const size_t nc = std::max<size_t>(1, (size_t)c->proj.rows_total * nvec);
   auto up = [](size_t b) { return (b + 255) / 256 * 256; };
-  const size_t bytes = up(ng * 8) + up(std::max<size_t>(nd, 1) * 16) + 2 * up(nc * el) +
+  gs->coef_bytes = up(nc * el);
+  const size_t bytes = up(ng * 8) + up(std::max<size_t>(nd, 1) * 16) + ncoef * gs->coef_bytes +
                        2 * up((size_t)nvec * 8);
   GBC_TRY(gbc_ensure_work(c, 9, bytes));
   char* p = (char*)c->work[9];
@@ -184,10 +179,8 @@ gbc_status grad_scratch(gbc_ctx* c, int nvec, GradScratch* gs) {
   p += up(ng * 8);
   gs->gD = (double2*)p;
   p += up(std::max<size_t>(nd, 1) * 16);
-  gs->Ca = p;
-  p += up(nc * el);
-  gs->Cb = p;
-  p += up(nc * el);
+  gs->coef = p;
+  p += ncoef * gs->coef_bytes;
   gs->wv = (double*)p;
   p += up((size_t)nvec * 8);
   gs->dots = (double*)p;
@@ -253,24 +246,28 @@ gbc_status filter_vjp_t(gbc_ctx* c, const cplx<T>* X0, const cplx<T>* GY, cplx<T
   auto blk = [&](int i) { return (C*)(pool + bb * (size_t)i); };
   C* Y = (C*)c->work[0];
   auto lam = [&](int j) { return blk(nck + nseg + (j % 3)); };
+  // P^H X_0 .. P^H X_{m-1} and P^H of the adjoint: the recurrence steps leave them, so the Delta
+  // gradient projects only X_{m-1} itself
   GradScratch gs;
-  GBC_TRY(grad_scratch(c, nvec, &gs));
+  GBC_TRY(grad_scratch(c, nvec, m + 1, &gs));
+  auto coef = [&](int k) { return (C*)(gs.coef + gs.coef_bytes * (size_t)k); };
   const size_t nq3 = (size_t)c->nq * c->nq * c->nq;
   GBC_CU(c, cudaMemsetAsync(gs.g, 0, sizeof(double) * c->mesh.E * 4 * nq3, s));
-  if (c->proj.natoms)
+  if (c->proj.natoms) {
     GBC_CU(c, cudaMemsetAsync(gs.gD, 0, sizeof(double2) * c->proj.delta_off[c->proj.natoms], s));
+    GBC_CU(c, cudaMemsetAsync(gs.coef, 0, gs.coef_bytes * (m + 1), s));
+  }
   GBC_CU(c, cudaMemsetAsync(Y, 0, bb, s));
-  const T* invmd = std::is_same<T, double>::value ? (const T*)c->d_invmd : (const T*)c->d_invmd32;
   const long long rows = 2 * c->mesh.M;
   // ---- forward, keeping the checkpoint pairs
   std::vector<C*> xp(m, nullptr);
   for (int j = 0; j < m; ++j) xp[j] = ck_slot[j] >= 0 ? blk(ck_slot[j]) : blk(nck + (j % 3));
   GBC_CU(c, launch_copy_block<T>(X0, xp[0], c->mesh.M, nvec, ldx, s));
   for (int k = 0; k + 1 < m; ++k) {
-    GBC_TRY(gbc_apply_h_dev(c, xp[k], Y, nvec, ldx, false, s));
-    GBC_CU(c, launch_cheb_step<T>(Y, xp[k], k ? xp[k - 1] : nullptr, xp[k + 1], invmd, c->mesh.M,
-                                  nvec, ldx, alpha[k] / e, cc, beta[k], s));
+    GBC_TRY(gbc_recur_dev(c, xp[k], k ? xp[k - 1] : nullptr, xp[k + 1], Y, nvec, ldx, alpha[k] / e, cc,
+                          beta[k], coef(k), s));
   }
+  if (c->proj.natoms) GBC_CU(c, launch_nl_project<T>(c, xp[m - 1], nvec, ldx, coef(m - 1), s));
   // ---- adjoint seed Lt_m = M_D^-1 G_Y
   k_rowscale<T><<<gfor(rows * nvec), 256, 0, s>>>(GY, lam(m), c->d_invmd, rows, nvec, ldx);
   GBC_CU(c, cudaGetLastError());
@@ -282,20 +279,18 @@ gbc_status filter_vjp_t(gbc_ctx* c, const cplx<T>* X0, const cplx<T>* GY, cplx<T
     for (int j = k0; j < k1; ++j) seg[j - k0] = ck_slot[j] >= 0 ? blk(ck_slot[j]) : blk(nck + (j - k0));
     for (int k = k0 + 1; k + 1 < k1; ++k) {      // recompute X_{k+1} from X_k, X_{k-1}
       if (ck_slot[k + 1] >= 0) continue;
-      GBC_TRY(gbc_apply_h_dev(c, seg[k - k0], Y, nvec, ldx, false, s));
-      GBC_CU(c, launch_cheb_step<T>(Y, seg[k - k0], seg[k - 1 - k0], seg[k + 1 - k0], invmd,
-                                    c->mesh.M, nvec, ldx, alpha[k] / e, cc, beta[k], s));
+      GBC_TRY(gbc_recur_dev(c, seg[k - k0], seg[k - 1 - k0], seg[k + 1 - k0], Y, nvec, ldx, alpha[k] / e,
+                            cc, beta[k], nullptr, s));
     }
     for (int k = k1 - 1; k >= k0; --k) {
       const double f = alpha[k] / e;
       C* Xk = seg[k - k0];
       C* Lt1 = lam(k + 1);
       GBC_CU(c, quad_grad<T>(c, Lt1, Xk, nullptr, f, nvec, ldx, gs.g, s));
-      GBC_TRY(delta_grad<T>(c, Lt1, Xk, nullptr, f, nvec, ldx, (C*)gs.Ca, (C*)gs.Cb, gs.gD, s));
-      GBC_TRY(gbc_apply_h_dev(c, Lt1, Y, nvec, ldx, false, s));
       const bool has2 = k + 2 <= m;
-      GBC_CU(c, launch_cheb_step<T>(Y, Lt1, has2 ? lam(k + 2) : nullptr, lam(k), invmd, c->mesh.M,
-                                    nvec, ldx, alpha[k] / e, cc, has2 ? beta[k + 1] : 0.0, s));
+      GBC_TRY(gbc_recur_dev(c, Lt1, has2 ? lam(k + 2) : nullptr, lam(k), Y, nvec, ldx, alpha[k] / e, cc,
+                            has2 ? beta[k + 1] : 0.0, coef(m), s));
+      GBC_TRY(delta_grad<T>(c, coef(m), coef(k), nullptr, f, nvec, gs.gD, s));
     }
   }
   // ---- grad_X0 = M_D Lt_0
@@ -308,7 +303,7 @@ template <typename T>
 gbc_status energy_grad_t(gbc_ctx* c, const cplx<T>* Y, const double* w, cplx<T>* GY, double* loss,
                          double* gV, double* gB, double* gDelta, int nvec, int ldx, cudaStream_t s) {
   GradScratch gs;
-  GBC_TRY(grad_scratch(c, nvec, &gs));
+  GBC_TRY(grad_scratch(c, nvec, 1, &gs));
   const size_t nq3 = (size_t)c->nq * c->nq * c->nq;
   GBC_CU(c, cudaMemsetAsync(gs.g, 0, sizeof(double) * c->mesh.E * 4 * nq3, s));
   if (c->proj.natoms)
@@ -333,7 +328,8 @@ gbc_status energy_grad_t(gbc_ctx* c, const cplx<T>* Y, const double* w, cplx<T>*
   k_colscale<T><<<gfor(rows * nvec), 256, 0, s>>>(GY, gs.wv, 2.0, rows, nvec, ldx);
   GBC_CU(c, cudaGetLastError());
   GBC_CU(c, quad_grad<T>(c, Y, Y, gs.wv, 1.0, nvec, ldx, gs.g, s));
-  GBC_TRY(delta_grad<T>(c, Y, Y, gs.wv, 1.0, nvec, ldx, (cplx<T>*)gs.Ca, (cplx<T>*)gs.Cb, gs.gD, s));
+  if (c->proj.natoms) GBC_CU(c, launch_nl_project<T>(c, Y, nvec, ldx, (cplx<T>*)gs.coef, s));
+  GBC_TRY(delta_grad<T>(c, (cplx<T>*)gs.coef, (cplx<T>*)gs.coef, gs.wv, 1.0, nvec, gs.gD, s));
   std::vector<double> dots(nvec);
   GBC_CU(c, cudaMemcpyAsync(dots.data(), gs.dots, sizeof(double) * nvec, cudaMemcpyDeviceToHost, s));
   GBC_TRY(grad_download(c, gs, gV, gB, gDelta, s));
@@ -384,7 +380,7 @@ gbc_status gbc_density(gbc_ctx* c, const void* X, const double* occ, double* rho
   if (!gbc_is_device_ptr(X)) return gbc_fail(c, GBC_EINVAL, "X must be device memory");
   cudaStream_t s = (cudaStream_t)stream;
   GradScratch gs;
-  GBC_TRY(grad_scratch(c, nvec, &gs));
+  GBC_TRY(grad_scratch(c, nvec, 1, &gs));
   GBC_CU(c, cudaMemcpyAsync(gs.wv, occ, sizeof(double) * nvec, cudaMemcpyHostToDevice, s));
   if (c->prec == GBC_FP64)
     GBC_CU(c, density_t<double>(c, (const double2*)X, gs.wv, gs.g, nvec, ldx, 0, s));
