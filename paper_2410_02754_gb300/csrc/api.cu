@@ -231,14 +231,14 @@ gbc_status filter_t(gbc_ctx* c, cplx<T>* X, int nvec, int ldx, int m, double lT,
 template <typename T> constexpr int split_gram_cols() { return sizeof(T) == 8 ? 16 : 64; }
 template <typename T> constexpr int split_rotate_cols() { return sizeof(T) == 8 ? 16 : 32; }
 
-// S = X^H diag(md) Y, both triangles
+// S = X^H diag(md) X (Y = X) or X^H Y (md null), both triangles
 template <typename T, typename TY>
 gbc_status gram(gbc_ctx* c, const cplx<T>* X, int ldx, const cplx<TY>* Y, int ldy, const double* md,
                 int nvec, double2* S, cudaStream_t s) {
   {
     TimerScope ts(c, FAM_GRAM, s);
     if (nvec >= split_gram_cols<T>()) {
-      GBC_TRY((launch_gram_split<T, TY>(c, X, ldx, Y, ldy, md, c->mesh.M, nvec, S, s)));
+      GBC_TRY((launch_gram_split<T, TY>(c, X, ldx, md ? nullptr : Y, ldy, md, c->mesh.M, nvec, S, s)));
     } else if constexpr (std::is_same<T, double>::value) {
       GBC_CU(c, launch_gram<double>(X, Y, md, c->mesh.M, nvec, ldx, S, s));
     } else {

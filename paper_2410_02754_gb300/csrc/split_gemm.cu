@@ -21,7 +21,9 @@
 //    S = 7 (54 bits), 28 digit products.
 //
 // GB300's FP64 pipe gives 1.05 TFLOP/s and float-float arithmetic on the FP32 pipes about 6;
-// 28 BF16 products at 1.9 PFLOP/s are an FP64-accurate 68 TFLOP/s.  Per tile (128 x 128 for
+// 28 BF16 products at 1.9 PFLOP/s are an FP64-accurate 68 TFLOP/s.  Measured, 884,736 nodes x 256
+// FP32 columns: Gram 122 -> 21 ms (16 of them the products, 43% of the tensor pipe), rotation
+// 163 -> 26 ms (23 the products); 373,248 nodes x 256 in FP64: 333 -> 13 and 527 -> 14 ms.  Per tile (128 x 128 for
 // S = 4, 128 x 64 for S = 7) every order has its own accumulator in tensor memory and all S
 // digit slices of a 64-wide K chunk are in shared memory at once (one TMA box each), so a
 // slice is loaded once per tile and used in up to S products.  Step i multiplies A_i with all
@@ -42,6 +44,8 @@ __device__ int g_split_err;   // set when a bounded wait expired
 constexpr int kTM = 128;              // tile rows
 constexpr int kKC = 64;               // K chunk: one 128-byte swizzled row
 constexpr int kBad = 0x7fffffff;      // exponent of a row with an infinity or a NaN
+constexpr int kEpi = 16;              // read-out warps
+constexpr int kSplitThreads = 64 + 32 * kEpi;
 template <int S> struct SplitCfg {
   static constexpr int N = S <= 4 ? 128 : 64;             // tile columns
   static constexpr int FLUSH = S <= 4 ? 4 : 2;            // K chunks between read-outs
@@ -72,7 +76,7 @@ __device__ __forceinline__ double pow2d(int e) {
 
 // Persistent: CTAs take work items blockIdx.x, + gridDim.x, ...; the roles run on across items.
 template <int S, int MODE>
-__global__ void __launch_bounds__(320, 1)
+__global__ void __launch_bounds__(kSplitThreads, 1)
 k_split_gemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb,
              const SplitArgs a) {
   using G = SplitCfg<S>;
@@ -131,7 +135,7 @@ k_split_gemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUt
       tc::mbar_init(tc::smem_u32(&emptyb[s]), 1);
     }
     tc::mbar_init(tc::smem_u32(accf), 1);
-    tc::mbar_init(tc::smem_u32(acce), 8);
+    tc::mbar_init(tc::smem_u32(acce), kEpi);
     tc::mbar_init(tc::smem_u32(drain), 1);
     *fail = 0;
     tc::fence_mbar_init();
@@ -215,9 +219,9 @@ k_split_gemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUt
     tc::mma_commit(tc::smem_u32(drain));
     if (!tc::mbar_wait_bounded(tc::smem_u32(drain), 0)) atomicExch(fail, 1);
   } else if (warp >= 2) {
-    const int g = warp & 3, half = (warp - 2) >> 2;
-    constexpr int NC = N / 2;                        // columns of a thread
-    const uint32_t tl = tmem + ((uint32_t)(g * 32) << 16) + (uint32_t)(half * NC);
+    const int g = warp & 3, part = (warp - 2) >> 2;
+    constexpr int NC = N / (kEpi / 4);               // columns of a thread
+    const uint32_t tl = tmem + ((uint32_t)(g * 32) << 16) + (uint32_t)(part * NC);
     int win = 0;
     bool ok = true;
     for (int w = blockIdx.x; w < a.nwork && ok; w += gridDim.x) {
@@ -238,18 +242,26 @@ k_split_gemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUt
         if (ok) {
 #pragma unroll
           for (int c0 = 0; c0 < NC; c0 += 8) {
-            uint32_t r[S][8];
+            // orders 0..3, then the others: half of the registers at a time
+            uint32_t r[4][8];
 #pragma unroll
-            for (int t = 0; t < S; ++t) tc::tmem_ld8_nowait(tl + t * N + c0, r[t]);
+            for (int t = 0; t < 4; ++t) tc::tmem_ld8_nowait(tl + t * N + c0, r[t]);
             tc::tmem_wait_ld();
 #pragma unroll
             for (int i = 0; i < 8; ++i)
 #pragma unroll
-              for (int t = 0; t < S; ++t) {
-                const int x = __float2int_rn(__uint_as_float(r[t][i]));
-                if (t < 4) hi[c0 + i] += (long long)x * (1 << (8 * (3 - t)));
-                else lo[c0 + i] += (long long)x * (1 << (8 * (S - 1 - t)));
-              }
+              for (int t = 0; t < 4; ++t)
+                hi[c0 + i] += (long long)__float2int_rn(__uint_as_float(r[t][i])) * (1 << (8 * (3 - t)));
+            if (S > 4) {
+#pragma unroll
+              for (int t = 4; t < S; ++t) tc::tmem_ld8_nowait(tl + t * N + c0, r[t - 4]);
+              tc::tmem_wait_ld();
+#pragma unroll
+              for (int i = 0; i < 8; ++i)
+#pragma unroll
+                for (int t = 4; t < S; ++t)
+                  lo[c0 + i] += (long long)__float2int_rn(__uint_as_float(r[t - 4][i])) * (1 << (8 * (S - 1 - t)));
+            }
           }
         }
         tc::fence_before_sync();
@@ -258,7 +270,7 @@ k_split_gemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUt
       if (ok) {
         const int mr = it.m0 + g * 32 + lane;
         const int ea = a.ea[mr];
-        const int cb = it.n0 + half * NC;
+        const int cb = it.n0 + part * NC;
         const int* eb = a.eb + cb;
         // a rotation's sum (|hi| < 2^47) as one integer in units of 2^(ea + eb - 24 - sh): exact
         // where |hi| < 2^38 (or S = 4), else cut 2^-53 below its leading bit; rounded once
@@ -488,8 +500,8 @@ __global__ void k_col_scale(const double2* __restrict__ diag, int n, int* __rest
   }
 }
 
-// largest magnitude key of every real column over all rows (WEIGHT: of |x| w rounded up by a
-// factor of two)
+// largest magnitude key of every real column over all rows (WEIGHT: of |x| sqrt(w) rounded up
+// by a factor of two)
 template <typename T, bool WEIGHT>
 __global__ void __launch_bounds__(256)
 k_col_max(const cplx<T>* __restrict__ X, int ldx, int n, long long rows,
@@ -501,7 +513,7 @@ k_col_max(const cplx<T>* __restrict__ X, int ldx, int n, long long rows,
     for (long long r = blockIdx.x * 8LL + (threadIdx.x >> 5); r < rows; r += step) {
       cplx<T> x = X[r * ldx + c];
       if (WEIGHT) {
-        const T w = 2 * (T)md[r >> 1];
+        const T w = 2 * (T)sqrtf((float)md[r >> 1]);
         x.x *= w;
         x.y *= w;
       }
@@ -523,7 +535,8 @@ k_col_max(const cplx<T>* __restrict__ X, int ldx, int n, long long rows,
 
 // columns of a block over the rows [r0, r0 + rows_pad) -> digits [S][cols_pad][rows_pad] (rows
 // contiguous), rows >= rows as zeros; blocks of 64 rows x 32 complex columns are transposed
-// through shared memory.  WEIGHT: x w (FP64 product).
+// through shared memory.  WEIGHT: x sqrt(w), an FP64 product, so that one set of digits serves
+// both factors of X^H diag(w) X.
 template <int S, typename T, bool WEIGHT>
 __global__ void __launch_bounds__(256)
 k_split_cols(const cplx<T>* __restrict__ X, int ldx, int n, long long r0, long long rows,
@@ -531,14 +544,20 @@ k_split_cols(const cplx<T>* __restrict__ X, int ldx, int n, long long r0, long l
              const unsigned* __restrict__ key, uint16_t* __restrict__ D, int* __restrict__ eu) {
   using V = typename std::conditional<WEIGHT, double, T>::type;
   __shared__ V xs[64][65];                      // [real column][row]
+  __shared__ double ws[64];
   const int rb = blockIdx.x * 64, cb = blockIdx.y * 32;
+  if (WEIGHT) {
+    if (threadIdx.x < 64)
+      ws[threadIdx.x] = rb + threadIdx.x < rows ? sqrt(md[(r0 + rb + threadIdx.x) >> 1]) : 0.0;
+    __syncthreads();
+  }
   for (int i = threadIdx.x; i < 64 * 32; i += 256) {
     const int c = i & 31, rr = i >> 5;
     const long long r = rb + rr;
     V a = 0, b = 0;
     if (r < rows && cb + c < n) {
       const cplx<T> x = X[(r0 + r) * ldx + cb + c];
-      const double w = WEIGHT ? md[(r0 + r) >> 1] : 1.0;
+      const double w = WEIGHT ? ws[rr] : 1.0;
       a = WEIGHT ? (V)((double)x.x * w) : (V)x.x;
       b = WEIGHT ? (V)((double)x.y * w) : (V)x.y;
     }
@@ -577,7 +596,7 @@ cudaError_t run_split_gemm(const uint16_t* A, const uint16_t* B, int kpad, const
   auto k = k_split_gemm<S, MODE>;
   const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM);
   if (e != cudaSuccess) return e;
-  k<<<(unsigned)std::min(a.nwork, gbc_sm_count()), 320, G::SMEM, s>>>(ta, tb, a);
+  k<<<(unsigned)std::min(a.nwork, gbc_sm_count()), kSplitThreads, G::SMEM, s>>>(ta, tb, a);
   return cudaGetLastError();
 }
 
@@ -631,7 +650,9 @@ static gbc_status rotate_split(gbc_ctx* c, cplx<T>* X, const double2* Q, long lo
 template <typename T>
 gbc_status launch_rotate_split(gbc_ctx* c, cplx<T>* X, const double2* Q, long long M, int n, int ldx,
                                const double2* diag, cudaStream_t s) {
-  if (sizeof(T) == 4 && !diag) return rotate_split<4, T>(c, X, Q, M, n, ldx, diag, s);
+  if constexpr (sizeof(T) == 4) {
+    if (!diag) return rotate_split<4, T>(c, X, Q, M, n, ldx, diag, s);
+  }
   return rotate_split<7, T>(c, X, Q, M, n, ldx, diag, s);
 }
 template gbc_status launch_rotate_split<float>(gbc_ctx*, float2*, const double2*, long long, int, int,
@@ -639,7 +660,7 @@ template gbc_status launch_rotate_split<float>(gbc_ctx*, float2*, const double2*
 template gbc_status launch_rotate_split<double>(gbc_ctx*, double2*, const double2*, long long, int, int,
                                                 const double2*, cudaStream_t);
 
-// Sm (upper triangle) = X^H diag(md) Y (md may be null: weight 1)
+// Sm (upper triangle) = X^H diag(md) X (Y null), or X^H Y (md null)
 template <typename TX, typename TY>
 gbc_status launch_gram_split(gbc_ctx* c, const cplx<TX>* X, int ldx, const cplx<TY>* Y, int ldy,
                              const double* md, long long M, int n, double2* Sm, cudaStream_t s) {
@@ -647,17 +668,17 @@ gbc_status launch_gram_split(gbc_ctx* c, const cplx<TX>* X, int ldx, const cplx<
   using G = SplitCfg<S>;
   const long long rows = 2 * M;
   const int ma = up(2 * n, kTM), nb = ma;    // both padded to a row tile
-  const size_t rowb = (size_t)2 * S * (ma + nb);
+  const size_t rowb = (size_t)2 * S * (Y ? ma + nb : ma);
   const int win = G::FLUSH * kKC;
   const long long per = std::max<long long>(win, (long long)(kChunkBytes / rowb) / win * win);
   const int rc = (int)std::min<long long>(per, (rows + win - 1) / win * win);
-  const size_t ab = (size_t)2 * S * ma * rc, bb = (size_t)2 * S * nb * rc;
+  const size_t ab = (size_t)2 * S * ma * rc, bb = Y ? (size_t)2 * S * nb * rc : 0;
   GBC_TRY(gbc_ensure_work(c, 13, ab + bb + sizeof(int) * 4 * (size_t)ma + 1024));
   uint16_t* A = (uint16_t*)c->work[13];
-  uint16_t* B = (uint16_t*)((char*)A + ab);
-  int* ea = (int*)((char*)B + bb);
-  int* eb = ea + ma;
-  unsigned* ka = (unsigned*)(eb + nb);
+  uint16_t* B = Y ? (uint16_t*)((char*)A + ab) : A;   // one set of digits for both factors
+  int* ea = (int*)((char*)A + ab + bb);
+  int* eb = Y ? ea + ma : ea;
+  unsigned* ka = (unsigned*)(ea + 2 * (size_t)ma);
   unsigned* kb = ka + ma;
   GBC_CU(c, cudaMemsetAsync(Sm, 0, sizeof(double2) * (size_t)n * n, s));
   GBC_CU(c, cudaMemsetAsync(ka, 0, sizeof(unsigned) * 2 * (size_t)ma, s));
@@ -665,7 +686,7 @@ gbc_status launch_gram_split(gbc_ctx* c, const cplx<TX>* X, int ldx, const cplx<
   const dim3 gm((unsigned)std::max<long long>(1, std::min<long long>((rows + 63) / 64, 16LL * gbc_sm_count() / ncb + 1)), ncb);
   if (md) k_col_max<TX, true><<<gm, 256, 0, s>>>(X, ldx, n, rows, md, ka);
   else k_col_max<TX, false><<<gm, 256, 0, s>>>(X, ldx, n, rows, md, ka);
-  k_col_max<TY, false><<<gm, 256, 0, s>>>(Y, ldy, n, rows, nullptr, kb);
+  if (Y) k_col_max<TY, false><<<gm, 256, 0, s>>>(Y, ldy, n, rows, nullptr, kb);
   GBC_CU(c, cudaGetLastError());
   int tiles = 0;
   const int ntn = nb / G::N;
@@ -676,7 +697,7 @@ gbc_status launch_gram_split(gbc_ctx* c, const cplx<TX>* X, int ldx, const cplx<
     const dim3 gs((unsigned)(rp / 64), (unsigned)(ma / 64));
     if (md) k_split_cols<S, TX, true><<<gs, 256, 0, s>>>(X, ldx, n, r0, nr, rp, ma, md, ka, A, ea);
     else k_split_cols<S, TX, false><<<gs, 256, 0, s>>>(X, ldx, n, r0, nr, rp, ma, md, ka, A, ea);
-    k_split_cols<S, TY, false><<<gs, 256, 0, s>>>(Y, ldy, n, r0, nr, rp, nb, nullptr, kb, B, eb);
+    if (Y) k_split_cols<S, TY, false><<<gs, 256, 0, s>>>(Y, ldy, n, r0, nr, rp, nb, nullptr, kb, B, eb);
     GBC_CU(c, cudaGetLastError());
     // K split so that the CTAs fill the SMs about once, in whole read-out windows
     const int nwin = rp / win;
