@@ -147,7 +147,7 @@ gbc_status apply_h_t(gbc_ctx* c, const cplx<T>* X, cplx<T>* Y, int nvec, int ldx
     cplx<T>* C2 = C1 + (size_t)c->proj.rows_total * nvec;
     {
       TimerScope ts(c, FAM_NONLOCAL, s);
-      e = launch_nonlocal<T>(c, X, Y, nvec, ldx, C ? C : C1, C2, s);
+      e = launch_nonlocal<T>(c, X, Y, nvec, ldx, C ? C : C1, C2, s, false, nullptr, true);
     }
     if (e != cudaSuccess) return gbc_cuda_fail(c, e, "nonlocal");
   }
@@ -632,9 +632,10 @@ gbc_status gbc_sync_status(gbc_ctx* c, void* stream) {
   cudaStream_t s = (cudaStream_t)stream;
   int err = 0;
   GBC_CU(c, tc_nonlocal_error(&err, s));
-  int err2 = 0;
+  int err2 = 0, err3 = 0;
   GBC_CU(c, tcl_error(&err2, s));
-  err |= err2;
+  GBC_CU(c, split_error(&err3, s));
+  err |= err2 | err3;
   if (err) {
     GBC_CU(c, tc_nonlocal_reset(s));
     GBC_CU(c, cudaStreamSynchronize(s));

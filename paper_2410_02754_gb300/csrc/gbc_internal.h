@@ -209,8 +209,8 @@ struct gbc_ctx {
   // 0 H.X accumulator, 1 second block, 2 nonlocal coefficients, 3 small dense,
   // 4-7 FP64 copies / residual-split blocks, 8 backward block pool, 9 backward
   // accumulators; deterministic mode: 10 per-cell results, 11 projection partials,
-  // 12 reduction partials; 13 digit slices of the split products
-  static constexpr int kWorkSlots = 14;
+  // 12 reduction partials; 13 digit slices of the split products, 14 those of the nonlocal step
+  static constexpr int kWorkSlots = 15;
   void* work[kWorkSlots] = {};
   size_t work_bytes[kWorkSlots] = {};
   bool deterministic = false;        // FP64 kernels: fixed-order sums instead of atomics
@@ -321,11 +321,12 @@ gbc_status tcl_apply(gbc_ctx* c, const float2* X, float2* Y, int nvec, int ldx, 
 cudaError_t tcl_error(int* err, cudaStream_t s);
 void tcl_free(TclState* t);
 // nonlocal.cu : Y += sum_a P Delta P^H X (overwrite: Y = sum_a P Delta P^H X on every
-// support row, other rows untouched)
+// support row, other rows untouched).  may_alloc: work slot 14 may be grown and used (not in the
+// allocation-free entry point)
 template <typename T>
 cudaError_t launch_nonlocal(gbc_ctx* c, const cplx<T>* X, cplx<T>* Y, int nvec, int ldx,
                             cplx<T>* Cbuf, cplx<T>* Cpbuf, cudaStream_t s, bool overwrite = false,
-                            void* bpre = nullptr);
+                            void* bpre = nullptr, bool may_alloc = false);
 // nonlocal workspace for nvec vectors of element size el: C, C' and (FP32 tensor-core
 // expansion) its B blocks; *bpre_off = their offset, 0 when not used
 size_t nl_work_bytes(const gbc_ctx* c, int nvec, int ldx, size_t el, size_t* bpre_off);
@@ -429,6 +430,11 @@ template <typename TX, typename TY>
 gbc_status launch_gram_split(gbc_ctx* c, const cplx<TX>* X, int ldx, const cplx<TY>* Y, int ldy,
                              const double* md, long long M, int n, double2* Sm, cudaStream_t s);
 cudaError_t split_error(int* err, cudaStream_t s);
+// the FP64 projector contractions in the same form: C1 += P^H X, Y += P C2, with
+// nl_split_bytes in work slot 14
+size_t nl_split_bytes(const gbc_ctx* c, int nvec);
+cudaError_t nl_split_project(gbc_ctx* c, const double2* X, int nvec, int ldx, double2* C1, cudaStream_t s);
+cudaError_t nl_split_expand(gbc_ctx* c, double2* Y, int nvec, int ldx, const double2* C2, cudaStream_t s);
 // residual-split filter kernels
 template <typename T>
 cudaError_t launch_split_init(const double2* HX, const double2* X64, const double* invmd,

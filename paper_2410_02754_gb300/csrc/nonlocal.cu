@@ -399,6 +399,36 @@ cudaError_t run_expand_add(const gbc_ctx* c, double2* Y, int nvec, int ldx, cons
   return cudaGetLastError();
 }
 
+// FP64 contractions as split products on the tensor cores (split_gemm.cu), with their workspace in
+// place, where that is faster.  The direct kernels run at the FP64 rate (578 FMAs per ns at 95% of
+// it; padded columns count), the split ones take, per support node, writing and reading its
+// digits and the MMAs of one 64-wide tile of projectors, whatever their number.  Times in ns, the
+// constants fitted to H.X of 122,514 and 329,884 support nodes (18 projectors, p = 6) and of 25,476
+// and 1458 nodes (3 and 18).  Direct / split H.X, cell apply included, k != 0:
+//   122,514 nodes: 8 vectors 1.05 / 1.20 ms, 16 2.01 / 1.70, 64 7.52 / 4.82, 200 23.7 / 14.1
+//   329,884 nodes: 8 vectors 3.54 / 3.61 ms, 16 6.86 / 5.70, 64 27.0 / 18.9, 200 82.5 / 58.4
+//   122,514 nodes at k = 0 (half the FP64 work): 16 vectors 1.36 / 1.59, 64 5.08 / 4.37 ms
+//   25,476 nodes x 3 projectors, 64 vectors 1.71 / 1.84; 1458 nodes, 64 vectors 0.18 / 0.32 ms
+// Where the workspace cannot be had (no memory left, or it would have to grow while the stream is
+// captured) the direct kernels run.
+bool use_split(gbc_ctx* c, int nvec, cudaStream_t s) {
+  if (c->deterministic) return false;
+  const ProjDev& pj = c->proj;
+  const double np = (double)pj.nnodes_total;
+  const int ct = nl_col_tile(nvec), dcols = (2 * nvec + ct - 1) / ct * ct, scols = (4 * nvec + 127) / 128 * 128;
+  const double direct = (double)pj.pv_off.back() * dcols * (real_tables(c) ? 4 : 8) / 578.0;
+  const double split = 120e3 + np * (4.0 + 0.02 * scols);
+  if (direct < split) return false;
+  const size_t bytes = nl_split_bytes(c, nvec);
+  if (c->work_bytes[14] >= bytes) return true;
+  cudaStreamCaptureStatus cap;
+  if (cudaStreamIsCapturing(s, &cap) == cudaSuccess) {
+    if (cap != cudaStreamCaptureStatusNone) return false;
+    if (gbc_ensure_work(c, 14, bytes) == GBC_OK) return true;
+  }
+  cudaGetLastError();   // not left for the next launch's check
+  return false;
+}
 bool use_tc(const gbc_ctx* c) { return c->nl_engine == GBC_NL_TENSOR && tc_nonlocal_supported(c->proj); }
 
 }  // namespace
@@ -406,10 +436,18 @@ bool use_tc(const gbc_ctx* c) { return c->nl_engine == GBC_NL_TENSOR && tc_nonlo
 template <typename T>
 cudaError_t launch_nonlocal(gbc_ctx* c, const cplx<T>* X, cplx<T>* Y, int nvec, int ldx,
                             cplx<T>* Cbuf, cplx<T>* Cpbuf, cudaStream_t s, bool overwrite,
-                            void* bpre) {
+                            void* bpre, bool may_alloc) {
   const ProjDev& pj = c->proj;
   if (pj.natoms == 0 || nvec == 0 || pj.nchunks == 0 || pj.nexp_chunks == 0) return cudaSuccess;
-  cudaError_t e = launch_nl_project<T>(c, X, nvec, ldx, Cbuf, s);
+  const bool split = std::is_same<T, double>::value && may_alloc && !overwrite && use_split(c, nvec, s);
+  cudaError_t e = cudaSuccess;
+  if constexpr (std::is_same<T, double>::value) {
+    if (split) {
+      e = cudaMemsetAsync(Cbuf, 0, sizeof(cplx<T>) * (size_t)pj.rows_total * nvec, s);
+      if (e == cudaSuccess) e = nl_split_project(c, X, nvec, ldx, Cbuf, s);
+    }
+  }
+  if (!split) e = launch_nl_project<T>(c, X, nvec, ldx, Cbuf, s);
   if (e != cudaSuccess) return e;
   const cplx<T>* D = std::is_same<T, double>::value ? (const cplx<T>*)pj.d_delta64
                                                     : (const cplx<T>*)pj.d_delta32;
@@ -420,6 +458,8 @@ cudaError_t launch_nonlocal(gbc_ctx* c, const cplx<T>* X, cplx<T>* Y, int nvec, 
   if (e != cudaSuccess) return e;
   if constexpr (std::is_same<T, float>::value) {
     if (use_tc(c)) return launch_tc_expand(pj, Y, nvec, ldx, Cpbuf, s, overwrite, bpre, c->d_cell_ctr);
+  } else if (split) {
+    return nl_split_expand(c, Y, nvec, ldx, Cpbuf, s);
   } else if (!overwrite && !c->deterministic) {
     if (pj.max_npj <= 4) return run_expand_add<4>(c, Y, nvec, ldx, Cpbuf, s);
     if (pj.max_npj <= 8) return run_expand_add<8>(c, Y, nvec, ldx, Cpbuf, s);
@@ -464,9 +504,9 @@ template cudaError_t launch_nl_project<double>(gbc_ctx*, const double2*, int, in
                                                cudaStream_t);
 
 template cudaError_t launch_nonlocal<float>(gbc_ctx*, const float2*, float2*, int, int, float2*,
-                                            float2*, cudaStream_t, bool, void*);
+                                            float2*, cudaStream_t, bool, void*, bool);
 template cudaError_t launch_nonlocal<double>(gbc_ctx*, const double2*, double2*, int, int,
-                                             double2*, double2*, cudaStream_t, bool, void*);
+                                             double2*, double2*, cudaStream_t, bool, void*, bool);
 
 size_t nl_work_bytes(const gbc_ctx* c, int nvec, int ldx, size_t el, size_t* bpre_off) {
   const size_t cb = el * (size_t)c->proj.rows_total * (size_t)nvec;

@@ -56,17 +56,24 @@ template <int S> struct SplitCfg {
   static_assert(SMEM <= 227 * 1024, "shared memory");
 };
 
-enum { ROT32 = 0, ROT64 = 1, GRAM = 2 };
+// PROJ, EXPD: the FP64 projector contractions C += P^H X and Y += P C' (see nl_split_project)
+enum { ROT32 = 0, ROT64 = 1, GRAM = 2, PROJ = 3, EXPD = 4 };
+constexpr int kNlRows = 1024;         // rows of a support chunk's place in the digit buffers
 struct SplitArgs {
   int rows_a, rows_b;      // rows of a slice of A and B
   int nchunk, kper;        // K chunks; chunks per work item (GRAM: a part of them)
   int ntn;                 // column tiles
   int ntiles, nwork;       // tiles; work items (tiles, GRAM: x K parts)
   const int *ea, *eb;      // unit exponents (E - 6) of the rows of A and B
-  long long rows;          // rotation: valid rows of the chunk
+  long long rows;          // rotation: valid rows of the chunk; EXPD: free nodes of the mesh
   int n;                   // complex columns
-  int ldo;                 // rotation: complex leading dimension of out
+  int ldo;                 // rotation, EXPD: complex leading dimension of out
   void* out;
+  // PROJ, EXPD: chunks (atom, first node, count, node offset of the atom), supports, projectors
+  // and first row of C of an atom
+  const int4* chunks;
+  const long long* nodes;
+  const int *npj, *c_off;
 };
 
 // 2^e as a double (|e| < 1000)
@@ -81,9 +88,13 @@ k_split_gemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUt
              const SplitArgs a) {
   using G = SplitCfg<S>;
   constexpr int N = G::N;
-  struct Item { int m0, n0, k0, nk; };
+  // orders kept: the nonlocal contractions keep one more (order S: digits 1 .. S-1 only), since
+  // projectors are far below their largest value on most of their support
+  constexpr int T = MODE == PROJ || MODE == EXPD ? S + 1 : S;
+  static_assert(T * N <= 512 && T <= 8, "tensor memory columns");
+  struct Item { int m0, n0, k0, nk, b; };   // b: chunk of the batch
   auto decode = [&](int w) {
-    Item it{0, 0, 0, a.nchunk};
+    Item it{0, 0, 0, a.nchunk, 0};
     if (MODE == GRAM) {   // tiles that reach the diagonal or above it, row by row
       int I = 0, t = w % a.ntiles, first = 0;
       while (t >= a.ntn - first) {
@@ -95,6 +106,18 @@ k_split_gemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUt
       it.n0 = (first + t) * N;
       it.k0 = (w / a.ntiles) * a.kper;
       it.nk = min(a.kper, a.nchunk - it.k0);
+    } else if (MODE == PROJ) {   // X columns x projectors over the chunk's nodes
+      it.b = w / a.ntn;
+      it.m0 = w % a.ntn * kTM;
+      it.k0 = it.b * (kNlRows / kKC);
+      it.nk = (a.chunks[it.b].z + 127) / 128 * (128 / kKC);
+    } else if (MODE == EXPD) {   // nodes x columns of C' over the atom's projectors (B per chunk)
+      const int mt = w / a.ntn;
+      it.b = mt / (kNlRows / kTM);
+      const int4 ch = a.chunks[it.b];
+      it.m0 = mt * kTM;
+      it.n0 = (it.b * a.ntn + w % a.ntn) * N;
+      it.nk = it.m0 - it.b * kNlRows < ch.z ? 1 : 0;
     } else {   // column tiles of a row tile next to each other (its digits stay in L2)
       it.m0 = w / a.ntn * kTM;
       it.n0 = w % a.ntn * N;
@@ -193,18 +216,25 @@ k_split_gemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUt
         for (int i = 0; i < S; ++i) {
           if (!tc::mbar_wait_bounded(tc::smem_u32(&fulla[i]), q & 1)) atomicExch(fail, 1);
           tc::fence_after_sync();
-          // A_i against B_0 .. B_{S-1-i} at once: the slices are consecutive rows of one operand
-          // and their orders i .. S-1 consecutive accumulators, so an instruction is up to 256
+          // A_i against B_0 .. B_{T-1-i} at once: the slices are consecutive rows of one operand
+          // and their orders i .. T-1 consecutive accumulators, so an instruction is up to 256
           // columns wide (64 columns take as long as 256)
 #pragma unroll
           for (int kk = 0; kk < 4; ++kk)
 #pragma unroll
-            for (int j = 0; j < S - i; j += 256 / N) {
+            for (int j = 0; j < (T - i < S ? T - i : S); j += 256 / N) {
               constexpr int W = 256 / N;
-              const int cnt = S - i - j < W ? S - i - j : W;
-              tc::mma_bf16(tmem + (i + j) * N, tc::sdesc_sw128(A(i) + kk * 32),
-                           tc::sdesc_sw128(B(buf, j) + kk * 32), tc::idesc_bf16(kTM, cnt * N),
-                           (first && i == 0 && kk == 0) ? 0u : 1u);
+              const int nb = T - i < S ? T - i : S, cnt = nb - j < W ? nb - j : W;
+              auto mma = [&](int j, int cnt, unsigned acc) {
+                tc::mma_bf16(tmem + (i + j) * N, tc::sdesc_sw128(A(i) + kk * 32),
+                             tc::sdesc_sw128(B(buf, j) + kk * 32), tc::idesc_bf16(kTM, cnt * N), acc);
+              };
+              if (T > S && i == 1 && kk == 0 && j + cnt == S && first) {   // order S starts here
+                if (cnt > 1) mma(j, cnt - 1, 1u);
+                mma(S - 1, 1, 0u);
+              } else {
+                mma(j, cnt, (first && i == 0 && kk == 0) ? 0u : 1u);
+              }
             }
           tc::mma_commit(tc::smem_u32(&emptya[i]));
         }
@@ -226,7 +256,7 @@ k_split_gemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUt
     bool ok = true;
     for (int w = blockIdx.x; w < a.nwork && ok; w += gridDim.x) {
       const Item it = decode(w);
-      // orders 0..3 and 4..S-1 as 64-bit integers, in units of 256^-3 and 256^-(S-1)
+      // orders 0..3 and 4..T-1 as 64-bit integers, in units of 256^-3 and 256^-(T-1)
       long long hi[NC], lo[S > 4 ? NC : 1];
 #pragma unroll
       for (int i = 0; i < NC; ++i) {
@@ -254,24 +284,28 @@ k_split_gemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUt
                 hi[c0 + i] += (long long)__float2int_rn(__uint_as_float(r[t][i])) * (1 << (8 * (3 - t)));
             if (S > 4) {
 #pragma unroll
-              for (int t = 4; t < S; ++t) tc::tmem_ld8_nowait(tl + t * N + c0, r[t - 4]);
+              for (int t = 4; t < T; ++t) tc::tmem_ld8_nowait(tl + t * N + c0, r[t - 4]);
               tc::tmem_wait_ld();
 #pragma unroll
               for (int i = 0; i < 8; ++i)
 #pragma unroll
-                for (int t = 4; t < S; ++t)
-                  lo[c0 + i] += (long long)__float2int_rn(__uint_as_float(r[t - 4][i])) * (1 << (8 * (S - 1 - t)));
+                for (int t = 4; t < T; ++t)
+                  lo[c0 + i] += (long long)__float2int_rn(__uint_as_float(r[t - 4][i])) * (1 << (8 * (T - 1 - t)));
             }
           }
         }
         tc::fence_before_sync();
         if (lane == 0) tc::mbar_arrive(tc::smem_u32(acce));
       }
-      if (ok) {
+      if (T > S) {   // back to units of 256^-(S-1)
+#pragma unroll
+        for (int i = 0; i < NC; ++i) lo[i] = (lo[i] + 128) >> 8;
+      }
+      if (ok && it.nk > 0) {
         const int mr = it.m0 + g * 32 + lane;
-        const int ea = a.ea[mr];
+        const int ea = a.ea[mr + (MODE == PROJ ? it.b * a.rows_a : 0)];
         const int cb = it.n0 + part * NC;
-        const int* eb = a.eb + cb;
+        const int* eb = a.eb + cb + (MODE == PROJ ? it.b * a.rows_b : 0);
         // a rotation's sum (|hi| < 2^47) as one integer in units of 2^(ea + eb - 24 - sh): exact
         // where |hi| < 2^38 (or S = 4), else cut 2^-53 below its leading bit; rounded once
         auto value = [&](int i, int& sh) {
@@ -301,9 +335,20 @@ k_split_gemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUt
             }
           }
         } else {
+          int4 ch{};
+          int cols = 2 * a.n, c0 = cb;   // valid real columns, the thread's first
+          if (MODE == PROJ) {
+            ch = a.chunks[it.b];
+            cols = mr < 4 * a.n ? 2 * a.npj[ch.x] : 0;
+          }
+          if (MODE == EXPD) {
+            ch = a.chunks[it.b];
+            c0 = cb - it.b * a.ntn * N;
+            cols = mr - it.b * kNlRows < ch.z ? 4 * a.n : 0;
+          }
 #pragma unroll
           for (int i = 0; i < NC; i += 2) {
-            if (cb + i >= 2 * a.n) break;
+            if (c0 + i >= cols) break;
             double v[2];
 #pragma unroll
             for (int q = 0; q < 2; ++q) {
@@ -321,6 +366,20 @@ k_split_gemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUt
             if (MODE == ROT64) {
               if (mr < a.rows)
                 reinterpret_cast<double2*>(a.out)[(size_t)mr * a.ldo + (cb + i) / 2] = make_double2(v[0], v[1]);
+            } else if (MODE == PROJ) {
+              // conj(p) x: re = pr xr + pi xi, im = pr xi - pi xr; the row is one part of x
+              const int xc = mr >> 1, sp = xc >= a.n, vec = xc - sp * a.n;
+              double2* o = reinterpret_cast<double2*>(a.out) +
+                           (size_t)(a.c_off[ch.x] + 2 * ((c0 + i) >> 1) + sp) * a.n + vec;
+              atomicAdd(&o->x, (mr & 1) ? v[1] : v[0]);
+              atomicAdd(&o->y, (mr & 1) ? v[0] : -v[1]);
+            } else if (MODE == EXPD) {
+              const int yc = (c0 + i) >> 1, sp = yc >= a.n, vec = yc - sp * a.n;
+              const long long node = a.nodes[ch.w + ch.y + mr - it.b * kNlRows];
+              if (!GBC_IN_RANGE(GBC_SITE_NL_NODE, node, a.rows)) break;
+              double2* o = reinterpret_cast<double2*>(a.out) + (node * 2 + sp) * a.ldo + vec;
+              atomicAdd(&o->x, v[0]);
+              atomicAdd(&o->y, v[1]);
             } else {
               // conj(x) y of complex columns (mr / 2, (cb + i) / 2): re = rr + ii, im = ri - ir
               const int ci = mr >> 1, cj = (cb + i) >> 1;
@@ -583,6 +642,114 @@ k_split_cols(const cplx<T>* __restrict__ X, int ldx, int n, long long r0, long l
   }
 }
 
+// Columns of a chunk's rows -> digits [S][cols_pad][kp] (rows contiguous; the chunk's at b *
+// kNlRows, zeros up to a multiple of 128) and exponents [b][cols_pad], the maximum taken over
+// the chunk.  X: row j, column s nvec + v is X[(node_j 2 + s) ldx + v]; PTAB: rows of the atom's P
+// table.  The second pass over the rows finds them in L2.
+template <int S, bool PTAB>
+__global__ void __launch_bounds__(256)
+k_split_nodes(const double2* __restrict__ src, int ldx, int nvec, const int4* __restrict__ chunks,
+              const long long* __restrict__ nodes, const int* __restrict__ atom_npj,
+              const int* __restrict__ atom_pv_off, long long M, int cols_pad, int kp,
+              uint16_t* __restrict__ D, int* __restrict__ eu) {
+  __shared__ double xs[64][65];
+  __shared__ unsigned sk[2][8][32];
+  __shared__ int se[64];
+  const int b = blockIdx.x, cb = blockIdx.y * 32, l = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int4 ch = chunks[b];
+  const int npj = atom_npj[ch.x], c = cb + l;
+  const bool ok = c < (PTAB ? npj : 2 * nvec);
+  const int sp = !PTAB && c >= nvec;
+  const double2* base = PTAB ? src + atom_pv_off[ch.x] + (size_t)ch.y * npj + c
+                             : src + (size_t)sp * ldx + (c - sp * nvec);
+  const long long* nd = nodes + ch.w + ch.y;
+  auto at = [&](int j) {
+    if (!ok || j >= ch.z) return make_double2(0, 0);
+    if (PTAB) return base[(size_t)j * npj];
+    const long long node = nd[j];
+    return GBC_IN_RANGE(GBC_SITE_NL_NODE, node, M) ? base[node * 2 * ldx] : make_double2(0, 0);
+  };
+  unsigned kx = 0, ky = 0;
+#pragma unroll 4
+  for (int j = w; j < ch.z; j += 8) {
+    const double2 x = at(j);
+    kx = max(kx, mag_key(x.x));
+    ky = max(ky, mag_key(x.y));
+  }
+  sk[0][w][l] = kx;
+  sk[1][w][l] = ky;
+  __syncthreads();
+  if (threadIdx.x < 64) {   // real column 2 l' + part
+    unsigned k = 0;
+    for (int i = 0; i < 8; ++i) k = max(k, sk[threadIdx.x & 1][i][threadIdx.x >> 1]);
+    const int E = key_exponent<double>(k);
+    se[threadIdx.x] = E;
+    eu[(size_t)b * cols_pad + 2 * cb + threadIdx.x] = E == kBad ? kBad : E - 6;
+  }
+  const int cc = threadIdx.x >> 2, q = threadIdx.x & 3;   // real column, group of 16 rows
+  for (int rb = 0; rb < ch.z; rb += 128) {
+#pragma unroll 1
+    for (int h = 0; h < 128; h += 64) {
+      __syncthreads();
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const double2 x = at(rb + h + w + 8 * i);
+        xs[2 * l][w + 8 * i] = x.x;
+        xs[2 * l + 1][w + 8 * i] = x.y;
+      }
+      __syncthreads();
+      const int E = se[cc];
+      unsigned long long d[16];
+#pragma unroll
+      for (int i = 0; i < 16; ++i) d[i] = digits<S>(E == kBad ? 0 : to_fixed<S>(xs[cc][q * 16 + i], E));
+#pragma unroll
+      for (int s = 0; s < S; ++s) {
+        uint4* o = reinterpret_cast<uint4*>(
+            &D[((size_t)s * cols_pad + 2 * cb + cc) * kp + (size_t)b * kNlRows + rb + h + q * 16]);
+        o[0] = make_uint4(pack2<S>(d[0], d[1], s), pack2<S>(d[2], d[3], s), pack2<S>(d[4], d[5], s),
+                          pack2<S>(d[6], d[7], s));
+        o[1] = make_uint4(pack2<S>(d[8], d[9], s), pack2<S>(d[10], d[11], s), pack2<S>(d[12], d[13], s),
+                          pack2<S>(d[14], d[15], s));
+      }
+    }
+  }
+}
+
+// one warp per row of up to 32 complex values -> digits [S][rows][64] and exponents.  COEF: the
+// right factor of the expansion, row (chunk, real column (s, v, part)) of its atom's C'; else
+// rows of the chunks' P tables (zeros up to a multiple of 128 rows of a chunk)
+template <int S, bool COEF>
+__global__ void __launch_bounds__(256)
+k_split_proj(const double2* __restrict__ src, int nvec, int rows, int cols, const int4* __restrict__ chunks,
+             const int* __restrict__ atom_npj, const int* __restrict__ atom_off,
+             uint16_t* __restrict__ D, int* __restrict__ eu) {
+  const int lane = threadIdx.x & 31;
+  const int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (r >= rows) return;
+  double2 x = make_double2(0, 0);
+  if (COEF) {
+    const int atom = chunks[r / cols].x, rc = r % cols;   // cols: padded real columns
+    const int yc = rc >> 1, sp = yc >= nvec, v = yc - sp * nvec;
+    if (lane < atom_npj[atom] && rc < 4 * nvec) {
+      x = src[(size_t)(atom_off[atom] + 2 * lane + sp) * nvec + v];
+      x = (rc & 1) ? make_double2(x.y, x.x) : make_double2(x.x, -x.y);
+    }
+  } else {
+    const int4 ch = chunks[r / kNlRows];
+    const int i = r % kNlRows, npj = atom_npj[ch.x];
+    if (i >= (ch.z + 127) / 128 * 128) return;
+    if (i < ch.z && lane < npj) x = src[atom_off[ch.x] + (size_t)(ch.y + i) * npj + lane];
+  }
+  const unsigned key = __reduce_max_sync(0xffffffffu, max(mag_key(x.x), mag_key(x.y)));
+  const int E = key_exponent<double>(key);
+  if (lane == 0) eu[r] = E == kBad ? kBad : E - 6;
+  const unsigned long long a = digits<S>(E == kBad ? 0 : to_fixed<S>(x.x, E)),
+                           b = digits<S>(E == kBad ? 0 : to_fixed<S>(x.y, E));
+#pragma unroll
+  for (int s = 0; s < S; ++s)
+    *reinterpret_cast<unsigned*>(&D[((size_t)s * rows + r) * 64 + 2 * lane]) = pack2<S>(a, b, s);
+}
+
 inline int up(int x, int m) { return (x + m - 1) / m * m; }
 
 template <int S, int MODE>
@@ -603,6 +770,8 @@ cudaError_t run_split_gemm(const uint16_t* A, const uint16_t* B, int kpad, const
 // digit buffer of a chunk of rows: 884,736 x 256 CholGS 72 / 66 ms at 80 / 256 MB (fewer, longer
 // launches; that the digits stay in L2 at 80 MB does not make up for it)
 constexpr size_t kChunkBytes = size_t(512) << 20;
+constexpr size_t kNlBytes = size_t(256) << 20;   // the same of a batch of support chunks
+static_assert(GBC_MAX_NPJ <= 32, "a row of projectors is one 64-wide K chunk");
 
 }  // namespace
 
@@ -715,3 +884,73 @@ template gbc_status launch_gram_split<float, double>(gbc_ctx*, const float2*, in
                                                      const double*, long long, int, double2*, cudaStream_t);
 template gbc_status launch_gram_split<double, double>(gbc_ctx*, const double2*, int, const double2*, int,
                                                       const double*, long long, int, double2*, cudaStream_t);
+
+// FP64 projector contractions as split products, in batches of support chunks (at most kNlRows
+// nodes of one atom each).  Projection: C1 += P^H X over the chunk's nodes, exponents per chunk
+// and column; expansion: Y += P C2 over the atom's projectors, exponents per node and per column
+// of C2.  C1 is zero on entry; both add with FP64 atomics, as the direct kernels do.  The digits
+// live in work slot 14: nl_split_bytes, which does not shrink with nvec, or nothing is run.
+static size_t nl_split_chunk(int nvec, bool project) {
+  constexpr int S = 7;
+  const size_t cols = up(4 * nvec, project ? kTM : SplitCfg<S>::N);
+  return project ? (2 * S * (size_t)kNlRows + sizeof(int)) * (cols + 64)
+                 : (2 * S * 64 + sizeof(int)) * (kNlRows + cols);
+}
+static int nl_split_batch(const gbc_ctx* c, size_t per) {
+  return (int)std::min<size_t>(c->proj.nchunks, std::max<size_t>(1, kNlBytes / per));
+}
+size_t nl_split_bytes(const gbc_ctx* c, int nvec) {
+  const size_t per = std::max(nl_split_chunk(nvec, true), nl_split_chunk(nvec, false));
+  return std::min(per * c->proj.nchunks, std::max(per, kNlBytes));
+}
+
+cudaError_t nl_split_project(gbc_ctx* c, const double2* X, int nvec, int ldx, double2* C1, cudaStream_t s) {
+  constexpr int S = 7;
+  const ProjDev& pj = c->proj;
+  const int cols = up(4 * nvec, kTM), nb = nl_split_batch(c, nl_split_chunk(nvec, true));
+  for (int b0 = 0; b0 < pj.nchunks; b0 += nb) {
+    const int n = std::min(nb, pj.nchunks - b0), kp = n * kNlRows;
+    uint16_t* A = (uint16_t*)c->work[14];
+    uint16_t* B = A + (size_t)S * kp * cols;
+    int* ea = (int*)(B + (size_t)S * kp * 64);
+    int* eb = ea + (size_t)n * cols;
+    const int4* ch = pj.d_chunks + b0;
+    // (rows of A past the last 64 columns stay as they are: nothing of theirs is used)
+    k_split_nodes<S, false><<<dim3(n, up(4 * nvec, 64) / 64), 256, 0, s>>>(
+        X, ldx, nvec, ch, pj.d_nodes, pj.d_atom_npj, pj.d_atom_pv_off, c->mesh.M, cols, kp, A, ea);
+    k_split_nodes<S, true><<<dim3(n, 1), 256, 0, s>>>(pj.d_P64, 0, 0, ch, pj.d_nodes, pj.d_atom_npj,
+                                                      pj.d_atom_pv_off, c->mesh.M, 64, kp, B, eb);
+    const int ntm = cols / kTM;
+    SplitArgs a{cols, 64, 0, 0, ntm, n * ntm, n * ntm, ea, eb, 0, nvec, 0, C1, ch, pj.d_nodes,
+                pj.d_atom_npj, pj.d_atom_c_off};
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) e = run_split_gemm<S, PROJ>(A, B, kp, a, s);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+cudaError_t nl_split_expand(gbc_ctx* c, double2* Y, int nvec, int ldx, const double2* C2, cudaStream_t s) {
+  constexpr int S = 7;
+  const ProjDev& pj = c->proj;
+  const int cols = up(4 * nvec, SplitCfg<S>::N), nb = nl_split_batch(c, nl_split_chunk(nvec, false));
+  for (int b0 = 0; b0 < pj.nchunks; b0 += nb) {
+    const int n = std::min(nb, pj.nchunks - b0), ra = n * kNlRows, rb = n * cols;
+    uint16_t* A = (uint16_t*)c->work[14];
+    uint16_t* B = A + (size_t)S * ra * 64;
+    int* ea = (int*)(B + (size_t)S * rb * 64);
+    int* eb = ea + ra;
+    const int4* ch = pj.d_chunks + b0;
+    k_split_proj<S, false><<<ra / 8, 256, 0, s>>>(pj.d_P64, nvec, ra, 0, ch, pj.d_atom_npj,
+                                                  pj.d_atom_pv_off, A, ea);
+    k_split_proj<S, true><<<rb / 8, 256, 0, s>>>(C2, nvec, rb, cols, ch, pj.d_atom_npj,
+                                                 pj.d_atom_c_off, B, eb);
+    const int ntn = cols / SplitCfg<S>::N, tiles = ra / kTM * ntn;
+    SplitArgs a{ra, rb, 1, 1, ntn, tiles, tiles, ea, eb, c->mesh.M, nvec, ldx, Y, ch, pj.d_nodes,
+                pj.d_atom_npj, pj.d_atom_c_off};
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) e = run_split_gemm<S, EXPD>(A, B, 64, a, s);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}

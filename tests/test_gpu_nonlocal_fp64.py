@@ -43,3 +43,42 @@ def test_fp64_nonlocal_tiles(g, npj, nvec, ldx):
         ctx.sync_status()
         got = Y[:, :, :nvec].cpu().numpy()
         assert np.linalg.norm(got - ref) <= 1e-12 * np.linalg.norm(ref)
+
+
+# larger contractions run as split products: column tiles of 32 and 16 vectors with remainders,
+# projector counts up to the largest, supports of several node chunks, several batches of chunks
+# (512 vectors: 8 chunks a batch).  Each size lies past the crossover with the direct kernels.
+@pytest.mark.parametrize("npj,nvec,ldx,k", [(32, 16, 16, 0.1), (18, 33, 40, 0.1), (9, 65, 65, -0.2), (18, 65, 66, 0.0),
+                                            (18, 512, 512, 0.1), (18, 512, 512, 0.0)])
+def test_fp64_nonlocal_split_products(g, npj, nvec, ldx, k):
+    chan = {9: (D, P, S), 18: syn.SPD_CHANNELS, 32: CHANNELS[27] + (D,)}[npj]
+    big = nvec < 100
+    prob = syn.make_problem(ncell=(5, 5, 4) if big else (4, 3, 3), h=(1.0, 1.1, 0.9), p=4 if big else 3,
+                            periodic=(1, 1, 0), k=(k, -2 * k, 0.0), natoms=4 if big else 10,
+                            rc=2.5 if big else 1.2, seed=npj, channels=chan)
+    assert prob.atoms[0].npj == npj
+    X = syn.random_block(prob.nnodes, nvec, 3)
+    X *= np.logspace(-8, 8, nvec)                    # columns of very different size
+    ref = fe.Discretisation(prob).apply_h(X)
+    Xd = torch.zeros((prob.nnodes, 2, ldx), dtype=torch.complex128, device="cuda")
+    Xd[:, :, :nvec] = torch.from_numpy(X).cuda()
+    ctx = g.Context(0)
+    ctx.set_problem(prob)
+    Y = torch.empty_like(Xd)
+    ctx.apply_h(Xd, Y, nvec=nvec)
+    ctx.sync_status()
+    got = Y[:, :, :nvec].cpu().numpy()
+    err = np.linalg.norm(got - ref, axis=(0, 1))
+    assert (err <= 1e-12 * np.linalg.norm(ref, axis=(0, 1))).all()
+    if not big:
+        return
+    # a NaN and an infinity reach their own columns only
+    Xd[prob.nnodes // 2, 0, 1] = float("nan")
+    Xd[prob.nnodes // 2, 1, 4] = float("inf")
+    ctx.apply_h(Xd, Y, nvec=nvec)
+    ctx.sync_status()
+    again = Y[:, :, :nvec].cpu().numpy()
+    assert set(np.flatnonzero(~np.isfinite(again).all(axis=(0, 1)))) == {1, 4}
+    rest = [v for v in range(nvec) if v not in (1, 4)]
+    again = again[:, :, rest]
+    assert np.linalg.norm(again - ref[:, :, rest]) <= 1e-12 * np.linalg.norm(ref[:, :, rest])
