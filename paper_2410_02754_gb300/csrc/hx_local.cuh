@@ -168,9 +168,12 @@ template <int NP, int VB> __host__ __device__ constexpr int cell_vpoints() {
 // Threads of a group: about one per pencil of a vector's x stage.  At p = 3 and 4 small
 // groups are worth more than full rounds (12^3 cells, p = 4, 96 vectors: 446 us a launch at
 // 128 threads, 642 at 256).
+// At p = 7 two groups of 128 threads and 2 vectors each are 115 KB of shared memory, one CTA per SM;
+// one group of 256 lets two CTAs in (11 x 9 x 8 cells, degree-6 filter without atoms: 150 vectors 15.10
+// -> 13.26 ms at k = 0, 14.79 -> 13.83 at k != 0; 3 vectors 0.46 -> 0.43 and 0.50 -> 0.46).
 template <int NP, int VB> __host__ __device__ constexpr int cell_group_threads() {
   constexpr int g4[9] = {0, 0, 0, 64, 128, 128, 256, 256, 256};
-  constexpr int g2[9] = {0, 0, 0, 32, 64, 64, 128, 128, 128};
+  constexpr int g2[9] = {0, 0, 0, 32, 64, 64, 128, 128, 256};
   return VB == 4 ? g4[NP] : g2[NP];
 }
 // Whether each warp owns whole z planes of a cell (see cell_body): where a plane's pencils
