@@ -53,7 +53,7 @@ typedef enum {
 typedef enum {
   GBC_FP64 = 0,          /* complex128 blocks, FP64 arithmetic everywhere               */
   GBC_FP32 = 1,          /* complex64 blocks, FP32 arithmetic in H.X and the filter;
-                            Gram matrices accumulated in FP64                           */
+                            Gram matrices to FP64 accuracy                              */
   GBC_TF32 = 2,          /* reserved: cell apply on the TF32 tensor cores (not built;
                             gbc_set_precision returns GBC_EUNSUPPORTED)                 */
   GBC_BF16X3 = 3         /* reserved: cell apply in split BF16 on the tensor cores (not
@@ -182,14 +182,14 @@ gbc_status gbc_filter(gbc_ctx* ctx, void* X, int nvec, int ldx, int degree, doub
 gbc_status gbc_filter_residual(gbc_ctx* ctx, void* X, int nvec, int ldx, int degree, double lT,
                                double lmax, double lmin, const double* ritz, void* stream);
 
-/* Cholesky-Gram-Schmidt in the M_D inner product: S = X^H M_D X accumulated in
- * FP64, S = L L^H, X <- X L^-H.  GBC_ENOTPD if S is not positive definite
+/* Cholesky-Gram-Schmidt in the M_D inner product: S = X^H M_D X to FP64
+ * accuracy, S = L L^H, X <- X L^-H.  GBC_ENOTPD if S is not positive definite
  * (X is then left unchanged).  Synchronous (reads the pivot status).
  * nvec <= 512. */
 gbc_status gbc_cholgs(gbc_ctx* ctx, void* X, int nvec, int ldx, void* stream);
 
 /* Rayleigh-Ritz for an M_D-orthonormal block (Sec. III.B.2): Hp = X^H H X
- * accumulated in FP64, Hp Q = Q Lambda by a Jacobi eigensolver on the device,
+ * to FP64 accuracy, Hp Q = Q Lambda by a Jacobi eigensolver on the device,
  * X <- X Q.  ritz: host array of nvec doubles, ascending.  Synchronous.
  * nvec <= 512.  GBC_ETIMEOUT if the eigensolver hits its sweep cap. */
 gbc_status gbc_rayleigh_ritz(gbc_ctx* ctx, void* X, int nvec, int ldx, double* ritz,
@@ -456,7 +456,7 @@ enum {
   GBC_FAM_HX_LOCAL = 0,   /* cell-level local apply + assembly            */
   GBC_FAM_NONLOCAL = 1,   /* C = P^H X, C' = Delta C, Y += P C'            */
   GBC_FAM_CHEB = 2,       /* fused Chebyshev recurrence epilogue           */
-  GBC_FAM_GRAM = 3,       /* FP64-accumulated Gram matrices                */
+  GBC_FAM_GRAM = 3,       /* FP64-accurate Gram matrices                   */
   GBC_FAM_ROTATE = 4,     /* block rotation X <- X Q                       */
   GBC_FAM_DENSE = 5       /* small dense Cholesky / eigensolver            */
 };

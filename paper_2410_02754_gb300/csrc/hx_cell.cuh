@@ -41,7 +41,8 @@
 // warp instructions per cell and vector pair.  The steps: five stages and 16-byte two-spin
 // pencils 9.29, index work once per pencil 9.07, items decoded once and fields staged 8.34,
 // planes owned by warps 7.62.  Other sizes: 12^3 cells, p = 5, 96 vectors 1144 -> 815 us;
-// p = 4 812 -> 460; 10^3 cells, p = 3, 128 vectors 460 -> 212; p = 7, 64 vectors 1167 -> 1048.
+// p = 4 812 -> 460; 10^3 cells, p = 3, 128 vectors 460 -> 212; p = 7, 64 vectors 1167 -> 1048
+// (at 3 or 7 vectors the partly filled last item leaves it up to 12% behind the seven-stage form).
 //
 // Assembly modes (per system):
 //  * accumulate: Y += H^loc X with FP32 atomics on every node;

@@ -5,7 +5,8 @@
 // done as three batched small contractions on the atom-support node lists:
 //   C   = P_a^H X        (per atom: npj x 2 x nvec, reduction over the support)
 //   C'  = Delta_a C      (2npj x 2npj times 2npj x nvec)
-//   Y  += P_a C'         (FP64: atom by atom with atomics; deterministic mode and the
+//   Y  += P_a C'         (FP64: atom by atom with atomics, both contractions as split
+//                         products where they are large (split_gemm.cu); deterministic mode and the
 //                         FP32 SIMT engine: node-centric, every support node sums its
 //                         atoms' terms, a plain read-modify-write of Y)
 // P_a is the node-based projector table (one row per distinct free node of the
