@@ -889,7 +889,14 @@ template gbc_status launch_gram_split<double, double>(gbc_ctx*, const double2*, 
 // nodes of one atom each).  Projection: C1 += P^H X over the chunk's nodes, exponents per chunk
 // and column; expansion: Y += P C2 over the atom's projectors, exponents per node and per column
 // of C2.  C1 is zero on entry; both add with FP64 atomics, as the direct kernels do.  The digits
-// live in work slot 14: nl_split_bytes, which does not shrink with nvec, or nothing is run.
+// live in work slot 14: nl_split_bytes, which does not shrink with nvec as long as it is used.
+// Batches keep the workspace bounded; within one the chunks are independent tiles.  Measured per
+// launch at 58 chunks x 64 vectors x 18 projectors: splitting X 0.17 ms and P 0.10 ms (latency of a
+// CTA's walk over its chunk), projection products 0.086 ms (tensor pipe 43%); the direct kernels
+// run both contractions at the FP64 rate.  Error against 80-bit and wider sums, relative to the
+// result: 1.58e-15 (direct 1.63e-15) at 6,300-node supports and 33 vectors, 2.07e-15 (2.06e-15) at
+// 17,000 nodes.  One order less (as in the Gram products) measured up to 1.17 times the direct
+// kernels' error.
 static size_t nl_split_chunk(int nvec, bool project) {
   constexpr int S = 7;
   const size_t cols = up(4 * nvec, project ? kTM : SplitCfg<S>::N);
