@@ -76,11 +76,6 @@ struct SplitArgs {
   const int *npj, *c_off;
 };
 
-// 2^e as a double (|e| < 1000)
-__device__ __forceinline__ double pow2d(int e) {
-  return __hiloint2double((1023 + max(-1000, min(1000, e))) << 20, 0);
-}
-
 // Persistent: CTAs take work items blockIdx.x, + gridDim.x, ...; the roles run on across items.
 template <int S, int MODE>
 __global__ void __launch_bounds__(kSplitThreads, 1)
@@ -354,7 +349,7 @@ k_split_gemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUt
             for (int q = 0; q < 2; ++q) {
               int sh = 0;
               if (MODE == GRAM)   // hi may use all of its 53 bits here: hi + 2^-24 lo, rounded once
-                v[q] = fma(__ll2double_rn(lo[S > 4 ? i + q : 0]), pow2d(-24), __ll2double_rn(hi[i + q]));
+                v[q] = fma(__ll2double_rn(lo[S > 4 ? i + q : 0]), 0x1p-24, __ll2double_rn(hi[i + q]));
               else
                 v[q] = __ll2double_rn(value(i + q, sh));
               const int e = eb[i + q], x = ea + e - 24 - sh;
@@ -436,7 +431,7 @@ template <int S, typename T> __device__ __forceinline__ long long to_fixed(T x, 
     sh = max(ex, 1) - 1075;
   }
   sh += 6 + 8 * (S - 1) - E;
-  if (sh >= 0) m <<= min(sh, 40);
+  if (sh >= 0) m = sh > 30 ? 0 : m << sh;   // more only for a subnormal that the exponent left out
   else m = sh < -60 ? 0 : (m + (1LL << (-sh - 1))) >> -sh;
   return neg ? -m : m;
 }
@@ -453,8 +448,18 @@ __device__ __forceinline__ unsigned pack2(unsigned long long a, unsigned long lo
   return __byte_perm(__float_as_uint(fa), __float_as_uint(fb), 0x7632);
 }
 
+// exponent of the larger part of a complex value that counts 2^c: kNone for zero, kBad for an
+// infinity or a NaN
+constexpr int kNone = -(1 << 30);
+template <typename T, typename V> __device__ __forceinline__ int scaled_exponent(V x, int c) {
+  const unsigned k = max(mag_key(x.x), mag_key(x.y));
+  const int e = key_exponent<T>(k);
+  return k == 0 ? kNone : e == kBad ? kBad : e + c;
+}
+
 // rows of a block (2n reals each) -> digits [S][rows_pad][kp] and unit exponents, one warp per
-// row; rows >= rows are written as zeros.  cs: exponents that multiply the columns (or null).
+// row; rows >= rows are written as zeros.  cs: exponents that multiply the columns (or null).  They
+// are added to the exponents and never multiplied in: they may be larger than the type's range.
 template <int S, typename T>
 __global__ void __launch_bounds__(256)
 k_split_rows(const cplx<T>* __restrict__ X, int ldx, int n, long long rows, int rows_pad, int kp,
@@ -464,7 +469,7 @@ k_split_rows(const cplx<T>* __restrict__ X, int ldx, int n, long long rows, int 
   if (r >= rows_pad) return;
   constexpr int IT = 512 / 64;                 // n <= 512: 64 complex columns per iteration
   T v[IT][4];
-  unsigned key = 0;
+  int E = kNone;
 #pragma unroll
   for (int i = 0; i < IT; ++i) {
     if (i * 128 >= kp) break;
@@ -472,21 +477,14 @@ k_split_rows(const cplx<T>* __restrict__ X, int ldx, int n, long long rows, int 
     for (int q = 0; q < 2; ++q) {
       const int c = i * 64 + 2 * lane + q;
       cplx<T> x = cmake<cplx<T>>(0, 0);
-      if (r < rows && c < n) {
-        x = X[r * ldx + c];
-        if (cs) {
-          const T f = (T)pow2d(cs[c]);
-          x.x *= f;
-          x.y *= f;
-        }
-      }
+      if (r < rows && c < n) x = X[r * ldx + c];
       v[i][2 * q] = x.x;
       v[i][2 * q + 1] = x.y;
-      key = max(key, max(mag_key(x.x), mag_key(x.y)));
+      E = max(E, scaled_exponent<T>(x, cs && c < n ? cs[c] : 0));
     }
   }
-  key = __reduce_max_sync(0xffffffffu, key);
-  const int E = key_exponent<T>(key);
+  E = __reduce_max_sync(0xffffffffu, E);
+  if (E == kNone) E = 0;
   if (lane == 0) eu[r] = E == kBad ? kBad : E - 6;
 #pragma unroll
   for (int i = 0; i < IT; ++i) {
@@ -495,7 +493,10 @@ k_split_rows(const cplx<T>* __restrict__ X, int ldx, int n, long long rows, int 
     if (k >= kp) continue;
     unsigned long long d[4];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) d[q] = digits<S>(E == kBad ? 0 : to_fixed<S>(v[i][q], E));
+    for (int q = 0; q < 4; ++q) {
+      const int c = i * 64 + 2 * lane + q / 2;
+      d[q] = digits<S>(E == kBad ? 0 : to_fixed<S>(v[i][q], E - (cs && c < n ? cs[c] : 0)));
+    }
 #pragma unroll
     for (int s = 0; s < S; ++s)
       *reinterpret_cast<uint2*>(&D[((size_t)s * rows_pad + r) * kp + k]) =
@@ -515,47 +516,40 @@ k_split_q(const double2* __restrict__ Q, int n, int rows_pad, int kp, const int*
   const int j = r >> 1, part = r & 1;
   auto at = [&](int i) {   // (factor of x_i.re, factor of x_i.im) in output part ``part``
     if (j >= n || i >= n) return make_double2(0, 0);
-    double2 q = Q[(size_t)i * n + j];
-    if (cs) {
-      const double f = pow2d(-cs[i]);
-      q.x *= f;
-      q.y *= f;
-    }
+    const double2 q = Q[(size_t)i * n + j];
     return part ? make_double2(q.y, q.x) : make_double2(q.x, -q.y);
   };
-  unsigned key = 0;
-  for (int i = lane; i < n; i += 32) {
-    const double2 q = at(i);
-    key = max(key, max(mag_key(q.x), mag_key(q.y)));
-  }
-  key = __reduce_max_sync(0xffffffffu, key);
-  const int E = key_exponent<double>(key);
+  int E = kNone;
+  for (int i = lane; i < n; i += 32) E = max(E, scaled_exponent<double>(at(i), cs ? -cs[i] : 0));
+  E = __reduce_max_sync(0xffffffffu, E);
+  if (E == kNone) E = 0;
   if (lane == 0) eu[r] = E == kBad ? kBad : E - 6;
   for (int i = lane; 2 * i < kp; i += 32) {
     const double2 q = at(i);
-    const unsigned long long a = digits<S>(E == kBad ? 0 : to_fixed<S>(q.x, E)),
-                             b = digits<S>(E == kBad ? 0 : to_fixed<S>(q.y, E));
+    const int Ei = cs && i < n && E != kBad ? E + cs[i] : E;
+    const unsigned long long a = digits<S>(E == kBad ? 0 : to_fixed<S>(q.x, Ei)),
+                             b = digits<S>(E == kBad ? 0 : to_fixed<S>(q.y, Ei));
 #pragma unroll
     for (int s = 0; s < S; ++s)
       *reinterpret_cast<unsigned*>(&D[((size_t)s * rows_pad + r) * kp + 2 * i]) = pack2<S>(a, b, s);
   }
 }
 
-// exponents that bring the columns to a common size: 2^cs[i] ~ max_j sqrt(S_jj) / sqrt(S_ii)
+// exponents that bring the columns to a common size: 2^cs[i] ~ max_j sqrt(S_jj) / sqrt(S_ii), over
+// the whole exponent range (a column that fell behind the common size would keep fewer digits)
 __global__ void k_col_scale(const double2* __restrict__ diag, int n, int* __restrict__ cs) {
   __shared__ int big;
-  if (threadIdx.x == 0) big = -100000;
+  if (threadIdx.x == 0) big = kNone;
   __syncthreads();
   auto half_exp = [&](int i) {   // exponent of the norm; a column that is zero or not finite: none
-    const unsigned k = mag_key(diag[i].x);
-    const int e = (int)(k >> 20);
-    return (e == 0 || e == 0x7ff) ? -100000 : (e - 1023) / 2;
+    const double d = diag[i].x;
+    return d > 0.0 && isfinite(d) ? ilogb(d) >> 1 : kNone;
   };
   for (int i = threadIdx.x; i < n; i += blockDim.x) atomicMax(&big, half_exp(i));
   __syncthreads();
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
     const int e = half_exp(i);
-    cs[i] = e == -100000 ? 0 : min(60, big - e);
+    cs[i] = e == kNone ? 0 : big - e;
   }
 }
 

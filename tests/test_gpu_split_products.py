@@ -66,6 +66,29 @@ def test_cholgs_tiles(g, prec, n, ldx):
     ctx.close()
 
 
+@pytest.mark.parametrize("prec,n", [(0, 16), (0, 65), (1, 65), (1, 130)])
+def test_cholgs_columns_of_any_size(g, prec, n):
+    """Column sizes over the type's range: CholGS does not depend on a column's size, so the same
+    block with its columns at 1, 2^-66, 2^-116 and 2^-200 (FP32: 2^-98, about 1e-30) of themselves
+    gives the same orthonormal block."""
+    ctx, prob = context(g, prec)
+    M = prob.nnodes
+    X = device(block(M, n, 3), prec, n).cpu().numpy().astype(np.complex128)
+    md = np.repeat(ctx.mass(), 2)[:, None]
+    f = X.reshape(2 * M, n)
+    L = np.linalg.cholesky(f.conj().T @ (md * f))
+    ref = np.linalg.solve(L.conj(), f.T).T
+    shift = np.array([0, -66, -116, -200] if prec == 0 else [0, -66, -98])
+    Xd = device(X * np.exp2(shift[np.arange(n) * 7 % len(shift)].astype(float)), prec, n)
+    ctx.cholgs(Xd)
+    Y = Xd.cpu().numpy().astype(np.complex128).reshape(2 * M, n)
+    if prec == 0:
+        assert np.abs(Y.conj().T @ (md * Y) - np.eye(n)).max() < 1e-12
+    err = np.linalg.norm(Y - ref, axis=0) / np.linalg.norm(ref, axis=0)
+    assert err.max() < (1e-12 if prec == 0 else 2.0 ** -23)
+    ctx.close()
+
+
 @pytest.mark.parametrize("prec", [0, 1])
 @pytest.mark.parametrize("n", [16, 63, 130])
 def test_rayleigh_ritz_tiles(g, prec, n):
