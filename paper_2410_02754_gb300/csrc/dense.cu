@@ -42,9 +42,11 @@ __global__ void k_chol_col(double2* A, double2* L, int n, int j, int* flag) {
     return;
   }
   const double2 aij = A[(size_t)i * n + j], akj = A[(size_t)k * n + j];
-  // aij * conj(akj) / d
-  const double re = (aij.x * akj.x + aij.y * akj.y) / d;
-  const double im = (aij.y * akj.x - aij.x * akj.y) / d;
+  // aij conj(akj / d): the quotient first, whose size is that of column k over column j (the product
+  // of the two entries leaves the range for columns 2^-256 of the largest)
+  const double kx = akj.x / d, ky = akj.y / d;
+  const double re = aij.x * kx + aij.y * ky;
+  const double im = aij.y * kx - aij.x * ky;
   double2* a = &A[(size_t)i * n + k];
   a->x -= re;
   a->y -= im;

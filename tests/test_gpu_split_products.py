@@ -69,7 +69,7 @@ def test_cholgs_tiles(g, prec, n, ldx):
 @pytest.mark.parametrize("prec,n", [(0, 16), (0, 65), (1, 65), (1, 130)])
 def test_cholgs_columns_of_any_size(g, prec, n):
     """Column sizes over the type's range: CholGS does not depend on a column's size, so the same
-    block with its columns at 1, 2^-66, 2^-116 and 2^-200 (FP32: 2^-98, about 1e-30) of themselves
+    block with its columns at 1, 2^-66, 2^-116 and 2^-332 (FP32: 2^-98, about 1e-30) of themselves
     gives the same orthonormal block."""
     ctx, prob = context(g, prec)
     M = prob.nnodes
@@ -78,7 +78,7 @@ def test_cholgs_columns_of_any_size(g, prec, n):
     f = X.reshape(2 * M, n)
     L = np.linalg.cholesky(f.conj().T @ (md * f))
     ref = np.linalg.solve(L.conj(), f.T).T
-    shift = np.array([0, -66, -116, -200] if prec == 0 else [0, -66, -98])
+    shift = np.array([0, -66, -116, -332] if prec == 0 else [0, -66, -98])
     Xd = device(X * np.exp2(shift[np.arange(n) * 7 % len(shift)].astype(float)), prec, n)
     ctx.cholgs(Xd)
     Y = Xd.cpu().numpy().astype(np.complex128).reshape(2 * M, n)
