@@ -13,18 +13,20 @@
 // row and per column of Q for a rotation, per column of the block (over all rows) for a Gram
 // matrix.  A row with an infinity or a NaN is marked and gives NaN, as in FP arithmetic.
 //
-//  * rotation of an orthonormal FP32 block by a unitary matrix (Rayleigh-Ritz): S = 4 (30 bits
-//    below the row's largest entry, an error of at most sqrt(n) 2^-33 of a column's norm), 10
-//    digit products, rounded to FP32 once;
-//  * everything else (Gram matrices, FP64 blocks, the triangular rotation of CholGS, whose
-//    terms can cancel; its columns are first brought to a common size by powers of two):
-//    S = 7 (54 bits), 28 digit products.
+// S = 7 digits: an entry is off by at most 2^-55 of its row's largest.  FP32 blocks are rounded to
+// FP32 once.  The rotation of CholGS, whose terms can cancel, takes its columns at a common size, by
+// powers of two; that of Rayleigh-Ritz rests on an M_D-orthonormal block, whose columns have one size.
+// Orders t <= T - 1 are summed.  What is left out of a sum over K terms is about sqrt(K) 2^-54 of
+// the largest entries' product at T = S, sqrt(K) 2^-62 at T = S + 1: the latter where a sum is
+// small against them, as in the rotation of a nearly converged block (Q close to the identity).  With
+// S = 4 = T (30 bits) such FP32 columns came out 6.2e-8 off at n = 256, with S = 7 the 2.5e-8 of
+// their rounding to FP32; 200 columns of 432,000 rows take 3.5 ms more for it.
 //
 // GB300's FP64 pipe gives 1.05 TFLOP/s and float-float arithmetic on the FP32 pipes about 6;
 // 28 BF16 products at 1.9 PFLOP/s are an FP64-accurate 68 TFLOP/s.  Measured, 884,736 nodes x 256
 // FP32 columns: Gram 122 -> 21 ms (16 of them the products, 43% of the tensor pipe), rotation
-// 163 -> 26 ms (23 the products); 373,248 nodes x 256 in FP64: 333 -> 13 and 527 -> 14 ms.  Per tile (128 x 128 for
-// S = 4, 128 x 64 for S = 7) every order has its own accumulator in tensor memory and all S
+// 163 -> 26 ms (23 the products); 373,248 nodes x 256 in FP64: 333 -> 13 and 527 -> 14 ms.  Per tile
+// (128 x 64) every order has its own accumulator in tensor memory and all S
 // digit slices of a 64-wide K chunk are in shared memory at once (one TMA box each), so a
 // slice is loaded once per tile and used in up to S products.  Step i multiplies A_i with all
 // of B_0 .. B_{S-1-i} in instructions of up to 256 columns (one product per instruction, 64
@@ -46,15 +48,13 @@ constexpr int kKC = 64;               // K chunk: one 128-byte swizzled row
 constexpr int kBad = 0x7fffffff;      // exponent of a row with an infinity or a NaN
 constexpr int kEpi = 16;              // read-out warps
 constexpr int kSplitThreads = 64 + 32 * kEpi;
-template <int S> struct SplitCfg {
-  static constexpr int N = S <= 4 ? 128 : 64;             // tile columns
-  static constexpr int FLUSH = S <= 4 ? 4 : 2;            // K chunks between read-outs
-  static constexpr int ABYTES = kTM * 128, BBYTES = N * 128;
-  static constexpr size_t SMEM = 1024 + (size_t)S * (ABYTES + 2 * BBYTES) + 256;
-  static_assert(S * N <= 512, "tensor memory columns");
-  static_assert((long long)S * FLUSH * kKC << 14 <= 1LL << 24, "exact accumulation");
-  static_assert(SMEM <= 227 * 1024, "shared memory");
-};
+constexpr int S = 7;                  // digits
+constexpr int kTN = 64;               // tile columns
+constexpr int kFlush = 2;             // K chunks between read-outs
+constexpr int kABytes = kTM * 128, kBBytes = kTN * 128;
+constexpr size_t kSplitSmem = 1024 + (size_t)S * (kABytes + 2 * kBBytes) + 256;
+static_assert((long long)S * kFlush * kKC << 14 <= 1LL << 24, "exact accumulation");
+static_assert(kSplitSmem <= 227 * 1024, "shared memory");
 
 // PROJ, EXPD: the FP64 projector contractions C += P^H X and Y += P C' (see nl_split_project)
 enum { ROT32 = 0, ROT64 = 1, GRAM = 2, PROJ = 3, EXPD = 4 };
@@ -77,15 +77,13 @@ struct SplitArgs {
 };
 
 // Persistent: CTAs take work items blockIdx.x, + gridDim.x, ...; the roles run on across items.
-template <int S, int MODE>
+template <int MODE>
 __global__ void __launch_bounds__(kSplitThreads, 1)
 k_split_gemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb,
              const SplitArgs a) {
-  using G = SplitCfg<S>;
-  constexpr int N = G::N;
-  // orders kept: the nonlocal contractions keep one more (order S: digits 1 .. S-1 only), since
-  // projectors are far below their largest value on most of their support
-  constexpr int T = MODE == PROJ || MODE == EXPD ? S + 1 : S;
+  constexpr int N = kTN;
+  // orders summed; order S: digits 1 .. S-1 only
+  constexpr int T = MODE == GRAM ? S : S + 1;
   static_assert(T * N <= 512 && T <= 8, "tensor memory columns");
   struct Item { int m0, n0, k0, nk, b; };   // b: chunk of the batch
   auto decode = [&](int w) {
@@ -122,7 +120,7 @@ k_split_gemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUt
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* st = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-  uint64_t* fulla = reinterpret_cast<uint64_t*>(st + S * (G::ABYTES + 2 * G::BBYTES));   // [S]
+  uint64_t* fulla = reinterpret_cast<uint64_t*>(st + S * (kABytes + 2 * kBBytes));   // [S]
   uint64_t* emptya = fulla + S;                                                          // [S]
   uint64_t* fullb = emptya + S;                                                          // [2]
   uint64_t* emptyb = fullb + 2;                                                          // [2]
@@ -133,9 +131,9 @@ k_split_gemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUt
   int* fail = reinterpret_cast<int*>(tslot + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // A: one buffer per digit slice; B: two buffers of all slices back to back
-  auto A = [&](int s) { return tc::smem_u32(st + s * G::ABYTES); };
+  auto A = [&](int s) { return tc::smem_u32(st + s * kABytes); };
   auto B = [&](int buf, int s) {
-    return tc::smem_u32(st + S * G::ABYTES + (buf * S + s) * G::BBYTES);
+    return tc::smem_u32(st + S * kABytes + (buf * S + s) * kBBytes);
   };
   auto failed = [&]() { return *reinterpret_cast<volatile int*>(fail) != 0; };
 
@@ -176,7 +174,7 @@ k_split_gemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUt
         if (q > 1 && !tc::mbar_wait_bounded(tc::smem_u32(&emptyb[buf]), (q / 2 - 1) & 1)) atomicExch(fail, 1);
         if (failed()) break;
         const uint32_t fb = tc::smem_u32(&fullb[buf]);
-        tc::mbar_arrive_expect_tx(fb, S * G::BBYTES);
+        tc::mbar_arrive_expect_tx(fb, S * kBBytes);
 #pragma unroll
         for (int s = 0; s < S; ++s) tc::tma_load_2d(B(buf, s), &tb, x, s * a.rows_b + it.n0, fb);
         ib = q + 1;
@@ -185,7 +183,7 @@ k_split_gemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUt
           if (q > 0 && !tc::mbar_wait_bounded(tc::smem_u32(&emptya[s]), (q - 1) & 1)) atomicExch(fail, 1);
           if (failed()) break;
           const uint32_t fa = tc::smem_u32(&fulla[s]);
-          tc::mbar_arrive_expect_tx(fa, G::ABYTES);
+          tc::mbar_arrive_expect_tx(fa, kABytes);
           tc::tma_load_2d(A(s), &ta, x, s * a.rows_a + it.m0, fa);
           ia[s] = q + 1;
         }
@@ -203,7 +201,7 @@ k_split_gemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUt
     for (int w = blockIdx.x; w < a.nwork && !failed(); w += gridDim.x) {
       const Item it = decode(w);
       for (int c = 0; c < it.nk && !failed(); ++c, ++q) {
-        const bool first = c % G::FLUSH == 0;
+        const bool first = c % kFlush == 0;
         if (first && win > 0 && !tc::mbar_wait_bounded(tc::smem_u32(acce), (win - 1) & 1)) atomicExch(fail, 1);
         const int buf = q & 1;
         if (!tc::mbar_wait_bounded(tc::smem_u32(&fullb[buf]), (q / 2) & 1)) atomicExch(fail, 1);
@@ -234,7 +232,7 @@ k_split_gemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUt
           tc::mma_commit(tc::smem_u32(&emptya[i]));
         }
         tc::mma_commit(tc::smem_u32(&emptyb[buf]));
-        if ((c + 1) % G::FLUSH == 0 || c + 1 == it.nk) {
+        if ((c + 1) % kFlush == 0 || c + 1 == it.nk) {
           tc::mma_commit(tc::smem_u32(accf));
           ++win;
         }
@@ -252,13 +250,13 @@ k_split_gemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUt
     for (int w = blockIdx.x; w < a.nwork && ok; w += gridDim.x) {
       const Item it = decode(w);
       // orders 0..3 and 4..T-1 as 64-bit integers, in units of 256^-3 and 256^-(T-1)
-      long long hi[NC], lo[S > 4 ? NC : 1];
+      long long hi[NC], lo[NC];
 #pragma unroll
       for (int i = 0; i < NC; ++i) {
         hi[i] = 0;
-        if (S > 4) lo[i] = 0;
+        lo[i] = 0;
       }
-      const int nwin = (it.nk + G::FLUSH - 1) / G::FLUSH;
+      const int nwin = (it.nk + kFlush - 1) / kFlush;
       for (int v = 0; v < nwin && ok; ++v, ++win) {
         ok = tc::mbar_wait_bounded(tc::smem_u32(accf), win & 1);
         if (!ok) atomicExch(fail, 1);
@@ -277,16 +275,14 @@ k_split_gemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUt
 #pragma unroll
               for (int t = 0; t < 4; ++t)
                 hi[c0 + i] += (long long)__float2int_rn(__uint_as_float(r[t][i])) * (1 << (8 * (3 - t)));
-            if (S > 4) {
 #pragma unroll
-              for (int t = 4; t < T; ++t) tc::tmem_ld8_nowait(tl + t * N + c0, r[t - 4]);
-              tc::tmem_wait_ld();
+            for (int t = 4; t < T; ++t) tc::tmem_ld8_nowait(tl + t * N + c0, r[t - 4]);
+            tc::tmem_wait_ld();
 #pragma unroll
-              for (int i = 0; i < 8; ++i)
+            for (int i = 0; i < 8; ++i)
 #pragma unroll
-                for (int t = 4; t < T; ++t)
-                  lo[c0 + i] += (long long)__float2int_rn(__uint_as_float(r[t - 4][i])) * (1 << (8 * (T - 1 - t)));
-            }
+              for (int t = 4; t < T; ++t)
+                lo[c0 + i] += (long long)__float2int_rn(__uint_as_float(r[t - 4][i])) * (1 << (8 * (T - 1 - t)));
           }
         }
         tc::fence_before_sync();
@@ -302,15 +298,11 @@ k_split_gemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUt
         const int cb = it.n0 + part * NC;
         const int* eb = a.eb + cb + (MODE == PROJ ? it.b * a.rows_b : 0);
         // a rotation's sum (|hi| < 2^47) as one integer in units of 2^(ea + eb - 24 - sh): exact
-        // where |hi| < 2^38 (or S = 4), else cut 2^-53 below its leading bit; rounded once
+        // where |hi| < 2^38, else cut 2^-53 below its leading bit; rounded once
         auto value = [&](int i, int& sh) {
-          if (S == 4) {
-            sh = 0;
-            return hi[i];
-          }
           const bool small = llabs(hi[i]) < (1LL << 38);
           sh = small ? 24 : 15;
-          return small ? (hi[i] << 24) + lo[S > 4 ? i : 0] : (hi[i] << 15) + (lo[S > 4 ? i : 0] >> 9);
+          return small ? (hi[i] << 24) + lo[i] : (hi[i] << 15) + (lo[i] >> 9);
         };
         if (MODE == ROT32) {
           if (mr < a.rows) {
@@ -349,7 +341,7 @@ k_split_gemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUt
             for (int q = 0; q < 2; ++q) {
               int sh = 0;
               if (MODE == GRAM)   // hi may use all of its 53 bits here: hi + 2^-24 lo, rounded once
-                v[q] = fma(__ll2double_rn(lo[S > 4 ? i + q : 0]), 0x1p-24, __ll2double_rn(hi[i + q]));
+                v[q] = fma(__ll2double_rn(lo[i + q]), 0x1p-24, __ll2double_rn(hi[i + q]));
               else
                 v[q] = __ll2double_rn(value(i + q, sh));
               const int e = eb[i + q], x = ea + e - 24 - sh;
@@ -413,7 +405,7 @@ template <typename T> __device__ __forceinline__ int key_exponent(unsigned k) {
   return k == 0 ? 0 : max((int)(k >> 20), 1) - 1022;
 }
 // x as a fixed-point integer with unit 2^(E - 6 - 8 (S - 1)), rounded to nearest
-template <int S, typename T> __device__ __forceinline__ long long to_fixed(T x, int E) {
+template <typename T> __device__ __forceinline__ long long to_fixed(T x, int E) {
   long long m;
   int sh;
   bool neg;
@@ -436,11 +428,10 @@ template <int S, typename T> __device__ __forceinline__ long long to_fixed(T x, 
   return neg ? -m : m;
 }
 // the biased digits of q (byte k of the result is digit S-1-k plus 128)
-template <int S> __device__ __forceinline__ unsigned long long digits(long long q) {
+__device__ __forceinline__ unsigned long long digits(long long q) {
   return (unsigned long long)q + (0x8080808080808080ULL >> (64 - 8 * S));
 }
 // digit s (0 = leading) of two values, as two BF16 (a low, b high)
-template <int S>
 __device__ __forceinline__ unsigned pack2(unsigned long long a, unsigned long long b, int s) {
   const int sh = 8 * (S - 1 - s);
   const float fa = __uint_as_float(0x4B000000u | ((unsigned)(a >> sh) & 255u)) - 8388736.f;
@@ -460,7 +451,7 @@ template <typename T, typename V> __device__ __forceinline__ int scaled_exponent
 // rows of a block (2n reals each) -> digits [S][rows_pad][kp] and unit exponents, one warp per
 // row; rows >= rows are written as zeros.  cs: exponents that multiply the columns (or null).  They
 // are added to the exponents and never multiplied in: they may be larger than the type's range.
-template <int S, typename T>
+template <typename T>
 __global__ void __launch_bounds__(256)
 k_split_rows(const cplx<T>* __restrict__ X, int ldx, int n, long long rows, int rows_pad, int kp,
              const int* __restrict__ cs, uint16_t* __restrict__ D, int* __restrict__ eu) {
@@ -495,18 +486,17 @@ k_split_rows(const cplx<T>* __restrict__ X, int ldx, int n, long long rows, int 
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const int c = i * 64 + 2 * lane + q / 2;
-      d[q] = digits<S>(E == kBad ? 0 : to_fixed<S>(v[i][q], E - (cs && c < n ? cs[c] : 0)));
+      d[q] = digits(E == kBad ? 0 : to_fixed(v[i][q], E - (cs && c < n ? cs[c] : 0)));
     }
 #pragma unroll
     for (int s = 0; s < S; ++s)
       *reinterpret_cast<uint2*>(&D[((size_t)s * rows_pad + r) * kp + k]) =
-          make_uint2(pack2<S>(d[0], d[1], s), pack2<S>(d[2], d[3], s));
+          make_uint2(pack2(d[0], d[1], s), pack2(d[2], d[3], s));
   }
 }
 
 // Q (n x n, rows scaled by 2^-cs) -> the real right factor of the rotation: row 2j + part of
 // output column j's part, over the reals k of a block row; one warp per output row
-template <int S>
 __global__ void __launch_bounds__(256)
 k_split_q(const double2* __restrict__ Q, int n, int rows_pad, int kp, const int* __restrict__ cs,
           uint16_t* __restrict__ D, int* __restrict__ eu) {
@@ -527,11 +517,11 @@ k_split_q(const double2* __restrict__ Q, int n, int rows_pad, int kp, const int*
   for (int i = lane; 2 * i < kp; i += 32) {
     const double2 q = at(i);
     const int Ei = cs && i < n && E != kBad ? E + cs[i] : E;
-    const unsigned long long a = digits<S>(E == kBad ? 0 : to_fixed<S>(q.x, Ei)),
-                             b = digits<S>(E == kBad ? 0 : to_fixed<S>(q.y, Ei));
+    const unsigned long long a = digits(E == kBad ? 0 : to_fixed(q.x, Ei)),
+                             b = digits(E == kBad ? 0 : to_fixed(q.y, Ei));
 #pragma unroll
     for (int s = 0; s < S; ++s)
-      *reinterpret_cast<unsigned*>(&D[((size_t)s * rows_pad + r) * kp + 2 * i]) = pack2<S>(a, b, s);
+      *reinterpret_cast<unsigned*>(&D[((size_t)s * rows_pad + r) * kp + 2 * i]) = pack2(a, b, s);
   }
 }
 
@@ -590,7 +580,7 @@ k_col_max(const cplx<T>* __restrict__ X, int ldx, int n, long long rows,
 // contiguous), rows >= rows as zeros; blocks of 64 rows x 32 complex columns are transposed
 // through shared memory.  WEIGHT: x sqrt(w), an FP64 product, so that one set of digits serves
 // both factors of X^H diag(w) X.
-template <int S, typename T, bool WEIGHT>
+template <typename T, bool WEIGHT>
 __global__ void __launch_bounds__(256)
 k_split_cols(const cplx<T>* __restrict__ X, int ldx, int n, long long r0, long long rows,
              int rows_pad, int cols_pad, const double* __restrict__ md,
@@ -625,14 +615,14 @@ k_split_cols(const cplx<T>* __restrict__ X, int ldx, int n, long long r0, long l
   unsigned long long d[16];
 #pragma unroll
   for (int i = 0; i < 16; ++i)
-    d[i] = digits<S>(E == kBad ? 0 : to_fixed<S>(xs[c][q * 16 + i], E));
+    d[i] = digits(E == kBad ? 0 : to_fixed(xs[c][q * 16 + i], E));
 #pragma unroll
   for (int s = 0; s < S; ++s) {
     uint4* o = reinterpret_cast<uint4*>(&D[((size_t)s * cols_pad + col) * rows_pad + rb + q * 16]);
-    o[0] = make_uint4(pack2<S>(d[0], d[1], s), pack2<S>(d[2], d[3], s), pack2<S>(d[4], d[5], s),
-                      pack2<S>(d[6], d[7], s));
-    o[1] = make_uint4(pack2<S>(d[8], d[9], s), pack2<S>(d[10], d[11], s), pack2<S>(d[12], d[13], s),
-                      pack2<S>(d[14], d[15], s));
+    o[0] = make_uint4(pack2(d[0], d[1], s), pack2(d[2], d[3], s), pack2(d[4], d[5], s),
+                      pack2(d[6], d[7], s));
+    o[1] = make_uint4(pack2(d[8], d[9], s), pack2(d[10], d[11], s), pack2(d[12], d[13], s),
+                      pack2(d[14], d[15], s));
   }
 }
 
@@ -640,7 +630,7 @@ k_split_cols(const cplx<T>* __restrict__ X, int ldx, int n, long long r0, long l
 // kNlRows, zeros up to a multiple of 128) and exponents [b][cols_pad], the maximum taken over
 // the chunk.  X: row j, column s nvec + v is X[(node_j 2 + s) ldx + v]; PTAB: rows of the atom's P
 // table.  The second pass over the rows finds them in L2.
-template <int S, bool PTAB>
+template <bool PTAB>
 __global__ void __launch_bounds__(256)
 k_split_nodes(const double2* __restrict__ src, int ldx, int nvec, const int4* __restrict__ chunks,
               const long long* __restrict__ nodes, const int* __restrict__ atom_npj,
@@ -695,15 +685,15 @@ k_split_nodes(const double2* __restrict__ src, int ldx, int nvec, const int4* __
       const int E = se[cc];
       unsigned long long d[16];
 #pragma unroll
-      for (int i = 0; i < 16; ++i) d[i] = digits<S>(E == kBad ? 0 : to_fixed<S>(xs[cc][q * 16 + i], E));
+      for (int i = 0; i < 16; ++i) d[i] = digits(E == kBad ? 0 : to_fixed(xs[cc][q * 16 + i], E));
 #pragma unroll
       for (int s = 0; s < S; ++s) {
         uint4* o = reinterpret_cast<uint4*>(
             &D[((size_t)s * cols_pad + 2 * cb + cc) * kp + (size_t)b * kNlRows + rb + h + q * 16]);
-        o[0] = make_uint4(pack2<S>(d[0], d[1], s), pack2<S>(d[2], d[3], s), pack2<S>(d[4], d[5], s),
-                          pack2<S>(d[6], d[7], s));
-        o[1] = make_uint4(pack2<S>(d[8], d[9], s), pack2<S>(d[10], d[11], s), pack2<S>(d[12], d[13], s),
-                          pack2<S>(d[14], d[15], s));
+        o[0] = make_uint4(pack2(d[0], d[1], s), pack2(d[2], d[3], s), pack2(d[4], d[5], s),
+                          pack2(d[6], d[7], s));
+        o[1] = make_uint4(pack2(d[8], d[9], s), pack2(d[10], d[11], s), pack2(d[12], d[13], s),
+                          pack2(d[14], d[15], s));
       }
     }
   }
@@ -712,7 +702,7 @@ k_split_nodes(const double2* __restrict__ src, int ldx, int nvec, const int4* __
 // one warp per row of up to 32 complex values -> digits [S][rows][64] and exponents.  COEF: the
 // right factor of the expansion, row (chunk, real column (s, v, part)) of its atom's C'; else
 // rows of the chunks' P tables (zeros up to a multiple of 128 rows of a chunk)
-template <int S, bool COEF>
+template <bool COEF>
 __global__ void __launch_bounds__(256)
 k_split_proj(const double2* __restrict__ src, int nvec, int rows, int cols, const int4* __restrict__ chunks,
              const int* __restrict__ atom_npj, const int* __restrict__ atom_off,
@@ -737,27 +727,26 @@ k_split_proj(const double2* __restrict__ src, int nvec, int rows, int cols, cons
   const unsigned key = __reduce_max_sync(0xffffffffu, max(mag_key(x.x), mag_key(x.y)));
   const int E = key_exponent<double>(key);
   if (lane == 0) eu[r] = E == kBad ? kBad : E - 6;
-  const unsigned long long a = digits<S>(E == kBad ? 0 : to_fixed<S>(x.x, E)),
-                           b = digits<S>(E == kBad ? 0 : to_fixed<S>(x.y, E));
+  const unsigned long long a = digits(E == kBad ? 0 : to_fixed(x.x, E)),
+                           b = digits(E == kBad ? 0 : to_fixed(x.y, E));
 #pragma unroll
   for (int s = 0; s < S; ++s)
-    *reinterpret_cast<unsigned*>(&D[((size_t)s * rows + r) * 64 + 2 * lane]) = pack2<S>(a, b, s);
+    *reinterpret_cast<unsigned*>(&D[((size_t)s * rows + r) * 64 + 2 * lane]) = pack2(a, b, s);
 }
 
 inline int up(int x, int m) { return (x + m - 1) / m * m; }
 
-template <int S, int MODE>
+template <int MODE>
 cudaError_t run_split_gemm(const uint16_t* A, const uint16_t* B, int kpad, const SplitArgs& a,
                            cudaStream_t s) {
-  using G = SplitCfg<S>;
   CUtensorMap ta, tb;
   if (!tc_make_map_bf16(&ta, A, (long long)S * a.rows_a, kpad, kTM) ||
-      !tc_make_map_bf16(&tb, B, (long long)S * a.rows_b, kpad, G::N))
+      !tc_make_map_bf16(&tb, B, (long long)S * a.rows_b, kpad, kTN))
     return cudaErrorInvalidValue;
-  auto k = k_split_gemm<S, MODE>;
-  const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM);
+  auto k = k_split_gemm<MODE>;
+  const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSplitSmem);
   if (e != cudaSuccess) return e;
-  k<<<(unsigned)std::min(a.nwork, gbc_sm_count()), kSplitThreads, G::SMEM, s>>>(ta, tb, a);
+  k<<<(unsigned)std::min(a.nwork, gbc_sm_count()), kSplitThreads, kSplitSmem, s>>>(ta, tb, a);
   return cudaGetLastError();
 }
 
@@ -777,14 +766,14 @@ cudaError_t split_error(int* err, cudaStream_t s) {
   return cudaMemcpyToSymbol(g_split_err, &zero, sizeof(int));
 }
 
-// X <- X Q in place, chunk of rows by chunk
-template <int S, typename T>
-static gbc_status rotate_split(gbc_ctx* c, cplx<T>* X, const double2* Q, long long M, int n, int ldx,
+// X <- X Q in place, chunk of rows by chunk.  diag: the diagonal of X's Gram matrix (the columns'
+// sizes squared), or null for columns of one size
+template <typename T>
+gbc_status launch_rotate_split(gbc_ctx* c, cplx<T>* X, const double2* Q, long long M, int n, int ldx,
                                const double2* diag, cudaStream_t s) {
   constexpr int MODE = sizeof(T) == 4 ? ROT32 : ROT64;
-  using G = SplitCfg<S>;
   const long long rows = 2 * M;
-  const int kp = up(2 * n, kKC), nb = up(2 * n, G::N);
+  const int kp = up(2 * n, kKC), nb = up(2 * n, kTN);
   const long long per = std::max<long long>(kTM, (long long)(kChunkBytes / (2 * S * (size_t)kp)) / kTM * kTM);
   const int rc = (int)std::min<long long>(per, (rows + kTM - 1) / kTM * kTM);
   const size_t ab = (size_t)2 * S * rc * kp, bb = (size_t)2 * S * nb * kp;
@@ -795,28 +784,18 @@ static gbc_status rotate_split(gbc_ctx* c, cplx<T>* X, const double2* Q, long lo
   int* eb = ea + rc;
   int* cs = diag ? eb + nb : nullptr;
   if (cs) k_col_scale<<<1, 256, 0, s>>>(diag, n, cs);
-  k_split_q<S><<<(nb + 7) / 8, 256, 0, s>>>(Q, n, nb, kp, cs, B, eb);
+  k_split_q<<<(nb + 7) / 8, 256, 0, s>>>(Q, n, nb, kp, cs, B, eb);
   GBC_CU(c, cudaGetLastError());
   for (long long r0 = 0; r0 < rows; r0 += rc) {
     const long long nr = std::min<long long>(rc, rows - r0);
     const int rp = up((int)nr, kTM);
-    k_split_rows<S, T><<<(rp + 7) / 8, 256, 0, s>>>(X + r0 * ldx, ldx, n, nr, rp, kp, cs, A, ea);
+    k_split_rows<T><<<(rp + 7) / 8, 256, 0, s>>>(X + r0 * ldx, ldx, n, nr, rp, kp, cs, A, ea);
     GBC_CU(c, cudaGetLastError());
-    const int ntn = nb / G::N, tiles = rp / kTM * ntn;
+    const int ntn = nb / kTN, tiles = rp / kTM * ntn;
     SplitArgs a{rp, nb, kp / kKC, kp / kKC, ntn, tiles, tiles, ea, eb, nr, n, ldx, X + r0 * ldx};
-    GBC_CU(c, (run_split_gemm<S, MODE>(A, B, kp, a, s)));
+    GBC_CU(c, run_split_gemm<MODE>(A, B, kp, a, s));
   }
   return GBC_OK;
-}
-// diag: the diagonal of X's Gram matrix (the columns' sizes squared), or null for orthonormal
-// columns and a unitary Q
-template <typename T>
-gbc_status launch_rotate_split(gbc_ctx* c, cplx<T>* X, const double2* Q, long long M, int n, int ldx,
-                               const double2* diag, cudaStream_t s) {
-  if constexpr (sizeof(T) == 4) {
-    if (!diag) return rotate_split<4, T>(c, X, Q, M, n, ldx, diag, s);
-  }
-  return rotate_split<7, T>(c, X, Q, M, n, ldx, diag, s);
 }
 template gbc_status launch_rotate_split<float>(gbc_ctx*, float2*, const double2*, long long, int, int,
                                                const double2*, cudaStream_t);
@@ -827,12 +806,10 @@ template gbc_status launch_rotate_split<double>(gbc_ctx*, double2*, const double
 template <typename TX, typename TY>
 gbc_status launch_gram_split(gbc_ctx* c, const cplx<TX>* X, int ldx, const cplx<TY>* Y, int ldy,
                              const double* md, long long M, int n, double2* Sm, cudaStream_t s) {
-  constexpr int S = 7;
-  using G = SplitCfg<S>;
   const long long rows = 2 * M;
   const int ma = up(2 * n, kTM), nb = ma;    // both padded to a row tile
   const size_t rowb = (size_t)2 * S * (Y ? ma + nb : ma);
-  const int win = G::FLUSH * kKC;
+  const int win = kFlush * kKC;
   const long long per = std::max<long long>(win, (long long)(kChunkBytes / rowb) / win * win);
   const int rc = (int)std::min<long long>(per, (rows + win - 1) / win * win);
   const size_t ab = (size_t)2 * S * ma * rc, bb = Y ? (size_t)2 * S * nb * rc : 0;
@@ -852,23 +829,23 @@ gbc_status launch_gram_split(gbc_ctx* c, const cplx<TX>* X, int ldx, const cplx<
   if (Y) k_col_max<TY, false><<<gm, 256, 0, s>>>(Y, ldy, n, rows, nullptr, kb);
   GBC_CU(c, cudaGetLastError());
   int tiles = 0;
-  const int ntn = nb / G::N;
-  for (int I = 0; I < ma / kTM; ++I) tiles += ntn - I * (kTM / G::N);
+  const int ntn = nb / kTN;
+  for (int I = 0; I < ma / kTM; ++I) tiles += ntn - I * (kTM / kTN);
   for (long long r0 = 0; r0 < rows; r0 += rc) {
     const long long nr = std::min<long long>(rc, rows - r0);
     const int rp = up((int)nr, win);
     const dim3 gs((unsigned)(rp / 64), (unsigned)(ma / 64));
-    if (md) k_split_cols<S, TX, true><<<gs, 256, 0, s>>>(X, ldx, n, r0, nr, rp, ma, md, ka, A, ea);
-    else k_split_cols<S, TX, false><<<gs, 256, 0, s>>>(X, ldx, n, r0, nr, rp, ma, md, ka, A, ea);
-    if (Y) k_split_cols<S, TY, false><<<gs, 256, 0, s>>>(Y, ldy, n, r0, nr, rp, nb, nullptr, kb, B, eb);
+    if (md) k_split_cols<TX, true><<<gs, 256, 0, s>>>(X, ldx, n, r0, nr, rp, ma, md, ka, A, ea);
+    else k_split_cols<TX, false><<<gs, 256, 0, s>>>(X, ldx, n, r0, nr, rp, ma, md, ka, A, ea);
+    if (Y) k_split_cols<TY, false><<<gs, 256, 0, s>>>(Y, ldy, n, r0, nr, rp, nb, nullptr, kb, B, eb);
     GBC_CU(c, cudaGetLastError());
     // K split so that the CTAs fill the SMs about once, in whole read-out windows
     const int nwin = rp / win;
     const int split = std::max(1, std::min(nwin, gbc_sm_count() / std::max(1, tiles)));
-    const int kper = (nwin + split - 1) / split * G::FLUSH;
+    const int kper = (nwin + split - 1) / split * kFlush;
     const int parts = (rp / kKC + kper - 1) / kper;
     SplitArgs a{ma, nb, rp / kKC, kper, ntn, tiles, tiles * parts, ea, eb, nr, n, 0, Sm};
-    GBC_CU(c, (run_split_gemm<S, GRAM>(A, B, rp, a, s)));
+    GBC_CU(c, run_split_gemm<GRAM>(A, B, rp, a, s));
   }
   return GBC_OK;
 }
@@ -892,8 +869,7 @@ template gbc_status launch_gram_split<double, double>(gbc_ctx*, const double2*, 
 // 17,000 nodes.  One order less (as in the Gram products) measured up to 1.17 times the direct
 // kernels' error.
 static size_t nl_split_chunk(int nvec, bool project) {
-  constexpr int S = 7;
-  const size_t cols = up(4 * nvec, project ? kTM : SplitCfg<S>::N);
+  const size_t cols = up(4 * nvec, project ? kTM : kTN);
   return project ? (2 * S * (size_t)kNlRows + sizeof(int)) * (cols + 64)
                  : (2 * S * 64 + sizeof(int)) * (kNlRows + cols);
 }
@@ -906,7 +882,6 @@ size_t nl_split_bytes(const gbc_ctx* c, int nvec) {
 }
 
 cudaError_t nl_split_project(gbc_ctx* c, const double2* X, int nvec, int ldx, double2* C1, cudaStream_t s) {
-  constexpr int S = 7;
   const ProjDev& pj = c->proj;
   const int cols = up(4 * nvec, kTM), nb = nl_split_batch(c, nl_split_chunk(nvec, true));
   for (int b0 = 0; b0 < pj.nchunks; b0 += nb) {
@@ -917,24 +892,23 @@ cudaError_t nl_split_project(gbc_ctx* c, const double2* X, int nvec, int ldx, do
     int* eb = ea + (size_t)n * cols;
     const int4* ch = pj.d_chunks + b0;
     // (rows of A past the last 64 columns stay as they are: nothing of theirs is used)
-    k_split_nodes<S, false><<<dim3(n, up(4 * nvec, 64) / 64), 256, 0, s>>>(
+    k_split_nodes<false><<<dim3(n, up(4 * nvec, 64) / 64), 256, 0, s>>>(
         X, ldx, nvec, ch, pj.d_nodes, pj.d_atom_npj, pj.d_atom_pv_off, c->mesh.M, cols, kp, A, ea);
-    k_split_nodes<S, true><<<dim3(n, 1), 256, 0, s>>>(pj.d_P64, 0, 0, ch, pj.d_nodes, pj.d_atom_npj,
+    k_split_nodes<true><<<dim3(n, 1), 256, 0, s>>>(pj.d_P64, 0, 0, ch, pj.d_nodes, pj.d_atom_npj,
                                                       pj.d_atom_pv_off, c->mesh.M, 64, kp, B, eb);
     const int ntm = cols / kTM;
     SplitArgs a{cols, 64, 0, 0, ntm, n * ntm, n * ntm, ea, eb, 0, nvec, 0, C1, ch, pj.d_nodes,
                 pj.d_atom_npj, pj.d_atom_c_off};
     cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess) e = run_split_gemm<S, PROJ>(A, B, kp, a, s);
+    if (e == cudaSuccess) e = run_split_gemm<PROJ>(A, B, kp, a, s);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
 }
 
 cudaError_t nl_split_expand(gbc_ctx* c, double2* Y, int nvec, int ldx, const double2* C2, cudaStream_t s) {
-  constexpr int S = 7;
   const ProjDev& pj = c->proj;
-  const int cols = up(4 * nvec, SplitCfg<S>::N), nb = nl_split_batch(c, nl_split_chunk(nvec, false));
+  const int cols = up(4 * nvec, kTN), nb = nl_split_batch(c, nl_split_chunk(nvec, false));
   for (int b0 = 0; b0 < pj.nchunks; b0 += nb) {
     const int n = std::min(nb, pj.nchunks - b0), ra = n * kNlRows, rb = n * cols;
     uint16_t* A = (uint16_t*)c->work[14];
@@ -942,15 +916,15 @@ cudaError_t nl_split_expand(gbc_ctx* c, double2* Y, int nvec, int ldx, const dou
     int* ea = (int*)(B + (size_t)S * rb * 64);
     int* eb = ea + ra;
     const int4* ch = pj.d_chunks + b0;
-    k_split_proj<S, false><<<ra / 8, 256, 0, s>>>(pj.d_P64, nvec, ra, 0, ch, pj.d_atom_npj,
+    k_split_proj<false><<<ra / 8, 256, 0, s>>>(pj.d_P64, nvec, ra, 0, ch, pj.d_atom_npj,
                                                   pj.d_atom_pv_off, A, ea);
-    k_split_proj<S, true><<<rb / 8, 256, 0, s>>>(C2, nvec, rb, cols, ch, pj.d_atom_npj,
+    k_split_proj<true><<<rb / 8, 256, 0, s>>>(C2, nvec, rb, cols, ch, pj.d_atom_npj,
                                                  pj.d_atom_c_off, B, eb);
-    const int ntn = cols / SplitCfg<S>::N, tiles = ra / kTM * ntn;
+    const int ntn = cols / kTN, tiles = ra / kTM * ntn;
     SplitArgs a{ra, rb, 1, 1, ntn, tiles, tiles, ea, eb, c->mesh.M, nvec, ldx, Y, ch, pj.d_nodes,
                 pj.d_atom_npj, pj.d_atom_c_off};
     cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess) e = run_split_gemm<S, EXPD>(A, B, 64, a, s);
+    if (e == cudaSuccess) e = run_split_gemm<EXPD>(A, B, 64, a, s);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;

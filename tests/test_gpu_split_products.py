@@ -109,6 +109,46 @@ def test_rayleigh_ritz_tiles(g, prec, n):
     ctx.close()
 
 
+def localised(prob, n):
+    """Columns peaked on one interior node of a cell each, a weak random tail everywhere."""
+    nx, ny, nz = prob.ncell
+    p, M = prob.p, prob.nnodes
+    cell = np.arange(n)
+    g = [c * p + 1 for c in (cell % nx, cell // nx % ny, cell // (nx * ny))]
+    X = 1e-4 * syn.random_block(M, n, 9)
+    X[(g[2] * ny * p + g[1]) * nx * p + g[0], 0, cell] += 1.0
+    return X
+
+
+@pytest.mark.parametrize("n,local", [(32, False), (256, False), (128, True), (512, True)])
+def test_ritz_rotation_of_a_converged_fp32_block(g, n, local):
+    """An FP32 block that is rotated close to the identity is rounded to FP32 once: what X Q leaves
+    over in the rotated block (least squares for Q) is at most 2^-24 of each column, however
+    delocalised or localised the columns are."""
+    ncell, p = ((8, 8, 8), 3) if local else ((3, 3, 3), 5)
+    prob = syn.make_problem(ncell=ncell, h=(1.0, 1.1, 0.9), p=p, seed=4)
+    if local:   # one potential per cell: the localised columns are close to eigenvectors
+        prob = prob.with_(veff=prob.veff + 0.5 * np.arange(512.0)[:, None])
+    ctx = g.Context(0)
+    ctx.set_problem(prob)
+    ctx.set_precision(1)
+    Xd = device(localised(prob, n) if local else block(prob.nnodes, n, 5), 1, n)
+    ctx.cholgs(Xd)
+    ctx.rayleigh_ritz(Xd)
+    # Ritz vectors turned a little, as a filter leaves them: the next Q is close to the identity
+    K = 1e-3 / n ** 0.5 * torch.randn((n, n), dtype=torch.complex128, device="cuda",
+                                      generator=torch.Generator("cuda").manual_seed(n))
+    Xd += (Xd.to(torch.complex128) @ (K - K.mH)).to(Xd.dtype)
+    ctx.cholgs(Xd)
+    X = Xd.to(torch.complex128).reshape(-1, n)
+    ctx.rayleigh_ritz(Xd)
+    Y = Xd.to(torch.complex128).reshape(-1, n)
+    Q = torch.linalg.solve(X.mH @ X, X.mH @ Y)
+    left = torch.linalg.vector_norm(Y - X @ Q, dim=0) / torch.linalg.vector_norm(Y, dim=0)
+    assert float(left.max()) < 2.0 ** -24
+    ctx.close()
+
+
 @pytest.mark.parametrize("prec", [0, 1])
 def test_cholgs_refuses_what_it_refused(g, prec):
     ctx, prob = context(g, prec, (2, 2, 2), 3)
