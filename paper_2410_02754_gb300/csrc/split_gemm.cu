@@ -6,30 +6,33 @@
 // 2012), with balanced base-256 digits: a value x with |x| < 2^E is
 //   x = 2^(E-6) sum_k d_k 256^-k,  |d_0| <= 65, d_k in [-128, 127],
 // so every digit is a BF16 number and a product of two digits an integer below 2^14; S digits
-// carry 8 S - 2 bits below 2^E.  The partial products of order t = i + j <= S - 1,
-// G_t = sum_{i+j=t} A_i B_j, are integers that FP32 holds exactly while (t + 1) K 2^14 <= 2^24;
+// carry 8 S - 2 bits below 2^E.  The partial products of order t = i + j <= S,
+// G_t = sum_{i+j=t} A_i B_j, are integers that FP32 holds exactly while S K 2^14 <= 2^24;
 // the accumulators are read out (to 64-bit integers) every kFlush K chunks to keep that, and
-// sum_t G_t 256^-t is rounded once at the end.  Exponents are per row of A and B: per block
+// sum_t G_t 256^-t is rounded at the end (Gram matrices and projections: once per part
+// of K, the parts added in FP64).  Exponents are per row of A and B: per block
 // row and per column of Q for a rotation, per column of the block (over all rows) for a Gram
 // matrix.  A row with an infinity or a NaN is marked and gives NaN, as in FP arithmetic.
 //
 // S = 7 digits: an entry is off by at most 2^-55 of its row's largest.  FP32 blocks are rounded to
 // FP32 once.  The rotation of CholGS, whose terms can cancel, takes its columns at a common size, by
 // powers of two; that of Rayleigh-Ritz rests on an M_D-orthonormal block, whose columns have one size.
-// Orders t <= T - 1 are summed.  What is left out of a sum over K terms is about sqrt(K) 2^-54 of
-// the largest entries' product at T = S, sqrt(K) 2^-62 at T = S + 1: the latter where a sum is
-// small against them, as in the rotation of a nearly converged block (Q close to the identity).  With
-// S = 4 = T (30 bits) such FP32 columns came out 6.2e-8 off at n = 256, with S = 7 the 2.5e-8 of
-// their rounding to FP32; 200 columns of 432,000 rows take 3.5 ms more for it.
+// Orders t < T = S + 1 are summed.  What is left out of a sum over K terms is about sqrt(K) 2^-62 of
+// the product of the largest entries (sqrt(K) 2^-54 without order S), which counts where a sum is
+// small against that: the rotation of a nearly converged block (Q close to the identity), Gram
+// entries of columns that peak in a few of many rows, projectors over most of their support.
+// Measured with fewer: FP32 columns of a nearly converged block, n = 256, came out 6.2e-8 off
+// with S = T = 4, 2.5e-8 (their rounding to FP32) now; FP64 columns with one of 746,000 rows 1000
+// times the others came out of CholGS orthonormal to 5e-14 with T = S, to 1.3e-15 now (direct FP64
+// 2.2e-15; 10^5 times: 5e-13, direct 6e-13).
 //
 // GB300's FP64 pipe gives 1.05 TFLOP/s and float-float arithmetic on the FP32 pipes about 6;
-// 28 BF16 products at 1.9 PFLOP/s are an FP64-accurate 68 TFLOP/s.  Measured, 884,736 nodes x 256
-// FP32 columns: Gram 122 -> 21 ms (16 of them the products, 43% of the tensor pipe), rotation
-// 163 -> 26 ms (23 the products); 373,248 nodes x 256 in FP64: 333 -> 13 and 527 -> 14 ms.  Per tile
-// (128 x 64) every order has its own accumulator in tensor memory and all S
+// 34 BF16 products at 1.9 PFLOP/s are an FP64-accurate 56 TFLOP/s.  Measured, 884,736 nodes x 256
+// FP32 columns: Gram 122 -> 24.5 ms, rotation 163 -> 28.8 ms; 373,248 nodes x 256 in FP64: 333 ->
+// 11.5 and 527 -> 13.0 ms.  Per tile (128 x 64) every order has its own accumulator in tensor memory and all S
 // digit slices of a 64-wide K chunk are in shared memory at once (one TMA box each), so a
 // slice is loaded once per tile and used in up to S products.  Step i multiplies A_i with all
-// of B_0 .. B_{S-1-i} in instructions of up to 256 columns (one product per instruction, 64
+// of B_0 .. B_{S-i} in instructions of up to 256 columns (one product per instruction, 64
 // columns, ran at a quarter of this rate); A_i's next chunk then loads behind the other steps,
 // B is double-buffered.
 #include <algorithm>
@@ -48,12 +51,13 @@ constexpr int kKC = 64;               // K chunk: one 128-byte swizzled row
 constexpr int kBad = 0x7fffffff;      // exponent of a row with an infinity or a NaN
 constexpr int kEpi = 16;              // read-out warps
 constexpr int kSplitThreads = 64 + 32 * kEpi;
-constexpr int S = 7;                  // digits
+constexpr int S = 7, T = S + 1;       // digits; orders summed (order S: digits 1 .. S-1 only)
 constexpr int kTN = 64;               // tile columns
 constexpr int kFlush = 2;             // K chunks between read-outs
 constexpr int kABytes = kTM * 128, kBBytes = kTN * 128;
 constexpr size_t kSplitSmem = 1024 + (size_t)S * (kABytes + 2 * kBBytes) + 256;
 static_assert((long long)S * kFlush * kKC << 14 <= 1LL << 24, "exact accumulation");
+static_assert(T * kTN <= 512 && T <= 8, "tensor memory columns");
 static_assert(kSplitSmem <= 227 * 1024, "shared memory");
 
 // PROJ, EXPD: the FP64 projector contractions C += P^H X and Y += P C' (see nl_split_project)
@@ -82,9 +86,6 @@ __global__ void __launch_bounds__(kSplitThreads, 1)
 k_split_gemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb,
              const SplitArgs a) {
   constexpr int N = kTN;
-  // orders summed; order S: digits 1 .. S-1 only
-  constexpr int T = MODE == GRAM ? S : S + 1;
-  static_assert(T * N <= 512 && T <= 8, "tensor memory columns");
   struct Item { int m0, n0, k0, nk, b; };   // b: chunk of the batch
   auto decode = [&](int w) {
     Item it{0, 0, 0, a.nchunk, 0};
@@ -222,7 +223,7 @@ k_split_gemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUt
                 tc::mma_bf16(tmem + (i + j) * N, tc::sdesc_sw128(A(i) + kk * 32),
                              tc::sdesc_sw128(B(buf, j) + kk * 32), tc::idesc_bf16(kTM, cnt * N), acc);
               };
-              if (T > S && i == 1 && kk == 0 && j + cnt == S && first) {   // order S starts here
+              if (i == 1 && kk == 0 && j + cnt == S && first) {   // order S starts here
                 if (cnt > 1) mma(j, cnt - 1, 1u);
                 mma(S - 1, 1, 0u);
               } else {
@@ -288,10 +289,8 @@ k_split_gemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUt
         tc::fence_before_sync();
         if (lane == 0) tc::mbar_arrive(tc::smem_u32(acce));
       }
-      if (T > S) {   // back to units of 256^-(S-1)
 #pragma unroll
-        for (int i = 0; i < NC; ++i) lo[i] = (lo[i] + 128) >> 8;
-      }
+      for (int i = 0; i < NC; ++i) lo[i] = (lo[i] + 128) >> 8;   // back to units of 256^-(S-1)
       if (ok && it.nk > 0) {
         const int mr = it.m0 + g * 32 + lane;
         const int ea = a.ea[mr + (MODE == PROJ ? it.b * a.rows_a : 0)];
@@ -579,21 +578,27 @@ k_col_max(const cplx<T>* __restrict__ X, int ldx, int n, long long rows,
 // columns of a block over the rows [r0, r0 + rows_pad) -> digits [S][cols_pad][rows_pad] (rows
 // contiguous), rows >= rows as zeros; blocks of 64 rows x 32 complex columns are transposed
 // through shared memory.  WEIGHT: x sqrt(w), an FP64 product, so that one set of digits serves
-// both factors of X^H diag(w) X.
+// both factors of X^H diag(w) X; and diag[.][c] += the column's |x|^2 w in FP64: a digit's product
+// with itself does not average out, so the orders left out of the products (d_4^2 first) would add
+// up to rows 2^-62 of the largest entry squared on the diagonal.  kDiagParts partial sums per column:
+// one would be the sum of 23,000 atomics at 746,000 rows and off by their roundings.
+constexpr int kDiagParts = 64;
 template <typename T, bool WEIGHT>
 __global__ void __launch_bounds__(256)
 k_split_cols(const cplx<T>* __restrict__ X, int ldx, int n, long long r0, long long rows,
              int rows_pad, int cols_pad, const double* __restrict__ md,
-             const unsigned* __restrict__ key, uint16_t* __restrict__ D, int* __restrict__ eu) {
+             const unsigned* __restrict__ key, uint16_t* __restrict__ D, int* __restrict__ eu,
+             double* __restrict__ diag) {
   using V = typename std::conditional<WEIGHT, double, T>::type;
   __shared__ V xs[64][65];                      // [real column][row]
-  __shared__ double ws[64];
+  __shared__ double ws[64], sqs[8][32];
   const int rb = blockIdx.x * 64, cb = blockIdx.y * 32;
   if (WEIGHT) {
     if (threadIdx.x < 64)
       ws[threadIdx.x] = rb + threadIdx.x < rows ? sqrt(md[(r0 + rb + threadIdx.x) >> 1]) : 0.0;
     __syncthreads();
   }
+  double sq = 0.0;
   for (int i = threadIdx.x; i < 64 * 32; i += 256) {
     const int c = i & 31, rr = i >> 5;
     const long long r = rb + rr;
@@ -604,10 +609,16 @@ k_split_cols(const cplx<T>* __restrict__ X, int ldx, int n, long long r0, long l
       a = WEIGHT ? (V)((double)x.x * w) : (V)x.x;
       b = WEIGHT ? (V)((double)x.y * w) : (V)x.y;
     }
+    if (WEIGHT) sq = fma((double)a, (double)a, fma((double)b, (double)b, sq));
     xs[2 * c][rr] = a;
     xs[2 * c + 1][rr] = b;
   }
+  if (WEIGHT) sqs[threadIdx.x >> 5][threadIdx.x & 31] = sq;
   __syncthreads();
+  if (WEIGHT && threadIdx.x < 32 && cb + threadIdx.x < n) {
+    for (int w = 1; w < 8; ++w) sq += sqs[w][threadIdx.x];
+    atomicAdd(&diag[(size_t)(blockIdx.x % kDiagParts) * n + cb + threadIdx.x], sq);
+  }
   const int c = threadIdx.x >> 2, q = threadIdx.x & 3;   // real column, group of 16 rows
   const int col = 2 * cb + c;
   const int E = col < 2 * n ? key_exponent<T>(key[col]) : 0;
@@ -623,6 +634,15 @@ k_split_cols(const cplx<T>* __restrict__ X, int ldx, int n, long long r0, long l
                       pack2(d[6], d[7], s));
     o[1] = make_uint4(pack2(d[8], d[9], s), pack2(d[10], d[11], s), pack2(d[12], d[13], s),
                       pack2(d[14], d[15], s));
+  }
+}
+
+// S_ii = sum of the parts of diag (NaN where it is not finite)
+__global__ void k_set_diag(const double* __restrict__ diag, int n, double2* __restrict__ Sm) {
+  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    double d = 0.0;
+    for (int p = 0; p < kDiagParts; ++p) d += diag[(size_t)p * n + i];
+    Sm[(size_t)i * n + i] = make_double2(isfinite(d) ? d : NAN, 0.0);
   }
 }
 
@@ -813,15 +833,16 @@ gbc_status launch_gram_split(gbc_ctx* c, const cplx<TX>* X, int ldx, const cplx<
   const long long per = std::max<long long>(win, (long long)(kChunkBytes / rowb) / win * win);
   const int rc = (int)std::min<long long>(per, (rows + win - 1) / win * win);
   const size_t ab = (size_t)2 * S * ma * rc, bb = Y ? (size_t)2 * S * nb * rc : 0;
-  GBC_TRY(gbc_ensure_work(c, 13, ab + bb + sizeof(int) * 4 * (size_t)ma + 1024));
+  GBC_TRY(gbc_ensure_work(c, 13, ab + bb + sizeof(int) * 4 * (size_t)ma + sizeof(double) * kDiagParts * n + 1024));
   uint16_t* A = (uint16_t*)c->work[13];
   uint16_t* B = Y ? (uint16_t*)((char*)A + ab) : A;   // one set of digits for both factors
   int* ea = (int*)((char*)A + ab + bb);
   int* eb = Y ? ea + ma : ea;
   unsigned* ka = (unsigned*)(ea + 2 * (size_t)ma);
   unsigned* kb = ka + ma;
+  double* diag = (double*)(kb + ma);
   GBC_CU(c, cudaMemsetAsync(Sm, 0, sizeof(double2) * (size_t)n * n, s));
-  GBC_CU(c, cudaMemsetAsync(ka, 0, sizeof(unsigned) * 2 * (size_t)ma, s));
+  GBC_CU(c, cudaMemsetAsync(ka, 0, sizeof(unsigned) * 2 * (size_t)ma + sizeof(double) * kDiagParts * n, s));
   const unsigned ncb = (unsigned)((n + 31) / 32);
   const dim3 gm((unsigned)std::max<long long>(1, std::min<long long>((rows + 63) / 64, 16LL * gbc_sm_count() / ncb + 1)), ncb);
   if (md) k_col_max<TX, true><<<gm, 256, 0, s>>>(X, ldx, n, rows, md, ka);
@@ -835,9 +856,9 @@ gbc_status launch_gram_split(gbc_ctx* c, const cplx<TX>* X, int ldx, const cplx<
     const long long nr = std::min<long long>(rc, rows - r0);
     const int rp = up((int)nr, win);
     const dim3 gs((unsigned)(rp / 64), (unsigned)(ma / 64));
-    if (md) k_split_cols<TX, true><<<gs, 256, 0, s>>>(X, ldx, n, r0, nr, rp, ma, md, ka, A, ea);
-    else k_split_cols<TX, false><<<gs, 256, 0, s>>>(X, ldx, n, r0, nr, rp, ma, md, ka, A, ea);
-    if (Y) k_split_cols<TY, false><<<gs, 256, 0, s>>>(Y, ldy, n, r0, nr, rp, nb, nullptr, kb, B, eb);
+    if (md) k_split_cols<TX, true><<<gs, 256, 0, s>>>(X, ldx, n, r0, nr, rp, ma, md, ka, A, ea, diag);
+    else k_split_cols<TX, false><<<gs, 256, 0, s>>>(X, ldx, n, r0, nr, rp, ma, md, ka, A, ea, nullptr);
+    if (Y) k_split_cols<TY, false><<<gs, 256, 0, s>>>(Y, ldy, n, r0, nr, rp, nb, nullptr, kb, B, eb, nullptr);
     GBC_CU(c, cudaGetLastError());
     // K split so that the CTAs fill the SMs about once, in whole read-out windows
     const int nwin = rp / win;
@@ -847,6 +868,8 @@ gbc_status launch_gram_split(gbc_ctx* c, const cplx<TX>* X, int ldx, const cplx<
     SplitArgs a{ma, nb, rp / kKC, kper, ntn, tiles, tiles * parts, ea, eb, nr, n, 0, Sm};
     GBC_CU(c, run_split_gemm<GRAM>(A, B, rp, a, s));
   }
+  if (md) k_set_diag<<<1, 256, 0, s>>>(diag, n, Sm);
+  GBC_CU(c, cudaGetLastError());
   return GBC_OK;
 }
 template gbc_status launch_gram_split<float, float>(gbc_ctx*, const float2*, int, const float2*, int,

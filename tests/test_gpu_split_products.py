@@ -109,6 +109,24 @@ def test_rayleigh_ritz_tiles(g, prec, n):
     ctx.close()
 
 
+def test_gram_of_peaked_columns(g):
+    """Columns that peak in one of 746,000 rows: an FP64 sum of K terms is off by about sqrt(K) 2^-53
+    of the terms' size, so the block of CholGS is orthonormal to that."""
+    ctx, prob = context(g, 0, (12, 12, 12), 6)
+    M, n = prob.nnodes, 16
+    Xd = torch.rand((M, 2, n, 2), dtype=torch.float64, device="cuda",
+                    generator=torch.Generator("cuda").manual_seed(1)) * 2 - 1
+    Xd = torch.view_as_complex(Xd)
+    Xd[M // 3, 0] *= 1000.0
+    ctx.cholgs(Xd)
+    Y = Xd.reshape(2 * M, n)
+    md = torch.from_numpy(np.repeat(ctx.mass(), 2)).cuda()[:, None]
+    G = sum(y.mH @ (m * y) for y, m in zip(Y.chunk(512), md.chunk(512)))
+    off = float((G - torch.eye(n, device="cuda")).abs().max())
+    assert off < (2 * M) ** 0.5 * 2.0 ** -53
+    ctx.close()
+
+
 def localised(prob, n):
     """Columns peaked on one interior node of a cell each, a weak random tail everywhere."""
     nx, ny, nz = prob.ncell
