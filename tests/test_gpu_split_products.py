@@ -110,8 +110,8 @@ def test_rayleigh_ritz_tiles(g, prec, n):
 
 
 def test_gram_of_peaked_columns(g):
-    """Columns that peak in one of 746,000 rows: an FP64 sum of K terms is off by about sqrt(K) 2^-53
-    of the terms' size, so the block of CholGS is orthonormal to that."""
+    """Columns that peak in one of 746,000 rows: an FP64 sum of K terms in 64 parts is off by about
+    sqrt(K / 64) 2^-53 of its value, and the block of CholGS is orthonormal to that."""
     ctx, prob = context(g, 0, (12, 12, 12), 6)
     M, n = prob.nnodes, 16
     Xd = torch.rand((M, 2, n, 2), dtype=torch.float64, device="cuda",
@@ -123,7 +123,7 @@ def test_gram_of_peaked_columns(g):
     md = torch.from_numpy(np.repeat(ctx.mass(), 2)).cuda()[:, None]
     G = sum(y.mH @ (m * y) for y, m in zip(Y.chunk(512), md.chunk(512)))
     off = float((G - torch.eye(n, device="cuda")).abs().max())
-    assert off < (2 * M) ** 0.5 * 2.0 ** -53
+    assert off < (2 * M / 64) ** 0.5 * 2.0 ** -53
     ctx.close()
 
 
