@@ -51,7 +51,19 @@ gbc_status gbc_ensure_work(gbc_ctx* c, int slot, size_t bytes) {
   if (c->work[slot]) cudaFree(c->work[slot]);
   c->work[slot] = nullptr;
   c->work_bytes[slot] = 0;
-  GBC_CU(c, cudaMalloc(&c->work[slot], bytes));
+  cudaError_t e = cudaMalloc(&c->work[slot], bytes);
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();   // not left for the next launch's check
+    c->work[slot] = nullptr;
+    if (slot != 13 && c->work[13]) {   // the digits of an earlier CholGS or Rayleigh-Ritz (synchronous calls)
+      cudaFree(c->work[13]);
+      c->work[13] = nullptr;
+      c->work_bytes[13] = 0;
+      e = cudaMalloc(&c->work[slot], bytes);
+      if (e != cudaSuccess) cudaGetLastError();
+    }
+  }
+  GBC_CU(c, e);
   c->work_bytes[slot] = bytes;
   return GBC_OK;
 }
@@ -223,11 +235,12 @@ gbc_status filter_t(gbc_ctx* c, cplx<T>* X, int nvec, int ldx, int m, double lT,
 }
 
 // Gram matrices and rotations: split products on the tensor cores (split_gemm.cu) from these
-// column counts on, below them FP64 (FP64 block) or float-float arithmetic (FP32 block).
-// Measured, split against direct: FP64 Gram at 16 columns 0.06 / 0.07 ms (1728 nodes) and
-// 1.36 / 5.22 ms (216,000 nodes), rotation 0.04 / 0.11 and 0.74 / 4.8 ms; FP32 Gram 1.34 /
-// 0.83 ms at 32 columns and 0.147 / 0.171 ms at 64 (216,000 and 13,824 nodes), FP32 rotation
-// 0.56 / 0.64 ms at 16 and 0.56 / 1.29 at 32 (216,000 nodes), 0.033 / 0.023 at 16 (1728).
+// column counts on, below them FP64 (FP64 block) or float-float arithmetic (FP32 block); the same
+// where the memory for the digits cannot be had.
+// Measured, split against direct: FP64 Gram at 16 columns 0.054 / 0.066 ms (1296 nodes) and
+// 0.86 / 5.22 ms (216,000 nodes), rotation 0.030 / 0.114 and 0.56 / 4.8 ms; FP32 Gram 1.34 /
+// 0.83 ms at 32 columns (216,000 nodes), 0.112 / 0.171 at 64 (13,824) and 0.92 / 2.32 (216,000), FP32
+// rotation 0.56 / 0.64 ms at 16 and 0.42 / 1.29 at 32 (216,000 nodes), 0.033 / 0.023 at 16 (1728).
 template <typename T> constexpr int split_gram_cols() { return sizeof(T) == 8 ? 16 : 64; }
 template <typename T> constexpr int split_rotate_cols() { return sizeof(T) == 8 ? 16 : 32; }
 
@@ -237,8 +250,11 @@ gbc_status gram(gbc_ctx* c, const cplx<T>* X, int ldx, const cplx<TY>* Y, int ld
                 int nvec, double2* S, cudaStream_t s) {
   {
     TimerScope ts(c, FAM_GRAM, s);
-    if (nvec >= split_gram_cols<T>()) {
-      GBC_TRY((launch_gram_split<T, TY>(c, X, ldx, md ? nullptr : Y, ldy, md, c->mesh.M, nvec, S, s)));
+    gbc_status st = GBC_ENOMEM;
+    if (nvec >= split_gram_cols<T>())
+      st = launch_gram_split<T, TY>(c, X, ldx, md ? nullptr : Y, ldy, md, c->mesh.M, nvec, S, s);
+    if (st != GBC_ENOMEM) {
+      GBC_TRY(st);
     } else if constexpr (std::is_same<T, double>::value) {
       GBC_CU(c, launch_gram<double>(X, Y, md, c->mesh.M, nvec, ldx, S, s));
     } else {
@@ -250,13 +266,14 @@ gbc_status gram(gbc_ctx* c, const cplx<T>* X, int ldx, const cplx<TY>* Y, int ld
 }
 
 // X <- X Q.  diag: the diagonal of X's Gram matrix (null: the columns have one size);
-// qsplit: 2 nvec^2 float2 of scratch
+// qsplit: 2 nvec^2 float2 of scratch (FP32 blocks)
 template <typename T>
 gbc_status rotate(gbc_ctx* c, cplx<T>* X, int nvec, int ldx, const double2* Q, const double2* diag,
                   float2* qsplit, cudaStream_t s) {
   if (nvec >= split_rotate_cols<T>()) {
     TimerScope ts(c, FAM_ROTATE, s);
-    return launch_rotate_split<T>(c, X, Q, c->mesh.M, nvec, ldx, diag, s);
+    const gbc_status st = launch_rotate_split<T>(c, X, Q, c->mesh.M, nvec, ldx, diag, s);
+    if (st != GBC_ENOMEM) return st;
   }
   GBC_TRY(gbc_ensure_work(c, 1, sizeof(cplx<T>) * 2 * (size_t)c->mesh.M * ldx));
   cplx<T>* W = (cplx<T>*)c->work[1];
@@ -280,19 +297,19 @@ gbc_status finish_dense(gbc_ctx* c, cudaStream_t s) {
 }
 
 // small dense scratch of CholGS / Rayleigh-Ritz (work slot 3): two n x n matrices, the FP32
-// pairs of Q, a diagonal and n doubles
+// pairs of Q (FP32 blocks), a diagonal and n doubles
 struct DenseScratch {
   double2 *S, *Q, *diag;
   float2* qsplit;
   double* ev;
 };
-gbc_status dense_scratch(gbc_ctx* c, int nvec, DenseScratch* d) {
-  const size_t nn = (size_t)nvec * nvec;
-  GBC_TRY(gbc_ensure_work(c, 3, sizeof(double2) * (3 * nn + nvec) + sizeof(double) * nvec + 256));
+template <typename T> gbc_status dense_scratch(gbc_ctx* c, int nvec, DenseScratch* d) {
+  const size_t nn = (size_t)nvec * nvec, nq = std::is_same<T, float>::value ? nn : 0;
+  GBC_TRY(gbc_ensure_work(c, 3, sizeof(double2) * (2 * nn + nq + nvec) + sizeof(double) * nvec + 256));
   d->S = (double2*)c->work[3];
   d->Q = d->S + nn;
   d->qsplit = (float2*)(d->Q + nn);
-  d->diag = d->Q + 2 * nn;
+  d->diag = d->Q + nn + nq;
   d->ev = (double*)(d->diag + nvec);
   return GBC_OK;
 }
@@ -303,7 +320,7 @@ gbc_status dense_scratch(gbc_ctx* c, int nvec, DenseScratch* d) {
 template <typename T>
 gbc_status cholgs_t(gbc_ctx* c, cplx<T>* X, int nvec, int ldx, cudaStream_t s) {
   DenseScratch d;
-  GBC_TRY(dense_scratch(c, nvec, &d));
+  GBC_TRY(dense_scratch<T>(c, nvec, &d));
   GBC_TRY((gram<T, T>(c, X, ldx, X, ldx, c->d_md, nvec, d.S, s)));
   GBC_CU(c, cudaMemcpy2DAsync(d.diag, sizeof(double2), d.S, sizeof(double2) * (nvec + 1), sizeof(double2),
                               nvec, cudaMemcpyDeviceToDevice, s));
@@ -324,7 +341,7 @@ gbc_status rr_t(gbc_ctx* c, cplx<T>* X, int nvec, int ldx, double* ritz, cudaStr
   const int ldh = f64 ? ldx : nvec;
   const size_t bytes = sizeof(double2) * 2 * (size_t)c->mesh.M * ldh;
   DenseScratch d;
-  GBC_TRY(dense_scratch(c, nvec, &d));
+  GBC_TRY(dense_scratch<T>(c, nvec, &d));
   GBC_TRY(gbc_ensure_work(c, 0, bytes));
   double2* HX = (double2*)c->work[0];
   const double2* X64;

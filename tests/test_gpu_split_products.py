@@ -183,3 +183,48 @@ def test_cholgs_refuses_what_it_refused(g, prec):
         assert e.value.status == 5                       # GBC_ENOTPD, the block unchanged
         assert torch.equal(torch.view_as_real(Xd).nan_to_num(), torch.view_as_real(keep).nan_to_num())
     ctx.close()
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+def test_no_memory_for_the_digits(g, prec):
+    """With too little device memory for the digits, CholGS and Rayleigh-Ritz run the direct kernels
+    (which need one more block), and the digits kept from an earlier call make room for other work."""
+    ctx, prob = context(g, prec, (6, 6, 6), 5)
+    M, n = prob.nnodes, 128
+    X0 = device(block(M, n, 3), prec, n)
+    want = X0.clone()
+    for m in (8, n):                                 # kernels loaded, reference block
+        few = device(block(M, m, 3), prec, m)
+        ctx.cholgs(few)
+        ctx.rayleigh_ritz(few)
+    ctx.cholgs(want)
+    ritz = ctx.rayleigh_ritz(want.clone())
+    del few
+    ctx.close()
+    ctx, _ = context(g, prec, (6, 6, 6), 5)
+    X = X0.clone()
+    ctx.apply_h(X, torch.empty_like(X))              # tables and coefficients in place
+
+    def starved(room, call):
+        torch.cuda.empty_cache()
+        hog = torch.empty(torch.cuda.mem_get_info()[0] - room, dtype=torch.uint8, device="cuda")
+        try:
+            return call()
+        finally:
+            del hog
+            torch.cuda.empty_cache()
+
+    # FP64 blocks take 105 MB, FP32 blocks 53, the digits 185 (Rayleigh-Ritz 369 for its Gram matrix)
+    starved(150 << 20, lambda: ctx.cholgs(X))
+    err = torch.linalg.vector_norm((X - want).reshape(-1, n), dim=0) / torch.linalg.vector_norm(want.reshape(-1, n), dim=0)
+    assert float(err.max()) < (1e-12 if prec == 0 else 2.0 ** -23)
+    got = starved(300 << 20, lambda: ctx.rayleigh_ritz(X))
+    assert np.abs(got - ritz).max() < (1e-11 if prec == 0 else 1e-6) * np.abs(ritz).max()
+    ctx.close()
+    # digits that an earlier call left (185 MB) make room for the blocks of a filter (two)
+    ctx, _ = context(g, prec, (6, 6, 6), 5)
+    ctx.apply_h(X, torch.empty_like(X))
+    ctx.cholgs(X0)
+    starved(50 << 20, lambda: ctx.filter(X, 2, 2.0, 80.0, -3.0))
+    ctx.sync_status()
+    ctx.close()
