@@ -130,8 +130,9 @@ gbc_status gbc_get_nonlocal_engine(const gbc_ctx* ctx, int* engine);
  * expired since the previous call (its results are then invalid); in the checked
  * build, GBC_ECHECK if a kernel met a node or row index out of range (the first one,
  * with its site, in gbc_last_error; the access was skipped, results are invalid);
- * GBC_ECUDA for a CUDA error, else GBC_OK.  Clears the recorded flags (they are
- * library-wide, not per context). */
+ * GBC_ECUDA for a CUDA error, else GBC_OK.  Clears the recorded flags.  They are
+ * library-wide, but for the waits of the FP64 products on the tensor cores (FP64 H.X
+ * and what is made of it, Gram matrices, rotations), which each context keeps. */
 gbc_status gbc_sync_status(gbc_ctx* ctx, void* stream);
 
 /* Number M of free FE nodes (spinor DOFs per vector = 2M).  gbc_get_ndof is the
@@ -185,7 +186,10 @@ gbc_status gbc_filter_residual(gbc_ctx* ctx, void* X, int nvec, int ldx, int deg
 /* Cholesky-Gram-Schmidt in the M_D inner product: S = X^H M_D X to FP64
  * accuracy, S = L L^H, X <- X L^-H.  GBC_ENOTPD if S is not positive definite
  * (X is then left unchanged).  Synchronous (reads the pivot status).
- * nvec <= 512. */
+ * nvec <= 512.  GBC_ETIMEOUT if a bounded wait of a tensor-core kernel of this
+ * context expired and gbc_sync_status has not reported it yet: X is unchanged, or
+ * invalid where the wait was the rotation's.  (gbc_rayleigh_ritz, gbc_filter_vjp
+ * and gbc_energy_grad report it likewise.) */
 gbc_status gbc_cholgs(gbc_ctx* ctx, void* X, int nvec, int ldx, void* stream);
 
 /* Rayleigh-Ritz for an M_D-orthonormal block (Sec. III.B.2): Hp = X^H H X
@@ -413,6 +417,8 @@ gbc_status gbc_tc_gemm_nt(const float* A, const float* B, float* D, int M, int N
  * next gbc_sync_status returns GBC_ETIMEOUT (and clears it) while the context
  * stays usable.  Synchronous; GBC_EINVAL for a cap out of range. */
 gbc_status gbc_tc_wait_selftest(int max_iter, void* stream);
+/* The same for the flag that ``ctx`` keeps (see gbc_sync_status). */
+gbc_status gbc_split_wait_selftest(gbc_ctx* ctx, int max_iter, void* stream);
 
 /* ---- deterministic mode ------------------------------------------------------------
  * With ``on`` != 0 the context's FP64 kernels add in a fixed order instead of with

@@ -288,11 +288,13 @@ gbc_status rotate(gbc_ctx* c, cplx<T>* X, int nvec, int ldx, const double2* Q, c
   return GBC_OK;
 }
 
-// waits for the stream; a bounded wait of the split products that expired
+// waits for the stream; a bounded wait of the rotation that expired (those of the Gram matrix are
+// looked at before the rotation, with the pivots and the sweeps: the block is then unchanged)
 gbc_status finish_dense(gbc_ctx* c, cudaStream_t s) {
   int err = 0;
-  GBC_CU(c, split_error(&err, s));
-  if (err) return gbc_fail(c, GBC_ETIMEOUT, "a tensor-core wait expired; the block is invalid");
+  GBC_CU(c, cudaMemcpyAsync(&err, c->d_flag + 1, sizeof(int), cudaMemcpyDeviceToHost, s));
+  GBC_CU(c, cudaStreamSynchronize(s));
+  if (err) return gbc_fail(c, GBC_ETIMEOUT, kSplitExpired);
   return GBC_OK;
 }
 
@@ -481,7 +483,8 @@ gbc_status gbc_create(gbc_ctx** out, int device_ordinal) {
   gbc_ctx* c = new (std::nothrow) gbc_ctx();
   if (!c) return GBC_ENOMEM;
   c->dev = device_ordinal;
-  if (cudaSetDevice(device_ordinal) != cudaSuccess || cudaMalloc(&c->d_flag, sizeof(int)) != cudaSuccess ||
+  if (cudaSetDevice(device_ordinal) != cudaSuccess || cudaMalloc(&c->d_flag, 2 * sizeof(int)) != cudaSuccess ||
+      cudaMemset(c->d_flag, 0, 2 * sizeof(int)) != cudaSuccess ||
       cudaMalloc(&c->d_cell_ctr, sizeof(unsigned long long)) != cudaSuccess) {
     cudaFree(c->d_flag);
     delete c;
@@ -651,10 +654,12 @@ gbc_status gbc_sync_status(gbc_ctx* c, void* stream) {
   GBC_CU(c, tc_nonlocal_error(&err, s));
   int err2 = 0, err3 = 0;
   GBC_CU(c, tcl_error(&err2, s));
-  GBC_CU(c, split_error(&err3, s));
+  GBC_CU(c, cudaMemcpyAsync(&err3, c->d_flag + 1, sizeof(int), cudaMemcpyDeviceToHost, s));
+  GBC_CU(c, cudaStreamSynchronize(s));
   err |= err2 | err3;
   if (err) {
     GBC_CU(c, tc_nonlocal_reset(s));
+    GBC_CU(c, cudaMemsetAsync(c->d_flag + 1, 0, sizeof(int), s));
     GBC_CU(c, cudaStreamSynchronize(s));
     return gbc_fail(c, GBC_ETIMEOUT, "a tensor-core wait expired; results since the last check are invalid");
   }

@@ -295,10 +295,11 @@ gbc_status dense_cholesky_inv_h(gbc_ctx* c, double2* S, int n, double2* Q, cudaS
     k_chol_col<<<nb(m), 256, 0, s>>>(S, L, n, j, c->d_flag);
   }
   GBC_CU(c, cudaGetLastError());
-  int flag = 0;
-  GBC_CU(c, cudaMemcpyAsync(&flag, c->d_flag, sizeof(int), cudaMemcpyDeviceToHost, s));
+  int flag[2] = {0, 0};
+  GBC_CU(c, cudaMemcpyAsync(flag, c->d_flag, sizeof flag, cudaMemcpyDeviceToHost, s));
   GBC_CU(c, cudaStreamSynchronize(s));
-  if (flag) return gbc_fail(c, GBC_ENOTPD, "Cholesky: non-positive pivot (overlap not positive definite)");
+  if (flag[1]) return gbc_fail(c, GBC_ETIMEOUT, kSplitExpired);
+  if (flag[0]) return gbc_fail(c, GBC_ENOTPD, "Cholesky: non-positive pivot (overlap not positive definite)");
   k_tri_inv<<<n, 256, 0, s>>>(L, Linv, n);
   GBC_CU(c, cudaGetLastError());
   k_conj_transpose<<<nb(nn), 256, 0, s>>>(Linv, Q, n);
@@ -332,10 +333,13 @@ gbc_status dense_eigh(gbc_ctx* c, double2* A, int n, double* evals_dev, double2*
     }
     GBC_CU(c, cudaGetLastError());
     double hn[2] = {0, 0};
+    int expired = 0;
     GBC_CU(c, cudaMemsetAsync(norms, 0, 2 * sizeof(double), s));
     k_offnorm<<<64, 256, 0, s>>>(a, n, norms);
     GBC_CU(c, cudaMemcpyAsync(hn, norms, 2 * sizeof(double), cudaMemcpyDeviceToHost, s));
+    if (sweep == 0) GBC_CU(c, cudaMemcpyAsync(&expired, c->d_flag + 1, sizeof(int), cudaMemcpyDeviceToHost, s));
     GBC_CU(c, cudaStreamSynchronize(s));
+    if (expired) return gbc_fail(c, GBC_ETIMEOUT, kSplitExpired);
     if (!(std::isfinite(hn[0]) && std::isfinite(hn[1])))
       return gbc_fail(c, GBC_EINVAL, "eigensolver: non-finite matrix entries");
     // converged when the off-diagonal part is at rounding level, or when it has

@@ -216,7 +216,8 @@ struct gbc_ctx {
   bool deterministic = false;        // FP64 kernels: fixed-order sums instead of atomics
   void* d_small = nullptr;           // small dense scratch (Gram, eigensolver)
   size_t small_bytes = 0;
-  int* d_flag = nullptr;
+  int* d_flag = nullptr;             // [0] Cholesky pivot; [1] an expired wait of the split products,
+                                     // set until gbc_sync_status reports it
   unsigned long long* d_cell_ctr = nullptr;   // work counter of the FP32 cell-apply launches
   int vb32 = 2;                      // FP64 kernel tile (vectors per CTA; fixed)
   int cell_var = 0;                  // FP32 cell-apply variant (GBC_CELL_VARIANTS), set by the tuner
@@ -419,6 +420,7 @@ cudaError_t launch_gram(const cplx<T>* X, const cplx<T>* Y, const double* md, lo
 template <typename T>
 cudaError_t launch_rotate(const cplx<T>* X, const double2* Q, cplx<T>* Out, long long M, int nvec,
                           int ldx, cudaStream_t s);
+constexpr const char* kSplitExpired = "a tensor-core wait of this context expired";
 // split_gemm.cu : Gram matrices and in-place rotations as exact split products on the tensor
 // cores (FP64-accurate; work slot 13)
 struct CUtensorMap_st;
@@ -429,7 +431,6 @@ gbc_status launch_rotate_split(gbc_ctx* c, cplx<T>* X, const double2* Q, long lo
 template <typename TX, typename TY>
 gbc_status launch_gram_split(gbc_ctx* c, const cplx<TX>* X, int ldx, const cplx<TY>* Y, int ldy,
                              const double* md, long long M, int n, double2* Sm, cudaStream_t s);
-cudaError_t split_error(int* err, cudaStream_t s);
 // the FP64 projector contractions in the same form: C1 += P^H X, Y += P C2, with
 // nl_split_bytes in work slot 14
 size_t nl_split_bytes(const gbc_ctx* c, int nvec);

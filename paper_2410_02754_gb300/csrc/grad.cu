@@ -204,7 +204,8 @@ gbc_status download_quad(gbc_ctx* c, const double* g, double* g0, double* g13, c
   return GBC_OK;
 }
 
-// copy g [E][4][q] to the four host arrays and the Hermitian-projected gD to host
+// copy g [E][4][q] to the four host arrays and the Hermitian-projected gD to host; a wait of the
+// split products (FP64) that expired
 gbc_status grad_download(gbc_ctx* c, const GradScratch& gs, double* gV, double* gB, double* gDelta,
                          cudaStream_t s) {
   const ProjDev& pj = c->proj;
@@ -216,7 +217,11 @@ gbc_status grad_download(gbc_ctx* c, const GradScratch& gs, double* gV, double* 
       GBC_CU(c, cudaMemcpyAsync(gDelta, gs.gD, sizeof(double2) * pj.delta_off[pj.natoms],
                                 cudaMemcpyDeviceToHost, s));
   }
-  return download_quad(c, gs.g, gV, gB, s);
+  int err = 0;
+  GBC_CU(c, cudaMemcpyAsync(&err, c->d_flag + 1, sizeof(int), cudaMemcpyDeviceToHost, s));
+  GBC_TRY(download_quad(c, gs.g, gV, gB, s));
+  if (err) return gbc_fail(c, GBC_ETIMEOUT, kSplitExpired);
+  return GBC_OK;
 }
 
 template <typename T>

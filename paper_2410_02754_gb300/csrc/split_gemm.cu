@@ -44,8 +44,6 @@
 
 namespace {
 
-__device__ int g_split_err;   // set when a bounded wait expired
-
 constexpr int kTM = 128;              // tile rows
 constexpr int kKC = 64;               // K chunk: one 128-byte swizzled row
 constexpr int kBad = 0x7fffffff;      // exponent of a row with an infinity or a NaN
@@ -73,6 +71,7 @@ struct SplitArgs {
   int n;                   // complex columns
   int ldo;                 // rotation, EXPD: complex leading dimension of out
   void* out;
+  int* err;                // the context's word for an expired wait
   // PROJ, EXPD: chunks (atom, first node, count, node offset of the atom), supports, projectors
   // and first row of C of an atom
   const int4* chunks;
@@ -382,7 +381,7 @@ k_split_gemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUt
   }
   tc::fence_before_sync();
   __syncthreads();
-  if (failed() && threadIdx.x == 0) atomicExch(&g_split_err, 1);
+  if (failed() && threadIdx.x == 0) atomicExch(a.err, 1);
   if (warp == 0) tc::tmem_dealloc(tmem, 512);
 }
 
@@ -778,12 +777,26 @@ static_assert(GBC_MAX_NPJ <= 32, "a row of projectors is one 64-wide K chunk");
 
 }  // namespace
 
-cudaError_t split_error(int* err, cudaStream_t s) {
-  cudaError_t e = cudaMemcpyFromSymbolAsync(err, g_split_err, sizeof(int), 0, cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  if (e != cudaSuccess || *err == 0) return e;
-  const int zero = 0;
-  return cudaMemcpyToSymbol(g_split_err, &zero, sizeof(int));
+// one warp waits on an mbarrier that nothing arrives at and gives up as k_split_gemm does
+__global__ void k_split_wait_selftest(uint32_t max_iter, int* err) {
+  __shared__ uint64_t bar;
+  if (threadIdx.x == 0) {
+    tc::mbar_init(tc::smem_u32(&bar), 1);
+    tc::fence_mbar_init();
+  }
+  __syncwarp();
+  if (!tc::mbar_wait_bounded(tc::smem_u32(&bar), 0, max_iter) && threadIdx.x == 0) atomicExch(err, 1);
+}
+
+extern "C" gbc_status gbc_split_wait_selftest(gbc_ctx* c, int max_iter, void* stream) {
+  if (!c) return GBC_EINVAL;
+  if (max_iter < 1 || max_iter > (1 << 20)) return gbc_fail(c, GBC_EINVAL, "max_iter must be in [1, 2^20]");
+  cudaStream_t s = (cudaStream_t)stream;
+  GBC_CU(c, cudaSetDevice(c->dev));
+  k_split_wait_selftest<<<1, 32, 0, s>>>((uint32_t)max_iter, c->d_flag + 1);
+  GBC_CU(c, cudaGetLastError());
+  GBC_CU(c, cudaStreamSynchronize(s));
+  return GBC_OK;
 }
 
 // X <- X Q in place, chunk of rows by chunk.  diag: the diagonal of X's Gram matrix (the columns'
@@ -812,7 +825,8 @@ gbc_status launch_rotate_split(gbc_ctx* c, cplx<T>* X, const double2* Q, long lo
     k_split_rows<T><<<(rp + 7) / 8, 256, 0, s>>>(X + r0 * ldx, ldx, n, nr, rp, kp, cs, A, ea);
     GBC_CU(c, cudaGetLastError());
     const int ntn = nb / kTN, tiles = rp / kTM * ntn;
-    SplitArgs a{rp, nb, kp / kKC, kp / kKC, ntn, tiles, tiles, ea, eb, nr, n, ldx, X + r0 * ldx};
+    SplitArgs a{rp, nb, kp / kKC, kp / kKC, ntn, tiles, tiles, ea, eb, nr, n, ldx, X + r0 * ldx,
+                c->d_flag + 1};
     GBC_CU(c, run_split_gemm<MODE>(A, B, kp, a, s));
   }
   return GBC_OK;
@@ -865,7 +879,7 @@ gbc_status launch_gram_split(gbc_ctx* c, const cplx<TX>* X, int ldx, const cplx<
     const int split = std::max(1, std::min(nwin, gbc_sm_count() / std::max(1, tiles)));
     const int kper = (nwin + split - 1) / split * kFlush;
     const int parts = (rp / kKC + kper - 1) / kper;
-    SplitArgs a{ma, nb, rp / kKC, kper, ntn, tiles, tiles * parts, ea, eb, nr, n, 0, Sm};
+    SplitArgs a{ma, nb, rp / kKC, kper, ntn, tiles, tiles * parts, ea, eb, nr, n, 0, Sm, c->d_flag + 1};
     GBC_CU(c, run_split_gemm<GRAM>(A, B, rp, a, s));
   }
   if (md) k_set_diag<<<1, 256, 0, s>>>(diag, n, Sm);
@@ -920,7 +934,7 @@ cudaError_t nl_split_project(gbc_ctx* c, const double2* X, int nvec, int ldx, do
     k_split_nodes<true><<<dim3(n, 1), 256, 0, s>>>(pj.d_P64, 0, 0, ch, pj.d_nodes, pj.d_atom_npj,
                                                       pj.d_atom_pv_off, c->mesh.M, 64, kp, B, eb);
     const int ntm = cols / kTM;
-    SplitArgs a{cols, 64, 0, 0, ntm, n * ntm, n * ntm, ea, eb, 0, nvec, 0, C1, ch, pj.d_nodes,
+    SplitArgs a{cols, 64, 0, 0, ntm, n * ntm, n * ntm, ea, eb, 0, nvec, 0, C1, c->d_flag + 1, ch, pj.d_nodes,
                 pj.d_atom_npj, pj.d_atom_c_off};
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = run_split_gemm<PROJ>(A, B, kp, a, s);
@@ -944,7 +958,7 @@ cudaError_t nl_split_expand(gbc_ctx* c, double2* Y, int nvec, int ldx, const dou
     k_split_proj<true><<<rb / 8, 256, 0, s>>>(C2, nvec, rb, cols, ch, pj.d_atom_npj,
                                                  pj.d_atom_c_off, B, eb);
     const int ntn = cols / kTN, tiles = ra / kTM * ntn;
-    SplitArgs a{ra, rb, 1, 1, ntn, tiles, tiles, ea, eb, c->mesh.M, nvec, ldx, Y, ch, pj.d_nodes,
+    SplitArgs a{ra, rb, 1, 1, ntn, tiles, tiles, ea, eb, c->mesh.M, nvec, ldx, Y, c->d_flag + 1, ch, pj.d_nodes,
                 pj.d_atom_npj, pj.d_atom_c_off};
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = run_split_gemm<EXPD>(A, B, 64, a, s);

@@ -34,7 +34,7 @@ EXPORTS = ["gbc_create", "gbc_destroy", "gbc_last_error", "gbc_version", "gbc_se
            "gbc_apply_h_noalloc", "gbc_batch_create", "gbc_batch_destroy",
            "gbc_batch_last_error", "gbc_batch_filter", "gbc_batch_launches", "gbc_tune",
            "gbc_get_tile", "gbc_filter_vjp", "gbc_energy_grad", "gbc_set_delta",
-           "gbc_tc_gemm_nt", "gbc_tc_wait_selftest", "gbc_set_nonlocal_engine", "gbc_get_nonlocal_engine",
+           "gbc_tc_gemm_nt", "gbc_tc_wait_selftest", "gbc_split_wait_selftest", "gbc_set_nonlocal_engine", "gbc_get_nonlocal_engine",
            "gbc_sync_status", "gbc_density", "gbc_density_dev", "gbc_fermi_occupations",
            "gbc_prolongate", "gbc_scf_fields", "gbc_anderson_mix", "gbc_get_ndof",
            "gbc_filter_backward", "gbc_alu_peak", "gbc_set_cell_variant",
@@ -103,6 +103,7 @@ def load_library(path: str = LIB_PATH):
         "gbc_anderson_mix": ([P, ct.POINTER(V), ct.POINTER(V), I, D, V, DP, DP, V], I),
         "gbc_tc_gemm_nt": ([V, V, V, I, I, I, V], I),
         "gbc_tc_wait_selftest": ([I, V], I),
+        "gbc_split_wait_selftest": ([P, I, V], I),
         "gbc_build_info": ([IP], I),
         "gbc_set_deterministic": ([P, I], I),
         "gbc_get_deterministic": ([P, IP], I),
@@ -254,6 +255,10 @@ class Context:
         e = ct.c_int()
         self._chk(self.lib.gbc_get_nonlocal_engine(self.h, ct.byref(e)))
         return e.value
+
+    def split_wait_selftest(self, max_iter=1000, stream=None):
+        """Make one bounded device wait expire on purpose (see gbc_split_wait_selftest)."""
+        self._chk(self.lib.gbc_split_wait_selftest(self.h, int(max_iter), _stream_ptr(stream)))
 
     def sync_status(self, stream=None):
         """Synchronise and raise if a device-side bounded wait expired."""

@@ -228,3 +228,30 @@ def test_no_memory_for_the_digits(g, prec):
     starved(50 << 20, lambda: ctx.filter(X, 2, 2.0, 80.0, -3.0))
     ctx.sync_status()
     ctx.close()
+
+
+def test_expired_wait_belongs_to_its_context(g):
+    """An expired wait of the split products is reported by the synchronous calls of its own context,
+    with the block unchanged, until gbc_sync_status has reported it, and by no other context."""
+    (a, prob), (b, _) = context(g, 0, (3, 3, 2), 3), context(g, 0, (3, 3, 2), 3)
+    X = device(block(prob.nnodes, 20, 3), 0, 20)
+    keep = X.clone()
+    a.split_wait_selftest()
+    b.sync_status()
+    Y = X.clone()
+    b.cholgs(Y)
+    ritz = b.rayleigh_ritz(Y)
+    bounds = (2.0, 80.0, -3.0)
+    calls = [lambda: a.cholgs(X), lambda: a.rayleigh_ritz(X),
+             lambda: a.filter_vjp(X, Y, torch.empty_like(X), 3, *bounds),
+             lambda: a.energy_grad(X, np.ones(20), torch.empty_like(X)), a.sync_status]
+    for call in calls:
+        with pytest.raises(g.GbcError) as e:
+            call()
+        assert e.value.status == 6                       # GBC_ETIMEOUT
+        assert torch.equal(X, keep)
+    a.sync_status()                                      # cleared
+    a.cholgs(X)
+    assert np.abs(a.rayleigh_ritz(X) - ritz).max() < 1e-11 * np.abs(ritz).max()
+    a.close()
+    b.close()
