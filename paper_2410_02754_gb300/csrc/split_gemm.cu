@@ -342,8 +342,10 @@ k_split_gemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUt
                 v[q] = fma(__ll2double_rn(lo[i + q]), 0x1p-24, __ll2double_rn(hi[i + q]));
               else
                 v[q] = __ll2double_rn(value(i + q, sh));
-              const int e = eb[i + q], x = ea + e - 24 - sh;
-              if (ea == kBad || e == kBad) v[q] = NAN;
+              const int e = eb[i + q];
+              const bool bad = ea == kBad || e == kBad;
+              const int x = bad ? 0 : ea + e - 24 - sh;
+              if (bad) v[q] = NAN;
               else if (abs(x) > 900) v[q] = scalbn(v[q], x);
               else if (v[q] != 0.0)   // a multiplication by 2^x on the integer pipe (2^-24 <= |v| < 2^63)
                 v[q] = __hiloint2double(__double2hiint(v[q]) + (x << 20), __double2loint(v[q]));
