@@ -7,8 +7,11 @@
 //   X_f[J] = sum_I N^{p_c}_I(r_J) X_c[I],
 //
 // per cell a tensor product of the 1-D matrix T[j][i] = l^{p_c}_i(x^{p_f}_j),
-// applied in three sum-factorised stages, each 1-D product in even-odd form (the GLL nodes are
-// symmetric).  p_f = p_c is the identity: a copy.
+// applied in three sum-factorised stages.  The first and last rows of T are unit rows (the GLL nodes
+// share their end points): those values are copied.  The other rows are dense products: with the
+// ends copied these take 30 paired multiply-adds a pencil at p = 5 -> 6, the even-odd form 33
+// instructions, and even-odd sums of entries that are close to 0 and 1 lose accuracy (relative error
+// on uniform random blocks 1.01e-7 at p = 5 -> 6, 8.0e-8 dense).  p_f = p_c is the identity: a copy.
 //
 // One CTA per (cell, tile of kLanes 16-byte elements a node row: 8 FP32 or 4 FP64 vectors), the
 // tiles of a cell next to each other so that they share its node rows' sectors in L2.  A thread
@@ -21,7 +24,9 @@
 // index < p_f in every direction); with the periodic wrap and the Dirichlet faces this writes
 // every free fine node exactly once, with no atomics.  HBM-bound in the limit (the coarse block
 // read and the fine block written once).  Measured on one GB300, 16^3 cells, p = 5 -> 6, 256 FP32
-// vectors: 2.91 ms with dense scalar products on 8-byte elements (issue-bound), 1.53 ms now.
+// vectors: 2.91 ms with scalar products of every row on 8-byte elements (issue-bound), 1.53 ms with
+// even-odd products on 16-byte elements, 1.37 ms now.  FP64, 64 vectors: p = 3 -> 4 on 20^3 cells 4.13,
+// 3.88, 2.63 ms; p = 6 -> 7 on 12^3 cells 6.98, 5.76, 6.10 ms.
 #include "hx_cell.cuh"
 
 namespace {
@@ -32,9 +37,10 @@ constexpr int kLanes = 4;       // 16-byte elements of a node row per CTA
 constexpr int kThreads = 192;
 
 template <typename T> __host__ __device__ constexpr int vecs_per_elem() { return sizeof(T) == 4 ? 2 : 1; }
-template <typename T, int NC, int NF> struct TwoGridTab;
-template <int NC, int NF> struct TwoGridTab<float, NC, NF> { EO2<NF, NC> t; };
-template <int NC, int NF> struct TwoGridTab<double, NC, NF> { EO<double, NF, NC> t; };
+// rows 1 .. NF-2 of T; FP32: every entry twice, the multiplier of a paired multiply-add on (re, im)
+template <typename T, int NC, int NF> struct TwoGridTab {
+  typename std::conditional<sizeof(T) == 4, float2, double>::type t[NF - 2][NC];
+};
 
 // asynchronous global -> shared copy of N bytes, of which src_bytes are read and the rest zero
 template <int N> __device__ __forceinline__ void cp_async_n(void* dst, const void* src, int src_bytes) {
@@ -51,28 +57,33 @@ template <int N> __device__ __forceinline__ void cp_async_n(void* dst, const voi
                  : "memory");
 }
 
-// one 1-D product: ld(j) -> the NC inputs, st(row, value) for the NF outputs
-template <int NC, int NF, typename L, typename S>
-__device__ __forceinline__ void line(const TwoGridTab<float, NC, NF>& tb, L ld, S st) {
-  Parts<NC> s;
-  load_parts<true>(s, ld);
-#pragma unroll
-  for (int i = 0; i < (NF + 1) / 2; ++i) {
-    Acc a;
-    row_sym<true, NF>(tb.t, i, s, a);
-    put_rows<true, NF>(i, a, st);
-  }
+__device__ __forceinline__ float4 t_mul(float2 m, float4 x) {
+  return cat2(p_mul(m, lo2(x)), p_mul(m, hi2(x)));
 }
-template <int NC, int NF, typename L, typename S>
-__device__ __forceinline__ void line(const TwoGridTab<double, NC, NF>& tb, L ld, S st) {
-  PartsD<NC> s;
-  load_parts(s, ld);
+__device__ __forceinline__ float4 t_fma(float2 m, float4 x, float4 a) {
+  return cat2(p_fma(m, lo2(x), lo2(a)), p_fma(m, hi2(x), hi2(a)));
+}
+__device__ __forceinline__ double2 t_mul(double m, double2 x) { return make_double2(m * x.x, m * x.y); }
+__device__ __forceinline__ double2 t_fma(double m, double2 x, double2 a) {
+  return make_double2(fma(m, x.x, a.x), fma(m, x.y, a.y));
+}
+
+// one 1-D product: ld(j) -> the NC inputs, st(row, value) for the NF outputs
+template <typename T, int NC, int NF, typename L, typename S>
+__device__ __forceinline__ void line(const TwoGridTab<T, NC, NF>& tb, L ld, S st) {
+  using E = decltype(ld(0));
+  E in[NC];
 #pragma unroll
-  for (int i = 0; i < (NF + 1) / 2; ++i) {
-    AccD a;
-    row_sym<true, NF>(tb.t, i, s, a);
-    put_rows<NF>(i, a, st);
+  for (int j = 0; j < NC; ++j) in[j] = ld(j);
+  st(0, in[0]);
+#pragma unroll
+  for (int i = 1; i < NF - 1; ++i) {
+    E a = t_mul(tb.t[i - 1][0], in[0]);
+#pragma unroll
+    for (int j = 1; j < NC; ++j) a = t_fma(tb.t[i - 1][j], in[j], a);
+    st(i, a);
   }
+  st(NF - 1, in[NC - 1]);
 }
 
 template <int NC> __host__ __device__ constexpr int odd_stride() { return NC | 1; }   // of A's x pencils
@@ -188,21 +199,17 @@ __global__ void k_copy_cols(const cplx<T>* __restrict__ X, int ldx, cplx<T>* __r
 template <typename T, int NC, int NF>
 cudaError_t launch_prolongate_t(const gbc_ctx* cc, const gbc_ctx* cf, const cplx<T>* Xc, int ldxc,
                                 cplx<T>* Xf, int ldxf, int nvec, cudaStream_t s) {
-  std::vector<double> m((size_t)NF * NC);   // coarse Lagrange basis at the fine GLL nodes
+  TwoGridTab<T, NC, NF> tb;   // coarse Lagrange basis at the fine GLL nodes
   const std::vector<double>& xc = cc->tab.gll_x;
   const std::vector<double>& xf = cf->tab.gll_x;
-  for (int j = 0; j < NF; ++j)
+  for (int j = 1; j < NF - 1; ++j)
     for (int i = 0; i < NC; ++i) {
       double l = 1.0;
       for (int k = 0; k < NC; ++k)
         if (k != i) l *= (xf[j] - xc[k]) / (xc[i] - xc[k]);
-      m[j * NC + i] = l;
+      if constexpr (sizeof(T) == 4) tb.t[j - 1][i] = make_float2((float)l, (float)l);
+      else tb.t[j - 1][i] = l;
     }
-  EO<T, NF, NC> eo;
-  if (!make_eo<T, NF, NC>(m, 1, &eo)) return cudaErrorInvalidValue;
-  TwoGridTab<T, NC, NF> tb;
-  if constexpr (sizeof(T) == 4) cvt_table(eo, tb.t);
-  else tb.t = eo;
   constexpr size_t smem = 16 * (size_t)kLanes * (points_a<NC, NF>() + NF * NC * NC);
   auto k = k_prolongate<T, NC, NF>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

@@ -114,3 +114,22 @@ def test_prolongate_argument_errors(g):
     assert not xf.abs().max().item()
     for c in (cc, cf, bad, far):
         c.close()
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("pc", [2, 3, 4, 5, 6])
+def test_shared_nodes_are_copied(g, pc, prec):
+    """The GLL nodes of both orders share the cell's end points, where the interpolation matrix has
+    unit rows: values at the cell vertices come over bit for bit."""
+    base = syn.make_problem(ncell=(2, 3, 2), h=(1.0, 0.9, 1.2), p=pc, natoms=0, seed=pc)
+    cc, cf = contexts(g, base, pc + 1, prec)
+    dt = torch.complex128 if prec == 0 else torch.complex64
+    xc = torch.from_numpy(syn.random_block(base.nnodes, 5, pc)).to(dt).cuda()
+    xf = torch.empty((cf.nnodes, 2, 5), dtype=dt, device="cuda")
+    cf.prolongate_from(cc, xc, xf)
+    box = [tuple(n * p for n in base.ncell[::-1]) + (2, 5) for p in (pc, pc + 1)]   # periodic
+    a = xc.reshape(box[0])[::pc, ::pc, ::pc]
+    b = xf.reshape(box[1])[::pc + 1, ::pc + 1, ::pc + 1]
+    assert torch.equal(a, b)
+    cc.close()
+    cf.close()
