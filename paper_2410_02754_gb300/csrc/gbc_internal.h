@@ -127,6 +127,7 @@ template <typename T, int NP, int NQ> struct Tables1D {
 struct HostTables {
   int p = 0, nq = 0;
   std::vector<double> gll_x, gll_w, gq_x, gq_w;
+  std::vector<double> gq_s;                    // FP32 tables: factor of the interpolation to a point
   std::vector<double> N1, D1;                  // [np][nq] values / d/dxi at Gauss points
   std::vector<double> Bh, Ah, Ch;              // [np][np] reference 1-D mass, stiffness, advection
 };

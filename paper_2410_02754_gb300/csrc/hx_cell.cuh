@@ -6,7 +6,7 @@
 // of Eq. FEHloc (per-cell Hermitian form), and Eq. chebfilt for the recurrence.
 //
 // Algorithm: with N' = N diag(sqrt(w_q)) (nodes x Gauss points, so that the 1-D mass is
-// (h/2) N' N'^T) and the 1-D kinetic / k operators G_d,
+// (h/2) N' N'^T; the tables split w_q unevenly, so that they round best to FP32) and the 1-D kinetic / k operators G_d,
 //   a  = N'_x^T X,  t1 = B_x X,  t2 = G_x X                      x pencils (n_p^2)
 //   u  = N'_y^T a;  c  = G_y t1 + B_y t2                          y pencils (n_q n_p; n_p^2)
 //   w  = N'_z F N'_z^T u + G'_z u;  k = B_z c                     z pencils (n_q^2; n_p^2)
@@ -77,8 +77,8 @@ template <int NP, int NQ, bool PACKED> struct CellTables {
   M<NP, NP> B[3];    // 1-D Gauss mass
   M<NP, NP> Gr[3];   // 1/2 A_d (z: times h_x h_y / 4)
   M<NP, NP> Gi[3];   // -1/2 k_d (C^ - C^T) (z: times h_x h_y / 4)
-  M<NQ, NP> Ni;      // N'^T: interpolation to the Gauss points times sqrt(w_q)
-  M<NP, NQ> Nt;      // N'
+  M<NQ, NP> Ni;      // N'^T: interpolation to the Gauss points times s_q (gq_s)
+  M<NP, NQ> Nt;      // N': times w_q / s_q
 };
 
 // One system of a launch.

@@ -83,8 +83,8 @@ template <typename T, int NP, int NQ> struct TablesEO {
   EO<T, NP, NP> B[3];    // 1-D Gauss mass h_d/2 B^               (symmetric)
   EO<T, NP, NP> Gr[3];   // 1/2 A_d (z: times h_x h_y / 4)          (symmetric)
   EO<T, NP, NP> Gi[3];   // -1/2 k_d (C^ - C^T) (z: the same)       (antisymmetric)
-  EO<T, NQ, NP> Ni;      // N'^T: interpolation times sqrt(w_q)      (symmetric)
-  EO<T, NP, NQ> Nt;      // N'                                       (symmetric)
+  EO<T, NQ, NP> Ni;      // N'^T: interpolation times sqrt(w_q), or s_q (FP32: gq_s)   (symmetric)
+  EO<T, NP, NQ> Nt;      // N': times w_q over that factor                             (symmetric)
 };
 
 // host: even-odd split of a dense row-major NO x NI matrix (checks the symmetry)
@@ -130,7 +130,10 @@ inline bool make_tables_eo(const gbc_ctx* c, TablesEO<T, NP, NQ>* t) {
   std::vector<double> Ni(NQ * NP), Nt(NP * NQ);
   for (int i = 0; i < NP; ++i)
     for (int q = 0; q < NQ; ++q) {
-      Ni[q * NP + i] = Nt[i * NQ + q] = h.N1[i * NQ + q] * std::sqrt(h.gq_w[q]);
+      const bool f32 = std::is_same<T, float>::value;
+      const double s = f32 ? h.gq_s[q] : std::sqrt(h.gq_w[q]);
+      Ni[q * NP + i] = h.N1[i * NQ + q] * s;
+      Nt[i * NQ + q] = h.N1[i * NQ + q] * (f32 ? h.gq_w[q] / s : s);
     }
   ok = ok && make_eo<T, NQ, NP>(Ni, 1, &t->Ni) && make_eo<T, NP, NQ>(Nt, 1, &t->Nt);
   return ok;

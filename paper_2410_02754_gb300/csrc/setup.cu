@@ -100,6 +100,39 @@ void lagrange_at(const std::vector<double>& xn, double t, std::vector<double>& L
 
 }  // namespace
 
+// The FP32 cell apply interpolates with N diag(s) and projects back with N diag(w / s); any s > 0,
+// symmetric like w, gives the same operator.  Which s is chosen decides how the even-odd entries of
+// the two tables round to FP32, and that rounding is most of the operator's error: with s = sqrt(w)
+// H.X is off by 1.14e-7 at p = 4, with the s of least squared rounding error among 256 within a
+// factor sqrt(2) of it by 8.6e-8 (uniform random vectors; p = 2, 3, 5, 6, 7: 1.43 -> 1.19, 0.96 -> 0.86,
+// 1.01 -> 0.89, 0.94 -> 0.87 and 0.95 -> 0.90e-7).
+static std::vector<double> interpolation_factors(const HostTables& t) {
+  const int np = t.p + 1, nq = t.nq;
+  auto sq = [](double v) { return (v - (float)v) * (v - (float)v); };
+  // squared rounding error of the even-odd entries of N[., q] f, relative to f
+  auto error = [&](int q, double f) {
+    double e = 0.0;
+    for (int i = 0; i < (np + 1) / 2; ++i) {
+      const double a = t.N1[i * nq + q] * f, b = t.N1[(np - 1 - i) * nq + q] * f;
+      e += i == np - 1 - i ? sq(a) : 2.0 * (sq(0.5 * (a + b)) + sq(0.5 * (a - b)));
+    }
+    return e / (f * f);
+  };
+  std::vector<double> s(nq);
+  for (int q = 0; q < (nq + 1) / 2; ++q) {
+    double best = 1e300;
+    for (int k = 0; k < 256; ++k) {
+      const double f = std::sqrt(t.gq_w[q]) * std::exp2(k / 256.0 - 0.5);
+      const double e = error(q, f) + error(q, t.gq_w[q] / f);
+      if (e < best) {
+        best = e;
+        s[q] = s[nq - 1 - q] = f;
+      }
+    }
+  }
+  return s;
+}
+
 gbc_status setup_tables(gbc_ctx* c) {
   HostTables& t = c->tab;
   const int p = c->mesh.p, np1 = p + 1, nq = c->nq;
@@ -132,6 +165,7 @@ gbc_status setup_tables(gbc_ctx* c) {
       t.Ah[i * np1 + j] = a;
       t.Ch[i * np1 + j] = cc;
     }
+  t.gq_s = interpolation_factors(t);
   return GBC_OK;
 }
 
@@ -154,7 +188,7 @@ __global__ void k_mass(const MeshDev m, const double* mx, const double* my, cons
 }
 
 // fields[e][q][c] = J * {V + |k|^2/2, bx, by, bz}[e][q] in FP64 and FP32 (the interpolation
-// tables carry sqrt(w_q) on both sides of them)
+// tables carry w_q)
 __global__ void k_fields(const double* raw, long long E, int nq, double jac, double k2half,
                          double* f64, float* f32) {
   const long long nq3 = (long long)nq * nq * nq;
