@@ -354,8 +354,8 @@ gbc_status gbc_batch_launches(const gbc_batch* batch, int* kernels_per_call);
  * mode, and, when the context has projectors the tensor-core engine takes, the
  * SIMT and tcgen05 nonlocal engines, on a scratch block of ``nvec`` vectors (CUDA
  * events, median of three after a warm-up), and keeps the fastest of each.  The
- * choice is cached per (device, FP32, p, k != 0, nvec rounded up to a power of
- * two) for the process and, when the environment variable GBC_TUNE_CACHE names a
+ * choice is cached per (device, version of the kernels, FP32, p, k != 0, nvec
+ * rounded up to a power of two) for the process and, when the environment variable GBC_TUNE_CACHE names a
  * file, across processes in that JSON file (with the measured times).
  * Synchronous.  Uses the context's workspace. */
 gbc_status gbc_tune(gbc_ctx* ctx, int nvec, void* stream);
@@ -364,7 +364,7 @@ gbc_status gbc_get_tile(const gbc_ctx* ctx, int* vectors_per_cta);
 /* Set (overriding the tuner) / read the FP32 cell-apply variant, 0 ..
  * GBC_CELL_VARIANTS - 1: 0 = 2 vectors per work item x 256 threads with registers
  * for 2 CTAs per SM, paired FP32 multiply-adds on (re, im); 1 = the same with
- * registers for 3 CTAs per SM; 2 and 3 = variants 0 and 1 with scalar FP32
+ * registers for 3 CTAs per SM (p <= 5; above, variant 0); 2 and 3 = variants 0 and 1 with scalar FP32
  * multiply-adds; 4 = 4 vectors x 512 threads, one CTA per SM, paired
  * multiply-adds.  A CTA's threads form independent groups that each work on one
  * item (one cell, 2 or 4 vectors) at a time.  gbc_get_cell_variant also returns

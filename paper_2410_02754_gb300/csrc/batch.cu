@@ -102,7 +102,11 @@ void tune_store() {
   std::fclose(fp);
 }
 
-// key: device, precision, order p, k != 0, vectors (rounded up to a power of two)
+// What a variant number stands for, and how fast it is, changes with the kernels: raise this then, and
+// times that an earlier library left in a cache file choose nothing.
+constexpr int kTuneVersion = 2;
+
+// key: device, kernel version, precision, order p, k != 0, vectors (rounded up to a power of two)
 std::string tune_key(const gbc_ctx* c, int nvec) {
   cudaDeviceProp prop;
   std::string dev = "gpu";
@@ -113,8 +117,8 @@ std::string tune_key(const gbc_ctx* c, int nvec) {
   int bucket = 1;
   while (bucket < nvec) bucket <<= 1;
   char buf[256];
-  std::snprintf(buf, sizeof buf, "%s/fp32/p%d/k%d/nvec%d", dev.c_str(), c->mesh.p, kpt ? 1 : 0,
-                bucket);
+  std::snprintf(buf, sizeof buf, "%.200s/v%d/fp32/p%d/k%d/nvec%d", dev.c_str(), kTuneVersion, c->mesh.p,
+                kpt ? 1 : 0, bucket);
   return buf;
 }
 

@@ -165,3 +165,30 @@ def test_every_cell_variant_matches_oracle(g, var, case):
     ref = oc.cheb_filter(d.apply_htilde, X, 3, *bounds)
     assert rel(Xd.cpu().numpy().astype(np.complex128), ref) < 2e-5
     c.close()
+
+
+def test_tuner_ignores_times_of_other_kernels(g, tmp_path):
+    """A cache file that a library with other kernels wrote (no version in the key) chooses nothing:
+    the variants are timed again."""
+    import json
+    import os
+    import subprocess
+    import sys
+    dev = torch.cuda.get_device_name(0).replace(" ", "_")
+    path = tmp_path / "tune.json"
+    old = {f"{dev}/fp32/p3/k0/nvec8": {"variant": 3, "nl_engine": -1, "ms": [9.0, 9.0, 9.0, 0.1, 9.0],
+                                       "nl_ms": [0.0, 0.0]}}
+    path.write_text("{\n" + ",\n".join(f'  "{k}": {json.dumps(v)}' for k, v in old.items()) + "\n}\n")
+    code = ("import synthetic as syn, paper_2410_02754_gb300 as g\n"
+            "c = g.Context(0)\n"
+            "c.set_problem(syn.make_problem(ncell=(3, 3, 3), h=(1.0, 1.0, 1.0), p=3, seed=1))\n"
+            "c.set_precision(1)\n"
+            "c.tune(8)\n"
+            "print(c.cell_variant()[0])\n")
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    out = subprocess.run([sys.executable, "-c", code], cwd=root, text=True, capture_output=True, check=True,
+                         env=dict(os.environ, GBC_TUNE_CACHE=str(path), PYTHONPATH=root))
+    data = json.loads(path.read_text())
+    new = [k for k in data if k not in old]
+    assert len(new) == 1 and new[0].endswith("/fp32/p3/k0/nvec8"), list(data)
+    assert data[new[0]]["variant"] == int(out.stdout) and min(data[new[0]]["ms"]) > 0
