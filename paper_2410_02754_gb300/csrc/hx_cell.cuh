@@ -759,10 +759,13 @@ cudaError_t launch_cell_group(const CellJob* jobs, int n, cudaStream_t s) {
     case 3: return launch_cell_group_p<4, VB, NT, MINB, PACKED>(jobs, n, s);
     case 4: return launch_cell_group_p<5, VB, NT, MINB, PACKED>(jobs, n, s);
     case 5: return launch_cell_group_p<6, VB, NT, MINB, PACKED>(jobs, n, s);
-    case 6: return launch_cell_group_p<7, VB, NT, MINB, PACKED>(jobs, n, s);
-    case 7: return launch_cell_group_p<8, VB, NT, MINB, PACKED>(jobs, n, s);
-    default: return cudaErrorInvalidValue;
+    default: break;
   }
+  if constexpr (MINB < 3) {   // see launch_cell_f32
+    if (jobs[0].c->mesh.p == 6) return launch_cell_group_p<7, VB, NT, MINB, PACKED>(jobs, n, s);
+    if (jobs[0].c->mesh.p == 7) return launch_cell_group_p<8, VB, NT, MINB, PACKED>(jobs, n, s);
+  }
+  return cudaErrorInvalidValue;
 }
 
 }  // namespace gbc

@@ -1,5 +1,6 @@
-// FP32 cell apply, variant 1: 2 vectors per item, 256 threads, registers sized for 3 CTAs per SM, paired FP32 multiply-adds
-// (p = 2..7, nq = p + 2).
+// FP32 cell apply, variant 1: 2 vectors per item, 256 threads, registers sized for 3 CTAs per SM,
+// paired FP32 multiply-adds
+// (p = 2..5, nq = p + 2).
 #include "hx_cell.cuh"
 
 cudaError_t launch_cell_f32_v1(const CellJob* jobs, int n, cudaStream_t s) {
