@@ -568,76 +568,90 @@ __device__ __forceinline__ void cell_body(const CellSys* __restrict__ sys, int n
     }
     psync();
 
-    // ---- x pencils: N' T1 + T2, assembled (vector fastest across threads)
-    for (int u = ut; u < VB * NP * nz; u += US) {
-      const int v = u % VB, pen = u / VB;
-      const int y = pen % NP, z = z0 + pen / NP;
-      const int vec = vbase + v;
-      if (vec >= d.nvec) continue;
-      float4 out[NP];
-      {
-        const float4* Q = T1b(v) + pq(0, y, z);
-        const float4* K = T2b(v) + pa(0, y, z);
-        Parts<NQ> s;
-        load_parts<PACKED>(s, [&](int j) { return Q[j]; });
+    // ---- x pencils: N' T1 + T2, assembled (vector fastest across threads; NS spins a thread)
+    auto assemble = [&](auto ns) {
+      constexpr int NS = decltype(ns)::value;
+      for (int u = ut; u < VB * NP * nz * (3 - NS); u += US) {
+        const int s0 = NS == 2 ? 0 : u / (VB * NP * NP);
+        const int v = u % VB, pen = (u - s0 * VB * NP * NP) / VB;
+        const int y = pen % NP, z = z0 + pen / NP;
+        const int vec = vbase + v;
+        if (vec >= d.nvec) continue;
+        float2 out[NS][NP];
+        {
+          const float4* Q = T1b(v) + pq(0, y, z);
+          const float4* K = T2b(v) + pa(0, y, z);
+          // both spins of a point, or one of them twice (what the second half would do is not compiled)
+          auto ld = [&](const float4* p) {
+            if (NS == 2) return *p;
+            const float2 a = reinterpret_cast<const float2*>(p)[s0];
+            return cat2(a, a);
+          };
+          Parts<NQ> s;
+          load_parts<PACKED>(s, [&](int j) { return ld(Q + j); });
 #pragma unroll
-        for (int i = 0; i < HP; ++i) {
-          Acc a;
-          row_sym<true, NP>(tb.Nt, i, s, a);
-          put_rows<PACKED, NP>(i, a, [&](int r, float4 val) {
-            const float4 k = K[r];
-            out[r] = cat2(c_add<PACKED>(lo2(val), lo2(k)), c_add<PACKED>(hi2(val), hi2(k)));
-          });
+          for (int i = 0; i < HP; ++i) {
+            Acc a;
+            row_sym<true, NP>(tb.Nt, i, s, a);
+            put_rows<PACKED, NP>(i, a, [&](int r, float4 val) {
+              const float4 k = ld(K + r);
+              out[0][r] = c_add<PACKED>(lo2(val), lo2(k));
+              if (NS == 2) out[NS - 1][r] = c_add<PACKED>(hi2(val), hi2(k));
+            });
+          }
         }
-      }
-      const bool yz_in = y > 0 && y < NP - 1 && z > 0 && z < NP - 1;
-      const int Iyz = no[8 + y] + no[16 + z];
+        const bool yz_in = y > 0 && y < NP - 1 && z > 0 && z < NP - 1;
+        const int Iyz = no[8 + y] + no[16 + z];
 #pragma unroll
-      for (int s = 0; s < 2; ++s) {
-        if (d.cheb && yz_in) {
-          // nodes x = 1 .. NP-2 of this pencil are interior to the cell: every load is
-          // issued before the first update (X_out may alias X_prev), so their latencies
-          // overlap
-          float2 yv[NIN], xv[NIN], pv[NIN];
-          const long long step = 2 * (long long)d.ldx;
-          const int I1 = Iyz + no[1];   // consecutive from here
-          const long long o1 = I1 * step + (long long)s * d.ldx + vec;
-          const float* w = wint + ((z - 1) * NIN + y - 1) * NIN;
+        for (int si = 0; si < NS; ++si) {
+          const int s = s0 + si;
+          if (d.cheb && yz_in) {
+            // nodes x = 1 .. NP-2 of this pencil are interior to the cell: every load is
+            // issued before the first update (X_out may alias X_prev), so their latencies
+            // overlap
+            float2 yv[NIN], xv[NIN], pv[NIN];
+            const long long step = 2 * (long long)d.ldx;
+            const int I1 = Iyz + no[1];   // consecutive from here
+            const long long o1 = I1 * step + (long long)s * d.ldx + vec;
+            const float* w = wint + ((z - 1) * NIN + y - 1) * NIN;
 #pragma unroll
-          for (int j = 0; j < NIN; ++j) {
-            const long long o = o1 + j * step;
-            if (GBC_IN_RANGE(GBC_SITE_CELL_STORE, I1 + j, d.mesh.M)) {
-              yv[j] = d.Y[o];
-              xv[j] = __ldg(&d.X[o]);
-              pv[j] = d.Xprev ? d.Xprev[o] : make_float2(0.f, 0.f);
-            } else {
-              yv[j] = xv[j] = pv[j] = make_float2(0.f, 0.f);
+            for (int j = 0; j < NIN; ++j) {
+              const long long o = o1 + j * step;
+              if (GBC_IN_RANGE(GBC_SITE_CELL_STORE, I1 + j, d.mesh.M)) {
+                yv[j] = d.Y[o];
+                xv[j] = __ldg(&d.X[o]);
+                pv[j] = d.Xprev ? d.Xprev[o] : make_float2(0.f, 0.f);
+              } else {
+                yv[j] = xv[j] = pv[j] = make_float2(0.f, 0.f);
+              }
+            }
+#pragma unroll
+            for (int j = 0; j < NIN; ++j) {
+              const long long o = o1 + j * step;
+              const float2 yt = p_add(yv[j], out[si][1 + j]);
+              const float2 xn = p_fma(dup(-d.cb), pv[j],
+                                      p_mul(dup(d.ca), p_fma(dup(-d.cc), xv[j], p_mul(dup(w[j]), yt))));
+              if (GBC_IN_RANGE(GBC_SITE_CELL_STORE, I1 + j, d.mesh.M)) d.Xout[o] = xn;
+            }
+#pragma unroll
+            for (int i = 0; i < NP; i += NP - 1) {   // the pencil's two face nodes
+              const int I = Iyz + no[i];
+              if (I >= 0 && GBC_IN_RANGE(GBC_SITE_CELL_STORE, I, d.mesh.M))
+                atomicAdd(&d.Y[((long long)I * 2 + s) * d.ldx + vec], out[si][i]);
+            }
+          } else {
+#pragma unroll
+            for (int i = 0; i < NP; ++i) {
+              const int I = Iyz + no[i];
+              if (I >= 0 && GBC_IN_RANGE(GBC_SITE_CELL_STORE, I, d.mesh.M))
+                atomicAdd(&d.Y[((long long)I * 2 + s) * d.ldx + vec], out[si][i]);
             }
           }
-#pragma unroll
-          for (int j = 0; j < NIN; ++j) {
-            const long long o = o1 + j * step;
-            const float2 yt = p_add(yv[j], s ? hi2(out[1 + j]) : lo2(out[1 + j]));
-            const float2 xn = p_fma(dup(-d.cb), pv[j],
-                                    p_mul(dup(d.ca), p_fma(dup(-d.cc), xv[j], p_mul(dup(w[j]), yt))));
-            if (GBC_IN_RANGE(GBC_SITE_CELL_STORE, I1 + j, d.mesh.M)) d.Xout[o] = xn;
-          }
-#pragma unroll
-          for (int i = 0; i < NP; i += NP - 1) {   // the pencil's two face nodes
-            const int I = Iyz + no[i];
-            if (I >= 0 && GBC_IN_RANGE(GBC_SITE_CELL_STORE, I, d.mesh.M))
-              atomicAdd(&d.Y[((long long)I * 2 + s) * d.ldx + vec], s ? hi2(out[i]) : lo2(out[i]));
-          }
-        } else {
-#pragma unroll
-          for (int i = 0; i < NP; ++i) {
-            const int I = Iyz + no[i];
-            if (I >= 0 && GBC_IN_RANGE(GBC_SITE_CELL_STORE, I, d.mesh.M))
-              atomicAdd(&d.Y[((long long)I * 2 + s) * d.ldx + vec], s ? hi2(out[i]) : lo2(out[i]));
-          }
         }
       }
-    }
+    };
+    if (cell_split_spins<NP, VB>() && d.cheb) assemble(std::integral_constant<int, cell_split_spins<NP, VB>() ? 1 : 2>());
+    else assemble(std::integral_constant<int, 2>());
   }
 }
 

@@ -185,6 +185,11 @@ template <int NP, int VB> __host__ __device__ constexpr int cell_group_threads()
 // p = 7 a plane has 36 pencils a vector quad and every warp a plane (1048 -> 1090 us), at
 // p <= 4 it leaves lanes idle (460 -> 575 us).
 template <int NP> __host__ __device__ constexpr bool cell_planes() { return NP == 6 || NP == 7; }
+// Whether a thread of the FP32 kernel's last stage has one spin of a pencil in recurrence mode: at p = 7
+// and 2 vectors 128 pencils are half of the group, and the update's loads wait for each other.  11 x 9 x 8
+// cells, k = 0: 7 vectors 112.9 -> 108.3 us a launch, 64 vectors 854 -> 852 (variant 2: 914 -> 885).  Without
+// the update the shared-memory accesses of half a point each cost more (64 vectors 654 -> 693).
+template <int NP, int VB> __host__ __device__ constexpr bool cell_split_spins() { return NP == 8 && VB == 2; }
 constexpr int kNoNode = -(1 << 29);   // offset of a direction with no free node (Dirichlet face)
 
 // ---------------------------------------------------------------------------

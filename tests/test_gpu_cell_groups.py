@@ -75,3 +75,35 @@ def test_local_apply_keeps_fp32_accuracy(g, p):
         c.apply_h(X, Y)
         assert float((Y - ref).norm() / ref.norm()) < 1.05e-7
     c.close()
+
+
+@pytest.mark.parametrize("p,ncell,nvec", [(2, (12, 10, 10), 17), (5, (8, 7, 6), 9), (6, (7, 6, 6), 11), (7, (7, 6, 5), 13)])
+def test_groups_take_many_items(g, p, ncell, nvec):
+    """More work items than the GPU has groups, so that every group reuses its item slots: H.X of both
+    precisions and the fused FP32 recurrence, with a ragged last vector chunk and Dirichlet faces."""
+    prob = syn.make_problem(ncell=ncell, h=(0.9, 1.0, 1.1), p=p, periodic=(1, 0, 1), k=(0.1, 0.0, -0.1), seed=p)
+    d = fe.Discretisation(prob)
+    X = syn.random_block(d.mesh.nnodes, nvec, 4)
+    want = d.apply_h(X)
+    bounds = (1.0, 300.0, -3.0)
+    c = g.Context(0)
+    c.set_problem(prob)
+    X64 = torch.from_numpy(X).cuda()
+    Y64 = torch.empty_like(X64)
+    c.apply_h(X64, Y64)
+    assert rel(Y64.cpu().numpy(), want) < 1e-12
+    F64 = X64.clone()
+    c.filter(F64, 3, *bounds)
+    c.set_precision(1)
+    X32 = X64.to(torch.complex64)
+    for var in (0, 2, 4):
+        c.set_cell_variant(var)
+        Y = torch.empty_like(X32)
+        c.apply_h(X32, Y)
+        c.sync_status()
+        assert rel(Y.cpu().numpy(), want) < 1e-5
+        F = X32.clone()
+        c.filter(F, 3, *bounds)
+        c.sync_status()
+        assert rel(F.cpu().numpy(), F64.cpu().numpy()) < 2e-5
+    c.close()
