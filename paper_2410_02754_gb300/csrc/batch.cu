@@ -155,23 +155,29 @@ extern "C" gbc_status gbc_tune(gbc_ctx* c, int nvec, void* stream) {
     if (it->second.nl_engine >= 0) c->nl_engine = it->second.nl_engine;
     return GBC_OK;
   }
-  // every candidate timed on a scratch block (work slots 0, 1, 2)
+  // every candidate timed on scratch blocks (work slots 0, 1, 4; 2)
   const size_t bytes = sizeof(float2) * 2 * (size_t)c->mesh.M * nvec;
   GBC_TRY(gbc_ensure_work(c, 0, bytes));
   GBC_TRY(gbc_ensure_work(c, 1, bytes));
   float2* X = (float2*)c->work[1];
   float2* Y = (float2*)c->work[0];
   GBC_CU(c, cudaMemsetAsync(X, 0, bytes, s));
+  // a third block for X_{k-1} and X_{k+1}: with fewer blocks the variants' times come out as their
+  // arithmetic, without the traffic that orders them in a filter (p = 7, 64 vectors, k = 0: 840 and 838 us
+  // a launch for variants 4 and 0, 892 and 854 in the filter)
+  float2* W = gbc_ensure_work(c, 4, bytes) == GBC_OK ? (float2*)c->work[4] : Y;
+  GBC_CU(c, cudaMemsetAsync(W, 0, bytes, s));
+  GBC_CU(c, cudaMemsetAsync(Y, 0, bytes, s));
   cudaEvent_t e0, e1;
   GBC_CU(c, cudaEventCreate(&e0));
   GBC_CU(c, cudaEventCreate(&e1));
   TuneEntry ent;
   float best = 1e30f;
   for (int var = 0; var < GBC_CELL_VARIANTS; ++var) {
-    // timed in the filter's recurrence mode (the scratch block is zero, so writing
-    // the update over it changes nothing); a variant whose shared memory does not
+    // timed in the filter's recurrence mode (the blocks are zero, so writing
+    // the update changes nothing); a variant whose shared memory does not
     // fit this order is skipped
-    CellJob j{c, X, Y, nvec, nvec, X, X, 0.0, 0.0, 0.0};
+    CellJob j{c, X, Y, nvec, nvec, W, W, 0.0, 0.0, 0.0};
     const float ms = time_median(c, s, e0, e1, [&] { return launch_cell_f32(&j, 1, var, s); });
     ent.ms[var] = ms;
     if (ms >= 0.f && ms < best) {
