@@ -288,11 +288,11 @@ gbc_status rotate(gbc_ctx* c, cplx<T>* X, int nvec, int ldx, const double2* Q, c
   return GBC_OK;
 }
 
-// waits for the stream; a bounded wait of the rotation that expired (those of the Gram matrix are
+// waits for the stream; a bounded wait of a split rotation that expired (those of the Gram matrix are
 // looked at before the rotation, with the pivots and the sweeps: the block is then unchanged)
-gbc_status finish_dense(gbc_ctx* c, cudaStream_t s) {
+gbc_status finish_dense(gbc_ctx* c, bool split, cudaStream_t s) {
   int err = 0;
-  GBC_CU(c, cudaMemcpyAsync(&err, c->d_flag + 1, sizeof(int), cudaMemcpyDeviceToHost, s));
+  if (split) GBC_CU(c, cudaMemcpyAsync(&err, c->d_flag + 1, sizeof(int), cudaMemcpyDeviceToHost, s));
   GBC_CU(c, cudaStreamSynchronize(s));
   if (err) return gbc_fail(c, GBC_ETIMEOUT, kSplitExpired);
   return GBC_OK;
@@ -324,14 +324,16 @@ gbc_status cholgs_t(gbc_ctx* c, cplx<T>* X, int nvec, int ldx, cudaStream_t s) {
   DenseScratch d;
   GBC_TRY(dense_scratch<T>(c, nvec, &d));
   GBC_TRY((gram<T, T>(c, X, ldx, X, ldx, c->d_md, nvec, d.S, s)));
-  GBC_CU(c, cudaMemcpy2DAsync(d.diag, sizeof(double2), d.S, sizeof(double2) * (nvec + 1), sizeof(double2),
-                              nvec, cudaMemcpyDeviceToDevice, s));
+  const bool split = nvec >= split_rotate_cols<T>();
+  if (split)
+    GBC_CU(c, cudaMemcpy2DAsync(d.diag, sizeof(double2), d.S, sizeof(double2) * (nvec + 1), sizeof(double2),
+                                nvec, cudaMemcpyDeviceToDevice, s));
   {
     TimerScope ts(c, FAM_DENSE, s);
     GBC_TRY(dense_cholesky_inv_h(c, d.S, nvec, d.Q, s));
   }
   GBC_TRY(rotate<T>(c, X, nvec, ldx, d.Q, d.diag, d.qsplit, s));
-  return finish_dense(c, s);
+  return finish_dense(c, split, s);
 }
 
 // Rayleigh-Ritz: Hp = X^H (H X), Hp Q = Q Lambda, X <- X Q.  HX is the FP64 H.X of X; an FP32
@@ -362,7 +364,7 @@ gbc_status rr_t(gbc_ctx* c, cplx<T>* X, int nvec, int ldx, double* ritz, cudaStr
   }
   GBC_TRY(rotate<T>(c, X, nvec, ldx, d.Q, nullptr, d.qsplit, s));
   GBC_CU(c, cudaMemcpyAsync(ritz, d.ev, sizeof(double) * nvec, cudaMemcpyDeviceToHost, s));
-  return finish_dense(c, s);
+  return finish_dense(c, nvec >= split_rotate_cols<T>(), s);
 }
 
 // Residual-split filter (Hamiltonian-times-residual form of the recurrence):
