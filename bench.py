@@ -153,11 +153,12 @@ def _eo_flops(no: int, ni: int) -> int:
 
 
 def flops_per_cell_vector(p: int, nq: int, kpt: bool) -> int:
-    """Algorithmic flops (FMA = 2) of the cell apply as implemented, for one cell
-    and one two-component vector: the kinetic/k part as 7 one-dimensional
+    """Flops (FMA = 2) of the cell operator with separate kinetic and potential passes,
+    for one cell and one two-component vector: the kinetic/k part as 7 one-dimensional
     contractions (complex G = Gr + i Gi when k != 0), 3 + 3 interpolation /
     testing contractions n <-> nq, the pointwise 2x2 spin operator at the nq^3
-    Gauss points, all 1-D contractions in even-odd form."""
+    Gauss points, all 1-D contractions in even-odd form.  The FP32 kernel does fewer:
+    cell_apply_flops."""
     n, q = p + 1, nq
     b = _eo_flops(n, n)
     g = b + (_eo_flops(n, n) + 2 * n if kpt else 0)
@@ -167,6 +168,41 @@ def flops_per_cell_vector(p: int, nq: int, kpt: bool) -> int:
     test = 2 * (q * q + q * n + n * n) * _eo_flops(n, q) + per_ps * 2 * n
     pointwise = q ** 3 * 32
     return kin + interp + test + pointwise
+
+
+def cell_apply_flops(p: int, nq: int, kpt: bool) -> int:
+    """Flops (FMA = 2) that the FP32 cell apply does for one cell and one two-component
+    vector (csrc/hx_cell.cuh): five stages, the z kinetic term on the interpolated field,
+    even-odd 1-D products that share the parts of their input and the sums of their output."""
+    n, q = p + 1, nq
+
+    def rows(no):                                 # (row pairs, middle row)
+        return no // 2, no % 2
+
+    def parts(ni):                                # even and odd parts of a complex pencil
+        return 4 * (ni // 2)
+
+    def sym(no, ni):                              # E e (+ Mid) of every row, O o of every pair
+        pairs, mid = rows(no)
+        return (pairs + mid) * 4 * (ni // 2 + ni % 2) + pairs * 4 * (ni // 2)
+
+    def anti(no, ni):                             # the same of a centro-antisymmetric i M, and its sums
+        pairs, mid = rows(no)
+        return (pairs + mid) * (4 * (ni // 2) + 2) + pairs * (4 * (ni // 2 + ni % 2) + 2) if kpt else 0
+
+    def out(no):                                  # rows i and no - 1 - i from their sums
+        return 4 * (no // 2)
+
+    g = sym(n, n) + anti(n, n)
+    x1 = parts(n) + sym(q, n) + out(q) + sym(n, n) + out(n) + g + out(n)
+    y1 = parts(n) + sym(q, n) + out(q)
+    y2 = 2 * parts(n) + g + sym(n, n) + out(n)
+    z1 = parts(n) + sym(q, n) + out(q) + parts(q) + sym(n, q) + g + out(n)
+    z2 = parts(n) + sym(n, n) + out(n)
+    y3 = parts(q) + sym(n, q) + out(n)
+    x2 = y3 + 2 * n
+    return (2 * (n * n * (x1 + y2 + z2 + x2) + n * q * (y1 + y3) + q * q * z1) +
+            22 * q ** 3)                          # the 2 x 2 spin operator
 
 
 def hbm_peak():
@@ -357,7 +393,7 @@ def run_gpu(args):
     loc = fams["hx_local"]
     avg_local_ms = loc[0] / loc[1]
     kpt = any(abs(x) > 0 for k in ks for x in k)
-    flops_launch = flops_per_cell_vector(prob.p, prob.nq, kpt) * prob.ncells * nvec
+    flops_launch = cell_apply_flops(prob.p, prob.nq, kpt) * prob.ncells * nvec
     clocks = clk.summary()
     fp32 = [v for k, v in peaks.items() if k in ("ffma", "ffma2") and isinstance(v, float)]
     if fp32:
@@ -555,7 +591,7 @@ def run_gpu(args):
             peak, peak_src = hbm_peak()
             gbs = by / (ms_t / 1e3) / 1e9
             out["twogrid"] = {
-                "ms": round(ms_t, 4), "kernel": f"k_prolongate<float,{pc + 1},{prob.p + 1},8>",
+                "ms": round(ms_t, 4), "kernel": f"k_prolongate<float,{pc + 1},{prob.p + 1}>",
                 "algorithmic_bytes": by, "achieved_gbs": round(gbs, 1),
                 "frac_hbm": round(gbs / peak, 4), "peak_gbs": peak, "peak_note": peak_src,
                 "how": f"order {pc} -> {prob.p} on the bench mesh, {nvec} vectors FP32, {nrep} "
@@ -602,7 +638,7 @@ def run_gpu(args):
     # ---- FP64 filter and accuracy of the mixed path at the same inputs (k-point 0):
     # three chains from the same seeded block -- FP64, mixed direct, mixed residual-split --
     # each cycle 0 (CholGS + RR) then ``--cycles`` x (filter, CholGS, RR); CholGS/RR
-    # run in FP64 in every chain.
+    # to FP64 accuracy in every chain (FP32 blocks rounded to FP32 after each rotation).
     if not args.no_fp64 and rank == 0:
         c64 = build_contexts(g, prob, ks[:1], g.FP64)[0]
         c32 = ctx32[0]
@@ -655,10 +691,10 @@ def run_gpu(args):
             "final_ha": {k: v[-1] for k, v in per_cycle.items()} if args.cycles else None,
             "target_ha": 1e-6,
             "how": f"k-point 0, cycle 0 + {args.cycles} x (filter degree {degree}, CholGS, RR); "
-                   "CholGS/RR in FP64 in every chain; lower half of the block",
+                   "CholGS/RR to FP64 accuracy in every chain; lower half of the block",
             "ms_per_filter": {k: round(min(v), 2) for k, v in ms.items() if v},
             "ms_per_cycle": {k: round(min(v), 2) for k, v in ms_cycle.items() if v},
-            "cycle_note": "filter + CholGS + Rayleigh-Ritz (the latter two in FP64 in every chain)",
+            "cycle_note": "filter + CholGS + Rayleigh-Ritz (the latter two to FP64 accuracy in every chain)",
             "lowest_ritz_ha": [float(x) for x in ritz["fp64"][:4]]}
         c64.close()
 

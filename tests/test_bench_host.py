@@ -58,3 +58,21 @@ def test_cell_traffic_scales_the_captured_variants_only():
     assert 4 in bench.CELL_TRAFFIC_32             # the variant the tuner picks at p = 6, 256 vectors
     t, note = bench.CELL_TRAFFIC(256, 0)
     assert t is None and "no ncu capture" in note
+
+
+def test_cell_apply_flops_of_the_five_stage_form():
+    """Against a count by hand at p = 6, n_q = 8 (n = 7, q = 8): a product of 7 or 8 rows and inputs
+    costs 4 (E, and Mid of an odd input) or 8 (with O) flops an entry, and each of the five stages
+    does the products it lists; fewer flops than the separate passes."""
+    s78, s87, s77 = 4 * 4 * 4 + 4 * 4 * 3, 4 * 4 * 4 + 3 * 4 * 4, 4 * 4 * 4 + 3 * 4 * 3   # (q,n), (n,q), (n,n)
+    a77 = 4 * (4 * 3 + 2) + 3 * (4 * 4 + 2)
+    pn, pq, on, oq = 12, 16, 12, 16
+    x1 = pn + s78 + oq + s77 + on + s77 + a77 + on
+    y2 = 2 * pn + 2 * s77 + a77 + on
+    z1 = pn + s78 + oq + pq + s87 + s77 + a77 + on
+    want = 2 * (49 * (x1 + y2 + (pn + s77 + on) + (pq + s87 + on + 14)) +
+                56 * ((pn + s78 + oq) + (pq + s87 + on)) + 64 * z1) + 22 * 512
+    assert bench.cell_apply_flops(6, 8, True) == want
+    assert bench.cell_apply_flops(6, 8, False) == want - 2 * a77 * (49 * 2 + 64)
+    for p in range(2, 8):
+        assert bench.cell_apply_flops(p, p + 2, True) < bench.flops_per_cell_vector(p, p + 2, True)
