@@ -51,13 +51,15 @@ typedef enum {
 } gbc_status;
 
 typedef enum {
-  GBC_FP64 = 0,          /* complex128 blocks, FP64 arithmetic everywhere               */
+  GBC_FP64 = 0,          /* complex128 blocks, FP64 arithmetic; Gram matrices, rotations
+                            and larger projector contractions as exact products of BF16
+                            digits (54 bits below the largest entry of a row or column,
+                            sums to FP64 accuracy; gbc_set_deterministic keeps the
+                            projector contractions in FP64 arithmetic)                  */
   GBC_FP32 = 1,          /* complex64 blocks, FP32 arithmetic in H.X and the filter;
                             Gram matrices to FP64 accuracy                              */
-  GBC_TF32 = 2,          /* reserved: cell apply on the TF32 tensor cores (not built;
-                            gbc_set_precision returns GBC_EUNSUPPORTED)                 */
-  GBC_BF16X3 = 3         /* reserved: cell apply in split BF16 on the tensor cores (not
-                            built; gbc_set_precision returns GBC_EUNSUPPORTED)          */
+  GBC_TF32 = 2,          /* complex64 blocks, cell apply as TF32 tensor-core GEMMs      */
+  GBC_BF16X3 = 3         /* complex64 blocks, cell apply as split BF16 tensor-core GEMMs */
 } gbc_precision;
 
 /* ---- context ----------------------------------------------------------- */
@@ -117,7 +119,8 @@ gbc_status gbc_set_precision(gbc_ctx* ctx, gbc_precision prec);
  *                      (default; used where the projector layout allows it:
  *                      npj <= 64 and at most 16 atoms over any 128 owned
  *                      support nodes, else the SIMT engine runs).
- * FP64 always runs on the SIMT cores.  GBC_EINVAL for another value. */
+ * The FP64 precision does not take this choice (GBC_FP64 above).  GBC_EINVAL for
+ * another value. */
 enum { GBC_NL_SIMT = 0, GBC_NL_TENSOR = 1 };
 gbc_status gbc_set_nonlocal_engine(gbc_ctx* ctx, int engine);
 /* Engine (GBC_NL_*) that the FP32 nonlocal step runs for the projectors set

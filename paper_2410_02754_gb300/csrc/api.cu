@@ -316,9 +316,9 @@ template <typename T> gbc_status dense_scratch(gbc_ctx* c, int nvec, DenseScratc
   return GBC_OK;
 }
 
-// Cholesky-Gram-Schmidt.  FP64 blocks: FP64 throughout.  The mixed path keeps complex64
-// blocks for the filter, but S = X^H M_D X and the rotation are FP64-accurate (the rotated
-// block is rounded to FP32 once).
+// Cholesky-Gram-Schmidt.  S = X^H M_D X and the rotation are FP64-accurate for both blocks (split
+// products from split_gram_cols / split_rotate_cols columns on, FP64 or float-float arithmetic
+// below); a rotated FP32 block is rounded to FP32 once.
 template <typename T>
 gbc_status cholgs_t(gbc_ctx* c, cplx<T>* X, int nvec, int ldx, cudaStream_t s) {
   DenseScratch d;

@@ -27,7 +27,7 @@
 cudaError_t launch_hx_local_f64(const gbc_ctx* c, const double2* X, double2* Y, int nvec, int ldx,
                                 cudaStream_t s, void* Ycell) {
   HxJob j{c, X, Y, nvec, ldx, Ycell};
-  return launch_hx_local_group_f64(&j, 1, 1, s);
+  return launch_hx_local_group_f64(&j, 1, s);
 }
 
 cudaError_t launch_hx_local_f32(const gbc_ctx* c, const float2* X, float2* Y, int nvec, int ldx,
@@ -392,7 +392,7 @@ gbc_status record_filters(gbc_batch* b, std::vector<SysRun>& runs, cudaStream_t 
         jobs.push_back(HxJob{runs[j].c, cur_of(runs[j]), runs[j].Y, runs[j].nvec, runs[j].ldx});
         done[j] = true;
       }
-      const cudaError_t e = launch_hx_local_group_f64(jobs.data(), (int)jobs.size(), 1, s);
+      const cudaError_t e = launch_hx_local_group_f64(jobs.data(), (int)jobs.size(), s);
       if (e != cudaSuccess) return bfail(b, GBC_ECUDA, std::string("cell apply: ") + cudaGetErrorString(e));
       ++count;
     }

@@ -288,7 +288,7 @@ struct HxJob {
   int nvec, ldx;
   void* Ycell = nullptr;   // non-null: per-cell results [E][n_p^3][2][nvec], no assembly
 };
-cudaError_t launch_hx_local_group_f64(const HxJob* jobs, int n, int vb, cudaStream_t s);
+cudaError_t launch_hx_local_group_f64(const HxJob* jobs, int n, cudaStream_t s);
 // Y += the per-cell results Ycell of launch_hx_local_group_f64, in a fixed order per node
 cudaError_t launch_cell_gather_f64(const gbc_ctx* c, const double2* Ycell, double2* Y, int nvec,
                                    int ldx, cudaStream_t s);
@@ -324,7 +324,7 @@ cudaError_t tcl_error(int* err, cudaStream_t s);
 void tcl_free(TclState* t);
 // nonlocal.cu : Y += sum_a P Delta P^H X (overwrite: Y = sum_a P Delta P^H X on every
 // support row, other rows untouched).  may_alloc: work slot 14 may be grown and used (not in the
-// allocation-free entry point)
+// allocation-free entry point, nor in the batch, whose graph is captured)
 template <typename T>
 cudaError_t launch_nonlocal(gbc_ctx* c, const cplx<T>* X, cplx<T>* Y, int nvec, int ldx,
                             cplx<T>* Cbuf, cplx<T>* Cpbuf, cudaStream_t s, bool overwrite = false,

@@ -14,7 +14,7 @@ static cudaError_t launch_hx_group(const HxJob* jobs, int n, cudaStream_t s) {
   }
 }
 
-cudaError_t launch_hx_local_group_f64(const HxJob* jobs, int n, int /*vb*/, cudaStream_t s) {
+cudaError_t launch_hx_local_group_f64(const HxJob* jobs, int n, cudaStream_t s) {
   return launch_hx_group(jobs, n, s);
 }
 

@@ -86,7 +86,6 @@ __device__ __forceinline__ void mma_tf32_ts(uint32_t d_tmem, uint32_t a_tmem, ui
       : "memory");
 }
 
-// BF16 operands (kind::f16), FP32 accumulation; one instruction takes K = 16 (32 bytes a row)
 // 2-D TMA box at element (x, y), completion counted on mbar in bytes (x * size a multiple of 16)
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const void* tmap, int x, int y,
                                             uint32_t mbar) {
@@ -97,6 +96,7 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const void* tmap, int 
       : "memory");
 }
 
+// BF16 operands (kind::f16), FP32 accumulation; one instruction takes K = 16 (32 bytes a row)
 __host__ __device__ constexpr uint32_t idesc_bf16(int M, int N) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) |
          ((uint32_t)(M >> 4) << 24);

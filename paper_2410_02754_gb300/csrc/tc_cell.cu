@@ -553,11 +553,12 @@ gbc_status tcl_apply(gbc_ctx* c, const float2* X, float2* Y, int nvec, int ldx, 
   return GBC_OK;
 }
 
-// bounded-wait flag of the tensor-core cell apply (cleared on read)
+// tensor map of a BF16 array [rows][cols] in boxes of box_rows x 64 (one 128-byte swizzled row)
 bool tc_make_map_bf16(CUtensorMap* m, const void* p, long long rows, int cols, int box_rows) {
   return make_map(m, p, rows, cols, box_rows, 1);
 }
 
+// bounded-wait flag of the tensor-core cell apply (cleared on read)
 cudaError_t tcl_error(int* err, cudaStream_t s) {
   cudaError_t e = cudaMemcpyFromSymbolAsync(err, g_tcl_err, sizeof(int), 0, cudaMemcpyDeviceToHost, s);
   if (e != cudaSuccess) return e;
