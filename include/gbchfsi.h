@@ -195,7 +195,8 @@ gbc_status gbc_filter_residual(gbc_ctx* ctx, void* X, int nvec, int ldx, int deg
  * and gbc_energy_grad report it likewise.) */
 gbc_status gbc_cholgs(gbc_ctx* ctx, void* X, int nvec, int ldx, void* stream);
 
-/* Rayleigh-Ritz for an M_D-orthonormal block (Sec. III.B.2): Hp = X^H H X
+/* Rayleigh-Ritz for an M_D-orthonormal block (Sec. III.B.2; a column far smaller than
+ * the others would be rotated with their accuracy, not its own): Hp = X^H H X
  * to FP64 accuracy, Hp Q = Q Lambda by a Jacobi eigensolver on the device,
  * X <- X Q.  ritz: host array of nvec doubles, ascending.  Synchronous.
  * nvec <= 512.  GBC_ETIMEOUT if the eigensolver hits its sweep cap. */
@@ -216,7 +217,8 @@ gbc_status gbc_rayleigh_ritz(gbc_ctx* ctx, void* X, int nvec, int ldx, double* r
  * gDelta (host, the concatenated Delta matrices, complex128, Hermitian part,
  * written; may be NULL).  p <= 6.  Synchronous.  Uses library workspace of
  * (2 ceil(degree/ckpt_every) + max(ckpt_every, 3) + 4) blocks and the projector
- * coefficients (2 npj per atom and vector) of every degree. */
+ * coefficients (2 npj per atom and vector) of every degree, or of one where there is
+ * no memory for them. */
 gbc_status gbc_filter_vjp(gbc_ctx* ctx, const void* X0, const void* GY, void* GX, double* gV,
                           double* gB, double* gDelta, int nvec, int ldx, int degree, double lT,
                           double lmax, double lmin, int ckpt_every, void* stream);

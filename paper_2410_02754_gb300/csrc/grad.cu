@@ -252,15 +252,20 @@ gbc_status filter_vjp_t(gbc_ctx* c, const cplx<T>* X0, const cplx<T>* GY, cplx<T
   C* Y = (C*)c->work[0];
   auto lam = [&](int j) { return blk(nck + nseg + (j % 3)); };
   // P^H X_0 .. P^H X_{m-1} and P^H of the adjoint: the recurrence steps leave them, so the Delta
-  // gradient projects only X_{m-1} itself
+  // gradient projects only X_{m-1} itself.  Where there is no memory for the coefficients of every
+  // degree, X_k is projected when its turn comes (set 0; the adjoint's is set 1).
   GradScratch gs;
-  GBC_TRY(grad_scratch(c, nvec, m + 1, &gs));
+  const gbc_status kept = grad_scratch(c, nvec, m + 1, &gs);
+  const bool keep = kept == GBC_OK;
+  if (kept == GBC_ENOMEM) GBC_TRY(grad_scratch(c, nvec, 2, &gs));
+  else GBC_TRY(kept);
+  const int nset = keep ? m + 1 : 2;
   auto coef = [&](int k) { return (C*)(gs.coef + gs.coef_bytes * (size_t)k); };
   const size_t nq3 = (size_t)c->nq * c->nq * c->nq;
   GBC_CU(c, cudaMemsetAsync(gs.g, 0, sizeof(double) * c->mesh.E * 4 * nq3, s));
   if (c->proj.natoms) {
     GBC_CU(c, cudaMemsetAsync(gs.gD, 0, sizeof(double2) * c->proj.delta_off[c->proj.natoms], s));
-    GBC_CU(c, cudaMemsetAsync(gs.coef, 0, gs.coef_bytes * (m + 1), s));
+    GBC_CU(c, cudaMemsetAsync(gs.coef, 0, gs.coef_bytes * nset, s));
   }
   GBC_CU(c, cudaMemsetAsync(Y, 0, bb, s));
   const long long rows = 2 * c->mesh.M;
@@ -270,9 +275,9 @@ gbc_status filter_vjp_t(gbc_ctx* c, const cplx<T>* X0, const cplx<T>* GY, cplx<T
   GBC_CU(c, launch_copy_block<T>(X0, xp[0], c->mesh.M, nvec, ldx, s));
   for (int k = 0; k + 1 < m; ++k) {
     GBC_TRY(gbc_recur_dev(c, xp[k], k ? xp[k - 1] : nullptr, xp[k + 1], Y, nvec, ldx, alpha[k] / e, cc,
-                          beta[k], coef(k), s));
+                          beta[k], keep ? coef(k) : nullptr, s));
   }
-  if (c->proj.natoms) GBC_CU(c, launch_nl_project<T>(c, xp[m - 1], nvec, ldx, coef(m - 1), s));
+  if (c->proj.natoms && keep) GBC_CU(c, launch_nl_project<T>(c, xp[m - 1], nvec, ldx, coef(m - 1), s));
   // ---- adjoint seed Lt_m = M_D^-1 G_Y
   k_rowscale<T><<<gfor(rows * nvec), 256, 0, s>>>(GY, lam(m), c->d_invmd, rows, nvec, ldx);
   GBC_CU(c, cudaGetLastError());
@@ -294,8 +299,9 @@ gbc_status filter_vjp_t(gbc_ctx* c, const cplx<T>* X0, const cplx<T>* GY, cplx<T
       GBC_CU(c, quad_grad<T>(c, Lt1, Xk, nullptr, f, nvec, ldx, gs.g, s));
       const bool has2 = k + 2 <= m;
       GBC_TRY(gbc_recur_dev(c, Lt1, has2 ? lam(k + 2) : nullptr, lam(k), Y, nvec, ldx, alpha[k] / e, cc,
-                            has2 ? beta[k + 1] : 0.0, coef(m), s));
-      GBC_TRY(delta_grad<T>(c, coef(m), coef(k), nullptr, f, nvec, gs.gD, s));
+                            has2 ? beta[k + 1] : 0.0, coef(nset - 1), s));
+      if (c->proj.natoms && !keep) GBC_CU(c, launch_nl_project<T>(c, Xk, nvec, ldx, coef(0), s));
+      GBC_TRY(delta_grad<T>(c, coef(nset - 1), coef(keep ? k : 0), nullptr, f, nvec, gs.gD, s));
     }
   }
   // ---- grad_X0 = M_D Lt_0

@@ -211,3 +211,49 @@ def test_full_size_fifty_direction_fd(g, capsys):
         print(f"  full-size FD, 50 joint directions, h = {h:g}: worst relative error {worst:.2e}; "
               f"loss reproducibility {noise:.1e}")
     assert worst <= 5e-6, worst
+
+
+@pytest.mark.parametrize("prec,tol", [(0, 1e-10), (1, 2e-4)])
+def test_vjp_of_many_projectors(g, prec, tol):
+    """40 atoms x 18 projectors on a small mesh, 64 vectors, degree 60: the FP64 contractions run as split
+    products (against fixed-order FP64 arithmetic), and the projector coefficients of every degree
+    (90 MB in FP64) are kept where there is memory for them; where there is not, the same gradients."""
+    prob = syn.make_problem(ncell=(4, 3, 3), h=(1.0, 1.1, 0.9), p=3, k=(0.1, -0.2, 0.0), natoms=40, rc=1.2,
+                            seed=3, channels=syn.SPD_CHANNELS, delta_std=0.02)
+    dt = torch.complex128 if prec == 0 else torch.complex64
+    X = torch.from_numpy(syn.random_block(prob.nnodes, 64, 1)).to(dt).cuda()
+    G = torch.from_numpy(syn.random_block(prob.nnodes, 64, 2)).to(dt).cuda()
+    H = torch.empty_like(X)
+    args = (60, 6.0, 90.0, -6.0)
+
+    def context():
+        c = g.Context(0)
+        c.set_problem(prob)
+        c.set_precision(prec)
+        c.apply_h(X, H)                              # tables in place
+        return c
+
+    def vjp(c):
+        out = torch.empty_like(X)
+        rest = c.filter_vjp(X, G, out, *args)
+        return [out.cpu().numpy()] + [np.asarray(a) for a in rest]
+
+    c = context()
+    want = vjp(c)
+    c.set_deterministic(True)
+    fixed = vjp(c)
+    c.close()
+    c = context()
+    torch.cuda.empty_cache()
+    el = X.element_size()
+    blocks = 33 * X.numel() * el
+    hog = torch.empty(torch.cuda.mem_get_info()[0] - blocks - (45 << 20) * el // 16, dtype=torch.uint8, device="cuda")
+    try:
+        starved = vjp(c)
+    finally:
+        del hog
+        torch.cuda.empty_cache()
+    c.close()
+    for a, b, d in zip(want, fixed, starved):
+        assert rel(b, a) < tol
+        assert rel(d, a) < tol
