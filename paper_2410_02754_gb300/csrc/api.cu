@@ -239,8 +239,8 @@ gbc_status filter_t(gbc_ctx* c, cplx<T>* X, int nvec, int ldx, int m, double lT,
 // where the memory for the digits cannot be had.
 // Measured, split against direct: FP64 Gram at 16 columns 0.054 / 0.066 ms (1296 nodes) and
 // 0.86 / 5.22 ms (216,000 nodes), rotation 0.030 / 0.114 and 0.56 / 4.8 ms; FP32 Gram 1.34 /
-// 0.83 ms at 32 columns (216,000 nodes), 0.112 / 0.171 at 64 (13,824) and 0.92 / 2.32 (216,000), FP32
-// rotation 0.56 / 0.64 ms at 16 and 0.42 / 1.29 at 32 (216,000 nodes), 0.033 / 0.023 at 16 (1728).
+// 0.83 ms at 32 columns (216,000 nodes), 0.109 / 0.171 at 64 (13,824) and 0.87 / 2.32 (216,000), FP32
+// rotation 0.56 / 0.64 ms at 16 and 0.41 / 1.29 at 32 (216,000 nodes), 0.033 / 0.023 at 16 (1728).
 template <typename T> constexpr int split_gram_cols() { return sizeof(T) == 8 ? 16 : 64; }
 template <typename T> constexpr int split_rotate_cols() { return sizeof(T) == 8 ? 16 : 32; }
 

@@ -6,7 +6,7 @@
 // 2012), with balanced base-256 digits: a value x with |x| < 2^E is
 //   x = 2^(E-6) sum_k d_k 256^-k,  |d_0| <= 65, d_k in [-128, 127],
 // so every digit is a BF16 number and a product of two digits an integer below 2^14; S digits
-// carry 8 S - 2 bits below 2^E.  The partial products of order t = i + j <= S,
+// carry 8 S - 2 bits below 2^E.  The partial products of order t = i + j < T,
 // G_t = sum_{i+j=t} A_i B_j, are integers that FP32 holds exactly while S K 2^14 <= 2^24;
 // the accumulators are read out (to 64-bit integers) every kFlush K chunks to keep that, and
 // sum_t G_t 256^-t is rounded at the end (Gram matrices and projections: once per part
@@ -17,22 +17,24 @@
 // S = 7 digits: an entry is off by at most 2^-55 of its row's largest.  FP32 blocks are rounded to
 // FP32 once.  The rotation of CholGS, whose terms can cancel, takes its columns at a common size, by
 // powers of two; that of Rayleigh-Ritz rests on an M_D-orthonormal block, whose columns have one size.
-// Orders t < T = S + 1 are summed.  What is left out of a sum over K terms is about sqrt(K) 2^-62 of
-// the product of the largest entries (sqrt(K) 2^-54 without order S), which counts where a sum is
+// Orders t < T are summed.  What is left out of a sum over K terms is about sqrt(K) 2^-54 of the
+// product of the largest entries at T = S, sqrt(K) 2^-62 at T = S + 1, which counts where a sum is
 // small against that: the rotation of a nearly converged block (Q close to the identity), Gram
-// entries of columns that peak in a few of many rows, projectors over most of their support.
-// Measured with fewer: FP32 columns of a nearly converged block, n = 256, came out 6.2e-8 off
-// with S = T = 4, 2.5e-8 (their rounding to FP32) now; FP64 columns with one of 746,000 rows 1000
-// times the others came out of CholGS orthonormal to 5e-14 with T = S, to 1.3e-15 now (direct FP64
-// 2.2e-15; 10^5 times: 5e-13, direct 6e-13).
+// entries of columns that peak in a few of many rows, projectors over most of their support.  FP64:
+// T = S + 1.  FP64 columns with one of 746,000 rows 1000 times the others came out of CholGS
+// orthonormal to 5e-14 with T = S, to 1.3e-15 now (direct FP64 2.2e-15; 10^5 times: 5e-13, direct
+// 6e-13).  FP32 blocks: T = S, which is closer than the float-float sums of before (Ritz values of
+// such FP32 columns 3.4e-15 of the largest, float-float 4.7e-14) and far below the rounding to
+// FP32.  S = T = 4 was not: columns of a nearly converged FP32 block of 256 came out 6.2e-8 off,
+// 2.5e-8 (their rounding) now.
 //
 // GB300's FP64 pipe gives 1.05 TFLOP/s and float-float arithmetic on the FP32 pipes about 6;
-// 34 BF16 products at 1.9 PFLOP/s are an FP64-accurate 56 TFLOP/s.  Measured, 884,736 nodes x 256
-// FP32 columns: Gram 122 -> 24.5 ms, rotation 163 -> 28.8 ms; 373,248 nodes x 256 in FP64: 333 ->
+// 28 (34) BF16 products at T = S (S + 1) and 1.9 PFLOP/s are an FP64-accurate 68 (56) TFLOP/s.  Measured, 884,736 nodes x 256
+// FP32 columns: Gram 122 -> 22.6 ms, rotation 163 -> 26.6 ms; 373,248 nodes x 256 in FP64: 333 ->
 // 11.5 and 527 -> 13.0 ms.  Per tile (128 x 64) every order has its own accumulator in tensor memory and all S
 // digit slices of a 64-wide K chunk are in shared memory at once (one TMA box each), so a
 // slice is loaded once per tile and used in up to S products.  Step i multiplies A_i with all
-// of B_0 .. B_{S-i} in instructions of up to 256 columns (one product per instruction, 64
+// of B_0 .. B_{T-1-i} in instructions of up to 256 columns (one product per instruction, 64
 // columns, ran at a quarter of this rate); A_i's next chunk then loads behind the other steps,
 // B is double-buffered.
 #include <algorithm>
@@ -49,17 +51,20 @@ constexpr int kKC = 64;               // K chunk: one 128-byte swizzled row
 constexpr int kBad = 0x7fffffff;      // exponent of a row with an infinity or a NaN
 constexpr int kEpi = 16;              // read-out warps
 constexpr int kSplitThreads = 64 + 32 * kEpi;
-constexpr int S = 7, T = S + 1;       // digits; orders summed (order S: digits 1 .. S-1 only)
+constexpr int S = 7;                  // digits
 constexpr int kTN = 64;               // tile columns
 constexpr int kFlush = 2;             // K chunks between read-outs
 constexpr int kABytes = kTM * 128, kBBytes = kTN * 128;
 constexpr size_t kSplitSmem = 1024 + (size_t)S * (kABytes + 2 * kBBytes) + 256;
 static_assert((long long)S * kFlush * kKC << 14 <= 1LL << 24, "exact accumulation");
-static_assert(T * kTN <= 512 && T <= 8, "tensor memory columns");
 static_assert(kSplitSmem <= 227 * 1024, "shared memory");
 
 // PROJ, EXPD: the FP64 projector contractions C += P^H X and Y += P C' (see nl_split_project)
-enum { ROT32 = 0, ROT64 = 1, GRAM = 2, PROJ = 3, EXPD = 4 };
+enum { ROT32, ROT64, GRAM32, GRAM64, PROJ, EXPD };
+// orders summed (order S: digits 1 .. S-1 only)
+template <int MODE> __host__ __device__ constexpr int split_orders() {
+  return MODE == ROT32 || MODE == GRAM32 ? S : S + 1;
+}
 constexpr int kNlRows = 1024;         // rows of a support chunk's place in the digit buffers
 struct SplitArgs {
   int rows_a, rows_b;      // rows of a slice of A and B
@@ -84,11 +89,13 @@ template <int MODE>
 __global__ void __launch_bounds__(kSplitThreads, 1)
 k_split_gemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb,
              const SplitArgs a) {
-  constexpr int N = kTN;
+  constexpr int N = kTN, T = split_orders<MODE>();
+  constexpr bool GRAM = MODE == GRAM32 || MODE == GRAM64;
+  static_assert(T * N <= 512 && T <= 8, "tensor memory columns");
   struct Item { int m0, n0, k0, nk, b; };   // b: chunk of the batch
   auto decode = [&](int w) {
     Item it{0, 0, 0, a.nchunk, 0};
-    if (MODE == GRAM) {   // tiles that reach the diagonal or above it, row by row
+    if (GRAM) {   // tiles that reach the diagonal or above it, row by row
       int I = 0, t = w % a.ntiles, first = 0;
       while (t >= a.ntn - first) {
         t -= a.ntn - first;
@@ -222,7 +229,7 @@ k_split_gemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUt
                 tc::mma_bf16(tmem + (i + j) * N, tc::sdesc_sw128(A(i) + kk * 32),
                              tc::sdesc_sw128(B(buf, j) + kk * 32), tc::idesc_bf16(kTM, cnt * N), acc);
               };
-              if (i == 1 && kk == 0 && j + cnt == S && first) {   // order S starts here
+              if (T > S && i == 1 && kk == 0 && j + cnt == S && first) {   // order S starts here
                 if (cnt > 1) mma(j, cnt - 1, 1u);
                 mma(S - 1, 1, 0u);
               } else {
@@ -288,8 +295,10 @@ k_split_gemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUt
         tc::fence_before_sync();
         if (lane == 0) tc::mbar_arrive(tc::smem_u32(acce));
       }
+      if (T > S) {   // back to units of 256^-(S-1)
 #pragma unroll
-      for (int i = 0; i < NC; ++i) lo[i] = (lo[i] + 128) >> 8;   // back to units of 256^-(S-1)
+        for (int i = 0; i < NC; ++i) lo[i] = (lo[i] + 128) >> 8;
+      }
       if (ok && it.nk > 0) {
         const int mr = it.m0 + g * 32 + lane;
         const int ea = a.ea[mr + (MODE == PROJ ? it.b * a.rows_a : 0)];
@@ -338,7 +347,7 @@ k_split_gemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUt
 #pragma unroll
             for (int q = 0; q < 2; ++q) {
               int sh = 0;
-              if (MODE == GRAM)   // hi may use all of its 53 bits here: hi + 2^-24 lo, rounded once
+              if (GRAM)   // hi may use all of its 53 bits here: hi + 2^-24 lo, rounded once
                 v[q] = fma(__ll2double_rn(lo[i + q]), 0x1p-24, __ll2double_rn(hi[i + q]));
               else
                 v[q] = __ll2double_rn(value(i + q, sh));
@@ -882,7 +891,7 @@ gbc_status launch_gram_split(gbc_ctx* c, const cplx<TX>* X, int ldx, const cplx<
     const int kper = (nwin + split - 1) / split * kFlush;
     const int parts = (rp / kKC + kper - 1) / kper;
     SplitArgs a{ma, nb, rp / kKC, kper, ntn, tiles, tiles * parts, ea, eb, nr, n, 0, Sm, c->d_flag + 1};
-    GBC_CU(c, run_split_gemm<GRAM>(A, B, rp, a, s));
+    GBC_CU(c, (run_split_gemm<sizeof(TX) == 4 ? GRAM32 : GRAM64>(A, B, rp, a, s)));
   }
   if (md) k_set_diag<<<1, 256, 0, s>>>(diag, n, Sm);
   GBC_CU(c, cudaGetLastError());
