@@ -42,7 +42,8 @@
 // pencils 9.29, index work once per pencil 9.07, items decoded once and fields staged 8.34,
 // planes owned by warps 7.62.  Other sizes: 12^3 cells, p = 5, 96 vectors 1144 -> 815 us;
 // p = 4 812 -> 460; 10^3 cells, p = 3, 128 vectors 460 -> 212; p = 7, 64 vectors 1167 -> 1048
-// (at 3 or 7 vectors the partly filled last item leaves it up to 12% behind the seven-stage form).
+// (in recurrence mode, tuned, 11 x 9 x 8 cells, k = 0: 3, 7 and 64 vectors 1.26, 1.58 and 6.63 ms a degree-6
+// filter in seven stages, 1.24, 1.59 and 6.48 now).
 //
 // Assembly modes (per system):
 //  * accumulate: Y += H^loc X with FP32 atomics on every node;
