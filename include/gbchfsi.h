@@ -191,8 +191,8 @@ gbc_status gbc_filter_residual(gbc_ctx* ctx, void* X, int nvec, int ldx, int deg
  * (X is then left unchanged).  Synchronous (reads the pivot status).
  * nvec <= 512.  GBC_ETIMEOUT if a bounded wait of a tensor-core kernel of this
  * context expired and gbc_sync_status has not reported it yet: X is unchanged, or
- * invalid where the wait was the rotation's.  (gbc_rayleigh_ritz, gbc_filter_vjp
- * and gbc_energy_grad report it likewise.) */
+ * invalid where the wait was the rotation's.  (gbc_rayleigh_ritz, gbc_filter_vjp,
+ * gbc_energy_grad and gbc_lanczos_bounds report it likewise.) */
 gbc_status gbc_cholgs(gbc_ctx* ctx, void* X, int nvec, int ldx, void* stream);
 
 /* Rayleigh-Ritz for an M_D-orthonormal block (Sec. III.B.2; a column far smaller than
