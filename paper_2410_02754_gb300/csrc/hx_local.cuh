@@ -41,7 +41,7 @@ struct SysDesc {
   double2* Ycell;        // non-null: per-cell results [E][n_p^3][2][nvec] instead of assembly
   const double* fields;  // [E][NQ^3][4] J (V + |k|^2/2), J B_x, J B_y, J B_z
   int ldx, nvec;
-  long long item0;       // work items (pairs of (cell, vector)s): [item0, item0 + ceil(E nvec / 2))
+  long long item0;       // work items (per (cell, vector)s each): [item0, item0 + ceil(E nvec / per))
   MeshDev mesh;
 };
 
@@ -274,7 +274,16 @@ template <int NP> __host__ __device__ constexpr size_t hx_group_smem() {
 }
 template <int NP> __host__ __device__ constexpr int hx_groups() { return kHxThreads / cell_group_threads<NP, 4>(); }
 
-template <int NP, int NQ, bool KPT>
+// Whether items of one (cell, vector) are there too, for launches that leave SMs idle or one pair ahead of
+// the others: at p = 4 and 7 half of the units is a round of the group's threads less (z stage: 144 on
+// 128 threads, 324 on 256), so an SM with one or three single items is done before one with one or two
+// pairs.  27 to 135 (cell, vector)s: p = 4 46 -> 36 us a launch, p = 7 141 -> 82; 400 to 420: p = 4 72 ->
+// 59, p = 7 148 -> 120 (one pair a CTA in seven stages: 46, 138, 67 and 148).  Two single items an SM are
+// no faster than one pair; at the other orders half of the units saves nothing (p = 5 at 420: 109 -> 152).
+template <int NP> __host__ __device__ constexpr bool hx_single_items() { return NP == 5 || NP == 8; }
+
+// PER: (cell, vector)s of an item
+template <int NP, int NQ, bool KPT, int PER>
 __global__ void __launch_bounds__(kHxThreads, 1)
 hx_local_kernel(const __grid_constant__ LocalArgs a, const __grid_constant__ TablesEO<double, NP, NQ> tb) {
   constexpr int GT = cell_group_threads<NP, 4>(), NW = GT / 32;
@@ -306,6 +315,8 @@ hx_local_kernel(const __grid_constant__ LocalArgs a, const __grid_constant__ Tab
     if (PL) __syncwarp();
     else sync();
   };
+  // lane vectors of an item: unit u is lane vector u & lm of pencil u >> lb
+  constexpr int lb = PER, lm = 2 * PER - 1;
   const long long ngroups = (long long)gridDim.x * hx_groups<NP>();
   // a CTA's groups take items gridDim.x apart, so few items spread over the SMs
   const long long first = (long long)group * gridDim.x + blockIdx.x;
@@ -322,8 +333,8 @@ hx_local_kernel(const __grid_constant__ LocalArgs a, const __grid_constant__ Tab
       for (int k = 1; k < a.nsys; ++k)
         if (it >= a.sys[k].item0) r.q = k;
       const SysDesc& g = a.sys[r.q];
-      const long long li = 2 * (it - g.item0), n2 = (long long)g.mesh.E * g.nvec;
-      for (int i = 0; i < 2; ++i)
+      const long long li = PER * (it - g.item0), n2 = (long long)g.mesh.E * g.nvec;
+      for (int i = 0; i < PER; ++i)
         if (li + i < n2) {
           r.e[i] = (int)((li + i) / g.nvec);
           r.v[i] = (int)((li + i) - (long long)r.e[i] * g.nvec);
@@ -351,8 +362,8 @@ hx_local_kernel(const __grid_constant__ LocalArgs a, const __grid_constant__ Tab
   auto gather = [&](int n) {
     const HxItem it = rec(n);
     const SysDesc& g = a.sys[it.q];
-    for (int i = ut; i < 4 * NP * nz; i += US) {
-      const int w = i & 3, pen = i >> 2, sl = w >> 1;
+    for (int i = ut; i < (NP * nz) << lb; i += US) {
+      const int w = i & lm, pen = i >> lb, sl = w >> 1;
       const int y = pen % NP, z = z0 + pen / NP;
       const int* no = noff(n, sl);
       const bool have = (sl ? it.e[1] : it.e[0]) >= 0;
@@ -385,8 +396,8 @@ hx_local_kernel(const __grid_constant__ LocalArgs a, const __grid_constant__ Tab
     psync();
 
     // ---- x pencils: T1 = N'^T X, A = B_x X (in place), T2 = G_x X
-    for (int u = ut; u < 4 * NP * nz; u += US) {
-      const int w = u & 3, pen = u >> 2;
+    for (int u = ut; u < (NP * nz) << lb; u += US) {
+      const int w = u & lm, pen = u >> lb;
       const int y = pen % NP, z = z0 + pen / NP;
       double2 *A = Ab(w) + pa(0, y, z), *K = T2b(w) + pa(0, y, z), *Q = T1b(w) + pq(0, y, z);
       PartsD<NP> s;
@@ -410,8 +421,8 @@ hx_local_kernel(const __grid_constant__ LocalArgs a, const __grid_constant__ Tab
     psync();
 
     // ---- y pencils (in place): T1 = N'^T T1; T2 = G_y A + B_y T2
-    for (int u = ut; u < 4 * NQ * nz; u += US) {
-      double2* Q = T1b(u & 3) + pq((u >> 2) % NQ, 0, z0 + (u >> 2) / NQ);
+    for (int u = ut; u < (NQ * nz) << lb; u += US) {
+      double2* Q = T1b(u & lm) + pq((u >> lb) % NQ, 0, z0 + (u >> lb) / NQ);
       PartsD<NP> s;
       load_parts(s, [&](int j) { return Q[j * L::QY]; });
 #pragma unroll
@@ -421,8 +432,8 @@ hx_local_kernel(const __grid_constant__ LocalArgs a, const __grid_constant__ Tab
         put_rows<NQ>(i, r, [&](int k, double2 v) { Q[k * L::QY] = v; });
       }
     }
-    for (int u = (ut + US - 4 * NQ * nz % US) % US; u < 4 * NP * nz; u += US) {
-      const int w = u & 3, o = pa((u >> 2) % NP, 0, z0 + (u >> 2) / NP);
+    for (int u = (ut + US - ((NQ * nz) << lb) % US) % US; u < (NP * nz) << lb; u += US) {
+      const int w = u & lm, o = pa((u >> lb) % NP, 0, z0 + (u >> lb) / NP);
       const double2* A = Ab(w) + o;
       double2* K = T2b(w) + o;
       PartsD<NP> s1, s2;
@@ -444,13 +455,13 @@ hx_local_kernel(const __grid_constant__ LocalArgs a, const __grid_constant__ Tab
 
     // ---- z pencils (in place): T1 = N' F N'^T T1 + G'_z T1; the two spins of a pencil are on
     // neighbouring lanes and swap their values by shuffle
-    constexpr int UZ = 4 * NQ * NQ, ROUNDS = (UZ + GT - 1) / GT;
+    constexpr int UZ = (NQ * NQ) << lb;
 #pragma unroll 1
-    for (int rd = 0; rd < ROUNDS; ++rd) {
-      const int uu = tid + rd * GT;
+    for (int rd = 0; rd < UZ; rd += GT) {
+      const int uu = tid + rd;
       const bool act = uu < UZ;
       const int u = act ? uu : (uu & 1);
-      const int w = u & 3, x = (u >> 2) % NQ, y = (u >> 2) / NQ;
+      const int w = u & lm, x = (u >> lb) % NQ, y = (u >> lb) / NQ;
       double2* Q = T1b(w) + pq(x, y, 0);
       const int e = max(0, (w >> 1) ? item.e[1] : item.e[0]);
       const double2* __restrict__ fld = reinterpret_cast<const double2*>(d.fields) + 2 * (size_t)e * NQ3;
@@ -488,8 +499,8 @@ hx_local_kernel(const __grid_constant__ LocalArgs a, const __grid_constant__ Tab
       }
     }
     // T2 = B_z T2 (the threads left idle by the last round above take the first units)
-    for (int u = (tid + GT - UZ % GT) % GT; u < 4 * NP * NP; u += GT) {
-      double2* K = T2b(u & 3) + pa((u >> 2) % NP, (u >> 2) / NP, 0);
+    for (int u = (tid + GT - UZ % GT) % GT; u < (NP * NP) << lb; u += GT) {
+      double2* K = T2b(u & lm) + pa((u >> lb) % NP, (u >> lb) / NP, 0);
       PartsD<NP> s;
       load_parts(s, [&](int j) { return K[j * L::AZ]; });
 #pragma unroll
@@ -503,8 +514,8 @@ hx_local_kernel(const __grid_constant__ LocalArgs a, const __grid_constant__ Tab
     sync();
 
     // ---- y pencils (in place): T1 = N' T1
-    for (int u = ut; u < 4 * NQ * nz; u += US) {
-      double2* Q = T1b(u & 3) + pq((u >> 2) % NQ, 0, z0 + (u >> 2) / NQ);
+    for (int u = ut; u < (NQ * nz) << lb; u += US) {
+      double2* Q = T1b(u & lm) + pq((u >> lb) % NQ, 0, z0 + (u >> lb) / NQ);
       PartsD<NQ> s;
       load_parts(s, [&](int j) { return Q[j * L::QY]; });
 #pragma unroll
@@ -517,8 +528,8 @@ hx_local_kernel(const __grid_constant__ LocalArgs a, const __grid_constant__ Tab
     psync();
 
     // ---- x pencils: N' T1 + T2, assembled
-    for (int u = ut; u < 4 * NP * nz; u += US) {
-      const int w = u & 3, pen = u >> 2, sl = w >> 1, sp = w & 1;
+    for (int u = ut; u < (NP * nz) << lb; u += US) {
+      const int w = u & lm, pen = u >> lb, sl = w >> 1, sp = w & 1;
       const int y = pen % NP, z = z0 + pen / NP;
       const int e = sl ? item.e[1] : item.e[0], vec = sl ? item.v[1] : item.v[0];
       if (e < 0) continue;
@@ -551,6 +562,10 @@ cudaError_t launch_hx_group_p(const HxJob* jobs, int n, cudaStream_t s) {
   constexpr int NQ = NP + 1;   // nq = p + 2
   if (n < 1 || n > GBC_MAX_BATCH) return cudaErrorInvalidValue;
   LocalArgs a;
+  long long all = 0;
+  for (int i = 0; i < n; ++i) all += (long long)jobs[i].c->mesh.E * jobs[i].nvec;
+  const long long nsm = gbc_sm_count(), ones = (all + nsm - 1) / nsm, twos = (all + 2 * nsm - 1) / (2 * nsm);
+  const int per = hx_single_items<NP>() && ones <= 3 && ones < 2 * twos ? 1 : 2;
   long long item = 0;
   for (int i = 0; i < GBC_MAX_BATCH; ++i) {
     SysDesc& d = a.sys[i];
@@ -568,7 +583,7 @@ cudaError_t launch_hx_group_p(const HxJob* jobs, int n, cudaStream_t s) {
     d.nvec = jobs[i].nvec;
     d.item0 = item;
     d.mesh = c->mesh;
-    item += ((long long)c->mesh.E * d.nvec + 1) / 2;
+    item += ((long long)c->mesh.E * d.nvec + per - 1) / per;
   }
   a.nsys = n;
   a.nitems = item;
@@ -586,8 +601,10 @@ cudaError_t launch_hx_group_p(const HxJob* jobs, int n, cudaStream_t s) {
     kern<<<(unsigned)nblk, kHxThreads, smem, s>>>(a, tb);
     return cudaGetLastError();
   };
-  if (kpt) return run(hx_local_kernel<NP, NQ, true>);
-  return run(hx_local_kernel<NP, NQ, false>);
+  if constexpr (hx_single_items<NP>()) {
+    if (per == 1) return kpt ? run(hx_local_kernel<NP, NQ, true, 1>) : run(hx_local_kernel<NP, NQ, false, 1>);
+  }
+  return kpt ? run(hx_local_kernel<NP, NQ, true, 2>) : run(hx_local_kernel<NP, NQ, false, 2>);
 }
 
 // Deterministic assembly: Y[I][s][v] += the results of every cell holding node I, added

@@ -41,3 +41,22 @@ def test_fp64_cell_pairs(g, p, ncell, per, nvec, ldx):
         ctx.sync_status()
         got = Y[:, :, :nvec].cpu().numpy()
         assert np.linalg.norm(got - ref) <= 1e-12 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("p", [4, 7])
+def test_fp64_items_of_one_and_two(g, p):
+    """The numbers of (cell, vector)s at which the items of the cell apply change from one to two and
+    back: around 1, 2 and 3 for every SM, odd and even."""
+    sm = torch.cuda.get_device_properties(0).multi_processor_count
+    for n in (1, sm, sm + 1, 2 * sm, 2 * sm + 1, 3 * sm, 3 * sm + 1):
+        prob = syn.make_problem(ncell=(n, 1, 1), h=(0.9, 1.3, 1.1), p=p, periodic=(1, 1, 0),
+                                k=(0.1, 0.0, 0.0) if n % 2 else (0.0, 0.0, 0.0), seed=n)
+        X = syn.random_block(prob.nnodes, 1, 3)
+        ref = fe.Discretisation(prob).apply_h(X)
+        ctx = g.Context(0)
+        ctx.set_problem(prob)
+        Xd = torch.from_numpy(X).cuda()
+        Y = torch.empty_like(Xd)
+        ctx.apply_h(Xd, Y)
+        assert np.linalg.norm(Y.cpu().numpy() - ref) <= 1e-12 * np.linalg.norm(ref)
+        ctx.close()
