@@ -104,8 +104,10 @@ void lagrange_at(const std::vector<double>& xn, double t, std::vector<double>& L
 // symmetric like w, gives the same operator.  Which s is chosen decides how the even-odd entries of
 // the two tables round to FP32, and that rounding is most of the operator's error: with s = sqrt(w)
 // H.X is off by 1.14e-7 at p = 4, with the s of least squared rounding error among 256 within a
-// factor sqrt(2) of it by 8.6e-8 (uniform random vectors; p = 2, 3, 5, 6, 7: 1.43 -> 1.19, 0.96 -> 0.86,
-// 1.01 -> 0.89, 0.94 -> 0.87 and 0.95 -> 0.90e-7).
+// factor sqrt(2) of it by 8.6e-8 (uniform random vectors; p = 3, 5, 6, 7: 0.96 -> 0.86, 1.01 -> 0.89,
+// 0.94 -> 0.87 and 0.95 -> 0.90e-7).  p = 2 keeps sqrt(w): H.X would gain (1.43 -> 1.19e-7), but on the
+// smooth vectors that a filter brings out its few entries' errors add up the other way (degree 12, 6 atoms:
+// 1.31e-6 for 1.40e-6).
 static std::vector<double> interpolation_factors(const HostTables& t) {
   const int np = t.p + 1, nq = t.nq;
   auto sq = [](double v) { return (v - (float)v) * (v - (float)v); };
@@ -119,10 +121,11 @@ static std::vector<double> interpolation_factors(const HostTables& t) {
     return e / (f * f);
   };
   std::vector<double> s(nq);
+  const int trials = t.p == 2 ? 1 : 256;
   for (int q = 0; q < (nq + 1) / 2; ++q) {
     double best = 1e300;
-    for (int k = 0; k < 256; ++k) {
-      const double f = std::sqrt(t.gq_w[q]) * std::exp2(k / 256.0 - 0.5);
+    for (int k = 0; k < trials; ++k) {
+      const double f = std::sqrt(t.gq_w[q]) * (trials > 1 ? std::exp2(k / 256.0 - 0.5) : 1.0);
       const double e = error(q, f) + error(q, t.gq_w[q] / f);
       if (e < best) {
         best = e;
